@@ -1,0 +1,377 @@
+// k_depth.cu -- the depth order of the visible Gaussians (paper Sec. 3.1
+// 'Sorting') by one partition and one sort per bucket, and each Gaussian's
+// first pair slot.
+//
+// The order is (FP32 depth key, node id), i.e. (key, in-front index), and a
+// pair (key, index) is unique, so no step needs to be stable and none needs a
+// look-back chain:
+//  * preprocess counts the visible keys in DEPTH_BINS bins of a monotone
+//    function of the key (half of the bins logarithmic in z, half linear, over
+//    the depth range the scene's bounds allow: depth_bin);
+//  * k_depth_part scans the bins (every CTA for itself), joins neighbouring
+//    bins into buckets of about 2^q keys (bucket of a bin = its exclusive
+//    prefix >> q, so no bucket holds more than 2^q + its largest bin), and
+//    writes each (key, index << 8 | slot count) to its bucket, at a place
+//    reserved with one atomic per CTA and bucket; the same atomic adds up the
+//    bucket's candidate slots;
+//  * k_depth_local gives each bucket to one CTA: a counting sort by 4096
+//    sub-bins of the bucket's own key range in shared memory leaves runs of
+//    one or two keys, whose members rank themselves by (key, index); a bucket
+//    with a long run (many equal keys) is sorted by a bitonic network instead.
+//    The slot counts travel with the keys, so the CTA also writes the first
+//    slot of each of its Gaussians (the sum of the earlier buckets' slots plus
+//    a scan of its own).
+// Four stable radix passes and a scan of the slot counts did this before; each
+// pass was a chain of look-back round trips (15-21 us for 550K keys whatever
+// the traffic).  Depth order and slots, 1M-leaf box at 1080p (552K visible):
+// 96 -> 29 us; city at 1080p (2.67M visible): 153 -> 79 us.  Bound now by the
+// shared-memory atomics and barriers of a CTA's steps (issue slots 35-45 %).
+// A bucket that does not fit a CTA (F_SORT_SKEW: thousands of Gaussians in one
+// bin) makes the host replay the frame with the radix passes of k_sort.cu.
+#include "vgr_internal.cuh"
+#include "vgr_launch.h"
+
+namespace vgr {
+
+constexpr int DP_THREADS = 512;
+constexpr int DP_ITEMS = 16;
+constexpr int DP_TILE = DP_THREADS * DP_ITEMS;  // entries a CTA partitions at a time
+constexpr int DP_BPT = DEPTH_BINS / DP_THREADS;  // bins per thread
+constexpr uint32_t DP_Q_MIN = 8, DP_Q_MAX = 11;
+constexpr uint32_t DP_BUCKETS = 320;             // buckets aimed at while they stay below 2^DP_Q_MAX keys
+static_assert(DP_BPT % 4 == 0, "bins are read as uint4");
+
+constexpr int DL_THREADS = 512;
+constexpr int DL_WARPS = DL_THREADS / 32;
+constexpr uint32_t DL_CAP = 8192;       // keys of a bucket sorted in shared memory
+constexpr int DL_ITEMS = DL_CAP / DL_THREADS;
+constexpr uint32_t DL_SUB_BITS = 12, DL_SUB = 1u << DL_SUB_BITS;
+constexpr uint32_t DL_RUN_MAX = 48;     // longest run ranked by comparing its members
+constexpr int DL_SPT = DL_SUB / DL_THREADS;
+
+// log2 of the bucket size for n keys, and the number of bucket ids it makes
+__host__ __device__ inline uint32_t depth_q(uint32_t n) {
+    uint32_t q = DP_Q_MIN;
+    while (q < DP_Q_MAX && (n >> q) > DP_BUCKETS) ++q;
+    return q;
+}
+__host__ __device__ inline uint32_t depth_buckets(uint32_t n) { return (n >> depth_q(n)) + 1u; }
+
+uint32_t depth_bucket_cap(uint32_t cap_vis) {
+    const uint32_t a = DP_BUCKETS + 2u, b = (cap_vis >> DP_Q_MAX) + 2u;
+    return a > b ? a : b;
+}
+
+__global__ void __launch_bounds__(DP_THREADS, 2) k_depth_part(const uint32_t* __restrict__ depth,
+                                                              const uint32_t* __restrict__ ntile, uint32_t cap,
+                                                              const uint32_t* __restrict__ bins,
+                                                              uint32_t* __restrict__ bstart,
+                                                              unsigned long long* __restrict__ cursor,
+                                                              uint2* __restrict__ part, uint32_t cap_buckets,
+                                                              Counters* __restrict__ ctr,
+                                                              const FrameParams* __restrict__ fp) {
+    pdl_wait();
+    extern __shared__ uint32_t sm[];
+    uint16_t* s_bucket = reinterpret_cast<uint16_t*>(sm);  // [DEPTH_BINS] bucket of each bin
+    uint32_t* s_start = sm + DEPTH_BINS / 2;               // [nb + 1] first position of each bucket
+    uint32_t* s_base = s_start + cap_buckets + 1;          // [nb] keys of this tile, then their first position
+    uint32_t* s_slot = s_base + cap_buckets;               // [nb] candidate slots of this tile
+    __shared__ uint32_t s_scan[DP_THREADS / 32 + 1];
+    __shared__ uint32_t s_last[DP_THREADS];
+    const uint32_t t = threadIdx.x;
+    const uint32_t n = min(ctr->n_front, cap);
+    // contiguous chunks, whole rows of DP_THREADS entries
+    uint32_t chunk = (n + gridDim.x - 1) / gridDim.x;
+    chunk = max((chunk + DP_THREADS - 1) / DP_THREADS, 2u) * DP_THREADS;
+    const uint32_t first = blockIdx.x * chunk;
+    if (blockIdx.x == 0 && t == 0 && ctr->n_front > MAX_RANKS) atomicOr(&ctr->flags, F_OVF_VIS);
+    if (blockIdx.x != 0 && first >= n) return;
+    const uint32_t end = min(first + chunk, n);
+    const DepthMap map = fp->depth;
+    uint32_t key[DP_ITEMS];  // the first tile's keys are in flight during the scan of the bins
+#pragma unroll
+    for (int k = 0; k < DP_ITEMS; ++k) {
+        const uint32_t i = first + k * DP_THREADS + t;
+        key[k] = i < end ? depth[i] : NONE;
+    }
+    uint32_t total, nb;
+    {
+        uint32_t c[DP_BPT];
+#pragma unroll
+        for (int k = 0; k < DP_BPT / 4; ++k) {
+            const uint4 v = reinterpret_cast<const uint4*>(bins)[t * (DP_BPT / 4) + k];
+            c[4 * k] = v.x; c[4 * k + 1] = v.y; c[4 * k + 2] = v.z; c[4 * k + 3] = v.w;
+        }
+        uint32_t sum = 0;
+#pragma unroll
+        for (int k = 0; k < DP_BPT; ++k) sum += c[k];
+        s_last[t] = c[DP_BPT - 1];
+        uint32_t pre = block_excl_scan<DP_THREADS / 32>(sum, s_scan, &total);
+        const uint32_t q = depth_q(total);
+        nb = min((total >> q) + 1u, cap_buckets);
+        // bucket ids above the previous bin's start at this bin
+        uint32_t id = t == 0 ? NONE : (pre - s_last[t - 1]) >> q;  // NONE + 1 == 0
+#pragma unroll
+        for (int k = 0; k < DP_BPT; ++k) {
+            const uint32_t b = min(pre >> q, nb - 1u);
+            s_bucket[t * DP_BPT + k] = (uint16_t)b;
+            while (id != b) s_start[++id] = pre;
+            pre += c[k];
+        }
+        if (t == DP_THREADS - 1)
+            while (id != nb) s_start[++id] = total;
+    }
+    for (uint32_t b = t; b < nb; b += DP_THREADS) s_base[b] = s_slot[b] = 0u;
+    __syncthreads();
+    if (blockIdx.x == 0) {
+        bool skew = false;
+        for (uint32_t b = t; b <= nb; b += DP_THREADS) {
+            bstart[b] = s_start[b];
+            skew = skew || (b < nb && s_start[b + 1] - s_start[b] > DL_CAP);
+        }
+        if (skew) atomicOr(&ctr->flags, F_SORT_SKEW);
+    }
+    for (uint32_t base = first;;) {
+        uint32_t at[DP_ITEMS];         // bucket << 13 | place in this tile's share of it
+        uint32_t cnt[DP_ITEMS / 4];    // slot counts, saturated at 255
+#pragma unroll
+        for (int k = 0; k < DP_ITEMS / 4; ++k) cnt[k] = 0u;
+#pragma unroll
+        for (int k = 0; k < DP_ITEMS; ++k) {
+            const uint32_t i = base + k * DP_THREADS + t;
+            at[k] = NONE;
+            if (i < end && key[k] != NONE) {  // culled entries carry all ones
+                const uint32_t b = s_bucket[depth_bin(map, key[k])];
+                const uint32_t c = ntile[i];
+                at[k] = (b << 13) | atomicAdd(&s_base[b], 1u);
+                atomicAdd(&s_slot[b], c);
+                cnt[k / 4] |= min(c, 255u) << (8 * (k % 4));
+            }
+        }
+        __syncthreads();
+        for (uint32_t b = t; b < nb; b += DP_THREADS) {
+            const uint32_t c = s_base[b];
+            if (c) {
+                const unsigned long long add = (unsigned long long)s_slot[b] << 32 | c;
+                s_base[b] = s_start[b] + (uint32_t)atomicAdd(&cursor[b], add);
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < DP_ITEMS; ++k) {
+            if (at[k] != NONE) {
+                const uint32_t i = base + k * DP_THREADS + t;
+                const uint32_t pos = s_base[at[k] >> 13] + (at[k] & 8191u);
+                part[pos] = make_uint2(key[k], (i << 8) | ((cnt[k / 4] >> (8 * (k % 4))) & 255u));
+            }
+        }
+        base += DP_TILE;
+        if (base >= end) break;
+        __syncthreads();
+        for (uint32_t b = t; b < nb; b += DP_THREADS) s_base[b] = s_slot[b] = 0u;
+#pragma unroll
+        for (int k = 0; k < DP_ITEMS; ++k) {
+            const uint32_t i = base + k * DP_THREADS + t;
+            key[k] = i < end ? depth[i] : NONE;
+        }
+        __syncthreads();
+    }
+}
+
+__device__ __forceinline__ unsigned long long warp_sum64(unsigned long long v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+    return v;
+}
+
+__global__ void __launch_bounds__(DL_THREADS, 2) k_depth_local(const uint2* __restrict__ part,
+                                                               const uint32_t* __restrict__ bstart,
+                                                               const unsigned long long* __restrict__ cursor,
+                                                               const uint32_t* __restrict__ ntile, uint32_t cap_vis,
+                                                               uint32_t* __restrict__ order,
+                                                               uint32_t* __restrict__ off, uint64_t cap_pairs,
+                                                               Counters* __restrict__ ctr) {
+    pdl_wait();
+    extern __shared__ uint2 s_kv[];                                  // [DL_CAP] the bucket, by sub-bin
+    uint32_t* s_sub = reinterpret_cast<uint32_t*>(s_kv + DL_CAP);    // [DL_SUB + 1] counts, then first places
+    uint32_t* s_fin = s_sub + DL_SUB + 1;                            // [DL_CAP] index << 8 | slots, in order
+    __shared__ uint32_t s_scan[DL_WARPS + 1];
+    __shared__ uint32_t s_min[DL_WARPS], s_max[DL_WARPS];
+    __shared__ unsigned long long s_sum[DL_WARPS];
+    const uint32_t t = threadIdx.x, lane = lane_id(), warp = t >> 5;
+    if (ctr->flags & F_SORT_SKEW) return;
+    const uint32_t n_vis = min(ctr->n_vis, cap_vis);
+    const uint32_t nb = depth_buckets(n_vis);
+    unsigned long long slots = 0ull;  // candidate slots of the buckets before b
+    uint32_t seen = 0;
+    for (uint32_t b = blockIdx.x; b < nb; b += gridDim.x) {
+        const uint32_t start = bstart[b], n = min(bstart[b + 1] - start, DL_CAP);
+        uint2 e[DL_ITEMS];
+        uint32_t lo = NONE, hi = 0u;
+#pragma unroll
+        for (int k = 0; k < DL_ITEMS; ++k) {
+            const uint32_t j = k * DL_THREADS + t;
+            if (j < n) {
+                e[k] = part[start + j];
+                lo = min(lo, e[k].x);
+                hi = max(hi, e[k].x);
+            }
+        }
+        unsigned long long sum = 0ull;
+        for (uint32_t p = seen + t; p < b; p += DL_THREADS) sum += cursor[p] >> 32;
+        seen = b;
+#pragma unroll
+        for (int k = 0; k < DL_SPT; ++k) s_sub[k * DL_THREADS + t] = 0u;
+        lo = __reduce_min_sync(0xFFFFFFFFu, lo);
+        hi = __reduce_max_sync(0xFFFFFFFFu, hi);
+        sum = warp_sum64(sum);
+        if (lane == 0) {
+            s_min[warp] = lo;
+            s_max[warp] = hi;
+            s_sum[warp] = sum;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int w = 0; w < DL_WARPS; ++w) {
+            lo = min(lo, s_min[w]);
+            hi = max(hi, s_max[w]);
+            slots += s_sum[w];
+        }
+        const uint32_t bits = n ? 32u - __clz(hi - lo) : 0u;  // __clz(0) is 32
+        const uint32_t sh = bits > DL_SUB_BITS ? bits - DL_SUB_BITS : 0u;
+        // counting sort by sub-bin, in any order within one
+        uint32_t place[DL_ITEMS];
+#pragma unroll
+        for (int k = 0; k < DL_ITEMS; ++k)
+            if (k * DL_THREADS + t < n) place[k] = atomicAdd(&s_sub[(e[k].x - lo) >> sh], 1u);
+        __syncthreads();
+        bool longrun = false;
+        {
+            uint32_t c[DL_SPT], s = 0, total;
+#pragma unroll
+            for (int k = 0; k < DL_SPT; ++k) {
+                c[k] = s_sub[DL_SPT * t + k];
+                longrun = longrun || c[k] > DL_RUN_MAX;
+                s += c[k];
+            }
+            uint32_t pre = block_excl_scan<DL_WARPS>(s, s_scan, &total);
+#pragma unroll
+            for (int k = 0; k < DL_SPT; ++k) {
+                s_sub[DL_SPT * t + k] = pre;
+                pre += c[k];
+            }
+            if (t == 0) s_sub[DL_SUB] = n;
+        }
+        longrun = __syncthreads_or(longrun);
+#pragma unroll
+        for (int k = 0; k < DL_ITEMS; ++k)
+            if (k * DL_THREADS + t < n) s_kv[s_sub[(e[k].x - lo) >> sh] + place[k]] = e[k];
+        if (!longrun) {
+            __syncthreads();
+            for (uint32_t j = t; j < n; j += DL_THREADS) {
+                const uint2 kv = s_kv[j];
+                const uint32_t sub = (kv.x - lo) >> sh;
+                const uint32_t r0 = s_sub[sub], r1 = s_sub[sub + 1];
+                uint32_t at = r0;
+                if (r1 - r0 > 1u)
+                    for (uint32_t r = r0; r < r1; ++r) {
+                        const uint2 o = s_kv[r];
+                        at += (o.x < kv.x || (o.x == kv.x && o.y < kv.y)) ? 1u : 0u;
+                    }
+                s_fin[at] = kv.y;
+            }
+        } else {
+            // many equal keys: a bitonic network over (key, index), padded with all ones
+            uint32_t p2 = 1;
+            while (p2 < n) p2 <<= 1;
+            for (uint32_t j = n + t; j < p2; j += DL_THREADS) s_kv[j] = make_uint2(NONE, NONE);
+            for (uint32_t k = 2; k <= p2; k <<= 1)
+                for (uint32_t d = k >> 1; d > 0; d >>= 1) {
+                    __syncthreads();
+                    for (uint32_t c = t; c < p2 / 2; c += DL_THREADS) {
+                        const uint32_t i = 2u * c - (c & (d - 1u)), j = i + d;
+                        const uint2 x = s_kv[i], y = s_kv[j];
+                        const bool gt = x.x > y.x || (x.x == y.x && x.y > y.y);
+                        if (gt == ((i & k) == 0u)) {
+                            s_kv[i] = y;
+                            s_kv[j] = x;
+                        }
+                    }
+                }
+            __syncthreads();
+            for (uint32_t j = t; j < n; j += DL_THREADS) s_fin[j] = s_kv[j].y;
+        }
+        __syncthreads();
+        // write the order and the first slots: warp w takes the rows of 32 from w R on
+        const uint32_t R = ((n + 31u) / 32u + DL_WARPS - 1u) / DL_WARPS;  // at most DL_ITEMS
+        uint32_t x[DL_ITEMS], carry = 0;
+#pragma unroll
+        for (int r = 0; r < DL_ITEMS; ++r) {
+            if (r < R) {
+                const uint32_t j = (warp * R + r) * 32u + lane;
+                uint32_t c = 0;
+                if (j < n) {
+                    const uint32_t v = s_fin[j];
+                    c = v & 255u;
+                    if (c == 255u) c = ntile[v >> 8];
+                }
+                uint32_t rowsum;
+                x[r] = carry + warp_excl_scan(c, &rowsum);
+                carry += rowsum;
+            }
+        }
+        if (lane == 0) s_scan[warp] = carry;
+        __syncthreads();
+        uint32_t mine = (uint32_t)slots, all = 0;
+#pragma unroll
+        for (int w = 0; w < DL_WARPS; ++w) {
+            const uint32_t v = s_scan[w];
+            mine += (uint32_t)w < warp ? v : 0u;
+            all += v;
+        }
+#pragma unroll
+        for (int r = 0; r < DL_ITEMS; ++r) {
+            if (r < R) {
+                const uint32_t j = (warp * R + r) * 32u + lane;
+                if (j < n) {
+                    order[start + j] = s_fin[j] >> 8;
+                    off[start + j] = mine + x[r];
+                }
+            }
+        }
+        if (b == nb - 1u && t == 0) {
+            const unsigned long long ns = slots + all;
+            off[n_vis] = (uint32_t)ns;
+            ctr->n_cand = ns;
+            if (ns > cap_pairs) atomicOr(&ctr->flags, F_OVF_PAIRS);
+        }
+        __syncthreads();  // the shared buffers are rewritten by the next bucket
+    }
+}
+
+size_t depth_local_smem() { return DL_CAP * sizeof(uint2) + (DL_SUB + 1 + DL_CAP) * sizeof(uint32_t); }
+size_t depth_part_smem(uint32_t cap_buckets) {
+    return DEPTH_BINS * sizeof(uint16_t) + (3 * (size_t)cap_buckets + 1) * sizeof(uint32_t);
+}
+
+cudaError_t depth_sort_init() {
+    cudaError_t e = cudaFuncSetAttribute(k_depth_local, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)depth_local_smem());
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_depth_part, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)depth_part_smem(depth_bucket_cap(MAX_RANKS)));
+    return e;
+}
+
+void launch_depth_sort(const VisBuffers& vis, uint32_t cap_vis, const uint32_t* bins, uint32_t* bstart,
+                       unsigned long long* cursor, uint2* part, uint32_t* order, uint32_t* slot_off,
+                       uint64_t cap_pairs, Counters* ctr, const FrameParams* fp, int sms, cudaStream_t s) {
+    const uint32_t cap = cap_vis < MAX_RANKS ? cap_vis : MAX_RANKS;
+    const uint32_t cb = depth_bucket_cap(cap);
+    launch_ks(k_depth_part, 2 * sms, DP_THREADS, depth_part_smem(cb), s, (const uint32_t*)vis.depth,
+              (const uint32_t*)vis.ntile, cap, bins, bstart, cursor, part, cb, ctr, fp);
+    launch_ks(k_depth_local, 2 * sms, DL_THREADS, depth_local_smem(), s, (const uint2*)part, (const uint32_t*)bstart,
+              (const unsigned long long*)cursor, (const uint32_t*)vis.ntile, cap, order, slot_off, cap_pairs, ctr);
+}
+
+}  // namespace vgr

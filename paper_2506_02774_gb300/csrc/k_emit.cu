@@ -234,12 +234,16 @@ __global__ void __launch_bounds__(EM_THREADS, 4) k_emit(const uint32_t* __restri
     }
 }
 
-void launch_emit(const uint32_t* order, uint32_t cap_vis, VisBuffers vis, uint32_t* slot_off, uint32_t* pair_key,
-                 uint32_t* pair_val, uint64_t cap_pairs, int tile_passes, uint32_t sentinel,
-                 unsigned long long* status, Counters* ctr, const FrameParams* fp, int grid_scan, int grid,
-                 cudaStream_t s) {
-    launch_k(k_slot_scan, grid_scan, SS_THREADS, s, order, cap_vis, (const uint32_t*)vis.ntile, slot_off, cap_pairs,
+void launch_slot_scan(const uint32_t* order, uint32_t cap_vis, const VisBuffers& vis, uint32_t* slot_off,
+                      uint64_t cap_pairs, unsigned long long* status, Counters* ctr, const FrameParams* fp, int grid,
+                      cudaStream_t s) {
+    launch_k(k_slot_scan, grid, SS_THREADS, s, order, cap_vis, (const uint32_t*)vis.ntile, slot_off, cap_pairs,
              status, ctr, fp);
+}
+
+void launch_emit(const uint32_t* order, uint32_t cap_vis, VisBuffers vis, uint32_t* slot_off, uint32_t* pair_key,
+                 uint32_t* pair_val, uint64_t cap_pairs, int tile_passes, uint32_t sentinel, Counters* ctr,
+                 const FrameParams* fp, int grid, cudaStream_t s) {
     launch_k(k_emit, grid, EM_THREADS, s, order, cap_vis, vis, (const uint32_t*)slot_off, pair_key, pair_val, cap_pairs,
              tile_passes, sentinel, ctr, fp);
 }

@@ -5,8 +5,10 @@
 // One thread per cut node in front of the near plane (the LoD stage lists
 // them, in ascending node id), dense and barrier-free: every entry's record
 // is written at its own index, and a culled entry gets the depth key
-// 0xFFFFFFFF.  The stable depth sort then puts the visible Gaussians first,
-// ordered by (depth key, node id), with no compaction pass at all.
+// 0xFFFFFFFF.  The depth sort then orders the visible Gaussians by (depth key,
+// node id), with no compaction pass at all; the histogram that its partition
+// needs (visible keys per depth bin) is counted here, one shared-memory atomic
+// per visible entry.
 //
 // Per node: p = R (mu - C); depth key = FP32 bits of
 // ((R20 dx + R21 dy) + R22 dz) with single-rounded operations; culled when
@@ -128,13 +130,15 @@ template <int DEG, int STORE, bool INTERP>
 __global__ void __launch_bounds__(PRE_THREADS, 2) k_preprocess(SceneDev sc, const uint32_t* __restrict__ front,
                                                             const uint32_t* __restrict__ n_front_p, uint32_t cap,
                                                             const FrameParams* __restrict__ fp, VisBuffers vis,
-                                                            Counters* __restrict__ ctr) {
+                                                            Counters* __restrict__ ctr,
+                                                            uint32_t* __restrict__ depth_bins) {
     pdl_wait();
     constexpr int K = (DEG + 1) * (DEG + 1);  // SH coefficients per channel
     constexpr int NSH = ((3 * K + 7) / 8) * 8;
-    __shared__ uint32_t s_hist[4][256];  // digit histograms of the depth keys (the sort's passes)
-    for (int i = threadIdx.x; i < 4 * 256; i += blockDim.x) (&s_hist[0][0])[i] = 0u;
+    __shared__ uint32_t s_bins[DEPTH_BINS];  // visible keys per depth bin (k_depth.cu)
+    for (int i = threadIdx.x; i < DEPTH_BINS; i += PRE_THREADS) s_bins[i] = 0u;
     __syncthreads();
+    const DepthMap dmap = fp->depth;
     const uint32_t n_front = min(*n_front_p, cap);
     const float R0 = fp->R[0], R1 = fp->R[1], R2 = fp->R[2], R3 = fp->R[3], R4 = fp->R[4], R5 = fp->R[5];
     const float R6 = fp->R[6], R7 = fp->R[7], R8 = fp->R[8];
@@ -278,13 +282,7 @@ __global__ void __launch_bounds__(PRE_THREADS, 2) k_preprocess(SceneDev sc, cons
             }
         }
         n_visible += __popc(__ballot_sync(0xFFFFFFFFu, v));
-        // one shared-memory atomic per digit: equal digits within the warp (the
-        // high bytes of neighbouring nodes' depths) are combined by the hardware,
-        // cheaper than finding the peers first
-        if (i < n_front) {
-#pragma unroll
-            for (int p = 0; p < 4; ++p) atomicAdd(&s_hist[p][(zbits >> (8 * p)) & 255u], 1u);
-        }
+        if (v) atomicAdd(&s_bins[depth_bin(dmap, zbits)], 1u);
         if (i < n_front) {
             vis.depth[i] = zbits;  // culled: all ones, sorted behind every visible key
             vis.ntile[i] = v ? (uint32_t)(tx1 - tx0 + 1) * (uint32_t)(ty1 - ty0 + 1) : 0u;
@@ -296,9 +294,9 @@ __global__ void __launch_bounds__(PRE_THREADS, 2) k_preprocess(SceneDev sc, cons
     }
     if (lane_id() == 0 && n_visible) atomicAdd(&ctr->n_vis, n_visible);
     __syncthreads();
-    for (int i = threadIdx.x; i < 4 * 256; i += blockDim.x) {
-        const uint32_t c = (&s_hist[0][0])[i];
-        if (c) atomicAdd(&ctr->depth_hist[0][0] + i, c);
+    for (int i = threadIdx.x; i < DEPTH_BINS; i += PRE_THREADS) {
+        const uint32_t c = s_bins[i];
+        if (c) atomicAdd(&depth_bins[i], c);
     }
 }
 
@@ -320,10 +318,11 @@ void prepare_scene_half(float4* covB, uint32_t n, cudaStream_t s) {
 }
 
 void launch_preprocess(const SceneDev& sc, const uint32_t* front, const uint32_t* n_front, uint32_t cap,
-                       const FrameParams* fp, VisBuffers vis, Counters* ctr, bool interp, int grid, cudaStream_t s) {
+                       const FrameParams* fp, VisBuffers vis, Counters* ctr, uint32_t* depth_bins, bool interp,
+                       int grid, cudaStream_t s) {
     const bool half = sc.storage == VGR_STORE_HALF;
 #define VGR_PRE_LAUNCH(D, ST, IN) \
-    launch_k(k_preprocess<D, ST, IN>, grid, PRE_THREADS, s, sc, front, n_front, cap, fp, vis, ctr)
+    launch_k(k_preprocess<D, ST, IN>, grid, PRE_THREADS, s, sc, front, n_front, cap, fp, vis, ctr, depth_bins)
 #define VGR_PRE_CASE(D)                                            \
     case D:                                                        \
         if (interp) {                                              \

@@ -1,7 +1,8 @@
 // vgr_capi.cu -- the C ABI (include/vgr.h): hierarchy upload and validation,
 // per-view buffers, and the per-frame launch sequence
 //   LoD (temporal update or top-down levels) -> cut compaction ->
-//   preprocess (with colour) -> depth sort -> emission -> tile sort (its last
+//   preprocess (with colour) -> depth partition and buckets (or radix passes
+//   when a bucket would not fit) -> emission -> tile sort (its last
 //   pass records the tile ranges) -> blend order -> blend
 // all enqueued on the view's stream (or replayed as one captured graph).
 // Counts stay on the device (every kernel reads its element count from
@@ -111,6 +112,7 @@ struct vgr_hierarchy {
     void* sh = nullptr;
     uint32_t n_nodes = 0, max_depth = 0;
     uint64_t bytes = 0;
+    float mean_lo[3] = {0.f, 0.f, 0.f}, mean_hi[3] = {0.f, 0.f, 0.f};  // bounds of the node centres
     int device = 0;
     int num_sms = 0;
 };
@@ -120,6 +122,7 @@ struct PendingFrame {
     vgr_camera cam{};
     float tau = 0.f, f = 0.f, t = 0.f, k = 0.f;
     bool scratch = false;
+    bool radix_depth = false;   // depth order by radix passes instead of the partition
     int tile_passes = 1;
     uint32_t kernels = 0;
     float* host = nullptr;
@@ -146,8 +149,14 @@ struct vgr_view {
     uint32_t n_words = 0;
     uint32_t* frontier[2] = {nullptr, nullptr};
     VisBuffers vis{};
-    uint32_t* sortK[2] = {nullptr, nullptr};
-    uint32_t* sortV[2] = {nullptr, nullptr};
+    // depth sort: the partition's (key, value) pairs fill all of sort_kv; the
+    // radix passes use its halves as their key buffers
+    uint32_t* sort_kv = nullptr;
+    uint32_t* sortV[2] = {nullptr, nullptr};  // sortV[1] receives the order
+    uint32_t* depth_bins = nullptr;           // [DEPTH_BINS], after the counters (one clear per frame)
+    unsigned long long* bucket_cursor = nullptr;  // [depth_bucket_cap], after the bins
+    uint32_t* bucket_start = nullptr;
+    int radix_frames = 0;  // frames left that order depths by radix passes (a bucket did not fit)
     uint32_t* slot_off = nullptr;  // first pair slot of each visible Gaussian by depth rank (cap_vis + 1)
     uint32_t* pairK[2] = {nullptr, nullptr};
     uint32_t* pairV[2] = {nullptr, nullptr};
@@ -190,7 +199,7 @@ struct vgr_view {
     // grid, and the per-frame values travel through fp_host (read by the
     // captured host-to-device copy at replay), so a graph stays valid until a
     // buffer is reallocated or the tile grid changes
-    cudaGraphExec_t graph[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
+    cudaGraphExec_t graph[2][2][2] = {};  // [radix depth order?][top-down cut?][buffer parity]
     uint32_t graph_tiles = 0;
     // frame in flight between submit and finish
     bool pending = false;
@@ -260,8 +269,13 @@ vgr_status vgr_load_hierarchy(const vgr_scene_desc* d, vgr_hierarchy** out) {
     }
     if (expect != N) return fail(VGR_E_INVALID, "not every node is reachable from the root (%llu of %u)",
                                  (unsigned long long)expect, N);
+    float lo[3] = {d->mean[0], d->mean[1], d->mean[2]}, hi[3] = {lo[0], lo[1], lo[2]};
     for (uint32_t n = 0; n < N; ++n) {
         const float* m = d->mean + 3 * (size_t)n;
+        for (int a = 0; a < 3; ++a) {
+            lo[a] = std::min(lo[a], m[a]);
+            hi[a] = std::max(hi[a], m[a]);
+        }
         if (!std::isfinite(m[0]) || !std::isfinite(m[1]) || !std::isfinite(m[2]))
             return fail(VGR_E_INVALID, "mean of node %u is not finite", n);
         const float op = d->opacity[n];
@@ -305,6 +319,10 @@ vgr_status vgr_load_hierarchy(const vgr_scene_desc* d, vgr_hierarchy** out) {
     h->max_depth = maxd;
     h->device = dev;
     h->num_sms = prop.multiProcessorCount;
+    for (int a = 0; a < 3; ++a) {
+        h->mean_lo[a] = lo[a];
+        h->mean_hi[a] = hi[a];
+    }
     const uint32_t K3 = 3u * (d->sh_degree + 1) * (d->sh_degree + 1);
     const bool half = d->storage == VGR_STORE_HALF;
     const uint32_t stride = half ? (K3 + 7u) / 8u * 8u : (K3 + 3u) / 4u * 4u;
@@ -510,13 +528,14 @@ std::mutex g_batch_mu;
 std::vector<BatchGraph> g_batches;
 uint64_t g_batch_clock = 0;
 constexpr size_t BATCH_GRAPHS_KEPT = 8;
+constexpr size_t BATCH_KEY_FIELDS = 7;  // per view, after the number of chains
 std::atomic<uint32_t> g_batch_chains{0};  // parallel chains of a captured batch (0: one per view)
 
 void forget_batches(uint64_t uid) {
     std::lock_guard<std::mutex> lk(g_batch_mu);
     for (size_t i = 0; i < g_batches.size();) {
         bool hit = false;
-        for (size_t k = 0; k < g_batches[i].key.size(); k += 6)
+        for (size_t k = 1; k < g_batches[i].key.size(); k += BATCH_KEY_FIELDS)
             if (g_batches[i].key[k] == uid) hit = true;
         if (hit) {
             destroy_batch(g_batches[i]);
@@ -528,9 +547,10 @@ void forget_batches(uint64_t uid) {
 }
 
 void drop_graphs(vgr_view* v) {
-    for (auto& row : v->graph)
-        for (auto& g : row)
-            if (g) { cudaGraphExecDestroy(g); g = nullptr; }
+    for (auto& mode : v->graph)
+        for (auto& row : mode)
+            for (auto& g : row)
+                if (g) { cudaGraphExecDestroy(g); g = nullptr; }
     ++v->gen;  // batch graphs holding this view's buffers no longer match
 }
 
@@ -538,7 +558,8 @@ void free_vis(vgr_view* v) {
     drop_graphs(v);
     dfree(v->vis.depth); dfree(v->vis.ntile); dfree(v->vis.rect);
     dfree(v->vis.recA); dfree(v->vis.recB); dfree(v->vis.rgb); dfree(v->vis.lw);
-    for (int i = 0; i < 2; ++i) { dfree(v->sortK[i]); dfree(v->sortV[i]); }
+    dfree(v->sort_kv);
+    for (int i = 0; i < 2; ++i) dfree(v->sortV[i]);
     dfree(v->slot_off);
     v->vis_bytes = 0;
 }
@@ -551,8 +572,7 @@ vgr_status alloc_vis(vgr_view* v, uint32_t cap) {
         (s = dalloc(&v->vis.ntile, cap, &b)) || (s = dalloc(&v->vis.rect, cap, &b)) ||
         (s = dalloc(&v->vis.recA, cap, &b)) || (s = dalloc(&v->vis.recB, cap, &b)) ||
         (s = dalloc(&v->vis.rgb, cap, &b)) || (s = dalloc(&v->vis.lw, cap, &b)) ||
-        (s = dalloc(&v->sortK[0], cap, &b)) ||
-        (s = dalloc(&v->sortK[1], cap, &b)) || (s = dalloc(&v->sortV[0], cap, &b)) ||
+        (s = dalloc(&v->sort_kv, 2 * (size_t)cap, &b)) || (s = dalloc(&v->sortV[0], cap, &b)) ||
         (s = dalloc(&v->sortV[1], cap, &b)) || (s = dalloc(&v->slot_off, (size_t)cap + 1, &b))) {
         free_vis(v);
         return s;
@@ -621,6 +641,14 @@ vgr_status alloc_status(vgr_view* v) {
     return s;
 }
 
+// Bytes cleared at the start of a frame: the counters, the depth bins and the
+// cursors of the buckets that cap_vis entries can make.
+constexpr size_t CTR_BYTES = (sizeof(Counters) + 15) / 16 * 16;
+size_t cleared_bytes(uint32_t cap_vis) {
+    return CTR_BYTES + DEPTH_BINS * sizeof(uint32_t) +
+           depth_bucket_cap(std::min(cap_vis, MAX_RANKS)) * sizeof(unsigned long long);
+}
+
 uint32_t tile_of(const vgr_view* v) { return v->opts.tile_size ? v->opts.tile_size : TILE_DEFAULT; }
 uint32_t tiles_for(uint32_t W, uint32_t H, uint32_t T) { return ((W + T - 1) / T) * ((H + T - 1) / T); }
 
@@ -681,7 +709,7 @@ void destroy_view(vgr_view* v) {
     free_cut(v);
     dfree(v->bitmap); dfree(v->front_bm); dfree(v->frontier[0]); dfree(v->frontier[1]);
     dfree(v->ranges); dfree(v->tile_order); dfree(v->image); dfree(v->lut); dfree(v->status);
-    dfree(v->ctr); dfree(v->vstate); dfree(v->fp_dev);
+    dfree(v->ctr); dfree(v->bucket_start); dfree(v->vstate); dfree(v->fp_dev);
     if (v->fp_host) cudaFreeHost(v->fp_host);
     if (v->ctr_host) cudaFreeHost(v->ctr_host);
     if (v->vstate_host) cudaFreeHost(v->vstate_host);
@@ -767,7 +795,18 @@ vgr_status vgr_create_view(vgr_hierarchy* h, const vgr_view_opts* opts, vgr_view
     VGR_VTRY(dalloc(&v->front_bm, v->n_words, &v->fixed_bytes));
     VGR_VTRY(dalloc(&v->frontier[0], N, &v->fixed_bytes));
     VGR_VTRY(dalloc(&v->frontier[1], N, &v->fixed_bytes));
-    VGR_VTRY(dalloc(&v->ctr, 1, &v->fixed_bytes));
+    {  // the counters, the depth bins and the buckets' cursors: cleared together every frame
+        unsigned char* z = nullptr;
+        VGR_VTRY(dalloc(&z, cleared_bytes(MAX_RANKS), &v->fixed_bytes));
+        v->ctr = reinterpret_cast<Counters*>(z);
+        v->depth_bins = reinterpret_cast<uint32_t*>(z + CTR_BYTES);
+        v->bucket_cursor = reinterpret_cast<unsigned long long*>(z + CTR_BYTES + DEPTH_BINS * sizeof(uint32_t));
+    }
+    VGR_VTRY(dalloc(&v->bucket_start, depth_bucket_cap(MAX_RANKS) + 1, &v->fixed_bytes));
+    {
+        cudaError_t ce = depth_sort_init();
+        if (ce != cudaSuccess) { destroy_view(v); return fail(VGR_E_CUDA, "depth sort: %s", cudaGetErrorString(ce)); }
+    }
     VGR_VTRY(dalloc(&v->vstate, 1, &v->fixed_bytes));
     VGR_VTRY(dalloc(&v->fp_dev, 1, &v->fixed_bytes));
     VGR_VTRY(dalloc(&v->lut, 260, &v->fixed_bytes));
@@ -862,7 +901,7 @@ vgr_status vgr_view_bytes_estimate(const vgr_hierarchy* h, const vgr_view_opts* 
     const uint32_t T = o.tile_size ? o.tile_size : TILE_DEFAULT;
     const uint64_t tiles = (uint64_t)((width + T - 1) / T) * ((height + T - 1) / T);
     uint64_t b = 3 * 4 * cap_cut + per_vis * cap_vis + 4 * 4 * cap_pairs + 2 * 4 * n_words + 2 * 4 * N +
-                 sizeof(Counters) + sizeof(ViewState) + sizeof(FrameParams) + 260 * 4 + 8 * status_words;
+                 cleared_bytes(MAX_RANKS) + 4 * (depth_bucket_cap(MAX_RANKS) + 1) + sizeof(ViewState) + sizeof(FrameParams) + 260 * 4 + 8 * status_words;
     b += (uint64_t)width * height * 3 * 4 + tiles * (sizeof(uint2) + 4);
     *bytes = b;
     return VGR_OK;
@@ -891,10 +930,15 @@ int tile_passes_for(uint32_t n_tiles) {
 // 0.199 ms on the city against 0.221 at six CTAs per SM and 40 registers).
 constexpr int EMIT_GRID_NUM = 4;
 
-uint32_t frame_kernels(const vgr_view* v, bool scratch, int tile_passes) {
+// After a depth bucket did not fit a CTA, this many frames of the view order
+// their depths by radix passes before the partition is tried again.
+constexpr int RADIX_FRAMES = 64;
+
+uint32_t frame_kernels(const vgr_view* v, bool scratch, bool radix_depth, int tile_passes) {
     const uint32_t lod = scratch ? v->h->max_depth + 1u : 1u;
-    return lod + 1u /*compact*/ + 1u /*preprocess, with colour*/ + 4u /*depth passes*/ +
-           2u /*slot scan, emit*/ + (uint32_t)tile_passes + 1u /*tile order (finishes the ranges)*/ + 1u /*blend*/;
+    return lod + 1u /*compact*/ + 1u /*preprocess, with colour*/ +
+           (radix_depth ? 6u /*histogram, 4 passes, slot scan*/ : 2u /*partition, buckets*/) + 1u /*emit*/ +
+           (uint32_t)tile_passes + 1u /*tile order (finishes the ranges)*/ + 1u /*blend*/;
 }
 
 // The frame's status block and cut sizes, read back after its last kernel.
@@ -907,7 +951,7 @@ void frame_readback(vgr_view* v, cudaStream_t s) {
 // the frame stops before the blend, which a batch runs over all its views
 // (frame_readback then follows that blend).  Returns the number of kernels
 // launched.
-uint32_t enqueue_frame(vgr_view* v, bool scratch, int tile_passes, bool own_blend = true) {
+uint32_t enqueue_frame(vgr_view* v, bool scratch, bool radix_depth, int tile_passes, bool own_blend = true) {
     const SceneDev& sc = v->h->dev;
     cudaStream_t s = v->stream;
     const bool timing = v->opts.timing != 0;
@@ -915,7 +959,7 @@ uint32_t enqueue_frame(vgr_view* v, bool scratch, int tile_passes, bool own_blen
     const FrameParams& fh = *v->fp_host;
     const uint32_t n_tiles = fh.tiles_x * fh.tiles_y;
     cudaMemcpyAsync(v->fp_dev, v->fp_host, sizeof(FrameParams), cudaMemcpyHostToDevice, s);
-    cudaMemsetAsync(v->ctr, 0, sizeof(Counters), s);
+    cudaMemsetAsync(v->ctr, 0, cleared_bytes(v->cap_vis), s);
     cudaMemsetAsync(v->ranges, 0xFF, (size_t)n_tiles * sizeof(uint2), s);  // (start, ~end): both all ones
     // the first kernel waits for the copies above in plain stream order; with
     // stage events between the kernels none of them is launched early
@@ -936,26 +980,37 @@ uint32_t enqueue_frame(vgr_view* v, bool scratch, int tile_passes, bool own_blen
                        &v->vstate->n_cut[cur], v->status + v->st_compact, v->status + v->st_front, v->ctr, v->fp_dev,
                        v->grid_scan, s);
     mark(VGR_STAGE_PREPROCESS);
-    launch_preprocess(sc, v->front_list, &v->ctr->n_front, v->cap_cut, v->fp_dev, v->vis, v->ctr, fh.lod_interp != 0,
-                      v->grid_wide, s);
+    launch_preprocess(sc, v->front_list, &v->ctr->n_front, v->cap_cut, v->fp_dev, v->vis, v->ctr, v->depth_bins,
+                      fh.lod_interp != 0, std::min(v->grid_wide, 2 * v->h->num_sms), s);
     mark(VGR_STAGE_DEPTH_SORT);
-    // every potentially visible entry is sorted; culled ones carry the key
-    // 0xFFFFFFFF and land last (the digit histograms come from preprocess)
-    for (int p = 0; p < 4; ++p) {
-        const uint32_t* kin = p == 0 ? v->vis.depth : v->sortK[(p + 1) & 1];
-        const uint32_t* vin = p == 0 ? nullptr : v->sortV[(p + 1) & 1];
-        // the last pass writes only the permutation (the sorted keys are not read)
-        launch_radix_pass(kin, vin, p == 3 ? nullptr : v->sortK[p & 1], v->sortV[p & 1], &v->ctr->n_front, nullptr,
-                          v->cap_vis, 8 * p,
-                          v->ctr->depth_hist[p], v->status + v->st_depth + p * v->st_depth_stride,
-                          &v->ctr->tickets[TK_SORT0 + p], v->fp_dev, v->ctr, v->grid_scan, s, p == 3 ? 1 : 0);
+    uint32_t* order = v->sortV[1];
+    if (!radix_depth) {
+        launch_depth_sort(v->vis, v->cap_vis, v->depth_bins, v->bucket_start, v->bucket_cursor,
+                          reinterpret_cast<uint2*>(v->sort_kv), order, v->slot_off, v->cap_pairs, v->ctr, v->fp_dev,
+                          v->h->num_sms, s);
+    } else {
+        // every potentially visible entry is sorted; culled ones carry the key
+        // 0xFFFFFFFF and land last
+        uint32_t* const sortK[2] = {v->sort_kv, v->sort_kv + v->cap_vis};
+        launch_radix_hist(v->vis.depth, &v->ctr->n_front, nullptr, v->cap_vis, 4, &v->ctr->depth_hist[0][0],
+                          v->grid_scan, s);
+        for (int p = 0; p < 4; ++p) {
+            const uint32_t* kin = p == 0 ? v->vis.depth : sortK[(p + 1) & 1];
+            const uint32_t* vin = p == 0 ? nullptr : v->sortV[(p + 1) & 1];
+            // the last pass writes only the permutation (the sorted keys are not read)
+            launch_radix_pass(kin, vin, p == 3 ? nullptr : sortK[p & 1], v->sortV[p & 1], &v->ctr->n_front, nullptr,
+                              v->cap_vis, 8 * p,
+                              v->ctr->depth_hist[p], v->status + v->st_depth + p * v->st_depth_stride,
+                              &v->ctr->tickets[TK_SORT0 + p], v->fp_dev, v->ctr, v->grid_scan, s, p == 3 ? 1 : 0);
+        }
+        launch_slot_scan(order, v->cap_vis, v->vis, v->slot_off, v->cap_pairs, v->status + v->st_emit, v->ctr,
+                         v->fp_dev, v->grid_scan, s);
     }
-    const uint32_t* order = v->sortV[1];  // after 4 passes
     mark(VGR_STAGE_COLOR);  // (evaluated in preprocess: the stage is empty)
     mark(VGR_STAGE_EMIT);
     const uint32_t sentinel = (uint32_t)((1ull << (8 * tile_passes)) - 1ull);
     launch_emit(order, v->cap_vis, v->vis, v->slot_off, v->pairK[0], v->pairV[0], v->cap_pairs, tile_passes, sentinel,
-                v->status + v->st_emit, v->ctr, v->fp_dev, v->grid_scan, v->grid_scan * EMIT_GRID_NUM / 4, s);
+                v->ctr, v->fp_dev, v->grid_scan * EMIT_GRID_NUM / 4, s);
     mark(VGR_STAGE_TILE_SORT);
     // (the last pass also records each tile's range)
     for (int p = 0; p < tile_passes; ++p) {
@@ -968,22 +1023,23 @@ uint32_t enqueue_frame(vgr_view* v, bool scratch, int tile_passes, bool own_blen
     v->last_tile_buf = tile_passes & 1;
     mark(VGR_STAGE_RANGES);
     launch_tile_order(v->ranges, n_tiles, v->tile_order, v->ctr, s);
-    if (!own_blend) return frame_kernels(v, scratch, tile_passes) - 1u;  // a batch blend follows
+    if (!own_blend) return frame_kernels(v, scratch, radix_depth, tile_passes) - 1u;  // a batch blend follows
     mark(VGR_STAGE_BLEND);
     launch_blend(v->fp_dev, nullptr, v->tile_order, n_tiles, &v->ctr->blend_next,
                  v->h->num_sms * blend_ctas_per_sm(v->opts.filter, v->opts.exp_mode, v->opts.blend_depth, fh.tile),
                  v->opts.filter, v->opts.exp_mode, v->opts.blend_depth, fh.tile, s);
     mark(VGR_N_STAGES);
     frame_readback(v, s);
-    return frame_kernels(v, scratch, tile_passes);
+    return frame_kernels(v, scratch, radix_depth, tile_passes);
 }
 
 // One frame on the view's stream: the plain launch sequence, or (use_graph,
 // no stage timing) the replay of the captured sequence for this
 // (top-down?, parity) pair, captured on first use.
-vgr_status run_frame(vgr_view* v, bool scratch, int tile_passes, uint32_t n_tiles, uint32_t* kernels) {
+vgr_status run_frame(vgr_view* v, bool scratch, bool radix_depth, int tile_passes, uint32_t n_tiles,
+                     uint32_t* kernels) {
     if (!v->opts.use_graph || v->opts.timing) {
-        *kernels += enqueue_frame(v, scratch, tile_passes);
+        *kernels += enqueue_frame(v, scratch, radix_depth, tile_passes);
         VGR_CK(cudaGetLastError());
         return VGR_OK;
     }
@@ -991,10 +1047,10 @@ vgr_status run_frame(vgr_view* v, bool scratch, int tile_passes, uint32_t n_tile
         drop_graphs(v);
         v->graph_tiles = n_tiles;
     }
-    cudaGraphExec_t& ge = v->graph[scratch ? 1 : 0][v->parity];
+    cudaGraphExec_t& ge = v->graph[radix_depth ? 1 : 0][scratch ? 1 : 0][v->parity];
     if (!ge) {
         VGR_CK(cudaStreamBeginCapture(v->stream, cudaStreamCaptureModeThreadLocal));
-        enqueue_frame(v, scratch, tile_passes);
+        enqueue_frame(v, scratch, radix_depth, tile_passes);
         cudaGraph_t g = nullptr;
         cudaError_t e = cudaStreamEndCapture(v->stream, &g);
         if (e == cudaSuccess) e = cudaGetLastError();
@@ -1008,7 +1064,7 @@ vgr_status run_frame(vgr_view* v, bool scratch, int tile_passes, uint32_t n_tile
     }
     v->last_tile_buf = tile_passes & 1;
     VGR_CK(cudaGraphLaunch(ge, v->stream));
-    *kernels += frame_kernels(v, scratch, tile_passes);
+    *kernels += frame_kernels(v, scratch, radix_depth, tile_passes);
     return VGR_OK;
 }
 
@@ -1074,6 +1130,33 @@ void frustum_planes(const vgr_camera* cam, float guard, float out[5][4]) {
     }
 }
 
+// The bins of the depth partition: half of them logarithmic, half linear over
+// the depths that the camera can see of the box of the node centres.  Keys
+// outside (by rounding) fall in the first or last bin, so these bounds shape
+// the bins' balance, not the order.
+DepthMap depth_map(const vgr_hierarchy* h, const vgr_camera* cam) {
+    double zmin = INFINITY, zmax = -INFINITY;
+    for (int c = 0; c < 8; ++c) {
+        double z = 0.0;
+        for (int a = 0; a < 3; ++a)
+            z += (double)cam->R[6 + a] * ((double)((c >> a) & 1 ? h->mean_hi[a] : h->mean_lo[a]) - (double)cam->pos[a]);
+        zmin = std::min(zmin, z);
+        zmax = std::max(zmax, z);
+    }
+    DepthMap m;
+    const float lo = (float)std::min(std::max(zmin, (double)cam->z_near), 1e38);
+    const float hi = (float)std::min(std::max(zmax, 1.0001 * (double)lo), 3e38);
+    uint32_t klo, khi;
+    memcpy(&klo, &lo, 4);
+    memcpy(&khi, &hi, 4);
+    const float half = 0.5f * (float)DEPTH_BINS - 1.0f;
+    m.key_lo = klo;
+    m.z_lo = lo;
+    m.c_log = half / (float)std::max(khi - klo, 1u);
+    m.c_lin = std::min(std::max(half / std::max(hi - lo, 1e-38f), 1e-37f), 1e37f);
+    return m;
+}
+
 void fill_params(vgr_view* v, const vgr_camera* cam, float t, float k, float* host_dev, int tile_passes) {
     const uint32_t W = cam->width, H = cam->height;
     FrameParams& p = *v->fp_host;
@@ -1099,6 +1182,7 @@ void fill_params(vgr_view* v, const vgr_camera* cam, float t, float k, float* ho
     p.lod_frustum = v->opts.lod_frustum ? 1u : 0u;
     p.lod_interp = v->opts.lod_interp ? 1u : 0u;
     p.lod_t = t;
+    p.depth = depth_map(v->h, cam);
     if (p.lod_frustum) frustum_planes(cam, v->opts.lod_frustum_guard, p.frustum);
     // the blend's buffers: the tile sort's last pass leaves the pairs in
     // buffer (passes & 1)
@@ -1157,6 +1241,8 @@ vgr_status prepare_frame(vgr_view* v, const vgr_camera* cam, float tau, float* h
     q.t = t;
     q.k = k;
     q.scratch = !v->has_prev || !v->opts.temporal || tau != v->prev_tau || q.f != v->prev_f;
+    // (the withheld look-back word is the radix path's slot scan's)
+    q.radix_depth = v->radix_frames > 0 || (v->opts.test_hooks & (VGR_HOOK_WITHHOLD_LOOKBACK | VGR_HOOK_RADIX_DEPTH));
     q.host_dev = pipe ? nullptr : mapped_host(v, host_rgb);
     fill_params(v, cam, q.t, q.k, q.host_dev, q.tile_passes);
     return VGR_OK;
@@ -1185,8 +1271,8 @@ vgr_status submit_impl(vgr_view* v, const vgr_camera* cam, float tau, float* hos
     vgr_status s = prepare_frame(v, cam, tau, host_rgb, pipe);
     if (s != VGR_OK) return s;
     PendingFrame& q = v->pend;
-    if ((s = run_frame(v, q.scratch, q.tile_passes, tiles_for(q.cam.width, q.cam.height, tile_of(v)), &q.kernels)) !=
-        VGR_OK)
+    if ((s = run_frame(v, q.scratch, q.radix_depth, q.tile_passes, tiles_for(q.cam.width, q.cam.height, tile_of(v)),
+                       &q.kernels)) != VGR_OK)
         return s;
     return close_frame(v, v->stream);
 }
@@ -1250,14 +1336,14 @@ vgr_status launch_batch_graph(vgr_view* const* views, uint32_t n) {
     for (int i : chain_last)
         if (i >= 0) tail[i] = 1;
     std::vector<uint64_t> key;
-    key.reserve((size_t)n * 6 + 1);
+    key.reserve((size_t)n * BATCH_KEY_FIELDS + 1);
     key.push_back(k);
     for (uint32_t i = 0; i < n; ++i) {
         const vgr_view* v = views[i];
         const PendingFrame& q = v->pend;
         const uint64_t tiles = tiles_for(q.cam.width, q.cam.height, tile_of(v));
-        key.insert(key.end(), {v->uid, v->gen, (uint64_t)q.scratch, (uint64_t)v->parity, tiles,
-                               (uint64_t)q.tile_passes});
+        key.insert(key.end(), {v->uid, v->gen, (uint64_t)q.scratch, (uint64_t)q.radix_depth, (uint64_t)v->parity,
+                               tiles, (uint64_t)q.tile_passes});
     }
     const std::vector<uint32_t> sh = batch_blend_views(views, n);
     std::vector<char> shared(n, 0);
@@ -1307,7 +1393,7 @@ vgr_status launch_batch_graph(vgr_view* const* views, uint32_t n) {
             vgr_view* v = views[i];
             e = cudaStreamWaitEvent(v->stream, prev[i] < 0 ? bs.fork : views[prev[i]]->join_ev, 0);
             if (e != cudaSuccess) break;
-            enqueue_frame(v, v->pend.scratch, v->pend.tile_passes, !shared[i]);
+            enqueue_frame(v, v->pend.scratch, v->pend.radix_depth, v->pend.tile_passes, !shared[i]);
             e = cudaEventRecord(v->join_ev, v->stream);
             if (e == cudaSuccess && tail[i]) e = cudaStreamWaitEvent(bs.s, v->join_ev, 0);
         }
@@ -1355,7 +1441,8 @@ vgr_status launch_batch_graph(vgr_view* const* views, uint32_t n) {
     for (uint32_t i = 0; i < n; ++i) {
         vgr_view* v = views[i];
         v->last_tile_buf = v->pend.tile_passes & 1;
-        v->pend.kernels += frame_kernels(v, v->pend.scratch, v->pend.tile_passes) - (shared[i] ? 1u : 0u);
+        v->pend.kernels += frame_kernels(v, v->pend.scratch, v->pend.radix_depth, v->pend.tile_passes) -
+                           (shared[i] ? 1u : 0u);
         if (!sh.empty() && i == sh[0]) v->pend.kernels += 3u;  // class offsets, tile placement, the batch blend
         vgr_status s = close_frame(v, bs.s);
         if (s != VGR_OK) return s;
@@ -1411,12 +1498,16 @@ vgr_status finish_impl(vgr_view* v, vgr_frame* out) {
                 return s;
             }
             again = true;
+        } else if (flags & F_SORT_SKEW) {
+            v->radix_frames = RADIX_FRAMES;
+            q.radix_depth = true;
+            again = true;
         }
         if (!again) break;
         if (attempt >= 12) return fail(VGR_E_OVERFLOW, "frame did not settle after %d replays", attempt + 1);
         ++replays;
         fill_params(v, &q.cam, q.t, q.k, q.host_dev, q.tile_passes);
-        if ((s = run_frame(v, q.scratch, q.tile_passes, TW * TH, &q.kernels)) != VGR_OK) return s;
+        if ((s = run_frame(v, q.scratch, q.radix_depth, q.tile_passes, TW * TH, &q.kernels)) != VGR_OK) return s;
         if (q.host && !q.host_dev && !q.pipe)
             VGR_CK(cudaMemcpyAsync(q.host, v->cur_image, (size_t)W * H * 3 * sizeof(float), cudaMemcpyDeviceToHost,
                                    v->stream));
@@ -1433,6 +1524,7 @@ vgr_status finish_impl(vgr_view* v, vgr_frame* out) {
         v->img_sel ^= 1;
     }
     const int cur = v->parity ^ 1;
+    if (v->radix_frames > 0) --v->radix_frames;
     v->parity = cur;
     v->has_prev = true;
     v->prev_tau = q.tau;

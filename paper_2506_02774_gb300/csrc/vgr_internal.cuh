@@ -26,6 +26,7 @@ constexpr uint32_t CHILD_MASK = (1u << CHILD_SHIFT) - 1u;
 constexpr int RADIX_THREADS = 256;            // one radix-sort tile: 256 threads x 15 keys
 constexpr int RADIX_ITEMS = 15;
 constexpr int RADIX_TILE = RADIX_THREADS * RADIX_ITEMS;
+constexpr int DEPTH_BINS = 8192;              // bins of the depth keys' histogram (k_depth.cu)
 
 // flags in Counters::flags
 enum : uint32_t {
@@ -36,12 +37,22 @@ enum : uint32_t {
     F_OVF_VIS = 16u,       // more visible Gaussians than a pair value's 24-bit rank holds
     F_OVF_PAIRS = 32u,
     F_OVF_FRONTIER = 64u,
+    F_SORT_SKEW = 128u,    // a depth bucket too large for one CTA: redo the frame with the radix passes
 };
 
 // ticket slots (dynamic tile order for the chained scans)
 enum : int { TK_COMPACT = 0, TK_PRE = 1, TK_EMIT = 2, TK_SORT0 = 3 /* .. TK_SORT0 + 7 */, TK_COUNT = 12 };
 
 struct Counters;
+
+// Monotone map from depth keys to bins: half of the bins logarithmic in z
+// (the key's bits rise like log2 z), half linear, over the depths the scene's
+// bounds allow; keys outside go to the first or last bin.
+struct DepthMap {
+    uint32_t key_lo;   // bits of z_lo
+    float z_lo;
+    float c_log, c_lin;  // bins per unit of key and of z
+};
 
 // Per-frame parameters, uploaded once per frame (a graph replays them).
 struct FrameParams {
@@ -63,6 +74,7 @@ struct FrameParams {
     float* host_image;    // device-accessible pinned host image the blend also writes, or null
     uint32_t lod_frustum; // frustum-aware expansion on (needs node boxes)
     uint32_t lod_interp;  // parent-child weight interpolation on
+    DepthMap depth;       // bins of the depth partition
     float lod_t;          // fl(tau / f), the size ratio the interpolation weight is measured against
     // its planes: world normal w (xyz) and offset o (w), inside iff w.x - o >= 0 (read as float4)
     alignas(16) float frustum[5][4];
@@ -267,6 +279,15 @@ __device__ __forceinline__ uint32_t lookback_warp(unsigned long long* status, ui
 __device__ __forceinline__ float depth_key(float4 m, float R6, float R7, float R8, float Cx, float Cy, float Cz) {
     const float dx = __fsub_rn(m.x, Cx), dy = __fsub_rn(m.y, Cy), dz = __fsub_rn(m.z, Cz);
     return __fadd_rn(__fadd_rn(__fmul_rn(R6, dx), __fmul_rn(R7, dy)), __fmul_rn(R8, dz));
+}
+
+// The key's bin.  Every step is a correctly rounded monotone operation, so the
+// bin never falls as the key rises; single intrinsics give every kernel the
+// same bin.
+__device__ __forceinline__ uint32_t depth_bin(const DepthMap& m, uint32_t key) {
+    const float a = __fmul_rn(__uint2float_rn(key > m.key_lo ? key - m.key_lo : 0u), m.c_log);
+    const float b = __fmul_rn(fmaxf(__fsub_rn(__uint_as_float(key), m.z_lo), 0.f), m.c_lin);
+    return min(__float2uint_rz(__fadd_rn(a, b)), (uint32_t)DEPTH_BINS - 1u);
 }
 
 // The granularity test, single-rounded FP32 (no contraction): expand iff

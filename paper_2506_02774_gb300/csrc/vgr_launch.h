@@ -84,10 +84,20 @@ struct VisBuffers {
     float* lw;      // parent weight of the interpolated Gaussian (weight interpolation only)
 };
 void launch_preprocess(const SceneDev& sc, const uint32_t* front, const uint32_t* n_front, uint32_t cap,
-                       const FrameParams* fp, VisBuffers vis, Counters* ctr, bool interp, int grid, cudaStream_t s);
+                       const FrameParams* fp, VisBuffers vis, Counters* ctr, uint32_t* depth_bins, bool interp,
+                       int grid, cudaStream_t s);
 uint32_t preprocess_tile();
 void prepare_scene(float4* covB, uint32_t n, cudaStream_t s);
 void prepare_scene_half(float4* covB, uint32_t n, cudaStream_t s);
+
+// k_depth.cu
+// Depth order of the visible entries and their first pair slots: order[r] is
+// the in-front index of depth rank r, slot_off[r] its first slot (r <= n_vis).
+uint32_t depth_bucket_cap(uint32_t cap_vis);  // bucket ids a frame of cap_vis entries can have, plus one
+cudaError_t depth_sort_init();                // once per device: the kernels' shared-memory limits
+void launch_depth_sort(const VisBuffers& vis, uint32_t cap_vis, const uint32_t* bins, uint32_t* bstart,
+                       unsigned long long* cursor, uint2* part, uint32_t* order, uint32_t* slot_off,
+                       uint64_t cap_pairs, Counters* ctr, const FrameParams* fp, int sms, cudaStream_t s);
 
 // k_sort.cu
 uint32_t radix_tile();
@@ -100,11 +110,13 @@ void launch_radix_pass(const uint32_t* keys_in, const uint32_t* vals_in, uint32_
                        uint32_t n_ranges = 0);
 
 // k_emit.cu
-// k_slot_scan (slot offsets in depth order, into slot_off[cap_vis + 1]) then k_emit
+// slot offsets in depth order, into slot_off[cap_vis + 1], after a radix depth sort
+void launch_slot_scan(const uint32_t* order, uint32_t cap_vis, const VisBuffers& vis, uint32_t* slot_off,
+                      uint64_t cap_pairs, unsigned long long* status, Counters* ctr, const FrameParams* fp, int grid,
+                      cudaStream_t s);
 void launch_emit(const uint32_t* order, uint32_t cap_vis, VisBuffers vis, uint32_t* slot_off, uint32_t* pair_key,
                  uint32_t* pair_val, uint64_t cap_pairs, int tile_passes, uint32_t sentinel,
-                 unsigned long long* status, Counters* ctr, const FrameParams* fp, int grid_scan, int grid,
-                 cudaStream_t s);
+                 Counters* ctr, const FrameParams* fp, int grid, cudaStream_t s);
 uint32_t emit_tile();
 uint32_t slot_scan_tile();
 void launch_tile_order(uint2* ranges, uint32_t n_tiles, uint32_t* order, Counters* ctr, cudaStream_t s);
