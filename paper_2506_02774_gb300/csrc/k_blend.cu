@@ -84,8 +84,8 @@ constexpr float LOG2_ALPHA_MIN = -7.9943534368588578f;  // log2(1/255)
 // so the pixel need not look at the record.  The canonical mode (no Eq. 4
 // before Eq. 3) and 'full' mark every pixel.
 template <int MODE, int SR, int T>
-__device__ __forceinline__ uint32_t blend_prepare(float4& a, float4& b, float4& b2, float row0, float col0,
-                                                  bool full) {
+__device__ __forceinline__ uint32_t blend_prepare(float4& a, float4& b, float4& b2, float theta, float row0,
+                                                  float col0, bool full) {
     uint32_t pmask = 0xFFFFFFFFu;
     if (MODE != 1 && !full) {
         const uint32_t hw = __float_as_uint(b.w);
@@ -127,7 +127,7 @@ __device__ __forceinline__ uint32_t blend_prepare(float4& a, float4& b, float4& 
         if (SR == 2) b = make_float4(u, Ap, R[2 % (2 * SR)], R[3 % (2 * SR)]);
         return pmask;
     }
-    const float4 X = MODE == 0 ? make_float4(a.x, a.z * LOG2E, 0.f, 0.f) : make_float4(a.x, a.z, b.y, b.z);
+    const float4 X = MODE == 0 ? make_float4(a.x, a.z * LOG2E, 0.f, 0.f) : make_float4(a.x, a.z, b.y, theta);
     a = X;
     b = make_float4(R[0], R[1], SR > 1 ? R[2 % (2 * SR)] : 0.f, SR > 1 ? R[3 % (2 * SR)] : 0.f);
     if (SR > 2) b2 = make_float4(R[4 % (2 * SR)], R[5 % (2 * SR)], R[6 % (2 * SR)], R[7 % (2 * SR)]);
@@ -215,8 +215,7 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 // location occupy registers during the walk; and the warp's blend statistics.
 struct WarpItem {
     const uint32_t* pair_val;
-    const float4* recA;
-    const float4* recB;
+    const float4* rec;
     const float4* rgb;
     float* image;
     float* host_image;
@@ -346,8 +345,7 @@ __global__ void __launch_bounds__(BL_THREADS, BL_MIN_CTAS) k_blend(const FramePa
                     it.ctr = fp->bl_ctr;
                 }
                 it.pair_val = fp->bl_pair_val;
-                it.recA = fp->bl_recA;
-                it.recB = fp->bl_recB;
+                it.rec = fp->bl_rec;
                 it.rgb = fp->bl_rgb;
                 it.image = fp->bl_image;
                 it.host_image = fp->host_image;
@@ -410,16 +408,15 @@ __global__ void __launch_bounds__(BL_THREADS, BL_MIN_CTAS) k_blend(const FramePa
         // stage up to DEPTH queued hits into buffer buf; returns their number
         auto issue = [&](int buf) -> uint32_t {
             const uint32_t nh = min((uint32_t)DEPTH, tail - head);
-            const float4* rA = it.recA;
-            const float4* rB = it.recB;
+            const float4* rR = it.rec;
             const float4* rC = it.rgb;
 #pragma unroll
             for (int q = 0; q < (DEPTH + 31) / 32; ++q) {
                 const uint32_t sl = 32u * q + lane;
                 if (sl < nh) {
                     const uint32_t gi = ring[(head + sl) & (RING - 1)] >> 8;
-                    cp_async16(&sbuf[buf][0][warp][sl], rA + gi);
-                    cp_async16(&sbuf[buf][2][warp][sl], rB + gi);
+                    cp_async16(&sbuf[buf][0][warp][sl], rR + 2 * (size_t)gi);
+                    cp_async16(&sbuf[buf][2][warp][sl], rR + 2 * (size_t)gi + 1);
                     cp_async16(&sbuf[buf][1][warp][sl], rC + gi);
                 }
             }
@@ -444,7 +441,8 @@ __global__ void __launch_bounds__(BL_THREADS, BL_MIN_CTAS) k_blend(const FramePa
                 const uint32_t sl = 32u * q + lane;
                 if (sl < (uint32_t)DEPTH)  // each lane its own slots; empty slots reach no pixel
                     s_pm[warp][sl] = sl < nh ? blend_prepare<MODE, SR, T>(wA[sl], sbuf[buf][2][warp][sl],
-                                                                           sbuf[buf][NP - 1][warp][sl], rlo, clo,
+                                                                           sbuf[buf][NP - 1][warp][sl],
+                                                                           MODE != 0 ? wC[sl].w : 0.f, rlo, clo,
                                                                            full_walk)
                                              : 0u;
             }

@@ -189,11 +189,13 @@ __global__ void __launch_bounds__(DL_THREADS, 2) k_depth_local(const uint2* __re
                                                                const unsigned long long* __restrict__ cursor,
                                                                const uint32_t* __restrict__ ntile, uint32_t cap_vis,
                                                                uint32_t* __restrict__ order,
-                                                               uint32_t* __restrict__ off, uint64_t cap_pairs,
+                                                               uint32_t* __restrict__ off,
+                                                               uint32_t* __restrict__ owner, uint64_t cap_pairs,
                                                                Counters* __restrict__ ctr) {
     pdl_wait();
     extern __shared__ uint2 s_kv[];                                  // [DL_CAP] the bucket, by sub-bin
     uint32_t* s_sub = reinterpret_cast<uint32_t*>(s_kv + DL_CAP);    // [DL_SUB + 1] counts, then first places
+    uint4* s_sub4 = reinterpret_cast<uint4*>(s_sub);
     uint32_t* s_fin = s_sub + DL_SUB + 1;                            // [DL_CAP] index << 8 | slots, in order
     __shared__ uint32_t s_scan[DL_WARPS + 1];
     __shared__ uint32_t s_min[DL_WARPS], s_max[DL_WARPS];
@@ -211,6 +213,7 @@ __global__ void __launch_bounds__(DL_THREADS, 2) k_depth_local(const uint2* __re
 #pragma unroll
         for (int k = 0; k < DL_ITEMS; ++k) {
             const uint32_t j = k * DL_THREADS + t;
+            if (k * DL_THREADS >= n) break;
             if (j < n) {
                 e[k] = part[start + j];
                 lo = min(lo, e[k].x);
@@ -221,7 +224,7 @@ __global__ void __launch_bounds__(DL_THREADS, 2) k_depth_local(const uint2* __re
         for (uint32_t p = seen + t; p < b; p += DL_THREADS) sum += cursor[p] >> 32;
         seen = b;
 #pragma unroll
-        for (int k = 0; k < DL_SPT; ++k) s_sub[k * DL_THREADS + t] = 0u;
+        for (int k = 0; k < DL_SPT / 4; ++k) s_sub4[k * DL_THREADS + t] = make_uint4(0u, 0u, 0u, 0u);
         lo = __reduce_min_sync(0xFFFFFFFFu, lo);
         hi = __reduce_max_sync(0xFFFFFFFFu, hi);
         sum = warp_sum64(sum);
@@ -242,30 +245,42 @@ __global__ void __launch_bounds__(DL_THREADS, 2) k_depth_local(const uint2* __re
         // counting sort by sub-bin, in any order within one
         uint32_t place[DL_ITEMS];
 #pragma unroll
-        for (int k = 0; k < DL_ITEMS; ++k)
+        for (int k = 0; k < DL_ITEMS; ++k) {
+            if (k * DL_THREADS >= n) break;
             if (k * DL_THREADS + t < n) place[k] = atomicAdd(&s_sub[(e[k].x - lo) >> sh], 1u);
+        }
         __syncthreads();
         bool longrun = false;
         {
             uint32_t c[DL_SPT], s = 0, total;
 #pragma unroll
+            for (int k = 0; k < DL_SPT / 4; ++k) {
+                const uint4 q = s_sub4[DL_SPT / 4 * t + k];
+                c[4 * k] = q.x; c[4 * k + 1] = q.y; c[4 * k + 2] = q.z; c[4 * k + 3] = q.w;
+            }
+#pragma unroll
             for (int k = 0; k < DL_SPT; ++k) {
-                c[k] = s_sub[DL_SPT * t + k];
                 longrun = longrun || c[k] > DL_RUN_MAX;
                 s += c[k];
             }
             uint32_t pre = block_excl_scan<DL_WARPS>(s, s_scan, &total);
 #pragma unroll
-            for (int k = 0; k < DL_SPT; ++k) {
-                s_sub[DL_SPT * t + k] = pre;
-                pre += c[k];
+            for (int k = 0; k < DL_SPT / 4; ++k) {
+                uint4 q;
+                q.x = pre; pre += c[4 * k];
+                q.y = pre; pre += c[4 * k + 1];
+                q.z = pre; pre += c[4 * k + 2];
+                q.w = pre; pre += c[4 * k + 3];
+                s_sub4[DL_SPT / 4 * t + k] = q;
             }
             if (t == 0) s_sub[DL_SUB] = n;
         }
         longrun = __syncthreads_or(longrun);
 #pragma unroll
-        for (int k = 0; k < DL_ITEMS; ++k)
+        for (int k = 0; k < DL_ITEMS; ++k) {
+            if (k * DL_THREADS >= n) break;
             if (k * DL_THREADS + t < n) s_kv[s_sub[(e[k].x - lo) >> sh] + place[k]] = e[k];
+        }
         if (!longrun) {
             __syncthreads();
             for (uint32_t j = t; j < n; j += DL_THREADS) {
@@ -304,19 +319,16 @@ __global__ void __launch_bounds__(DL_THREADS, 2) k_depth_local(const uint2* __re
         __syncthreads();
         // write the order and the first slots: warp w takes the rows of 32 from w R on
         const uint32_t R = ((n + 31u) / 32u + DL_WARPS - 1u) / DL_WARPS;  // at most DL_ITEMS
+        const uint32_t cap_owner = (uint32_t)(cap_pairs / EMIT_SLOTS) + 1u;
+        auto slots_of = [&](uint32_t v) -> uint32_t { return (v & 255u) < 255u ? v & 255u : ntile[v >> 8]; };
         uint32_t x[DL_ITEMS], carry = 0;
 #pragma unroll
         for (int r = 0; r < DL_ITEMS; ++r) {
-            if (r < R) {
+            if (r >= R) break;
+            {
                 const uint32_t j = (warp * R + r) * 32u + lane;
-                uint32_t c = 0;
-                if (j < n) {
-                    const uint32_t v = s_fin[j];
-                    c = v & 255u;
-                    if (c == 255u) c = ntile[v >> 8];
-                }
                 uint32_t rowsum;
-                x[r] = carry + warp_excl_scan(c, &rowsum);
+                x[r] = carry + warp_excl_scan(j < n ? slots_of(s_fin[j]) : 0u, &rowsum);
                 carry += rowsum;
             }
         }
@@ -331,11 +343,14 @@ __global__ void __launch_bounds__(DL_THREADS, 2) k_depth_local(const uint2* __re
         }
 #pragma unroll
         for (int r = 0; r < DL_ITEMS; ++r) {
-            if (r < R) {
+            if (r >= R) break;
+            {
                 const uint32_t j = (warp * R + r) * 32u + lane;
                 if (j < n) {
-                    order[start + j] = s_fin[j] >> 8;
-                    off[start + j] = mine + x[r];
+                    const uint32_t v = s_fin[j], o = mine + x[r];
+                    order[start + j] = v >> 8;
+                    off[start + j] = o;
+                    emit_owner(owner, cap_owner, o, slots_of(v), start + j);
                 }
             }
         }
@@ -365,13 +380,13 @@ cudaError_t depth_sort_init() {
 
 void launch_depth_sort(const VisBuffers& vis, uint32_t cap_vis, const uint32_t* bins, uint32_t* bstart,
                        unsigned long long* cursor, uint2* part, uint32_t* order, uint32_t* slot_off,
-                       uint64_t cap_pairs, Counters* ctr, const FrameParams* fp, int sms, cudaStream_t s) {
+                       uint32_t* owner, uint64_t cap_pairs, Counters* ctr, const FrameParams* fp, int sms, cudaStream_t s) {
     const uint32_t cap = cap_vis < MAX_RANKS ? cap_vis : MAX_RANKS;
     const uint32_t cb = depth_bucket_cap(cap);
     launch_ks(k_depth_part, 2 * sms, DP_THREADS, depth_part_smem(cb), s, (const uint32_t*)vis.depth,
               (const uint32_t*)vis.ntile, cap, bins, bstart, cursor, part, cb, ctr, fp);
     launch_ks(k_depth_local, 2 * sms, DL_THREADS, depth_local_smem(), s, (const uint2*)part, (const uint32_t*)bstart,
-              (const unsigned long long*)cursor, (const uint32_t*)vis.ntile, cap, order, slot_off, cap_pairs, ctr);
+              (const unsigned long long*)cursor, (const uint32_t*)vis.ntile, cap, order, slot_off, owner, cap_pairs, ctr);
 }
 
 }  // namespace vgr

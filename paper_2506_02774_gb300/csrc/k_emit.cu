@@ -2,15 +2,20 @@
 // tile-level preemptive alpha test, and the blend's tile order (which also
 // finishes the per-tile ranges the last tile-sort pass records).
 //
-// Two kernels.  k_slot_scan gives every visible Gaussian, in depth order (the
-// output of the depth sort), the first of its pair slots: an exclusive scan of
-// the candidate-tile counts by decoupled look-back over tiles of 4096, whose
-// per-tile work is light, so the chain of tiles moves fast.  k_emit then takes
-// 512 Gaussians per CTA tile with no ticket and no look-back (their slot range
-// is known): it gathers their records, and walks the tile's slots with all 256
-// threads (slot -> Gaussian by a search over the CTA's offsets in shared
-// memory), so a Gaussian with thousands of candidate tiles costs no more per
-// thread than one with a single tile.  For each slot the tile-level form of
+// Every visible Gaussian has a range of pair slots (one per candidate tile) in
+// depth order; their first slots come with the depth order (k_depth.cu, or
+// k_slot_scan after the radix passes: an exclusive scan of the counts by
+// decoupled look-back over tiles of 4096), and so does, for every chunk of 1024
+// slots, the depth rank that owns its first slot.  k_emit gives each CTA whole
+// chunks, so a CTA's work does not depend on how the slots are spread over the
+// Gaussians (a near one can have thousands): it marks the slots at which a
+// Gaussian starts in a bitmap, a slot finds its Gaussian by counting the marks
+// up to it, and reads its record (one 32-byte sector, shared through L1 with
+// the Gaussian's other slots).  Chunks
+// of 512 Gaussians before this left the CTA with the near ones running alone
+// (SM cycles 43 % busy on average) and gathered three half-used sectors each;
+// 1M-leaf box at 1080p (981K slots): 53 -> 21 us, city at 1080p (4.26M slots):
+// 107 -> 61 us.  For each slot the tile-level form of
 // Eq. 4 (paper Sec. 4.2) decides: a kept slot gets key = tile id, a dropped one
 // the sentinel key, which the stable tile sort moves behind every real pair
 // (which stay in depth order within a tile, the sort being stable).  The slot's
@@ -31,11 +36,12 @@
 namespace vgr {
 
 constexpr int EM_THREADS = 256;
-constexpr int EM_ITEMS = 2;
-constexpr int EM_TILE = EM_THREADS * EM_ITEMS;  // Gaussians per CTA tile
-static_assert(EM_TILE == 512, "the owner search takes two ballots over 32 x 16 Gaussians");
+constexpr int EM_WARPS = EM_THREADS / 32;
+constexpr uint32_t EM_SLOTS = EMIT_SLOTS;   // slots per chunk: 32 runs of a warp
+constexpr uint32_t EM_GAUSS = EM_SLOTS + 1; // Gaussians that may be looked at for a chunk
+static_assert(EM_SLOTS == 1024, "32 words of start bits, one per lane of the scanning warp");
 
-uint32_t emit_tile() { return EM_TILE; }
+uint32_t emit_owner_cap(uint64_t cap_pairs) { return (uint32_t)(cap_pairs / EMIT_SLOTS) + 1u; }
 
 constexpr int SS_THREADS = 256;
 constexpr int SS_ITEMS = 16;
@@ -47,7 +53,8 @@ uint32_t slot_scan_tile() { return SS_TILE; }
 // off[n_vis] is the frame's candidate-slot count.
 __global__ void __launch_bounds__(SS_THREADS) k_slot_scan(const uint32_t* __restrict__ order, uint32_t cap_vis,
                                                           const uint32_t* __restrict__ ntile,
-                                                          uint32_t* __restrict__ off, uint64_t cap_pairs,
+                                                          uint32_t* __restrict__ off,
+                                                          uint32_t* __restrict__ owner, uint64_t cap_pairs,
                                                           unsigned long long* __restrict__ status,
                                                           Counters* __restrict__ ctr,
                                                           const FrameParams* __restrict__ fp) {
@@ -92,7 +99,10 @@ __global__ void __launch_bounds__(SS_THREADS) k_slot_scan(const uint32_t* __rest
         run += s_prefix;
 #pragma unroll
         for (int k = 0; k < SS_ITEMS; ++k) {
-            if (r0 + k < n_vis) off[r0 + k] = run;
+            if (r0 + k < n_vis) {
+                off[r0 + k] = run;
+                emit_owner(owner, (uint32_t)(cap_pairs / EMIT_SLOTS) + 1u, run, c[k], r0 + k);
+            }
             run += c[k];
         }
         if (tile == ntiles - 1 && threadIdx.x == 0) {
@@ -106,146 +116,113 @@ __global__ void __launch_bounds__(SS_THREADS) k_slot_scan(const uint32_t* __rest
 }
 
 __global__ void __launch_bounds__(EM_THREADS, 4) k_emit(const uint32_t* __restrict__ order, uint32_t cap_vis,
-                                                     VisBuffers vis, const uint32_t* __restrict__ slot_off,
+                                                     const float4* __restrict__ rec,
+                                                     const uint32_t* __restrict__ slot_off,
+                                                     const uint32_t* __restrict__ owner,
                                                      uint32_t* __restrict__ pair_key,
                                                      uint32_t* __restrict__ pair_val, uint64_t cap, int tile_passes,
                                                      uint32_t sentinel, Counters* __restrict__ ctr,
                                                      const FrameParams* __restrict__ fp) {
     pdl_wait();
-    __shared__ uint32_t s_off[EM_TILE + 1];   // exclusive slot offsets within the CTA tile, then its total
-    __shared__ float4 s_g[EM_TILE];           // u v a b
-    __shared__ float4 s_h[EM_TILE];           // c rx ry thre
-    __shared__ uint32_t s_rect[EM_TILE];      // x0 | y0 << 10 | width << 20 (tiles; 16384-px images: < 2^10)
-    __shared__ __half s_hh[EM_TILE];          // footprint half-height, rounded up
-    __shared__ uint32_t s_vi[EM_TILE];        // index in the in-front arrays
+    __shared__ uint2 s_g[EM_GAUSS];   // per Gaussian: index in the in-front arrays, first slot
+    __shared__ uint32_t s_bits[32];   // slots at which a Gaussian starts
     __shared__ uint32_t s_hist[4][256];
-    for (int i = threadIdx.x; i < 4 * 256; i += blockDim.x) (&s_hist[0][0])[i] = 0u;
+    const uint32_t lane = lane_id(), warp = threadIdx.x >> 5;
+    for (int i = threadIdx.x; i < tile_passes * 256; i += EM_THREADS) (&s_hist[0][0])[i] = 0u;
     const uint32_t n_vis = min(ctr->n_vis, cap_vis);
-    const uint32_t ntiles = (n_vis + EM_TILE - 1) / EM_TILE;
+    const uint64_t cand = ctr->n_cand;
+    const uint32_t ns = (uint32_t)(cand < cap ? cand : cap);
+    const uint32_t nchunks = n_vis ? (ns + EM_SLOTS - 1u) / EM_SLOTS : 0u;
     const uint32_t TW = fp->tiles_x;
     const int T = (int)fp->tile;
     const int MR = T >= 8 ? T / 8 : 1;  // tile rows per row-mask bit (8 bits)
     const float Wf = fp->width_f, Hf = fp->height_f;
     const bool canonical = fp->filter == VGR_FILTER_CANONICAL;
     uint32_t kept = 0;
-    __shared__ uint32_t s_tile;
-    __syncthreads();
-
-    for (;;) {
-        // tiles are claimed in order as CTAs free up: their slot counts vary widely
-        if (threadIdx.x == 0) s_tile = atomicAdd(&ctr->tickets[TK_PRE], 1u);
+    for (uint32_t ck = blockIdx.x; ck < nchunks; ck += gridDim.x) {
+        const uint32_t j0 = ck * EM_SLOTS, len = min(EM_SLOTS, ns - j0);
+        const uint32_t g0 = owner[ck];
+        const uint32_t g1 = ck + 1u < nchunks ? owner[ck + 1u] : n_vis - 1u;  // may start past the chunk
+        const uint32_t m = min(g1 - g0 + 1u, EM_GAUSS);
+        if (threadIdx.x < 32) s_bits[threadIdx.x] = threadIdx.x == 0 ? 1u : 0u;  // the chunk's first slot has an owner
         __syncthreads();
-        const uint32_t tile = s_tile;
-        if (tile >= ntiles) break;
-        const uint32_t g0 = tile * EM_TILE;
-        const uint32_t base32 = slot_off[g0];
-        // gather EM_ITEMS Gaussians per thread (independent loads in flight)
-#pragma unroll
-        for (int k = 0; k < EM_ITEMS; ++k) {
-            const uint32_t q = k * EM_THREADS + threadIdx.x;  // position in depth order within the CTA tile
-            const uint32_t r = g0 + q;
-            if (r < n_vis) {
-                const uint32_t vi = order[r];
-                s_vi[q] = vi;
-                const uint2 rect = vis.rect[vi];
-                const float4 A = vis.recA[vi];
-                const float4 B = vis.recB[vi];
-                // the conic is stored pre-scaled (A = -a/2, B = -b, C = -c/2): exact to undo
-                const float ca = -2.0f * A.z, cb = -A.w, cc = -2.0f * B.x;
-                s_g[q] = make_float4(A.x, A.y, ca, cb);
-                // edge optima dy* = (-b / c) dx, dx* = (-b / a) dy; an ulp or two of
-                // error moves rho_max by far less than the test's 2e-3 slack
-                s_h[q] = make_float4(cc, __fdividef(-cb, ca), __fdividef(-cb, cc), B.y - TILE_EPS);
-                const uint32_t x0 = rect.x & 0xFFFFu, y0 = rect.x >> 16;
-                s_rect[q] = x0 | (y0 << 10) | (((rect.y & 0xFFFFu) - x0 + 1u) << 20);
-                s_hh[q] = __ushort_as_half((unsigned short)(__float_as_uint(B.w) & 0xFFFFu));  // half-height
-            }
-            // offsets within the tile; past the last Gaussian: the tile's total
-            s_off[q] = slot_off[min(r, n_vis)] - base32;
+        for (uint32_t q = threadIdx.x; q < m; q += EM_THREADS) {
+            const uint32_t o = slot_off[g0 + q];
+            s_g[q] = make_uint2(order[g0 + q], o);
+            if (o > j0 && o - j0 < len) atomicOr(&s_bits[(o - j0) >> 5], 1u << (o & 31u));  // j0 is a multiple of 32
         }
-        if (threadIdx.x == 0) s_off[EM_TILE] = slot_off[min(g0 + EM_TILE, n_vis)] - base32;
         __syncthreads();
-        const uint32_t total = s_off[EM_TILE];
-        const uint64_t base = base32;
-        // slots in warp-sized runs: the owner of the run's first slot by a
-        // warp-wide search, the other lanes' owners by counting the
-        // Gaussians that start inside the run (every visible Gaussian has at
-        // least one slot, so starts are distinct)
-        const uint32_t lane = lane_id();
-        for (uint32_t j0 = (threadIdx.x & ~31u); j0 < total; j0 += EM_THREADS) {
-            // the last Gaussian starting at or before j0 (offsets ascend, so the
-            // test holds on a prefix): lane k tests Gaussian 16 k, then lanes 0..15
-            // the 16 Gaussians of the last such stride -- two ballots
-            const uint32_t cm = __ballot_sync(0xFFFFFFFFu, s_off[16u * lane] <= j0);  // bit 0: s_off[0] = 0
-            const uint32_t kc = 31u - __clz(cm);
-            const uint32_t fm = __ballot_sync(0xFFFFFFFFu, lane < 16u && s_off[16u * kc + (lane & 15u)] <= j0);
-            const uint32_t lo = 16u * kc + 31u - __clz(fm);
-            const uint32_t gi = lo + 1u + lane;
-            const uint32_t d = (gi <= (uint32_t)EM_TILE ? s_off[gi] : 0xFFFFFFFFu) - j0;  // >= 1
-            const uint32_t starts = __reduce_or_sync(0xFFFFFFFFu, d < 32u ? 1u << d : 0u);
-            const uint32_t j = j0 + lane;
-            const bool valid = j < total;
-            const uint32_t g = lo + __popc(starts & ((2u << lane) - 1u));
-            uint32_t key = 0xFFFFFFFFu;
-            bool keep = false;
-            uint32_t rows = 0xFFu;
-            if (valid) {
-                const uint32_t local = j - s_off[g];
-                const uint32_t rc = s_rect[g];
+        uint32_t total;
+        const uint32_t bits_l = s_bits[lane];
+        const uint32_t pre_l = warp_excl_scan(__popc(bits_l), &total);  // starts before word 'lane'
+#pragma unroll
+        for (uint32_t r = 0; r < EM_SLOTS / EM_THREADS; ++r) {
+            const uint32_t word = r * EM_WARPS + warp;
+            const uint32_t bits = __shfl_sync(0xFFFFFFFFu, bits_l, word);
+            const uint32_t before = __shfl_sync(0xFFFFFFFFu, pre_l, word);
+            const uint32_t j = j0 + 32u * word + lane;
+            if (32u * word + lane < len) {
+                // the last Gaussian that starts at or before this slot
+                const uint2 gv = s_g[before + __popc(bits & ((2u << lane) - 1u)) - 1u];
+                const float4 A = rec[2 * (size_t)gv.x], B = rec[2 * (size_t)gv.x + 1];
+                const uint32_t local = j - gv.y;
+                const uint32_t rc = __float_as_uint(B.z);
                 const uint32_t w = rc >> 20;
                 // local / w and local % w: local < 2^20 and w <= 2^10, so (local + 1/2) / w is
                 // at least 1 / 2^11 from an integer and its FP32 quotient floors exactly
                 const uint32_t qy = (uint32_t)(((float)local + 0.5f) * __frcp_rn((float)w));
                 const int tx = (int)(rc & 0x3FFu) + (int)(local - qy * w);
                 const int ty = (int)((rc >> 10) & 0x3FFu) + (int)qy;
-                keep = true;
+                bool keep = true;
+                uint32_t rows = 0xFFu;
                 if (!canonical) {
-                    const float4 G = s_g[g], Hh = s_h[g];
-                    keep = tile_keep(G.x, G.y, G.z, G.w, Hh.x, Hh.y, Hh.z, Hh.w, tx, ty, Wf, Hf, T);
+                    // the conic is stored pre-scaled (A = -a/2, B = -b, C = -c/2): exact to undo;
+                    // edge optima dy* = (-b / c) dx, dx* = (-b / a) dy: an ulp or two of
+                    // error moves rho_max by far less than the test's 2e-3 slack
+                    const float ca = -2.0f * A.z, cb = -A.w, cc = -2.0f * B.x;
+                    keep = tile_keep(A.x, A.y, ca, cb, cc, __fdividef(-cb, ca), __fdividef(-cb, cc), B.y - TILE_EPS,
+                                     tx, ty, Wf, Hf, T);
                     // tile rows r with |row0 + r - v| <= half-height, as groups of MR rows
-                    const float row0 = (float)(ty * T) + 0.5f, hh = __half2float(s_hh[g]);
-                    const float rlo = fmaxf(0.f, ceilf(G.y - hh - row0));
-                    const float rhi = fminf((float)(T - 1), floorf(G.y + hh - row0));
+                    const float row0 = (float)(ty * T) + 0.5f;
+                    const float hh = __half2float(__ushort_as_half((unsigned short)(__float_as_uint(B.w) & 0xFFFFu)));
+                    const float rlo = fmaxf(0.f, ceilf(A.y - hh - row0));
+                    const float rhi = fminf((float)(T - 1), floorf(A.y + hh - row0));
                     rows = 0u;
                     if (rlo <= rhi) {
                         const uint32_t w0 = (uint32_t)rlo / MR, w1 = (uint32_t)rhi / MR;
                         rows = ((2u << w1) - 1u) & ~((1u << w0) - 1u);
                     }
                 }
-                key = keep ? (uint32_t)ty * TW + (uint32_t)tx : sentinel;
+                const uint32_t key = keep ? (uint32_t)ty * TW + (uint32_t)tx : sentinel;
                 kept += keep;
-            }
-            const uint64_t pos = base + j;
-            const bool write = valid && pos < cap;
-            if (write) {
-                pair_key[pos] = key;
-                pair_val[pos] = (s_vi[g] << 8) | rows;
+                pair_key[j] = key;
+                pair_val[j] = (gv.x << 8) | rows;
                 for (int p = 0; p < tile_passes; ++p) atomicAdd(&s_hist[p][(key >> (8 * p)) & 255u], 1u);
             }
         }
         __syncthreads();
     }
     const uint32_t wk = __reduce_add_sync(0xFFFFFFFFu, kept);
-    if (lane_id() == 0 && wk) atomicAdd(&ctr->n_pairs, (unsigned long long)wk);
+    if (lane == 0 && wk) atomicAdd(&ctr->n_pairs, (unsigned long long)wk);
     __syncthreads();
-    for (int i = threadIdx.x; i < tile_passes * 256; i += blockDim.x) {
+    for (int i = threadIdx.x; i < tile_passes * 256; i += EM_THREADS) {
         const uint32_t c = (&s_hist[0][0])[i];
         if (c) atomicAdd(&ctr->tile_hist[0][0] + i, c);
     }
 }
 
 void launch_slot_scan(const uint32_t* order, uint32_t cap_vis, const VisBuffers& vis, uint32_t* slot_off,
-                      uint64_t cap_pairs, unsigned long long* status, Counters* ctr, const FrameParams* fp, int grid,
-                      cudaStream_t s) {
-    launch_k(k_slot_scan, grid, SS_THREADS, s, order, cap_vis, (const uint32_t*)vis.ntile, slot_off, cap_pairs,
+                      uint32_t* owner, uint64_t cap_pairs, unsigned long long* status, Counters* ctr,
+                      const FrameParams* fp, int grid, cudaStream_t s) {
+    launch_k(k_slot_scan, grid, SS_THREADS, s, order, cap_vis, (const uint32_t*)vis.ntile, slot_off, owner, cap_pairs,
              status, ctr, fp);
 }
 
-void launch_emit(const uint32_t* order, uint32_t cap_vis, VisBuffers vis, uint32_t* slot_off, uint32_t* pair_key,
-                 uint32_t* pair_val, uint64_t cap_pairs, int tile_passes, uint32_t sentinel, Counters* ctr,
-                 const FrameParams* fp, int grid, cudaStream_t s) {
-    launch_k(k_emit, grid, EM_THREADS, s, order, cap_vis, vis, (const uint32_t*)slot_off, pair_key, pair_val, cap_pairs,
-             tile_passes, sentinel, ctr, fp);
+void launch_emit(const uint32_t* order, uint32_t cap_vis, const VisBuffers& vis, const uint32_t* slot_off,
+                 const uint32_t* owner, uint32_t* pair_key, uint32_t* pair_val, uint64_t cap_pairs, int tile_passes,
+                 uint32_t sentinel, Counters* ctr, const FrameParams* fp, int grid, cudaStream_t s) {
+    launch_k(k_emit, grid, EM_THREADS, s, order, cap_vis, (const float4*)vis.rec, slot_off, owner, pair_key, pair_val,
+             cap_pairs, tile_passes, sentinel, ctr, fp);
 }
 
 // Blend order: tiles by descending pair count (classes of floor(log2(count+1)),

@@ -126,6 +126,13 @@ struct Store<VGR_STORE_HALF> {
     }
 };
 
+// An entry's record in one 32-byte store.
+__device__ __forceinline__ void store_record(float4* p, float4 a, float4 b) {
+    asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};\n" ::"l"(p), "f"(a.x), "f"(a.y), "f"(a.z),
+                 "f"(a.w), "f"(b.x), "f"(b.y), "f"(b.z), "f"(b.w)
+                 : "memory");
+}
+
 template <int DEG, int STORE, bool INTERP>
 __global__ void __launch_bounds__(PRE_THREADS, 2) k_preprocess(SceneDev sc, const uint32_t* __restrict__ front,
                                                             const uint32_t* __restrict__ n_front_p, uint32_t cap,
@@ -277,7 +284,7 @@ __global__ void __launch_bounds__(PRE_THREADS, 2) k_preprocess(SceneDev sc, cons
                     cg = fmaf(shc[3 * kk + 1], Y[kk], cg);
                     cbl = fmaf(shc[3 * kk + 2], Y[kk], cbl);
                 }
-                vis.rgb[i] = make_float4(fmaxf(cr, 0.f), fmaxf(cg, 0.f), fmaxf(cbl, 0.f), 0.f);
+                vis.rgb[i] = make_float4(fmaxf(cr, 0.f), fmaxf(cg, 0.f), fmaxf(cbl, 0.f), theta);
                 zbits = __float_as_uint(z);
             }
         }
@@ -286,9 +293,8 @@ __global__ void __launch_bounds__(PRE_THREADS, 2) k_preprocess(SceneDev sc, cons
         if (i < n_front) {
             vis.depth[i] = zbits;  // culled: all ones, sorted behind every visible key
             vis.ntile[i] = v ? (uint32_t)(tx1 - tx0 + 1) * (uint32_t)(ty1 - ty0 + 1) : 0u;
-            vis.rect[i] = make_uint2((uint32_t)tx0 | ((uint32_t)ty0 << 16), (uint32_t)tx1 | ((uint32_t)ty1 << 16));
-            vis.recA[i] = make_float4(u, vv, -0.5f * ca, -cb);
-            vis.recB[i] = make_float4(-0.5f * cc, thr, theta, __uint_as_float(box_hw));
+            store_record(vis.rec + 2 * (size_t)i, make_float4(u, vv, -0.5f * ca, -cb),
+                         make_float4(-0.5f * cc, thr, __uint_as_float(pack_rect(tx0, ty0, tx1)), __uint_as_float(box_hw)));
             if (INTERP) vis.lw[i] = lw;
         }
     }
@@ -345,5 +351,26 @@ void launch_preprocess(const SceneDev& sc, const uint32_t* front, const uint32_t
 }
 
 uint32_t preprocess_tile() { return PRE_THREADS; }
+
+// The visible entries' records as separate arrays (the debug view's layout).
+__global__ void k_debug_records(VisBuffers vis, uint32_t n, uint2* __restrict__ rect, float4* __restrict__ recA,
+                                float4* __restrict__ recB, float4* __restrict__ rgb) {
+    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        const uint32_t c = vis.ntile[i];
+        if (c == 0u) continue;
+        const float4 a = vis.rec[2 * (size_t)i], b = vis.rec[2 * (size_t)i + 1], col = vis.rgb[i];
+        const uint32_t rc = __float_as_uint(b.z);
+        const uint32_t x0 = rc & 0x3FFu, y0 = (rc >> 10) & 0x3FFu, w = rc >> 20;
+        rect[i] = make_uint2(x0 | (y0 << 16), (x0 + w - 1u) | ((y0 + c / w - 1u) << 16));
+        recA[i] = a;
+        recB[i] = make_float4(b.x, b.y, col.w, b.w);
+        rgb[i] = make_float4(col.x, col.y, col.z, 0.f);
+    }
+}
+
+void launch_debug_records(const VisBuffers& vis, uint32_t n, uint2* rect, float4* recA, float4* recB, float4* rgb,
+                          cudaStream_t s) {
+    if (n) k_debug_records<<<1024, 256, 0, s>>>(vis, n, rect, recA, recB, rgb);
+}
 
 }  // namespace vgr

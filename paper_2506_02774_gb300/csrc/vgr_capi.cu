@@ -149,6 +149,9 @@ struct vgr_view {
     uint32_t n_words = 0;
     uint32_t* frontier[2] = {nullptr, nullptr};
     VisBuffers vis{};
+    // vgr_view_debug's copies of the records, made on its first call
+    uint2* dbg_rect = nullptr;
+    float4 *dbg_recA = nullptr, *dbg_recB = nullptr, *dbg_rgb = nullptr;
     // depth sort: the partition's (key, value) pairs fill all of sort_kv; the
     // radix passes use its halves as their key buffers
     uint32_t* sort_kv = nullptr;
@@ -158,6 +161,7 @@ struct vgr_view {
     uint32_t* bucket_start = nullptr;
     int radix_frames = 0;  // frames left that order depths by radix passes (a bucket did not fit)
     uint32_t* slot_off = nullptr;  // first pair slot of each visible Gaussian by depth rank (cap_vis + 1)
+    uint32_t* slot_owner = nullptr;  // depth rank of the first slot of each emission chunk
     uint32_t* pairK[2] = {nullptr, nullptr};
     uint32_t* pairV[2] = {nullptr, nullptr};
     uint2* ranges = nullptr;
@@ -556,8 +560,9 @@ void drop_graphs(vgr_view* v) {
 
 void free_vis(vgr_view* v) {
     drop_graphs(v);
-    dfree(v->vis.depth); dfree(v->vis.ntile); dfree(v->vis.rect);
-    dfree(v->vis.recA); dfree(v->vis.recB); dfree(v->vis.rgb); dfree(v->vis.lw);
+    dfree(v->vis.depth); dfree(v->vis.ntile);
+    dfree(v->vis.rec); dfree(v->vis.rgb); dfree(v->vis.lw);
+    dfree(v->dbg_rect); dfree(v->dbg_recA); dfree(v->dbg_recB); dfree(v->dbg_rgb);
     dfree(v->sort_kv);
     for (int i = 0; i < 2; ++i) dfree(v->sortV[i]);
     dfree(v->slot_off);
@@ -569,8 +574,7 @@ vgr_status alloc_vis(vgr_view* v, uint32_t cap) {
     uint64_t b = 0;
     vgr_status s;
     if ((s = dalloc(&v->vis.depth, cap, &b)) ||
-        (s = dalloc(&v->vis.ntile, cap, &b)) || (s = dalloc(&v->vis.rect, cap, &b)) ||
-        (s = dalloc(&v->vis.recA, cap, &b)) || (s = dalloc(&v->vis.recB, cap, &b)) ||
+        (s = dalloc(&v->vis.ntile, cap, &b)) || (s = dalloc(&v->vis.rec, 2 * (size_t)cap, &b)) ||
         (s = dalloc(&v->vis.rgb, cap, &b)) || (s = dalloc(&v->vis.lw, cap, &b)) ||
         (s = dalloc(&v->sort_kv, 2 * (size_t)cap, &b)) || (s = dalloc(&v->sortV[0], cap, &b)) ||
         (s = dalloc(&v->sortV[1], cap, &b)) || (s = dalloc(&v->slot_off, (size_t)cap + 1, &b))) {
@@ -585,6 +589,7 @@ vgr_status alloc_vis(vgr_view* v, uint32_t cap) {
 void free_pairs(vgr_view* v) {
     drop_graphs(v);
     for (int i = 0; i < 2; ++i) { dfree(v->pairK[i]); dfree(v->pairV[i]); }
+    dfree(v->slot_owner);
     v->pair_bytes = 0;
 }
 
@@ -593,7 +598,8 @@ vgr_status alloc_pairs(vgr_view* v, uint64_t cap) {
     uint64_t b = 0;
     vgr_status s;
     if ((s = dalloc(&v->pairK[0], cap, &b)) || (s = dalloc(&v->pairK[1], cap, &b)) ||
-        (s = dalloc(&v->pairV[0], cap, &b)) || (s = dalloc(&v->pairV[1], cap, &b))) {
+        (s = dalloc(&v->pairV[0], cap, &b)) || (s = dalloc(&v->pairV[1], cap, &b)) ||
+        (s = dalloc(&v->slot_owner, emit_owner_cap(cap), &b))) {
         free_pairs(v);
         return s;
     }
@@ -630,7 +636,7 @@ vgr_status alloc_status(vgr_view* v) {
     v->st_compact = 0;
     v->st_front = v->st_compact + cut_compact_tiles(v->n_words) + 1;
     v->st_emit = v->st_front + cut_compact_tiles(v->n_words) + 1;
-    v->st_depth = v->st_emit + ceil_div(v->cap_vis, emit_tile()) + 1;
+    v->st_depth = v->st_emit + ceil_div(v->cap_vis, slot_scan_tile()) + 1;
     v->st_depth_stride = (size_t)(ceil_div(v->cap_vis, RT) + 1) * 256;
     v->st_tile = v->st_depth + 4 * v->st_depth_stride;
     v->st_tile_stride = (size_t)(ceil_div(v->cap_pairs, RT) + 1) * 256;
@@ -892,15 +898,14 @@ vgr_status vgr_view_bytes_estimate(const vgr_hierarchy* h, const vgr_view_opts* 
     const uint64_t cap_pairs = o.pair_capacity ? o.pair_capacity : 2 * cap_vis;
     const uint64_t TW = cut_compact_tile_words();
     const uint64_t n_words = ((N + 31) / 32 + TW - 1) / TW * TW;
-    const uint64_t per_vis = 3 * sizeof(uint32_t) + sizeof(uint2) + 3 * sizeof(float4) + sizeof(float) /* visible SoA */ +
-                             sizeof(uint32_t) /* slot offsets */ +
-                             4 * sizeof(uint32_t) /* depth-sort ping-pong */ + 3 * sizeof(float4) /* rank records */;
+    const uint64_t per_vis = 2 * sizeof(uint32_t) + 3 * sizeof(float4) + sizeof(float) /* visible SoA */ +
+                             sizeof(uint32_t) /* slot offsets */ + 4 * sizeof(uint32_t) /* depth sort */;
     const uint64_t RT = radix_tile();
-    const uint64_t status_words = 2 * (cut_compact_tiles((uint32_t)n_words) + 1) + ceil_div(cap_vis, emit_tile()) + 1 +
+    const uint64_t status_words = 2 * (cut_compact_tiles((uint32_t)n_words) + 1) + ceil_div(cap_vis, slot_scan_tile()) + 1 +
                                   4 * (ceil_div(cap_vis, RT) + 1) * 256 + 4 * (ceil_div(cap_pairs, RT) + 1) * 256;
     const uint32_t T = o.tile_size ? o.tile_size : TILE_DEFAULT;
     const uint64_t tiles = (uint64_t)((width + T - 1) / T) * ((height + T - 1) / T);
-    uint64_t b = 3 * 4 * cap_cut + per_vis * cap_vis + 4 * 4 * cap_pairs + 2 * 4 * n_words + 2 * 4 * N +
+    uint64_t b = 3 * 4 * cap_cut + per_vis * cap_vis + 4 * 4 * cap_pairs + 4 * emit_owner_cap(cap_pairs) + 2 * 4 * n_words + 2 * 4 * N +
                  cleared_bytes(MAX_RANKS) + 4 * (depth_bucket_cap(MAX_RANKS) + 1) + sizeof(ViewState) + sizeof(FrameParams) + 260 * 4 + 8 * status_words;
     b += (uint64_t)width * height * 3 * 4 + tiles * (sizeof(uint2) + 4);
     *bytes = b;
@@ -986,8 +991,8 @@ uint32_t enqueue_frame(vgr_view* v, bool scratch, bool radix_depth, int tile_pas
     uint32_t* order = v->sortV[1];
     if (!radix_depth) {
         launch_depth_sort(v->vis, v->cap_vis, v->depth_bins, v->bucket_start, v->bucket_cursor,
-                          reinterpret_cast<uint2*>(v->sort_kv), order, v->slot_off, v->cap_pairs, v->ctr, v->fp_dev,
-                          v->h->num_sms, s);
+                          reinterpret_cast<uint2*>(v->sort_kv), order, v->slot_off, v->slot_owner, v->cap_pairs,
+                          v->ctr, v->fp_dev, v->h->num_sms, s);
     } else {
         // every potentially visible entry is sorted; culled ones carry the key
         // 0xFFFFFFFF and land last
@@ -1003,13 +1008,13 @@ uint32_t enqueue_frame(vgr_view* v, bool scratch, bool radix_depth, int tile_pas
                               v->ctr->depth_hist[p], v->status + v->st_depth + p * v->st_depth_stride,
                               &v->ctr->tickets[TK_SORT0 + p], v->fp_dev, v->ctr, v->grid_scan, s, p == 3 ? 1 : 0);
         }
-        launch_slot_scan(order, v->cap_vis, v->vis, v->slot_off, v->cap_pairs, v->status + v->st_emit, v->ctr,
-                         v->fp_dev, v->grid_scan, s);
+        launch_slot_scan(order, v->cap_vis, v->vis, v->slot_off, v->slot_owner, v->cap_pairs, v->status + v->st_emit,
+                         v->ctr, v->fp_dev, v->grid_scan, s);
     }
     mark(VGR_STAGE_COLOR);  // (evaluated in preprocess: the stage is empty)
     mark(VGR_STAGE_EMIT);
     const uint32_t sentinel = (uint32_t)((1ull << (8 * tile_passes)) - 1ull);
-    launch_emit(order, v->cap_vis, v->vis, v->slot_off, v->pairK[0], v->pairV[0], v->cap_pairs, tile_passes, sentinel,
+    launch_emit(order, v->cap_vis, v->vis, v->slot_off, v->slot_owner, v->pairK[0], v->pairV[0], v->cap_pairs, tile_passes, sentinel,
                 v->ctr, v->fp_dev, v->grid_scan * EMIT_GRID_NUM / 4, s);
     mark(VGR_STAGE_TILE_SORT);
     // (the last pass also records each tile's range)
@@ -1188,8 +1193,7 @@ void fill_params(vgr_view* v, const vgr_camera* cam, float t, float k, float* ho
     // buffer (passes & 1)
     p.bl_ranges = v->ranges;
     p.bl_pair_val = v->pairV[tile_passes & 1];
-    p.bl_recA = v->vis.recA;
-    p.bl_recB = v->vis.recB;
+    p.bl_rec = v->vis.rec;
     p.bl_rgb = v->vis.rgb;
     p.bl_lut = v->lut;
     p.bl_image = v->cur_image;
@@ -1689,10 +1693,23 @@ vgr_status vgr_view_debug(vgr_view* v, vgr_debug_buffers* o) {
     o->vis_node = v->front_list;  // entry i's node id
     o->vis_depth = v->vis.depth;
     o->vis_ntile = v->vis.ntile;
-    o->vis_rect = reinterpret_cast<const uint32_t*>(v->vis.rect);
-    o->vis_recA = reinterpret_cast<const float*>(v->vis.recA);
-    o->vis_recB = reinterpret_cast<const float*>(v->vis.recB);
-    o->vis_rgb = reinterpret_cast<const float*>(v->vis.rgb);
+    // the records as separate arrays, made here (the frame keeps them in one 32-byte sector each)
+    vgr_status s = VGR_OK;
+    VGR_CK(cudaSetDevice(v->h->device));
+    if (!v->dbg_rgb &&
+        ((s = dalloc(&v->dbg_rect, v->cap_vis, nullptr)) || (s = dalloc(&v->dbg_recA, v->cap_vis, nullptr)) ||
+         (s = dalloc(&v->dbg_recB, v->cap_vis, nullptr)) || (s = dalloc(&v->dbg_rgb, v->cap_vis, nullptr)))) {
+        dfree(v->dbg_rect); dfree(v->dbg_recA); dfree(v->dbg_recB); dfree(v->dbg_rgb);
+        return s;
+    }
+    launch_debug_records(v->vis, std::min(v->last_n_front, v->cap_vis), v->dbg_rect, v->dbg_recA, v->dbg_recB,
+                         v->dbg_rgb, v->stream);
+    VGR_CK(cudaGetLastError());
+    VGR_CK(cudaStreamSynchronize(v->stream));
+    o->vis_rect = reinterpret_cast<const uint32_t*>(v->dbg_rect);
+    o->vis_recA = reinterpret_cast<const float*>(v->dbg_recA);
+    o->vis_recB = reinterpret_cast<const float*>(v->dbg_recB);
+    o->vis_rgb = reinterpret_cast<const float*>(v->dbg_rgb);
     o->depth_order = v->sortV[1];
     o->pair_tile = v->pairK[v->last_tile_buf];
     o->pair_val = v->pairV[v->last_tile_buf];

@@ -26,7 +26,7 @@ constexpr uint32_t CHILD_MASK = (1u << CHILD_SHIFT) - 1u;
 constexpr int RADIX_THREADS = 256;            // one radix-sort tile: 256 threads x 15 keys
 constexpr int RADIX_ITEMS = 15;
 constexpr int RADIX_TILE = RADIX_THREADS * RADIX_ITEMS;
-constexpr int DEPTH_BINS = 8192;              // bins of the depth keys' histogram (k_depth.cu)
+constexpr int DEPTH_BINS = 4096;              // bins of the depth keys' histogram (k_depth.cu)
 
 // flags in Counters::flags
 enum : uint32_t {
@@ -44,6 +44,23 @@ enum : uint32_t {
 enum : int { TK_COMPACT = 0, TK_PRE = 1, TK_EMIT = 2, TK_SORT0 = 3 /* .. TK_SORT0 + 7 */, TK_COUNT = 12 };
 
 struct Counters;
+
+constexpr uint32_t EMIT_SLOTS = 1024;  // pair slots per emission chunk
+
+// Record each multiple of EMIT_SLOTS in a Gaussian's slots [off, off + c): the
+// depth rank that owns the first slot of that chunk.
+__device__ __forceinline__ void emit_owner(uint32_t* owner, uint32_t cap_owner, uint32_t off, uint32_t c,
+                                           uint32_t rank) {
+    const uint64_t end = (uint64_t)off + c;
+    for (uint64_t k = ((uint64_t)off + EMIT_SLOTS - 1u) / EMIT_SLOTS; k * EMIT_SLOTS < end && k < cap_owner; ++k)
+        owner[k] = rank;
+}
+
+// Candidate tiles of an entry in one word: x0 | y0 << 10 | width << 20 (an
+// image has at most 2^10 tiles a side); the height is the count / width.
+__device__ __forceinline__ uint32_t pack_rect(int x0, int y0, int x1) {
+    return (uint32_t)x0 | ((uint32_t)y0 << 10) | ((uint32_t)(x1 - x0 + 1) << 20);
+}
 
 // Monotone map from depth keys to bins: half of the bins logarithmic in z
 // (the key's bits rise like log2 z), half linear, over the depths the scene's
@@ -82,8 +99,7 @@ struct FrameParams {
     // reaches every view's through these)
     const uint2* bl_ranges;      // [tiles] pair range of each tile
     const uint32_t* bl_pair_val; // sorted pair values (in-front index << 8 | row mask)
-    const float4* bl_recA;
-    const float4* bl_recB;
+    const float4* bl_rec;        // 2 per entry
     const float4* bl_rgb;
     const float* bl_lut;         // Eq. 5 table (m + 1 entries)
     float* bl_image;             // H x W x 3

@@ -77,16 +77,19 @@ uint32_t cut_compact_tile_words();
 struct VisBuffers {
     uint32_t* depth;
     uint32_t* ntile;
-    uint2* rect;
-    float4* recA;   // u v A B   (rho = A dx^2 + B dx dy + C dy^2)
-    float4* recB;   // C thr theta, and the footprint box's half-height | half-width << 16 (FP16 bits, rounded up)
-    float4* rgb;    // r g b 0
+    // 2 float4 per entry, one 32-byte sector: u v A B (rho = A dx^2 + B dx dy + C dy^2), then C, thr, the candidate
+    // tiles (pack_rect) and the footprint box's half-height | half-width << 16 (FP16 bits, rounded up)
+    float4* rec;
+    float4* rgb;    // r g b theta
     float* lw;      // parent weight of the interpolated Gaussian (weight interpolation only)
 };
 void launch_preprocess(const SceneDev& sc, const uint32_t* front, const uint32_t* n_front, uint32_t cap,
                        const FrameParams* fp, VisBuffers vis, Counters* ctr, uint32_t* depth_bins, bool interp,
                        int grid, cudaStream_t s);
 uint32_t preprocess_tile();
+// The records of n entries as vgr_debug_buffers lays them out
+void launch_debug_records(const VisBuffers& vis, uint32_t n, uint2* rect, float4* recA, float4* recB, float4* rgb,
+                          cudaStream_t s);
 void prepare_scene(float4* covB, uint32_t n, cudaStream_t s);
 void prepare_scene_half(float4* covB, uint32_t n, cudaStream_t s);
 
@@ -97,7 +100,7 @@ uint32_t depth_bucket_cap(uint32_t cap_vis);  // bucket ids a frame of cap_vis e
 cudaError_t depth_sort_init();                // once per device: the kernels' shared-memory limits
 void launch_depth_sort(const VisBuffers& vis, uint32_t cap_vis, const uint32_t* bins, uint32_t* bstart,
                        unsigned long long* cursor, uint2* part, uint32_t* order, uint32_t* slot_off,
-                       uint64_t cap_pairs, Counters* ctr, const FrameParams* fp, int sms, cudaStream_t s);
+                       uint32_t* owner, uint64_t cap_pairs, Counters* ctr, const FrameParams* fp, int sms, cudaStream_t s);
 
 // k_sort.cu
 uint32_t radix_tile();
@@ -112,12 +115,12 @@ void launch_radix_pass(const uint32_t* keys_in, const uint32_t* vals_in, uint32_
 // k_emit.cu
 // slot offsets in depth order, into slot_off[cap_vis + 1], after a radix depth sort
 void launch_slot_scan(const uint32_t* order, uint32_t cap_vis, const VisBuffers& vis, uint32_t* slot_off,
-                      uint64_t cap_pairs, unsigned long long* status, Counters* ctr, const FrameParams* fp, int grid,
+                      uint32_t* owner, uint64_t cap_pairs, unsigned long long* status, Counters* ctr, const FrameParams* fp, int grid,
                       cudaStream_t s);
-void launch_emit(const uint32_t* order, uint32_t cap_vis, VisBuffers vis, uint32_t* slot_off, uint32_t* pair_key,
-                 uint32_t* pair_val, uint64_t cap_pairs, int tile_passes, uint32_t sentinel,
-                 Counters* ctr, const FrameParams* fp, int grid, cudaStream_t s);
-uint32_t emit_tile();
+uint32_t emit_owner_cap(uint64_t cap_pairs);  // entries of the owner table (first rank of each emission chunk)
+void launch_emit(const uint32_t* order, uint32_t cap_vis, const VisBuffers& vis, const uint32_t* slot_off,
+                 const uint32_t* owner, uint32_t* pair_key, uint32_t* pair_val, uint64_t cap_pairs, int tile_passes,
+                 uint32_t sentinel, Counters* ctr, const FrameParams* fp, int grid, cudaStream_t s);
 uint32_t slot_scan_tile();
 void launch_tile_order(uint2* ranges, uint32_t n_tiles, uint32_t* order, Counters* ctr, cudaStream_t s);
 constexpr uint32_t BATCH_VIEWS_MAX = 1024;  // views of one batch blend (k_batch_offsets: one thread each)
