@@ -15,17 +15,18 @@
 //    reserved with one atomic per CTA and bucket; the same atomic adds up the
 //    bucket's candidate slots;
 //  * k_depth_local gives each bucket to one CTA: a counting sort by 4096
-//    sub-bins of the bucket's own key range in shared memory leaves runs of
-//    one or two keys, whose members rank themselves by (key, index); a bucket
-//    with a long run (many equal keys) is sorted by a bitonic network instead.
+//    sub-bins of the bucket's bins (finer steps of the same monotone function)
+//    in shared memory leaves runs of one or two keys, whose members rank
+//    themselves by (key, index); a bucket with a long run (many equal keys) is
+//    sorted by a bitonic network instead.
 //    The slot counts travel with the keys, so the CTA also writes the first
 //    slot of each of its Gaussians (the sum of the earlier buckets' slots plus
 //    a scan of its own).
 // Four stable radix passes and a scan of the slot counts did this before; each
 // pass was a chain of look-back round trips (15-21 us for 550K keys whatever
 // the traffic).  Depth order and slots, 1M-leaf box at 1080p (552K visible):
-// 96 -> 29 us; city at 1080p (2.67M visible): 153 -> 79 us.  Bound now by the
-// shared-memory atomics and barriers of a CTA's steps (issue slots 35-45 %).
+// 96 -> 26 us; city at 1080p (2.67M visible): 153 -> 67 us.  Bound now by the
+// shared-memory atomics and barriers of a CTA's steps (issue slots 35-50 %).
 // A bucket that does not fit a CTA (F_SORT_SKEW: thousands of Gaussians in one
 // bin) makes the host replay the frame with the radix passes of k_sort.cu.
 #include "vgr_internal.cuh"
@@ -43,7 +44,8 @@ static_assert(DP_BPT % 4 == 0, "bins are read as uint4");
 
 constexpr int DL_THREADS = 512;
 constexpr int DL_WARPS = DL_THREADS / 32;
-constexpr uint32_t DL_CAP = 8192;       // keys of a bucket sorted in shared memory
+constexpr uint32_t DL_CAP = 6144;       // keys of a bucket sorted in shared memory
+constexpr uint32_t DL_CAP_P2 = 8192;    // the bitonic network's size for DL_CAP keys
 constexpr int DL_ITEMS = DL_CAP / DL_THREADS;
 constexpr uint32_t DL_SUB_BITS = 12, DL_SUB = 1u << DL_SUB_BITS;
 constexpr uint32_t DL_RUN_MAX = 48;     // longest run ranked by comparing its members
@@ -65,7 +67,7 @@ uint32_t depth_bucket_cap(uint32_t cap_vis) {
 __global__ void __launch_bounds__(DP_THREADS, 2) k_depth_part(const uint32_t* __restrict__ depth,
                                                               const uint32_t* __restrict__ ntile, uint32_t cap,
                                                               const uint32_t* __restrict__ bins,
-                                                              uint32_t* __restrict__ bstart,
+                                                              uint2* __restrict__ bstart,
                                                               unsigned long long* __restrict__ cursor,
                                                               uint2* __restrict__ part, uint32_t cap_buckets,
                                                               Counters* __restrict__ ctr,
@@ -76,7 +78,7 @@ __global__ void __launch_bounds__(DP_THREADS, 2) k_depth_part(const uint32_t* __
     uint32_t* s_start = sm + DEPTH_BINS / 2;               // [nb + 1] first position of each bucket
     uint32_t* s_base = s_start + cap_buckets + 1;          // [nb] keys of this tile, then their first position
     uint32_t* s_slot = s_base + cap_buckets;               // [nb] candidate slots of this tile
-    __shared__ uint32_t s_scan[DP_THREADS / 32 + 1];
+    __shared__ uint32_t s_scan[DP_THREADS / 32];
     __shared__ uint32_t s_last[DP_THREADS];
     const uint32_t t = threadIdx.x;
     const uint32_t n = min(ctr->n_front, cap);
@@ -115,20 +117,23 @@ __global__ void __launch_bounds__(DP_THREADS, 2) k_depth_part(const uint32_t* __
         for (int k = 0; k < DP_BPT; ++k) {
             const uint32_t b = min(pre >> q, nb - 1u);
             s_bucket[t * DP_BPT + k] = (uint16_t)b;
-            while (id != b) s_start[++id] = pre;
+            while (id != b) {
+                s_start[++id] = pre;
+                if (blockIdx.x == 0) bstart[id] = make_uint2(pre, t * DP_BPT + k);
+            }
             pre += c[k];
         }
         if (t == DP_THREADS - 1)
-            while (id != nb) s_start[++id] = total;
+            while (id != nb) {
+                s_start[++id] = total;
+                if (blockIdx.x == 0) bstart[id] = make_uint2(total, DEPTH_BINS);
+            }
     }
     for (uint32_t b = t; b < nb; b += DP_THREADS) s_base[b] = s_slot[b] = 0u;
     __syncthreads();
     if (blockIdx.x == 0) {
         bool skew = false;
-        for (uint32_t b = t; b <= nb; b += DP_THREADS) {
-            bstart[b] = s_start[b];
-            skew = skew || (b < nb && s_start[b + 1] - s_start[b] > DL_CAP);
-        }
+        for (uint32_t b = t; b < nb; b += DP_THREADS) skew = skew || s_start[b + 1] - s_start[b] > DL_CAP;
         if (skew) atomicOr(&ctr->flags, F_SORT_SKEW);
     }
     for (uint32_t base = first;;) {
@@ -185,71 +190,66 @@ __device__ __forceinline__ unsigned long long warp_sum64(unsigned long long v) {
 }
 
 __global__ void __launch_bounds__(DL_THREADS, 2) k_depth_local(const uint2* __restrict__ part,
-                                                               const uint32_t* __restrict__ bstart,
+                                                               const uint2* __restrict__ bstart,
                                                                const unsigned long long* __restrict__ cursor,
                                                                const uint32_t* __restrict__ ntile, uint32_t cap_vis,
                                                                uint32_t* __restrict__ order,
                                                                uint32_t* __restrict__ off,
                                                                uint32_t* __restrict__ owner, uint64_t cap_pairs,
-                                                               Counters* __restrict__ ctr) {
+                                                               Counters* __restrict__ ctr,
+                                                               const FrameParams* __restrict__ fp) {
     pdl_wait();
-    extern __shared__ uint2 s_kv[];                                  // [DL_CAP] the bucket, by sub-bin
+    extern __shared__ uint2 s_kv[];                                  // [DL_CAP] the bucket by sub-bin, then first slots
+    uint32_t* s_off = reinterpret_cast<uint32_t*>(s_kv);
     uint32_t* s_sub = reinterpret_cast<uint32_t*>(s_kv + DL_CAP);    // [DL_SUB + 1] counts, then first places
     uint4* s_sub4 = reinterpret_cast<uint4*>(s_sub);
-    uint32_t* s_fin = s_sub + DL_SUB + 1;                            // [DL_CAP] index << 8 | slots, in order
-    __shared__ uint32_t s_scan[DL_WARPS + 1];
-    __shared__ uint32_t s_min[DL_WARPS], s_max[DL_WARPS];
+    uint32_t* s_fin = s_sub + DL_SUB + 4;                            // [DL_CAP] index << 8 | slots, in order
+    __shared__ uint32_t s_scan[DL_WARPS], s_scan2[DL_WARPS];
     __shared__ unsigned long long s_sum[DL_WARPS];
     const uint32_t t = threadIdx.x, lane = lane_id(), warp = t >> 5;
     if (ctr->flags & F_SORT_SKEW) return;
+    const DepthMap map = fp->depth;
     const uint32_t n_vis = min(ctr->n_vis, cap_vis);
     const uint32_t nb = depth_buckets(n_vis);
+    const uint32_t cap_owner = (uint32_t)(cap_pairs / EMIT_SLOTS) + 1u;
+    auto slots_of = [&](uint32_t v) -> uint32_t { return (v & 255u) < 255u ? v & 255u : ntile[v >> 8]; };
+#pragma unroll
+    for (int k = 0; k < DL_SPT / 4; ++k) s_sub4[k * DL_THREADS + t] = make_uint4(0u, 0u, 0u, 0u);
+    __syncthreads();
     unsigned long long slots = 0ull;  // candidate slots of the buckets before b
     uint32_t seen = 0;
     for (uint32_t b = blockIdx.x; b < nb; b += gridDim.x) {
-        const uint32_t start = bstart[b], n = min(bstart[b + 1] - start, DL_CAP);
+        const uint2 bs = bstart[b], be = bstart[b + 1];  // (first position, first bin)
+        const uint32_t start = bs.x, n = min(be.x - bs.x, DL_CAP);
+        if (n == 0u && b + 1u < nb) continue;
+        // sub-bins: equal steps of the bin coordinate over the bucket's bins
+        const float c0 = (float)bs.y, cs = __fdividef((float)DL_SUB, (float)max(be.y - bs.y, 1u));
+        auto sub_of = [&](uint32_t key) -> uint32_t {
+            return min(__float2uint_rz(__fmul_rn(__fsub_rn(depth_coord(map, key), c0), cs)), DL_SUB - 1u);
+        };
         uint2 e[DL_ITEMS];
-        uint32_t lo = NONE, hi = 0u;
+        uint32_t place[DL_ITEMS];  // sub-bin << 16 | place in it, in any order
 #pragma unroll
         for (int k = 0; k < DL_ITEMS; ++k) {
             const uint32_t j = k * DL_THREADS + t;
             if (k * DL_THREADS >= n) break;
-            if (j < n) {
-                e[k] = part[start + j];
-                lo = min(lo, e[k].x);
-                hi = max(hi, e[k].x);
-            }
+            if (j < n) e[k] = part[start + j];
         }
         unsigned long long sum = 0ull;
         for (uint32_t p = seen + t; p < b; p += DL_THREADS) sum += cursor[p] >> 32;
         seen = b;
 #pragma unroll
-        for (int k = 0; k < DL_SPT / 4; ++k) s_sub4[k * DL_THREADS + t] = make_uint4(0u, 0u, 0u, 0u);
-        lo = __reduce_min_sync(0xFFFFFFFFu, lo);
-        hi = __reduce_max_sync(0xFFFFFFFFu, hi);
-        sum = warp_sum64(sum);
-        if (lane == 0) {
-            s_min[warp] = lo;
-            s_max[warp] = hi;
-            s_sum[warp] = sum;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int w = 0; w < DL_WARPS; ++w) {
-            lo = min(lo, s_min[w]);
-            hi = max(hi, s_max[w]);
-            slots += s_sum[w];
-        }
-        const uint32_t bits = n ? 32u - __clz(hi - lo) : 0u;  // __clz(0) is 32
-        const uint32_t sh = bits > DL_SUB_BITS ? bits - DL_SUB_BITS : 0u;
-        // counting sort by sub-bin, in any order within one
-        uint32_t place[DL_ITEMS];
-#pragma unroll
         for (int k = 0; k < DL_ITEMS; ++k) {
             if (k * DL_THREADS >= n) break;
-            if (k * DL_THREADS + t < n) place[k] = atomicAdd(&s_sub[(e[k].x - lo) >> sh], 1u);
+            if (k * DL_THREADS + t < n) {
+                const uint32_t sub = sub_of(e[k].x);
+                place[k] = sub << 16 | atomicAdd(&s_sub[sub], 1u);
+            }
         }
+        sum = warp_sum64(sum);
+        if (lane == 0) s_sum[warp] = sum;
         __syncthreads();
+        // first place of each sub-bin
         bool longrun = false;
         {
             uint32_t c[DL_SPT], s = 0, total;
@@ -275,17 +275,20 @@ __global__ void __launch_bounds__(DL_THREADS, 2) k_depth_local(const uint2* __re
             }
             if (t == 0) s_sub[DL_SUB] = n;
         }
+#pragma unroll
+        for (int w = 0; w < DL_WARPS; ++w) slots += s_sum[w];
         longrun = __syncthreads_or(longrun);
 #pragma unroll
         for (int k = 0; k < DL_ITEMS; ++k) {
             if (k * DL_THREADS >= n) break;
-            if (k * DL_THREADS + t < n) s_kv[s_sub[(e[k].x - lo) >> sh] + place[k]] = e[k];
+            if (k * DL_THREADS + t < n) s_kv[s_sub[place[k] >> 16] + (place[k] & 0xFFFFu)] = e[k];
         }
+        __syncthreads();
         if (!longrun) {
-            __syncthreads();
+            // the members of a run (a sub-bin) rank themselves by (key, index)
             for (uint32_t j = t; j < n; j += DL_THREADS) {
                 const uint2 kv = s_kv[j];
-                const uint32_t sub = (kv.x - lo) >> sh;
+                const uint32_t sub = sub_of(kv.x);
                 const uint32_t r0 = s_sub[sub], r1 = s_sub[sub + 1];
                 uint32_t at = r0;
                 if (r1 - r0 > 1u)
@@ -298,7 +301,7 @@ __global__ void __launch_bounds__(DL_THREADS, 2) k_depth_local(const uint2* __re
         } else {
             // many equal keys: a bitonic network over (key, index), padded with all ones
             uint32_t p2 = 1;
-            while (p2 < n) p2 <<= 1;
+            while (p2 < n) p2 <<= 1;  // at most DL_CAP_P2: the padding may cover s_sub, which is done with
             for (uint32_t j = n + t; j < p2; j += DL_THREADS) s_kv[j] = make_uint2(NONE, NONE);
             for (uint32_t k = 2; k <= p2; k <<= 1)
                 for (uint32_t d = k >> 1; d > 0; d >>= 1) {
@@ -317,42 +320,23 @@ __global__ void __launch_bounds__(DL_THREADS, 2) k_depth_local(const uint2* __re
             for (uint32_t j = t; j < n; j += DL_THREADS) s_fin[j] = s_kv[j].y;
         }
         __syncthreads();
-        // write the order and the first slots: warp w takes the rows of 32 from w R on
-        const uint32_t R = ((n + 31u) / 32u + DL_WARPS - 1u) / DL_WARPS;  // at most DL_ITEMS
-        const uint32_t cap_owner = (uint32_t)(cap_pairs / EMIT_SLOTS) + 1u;
-        auto slots_of = [&](uint32_t v) -> uint32_t { return (v & 255u) < 255u ? v & 255u : ntile[v >> 8]; };
-        uint32_t x[DL_ITEMS], carry = 0;
-#pragma unroll
-        for (int r = 0; r < DL_ITEMS; ++r) {
-            if (r >= R) break;
-            {
-                const uint32_t j = (warp * R + r) * 32u + lane;
-                uint32_t rowsum;
-                x[r] = carry + warp_excl_scan(j < n ? slots_of(s_fin[j]) : 0u, &rowsum);
-                carry += rowsum;
-            }
+        // first slots: each thread an odd number of neighbours (no bank conflicts)
+        const uint32_t per = ((n + DL_THREADS - 1u) / DL_THREADS) | 1u, jb = t * per, je = min(jb + per, n);
+        uint32_t mine = 0, all;
+        for (uint32_t j = jb; j < je; ++j) mine += slots_of(s_fin[j]);
+        uint32_t run = (uint32_t)slots + block_excl_scan<DL_WARPS>(mine, s_scan2, &all);
+        for (uint32_t j = jb; j < je; ++j) {
+            const uint32_t c = slots_of(s_fin[j]);
+            s_off[j] = run;
+            emit_owner(owner, cap_owner, run, c, start + j);
+            run += c;
         }
-        if (lane == 0) s_scan[warp] = carry;
+#pragma unroll
+        for (int k = 0; k < DL_SPT / 4; ++k) s_sub4[k * DL_THREADS + t] = make_uint4(0u, 0u, 0u, 0u);
         __syncthreads();
-        uint32_t mine = (uint32_t)slots, all = 0;
-#pragma unroll
-        for (int w = 0; w < DL_WARPS; ++w) {
-            const uint32_t v = s_scan[w];
-            mine += (uint32_t)w < warp ? v : 0u;
-            all += v;
-        }
-#pragma unroll
-        for (int r = 0; r < DL_ITEMS; ++r) {
-            if (r >= R) break;
-            {
-                const uint32_t j = (warp * R + r) * 32u + lane;
-                if (j < n) {
-                    const uint32_t v = s_fin[j], o = mine + x[r];
-                    order[start + j] = v >> 8;
-                    off[start + j] = o;
-                    emit_owner(owner, cap_owner, o, slots_of(v), start + j);
-                }
-            }
+        for (uint32_t j = t; j < n; j += DL_THREADS) {
+            order[start + j] = s_fin[j] >> 8;
+            off[start + j] = s_off[j];
         }
         if (b == nb - 1u && t == 0) {
             const unsigned long long ns = slots + all;
@@ -360,11 +344,12 @@ __global__ void __launch_bounds__(DL_THREADS, 2) k_depth_local(const uint2* __re
             ctr->n_cand = ns;
             if (ns > cap_pairs) atomicOr(&ctr->flags, F_OVF_PAIRS);
         }
-        __syncthreads();  // the shared buffers are rewritten by the next bucket
+        // (the next bucket writes s_kv and s_fin only after barriers that follow these reads)
     }
 }
 
-size_t depth_local_smem() { return DL_CAP * sizeof(uint2) + (DL_SUB + 1 + DL_CAP) * sizeof(uint32_t); }
+size_t depth_local_smem() { return DL_CAP * sizeof(uint2) + (DL_SUB + 4 + DL_CAP) * sizeof(uint32_t); }
+static_assert(DL_CAP * 8 + (DL_SUB + 4) * 4 >= DL_CAP_P2 * 8, "the bitonic network fits in s_kv and s_sub");
 size_t depth_part_smem(uint32_t cap_buckets) {
     return DEPTH_BINS * sizeof(uint16_t) + (3 * (size_t)cap_buckets + 1) * sizeof(uint32_t);
 }
@@ -378,15 +363,16 @@ cudaError_t depth_sort_init() {
     return e;
 }
 
-void launch_depth_sort(const VisBuffers& vis, uint32_t cap_vis, const uint32_t* bins, uint32_t* bstart,
+void launch_depth_sort(const VisBuffers& vis, uint32_t cap_vis, const uint32_t* bins, uint2* bstart,
                        unsigned long long* cursor, uint2* part, uint32_t* order, uint32_t* slot_off,
                        uint32_t* owner, uint64_t cap_pairs, Counters* ctr, const FrameParams* fp, int sms, cudaStream_t s) {
     const uint32_t cap = cap_vis < MAX_RANKS ? cap_vis : MAX_RANKS;
     const uint32_t cb = depth_bucket_cap(cap);
     launch_ks(k_depth_part, 2 * sms, DP_THREADS, depth_part_smem(cb), s, (const uint32_t*)vis.depth,
               (const uint32_t*)vis.ntile, cap, bins, bstart, cursor, part, cb, ctr, fp);
-    launch_ks(k_depth_local, 2 * sms, DL_THREADS, depth_local_smem(), s, (const uint2*)part, (const uint32_t*)bstart,
-              (const unsigned long long*)cursor, (const uint32_t*)vis.ntile, cap, order, slot_off, owner, cap_pairs, ctr);
+    launch_ks(k_depth_local, 2 * sms, DL_THREADS, depth_local_smem(), s, (const uint2*)part, (const uint2*)bstart,
+              (const unsigned long long*)cursor, (const uint32_t*)vis.ntile, cap, order, slot_off, owner, cap_pairs, ctr,
+              fp);
 }
 
 }  // namespace vgr

@@ -29,6 +29,13 @@
 
 namespace vgr {
 
+constexpr int CC_TILE_WORDS = 256;             // bitmap words per tile of the compaction
+constexpr int CC_TILE_IDS = CC_TILE_WORDS * 32;
+// words between the tiles' counters: a line each, since the warps in flight
+// count into neighbouring tiles (in one line their atomics queue at one L2
+// slice: +24 us on the city)
+constexpr int CC_COUNT_STRIDE = 32;
+
 // A cut node joins the cut bitmap, and the potentially-visible bitmap when
 // its FP32 depth key is beyond the near plane (the same key and test as
 // preprocess) and its footprint can reach the image.  The footprint test is
@@ -64,6 +71,7 @@ __device__ __forceinline__ void warp_bitmap_set(uint32_t* bm, uint32_t n, bool p
 struct CutOut {
     uint32_t* cut_bm;
     uint32_t* front_bm;
+    uint32_t* counts;  // bits set per bitmap tile: cut | in front << 16
     const float* lmax;
     const float4* cr;
     const uint32_t* parent;
@@ -71,9 +79,32 @@ struct CutOut {
     float fx, fy, cx, cy, kx, ky, umax, vmax;
     bool canonical;
     bool interp;  // weight interpolation: bound the interpolated Gaussian, not the node's own
-    __device__ __forceinline__ void add(uint32_t n, float4 c) const {
-        bitmap_set(cut_bm, n);
-        if (visible(n, c, lmax[n])) bitmap_set(front_bm, n);
+    // an ancestor that several nodes may report: the one that sets a bit counts it
+    __device__ __forceinline__ void add_shared(uint32_t n, float4 c) const {
+        const uint32_t bit = 1u << (n & 31u);
+        uint32_t fresh = (atomicOr(&cut_bm[n >> 5], bit) & bit) ? 0u : 1u;
+        if (visible(n, c, lmax[n]) && !(atomicOr(&front_bm[n >> 5], bit) & bit)) fresh |= 1u << 16;
+        if (fresh) atomicAdd(&counts[n / CC_TILE_IDS * CC_COUNT_STRIDE], fresh);
+    }
+    // a node that only this thread reports; its counts are held back in
+    // (tile, held) while the thread stays in one tile (a subtree's nodes do)
+    __device__ __forceinline__ void add(uint32_t n, float4 c, uint32_t& tile, uint32_t& held) const {
+        const uint32_t bit = 1u << (n & 31u);
+        atomicOr(&cut_bm[n >> 5], bit);
+        uint32_t one = 1u;
+        if (visible(n, c, lmax[n])) {
+            atomicOr(&front_bm[n >> 5], bit);
+            one |= 1u << 16;
+        }
+        if (n / CC_TILE_IDS != tile) {
+            flush(tile, held);
+            tile = n / CC_TILE_IDS;
+        }
+        held += one;
+    }
+    __device__ __forceinline__ void flush(uint32_t tile, uint32_t& held) const {
+        if (held) atomicAdd(&counts[tile * CC_COUNT_STRIDE], held);
+        held = 0u;
     }
     // may the Gaussian rendered for cut node n (centre c, lm = lmax[n]) reach the image?
     __device__ __forceinline__ bool visible(uint32_t n, float4 c, float lm) const {
@@ -141,10 +172,40 @@ struct CutOut {
     }
 };
 
+// Count the warp's nodes n[0..U) that join the cut (and of those the ones in
+// front) per bitmap tile: one atomic per tile, and a warp's nodes are mostly in
+// one.  All 32 lanes call it; every node is reported once.
+template <int U>
+__device__ __forceinline__ void warp_tile_count(uint32_t* counts, const uint32_t* n, const bool* in_cut,
+                                                const bool* in_front) {
+    uint32_t left[U], vis[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        left[u] = __ballot_sync(0xFFFFFFFFu, in_cut[u]);
+        vis[u] = __ballot_sync(0xFFFFFFFFu, in_front[u]);
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        while (left[u]) {  // uniform: every lane takes part in every shuffle and ballot
+            const int lead = __ffs(left[u]) - 1;
+            const uint32_t tile = __shfl_sync(0xFFFFFFFFu, n[u] / CC_TILE_IDS, lead);
+            uint32_t c = 0;
+#pragma unroll
+            for (int v = u; v < U; ++v) {
+                const uint32_t same = __ballot_sync(0xFFFFFFFFu, n[v] / CC_TILE_IDS == tile) & left[v];
+                left[v] &= ~same;
+                c += (uint32_t)__popc(same) | ((uint32_t)__popc(vis[v] & same) << 16);
+            }
+            if ((int)lane_id() == lead) atomicAdd(&counts[tile * CC_COUNT_STRIDE], c);
+        }
+    }
+}
+
 template <bool IP>
 __device__ __forceinline__ CutOut make_cut_out(const FrameParams* fp, const SceneDev& sc, uint32_t* cut_bm,
-                                               uint32_t* front_bm) {
+                                               uint32_t* front_bm, uint32_t* counts) {
     CutOut o;
+    o.counts = counts;
     o.cut_bm = cut_bm;
     o.front_bm = front_bm;
     o.lmax = sc.lmax;
@@ -172,12 +233,12 @@ __global__ void __launch_bounds__(256) k_lod_update(const uint32_t* __restrict__
                                                     const uint32_t* __restrict__ n_prev_p, uint32_t cap_prev,
                                                     SceneDev sc, const FrameParams* __restrict__ fp,
                                                     uint32_t* __restrict__ bitmap, uint32_t* __restrict__ front,
-                                                    Counters* __restrict__ ctr) {
+                                                    uint32_t* __restrict__ counts, Counters* __restrict__ ctr) {
     pdl_wait();
     const uint32_t n_prev = min(*n_prev_p, cap_prev);
     const float px = fp->pos[0], py = fp->pos[1], pz = fp->pos[2], k = fp->k;
     const uint32_t budget = fp->lod_budget, max_depth = fp->max_depth;
-    const CutOut out = make_cut_out<IP>(fp, sc, bitmap, front);
+    const CutOut out = make_cut_out<IP>(fp, sc, bitmap, front, counts);
     LodFrustum fr;
     if (FR) fr.load(fp, sc.box);
     // the granularity test, and in the frustum-aware variant the box test
@@ -214,7 +275,7 @@ __global__ void __launch_bounds__(256) k_lod_update(const uint32_t* __restrict__
                 ca = cpa;
                 if (steps > max_depth) { flags |= F_LOD_FALLBACK; break; }
             }
-            out.add(a, ca);
+            out.add_shared(a, ca);
         } else if (en) {
             // expand: depth-first over n's subtree, children ranges on a stack
             uint32_t nxt[MAX_TREE_DEPTH], end[MAX_TREE_DEPTH];
@@ -222,7 +283,7 @@ __global__ void __launch_bounds__(256) k_lod_update(const uint32_t* __restrict__
             nxt[0] = c0 & CHILD_MASK;
             end[0] = nxt[0] + (c0 >> CHILD_SHIFT);
             int sp = 1;
-            uint32_t local = 0;
+            uint32_t local = 0, tile = NONE, held = 0;
             while (sp > 0) {
                 if (nxt[sp - 1] == end[sp - 1]) { --sp; continue; }
                 const uint32_t m = nxt[sp - 1]++;
@@ -235,9 +296,10 @@ __global__ void __launch_bounds__(256) k_lod_update(const uint32_t* __restrict__
                     end[sp] = nxt[sp] + (chm >> CHILD_SHIFT);
                     ++sp;
                 } else {
-                    out.add(m, cm);
+                    out.add(m, cm, tile, held);
                 }
             }
+            out.flush(tile, held);
             evals += local;
         } else {
             return true;  // stay
@@ -258,7 +320,7 @@ __global__ void __launch_bounds__(256) k_lod_update(const uint32_t* __restrict__
         uint32_t nn[LOD_UNROLL], pp[LOD_UNROLL];
         float4 cc[LOD_UNROLL], qq[LOD_UNROLL];
         float ll[LOD_UNROLL];
-        bool ok[LOD_UNROLL];
+        bool ok[LOD_UNROLL], in_cut[LOD_UNROLL], in_front[LOD_UNROLL];
 #pragma unroll
         for (int u = 0; u < LOD_UNROLL; ++u) {
             const uint32_t i = b0 + u * stride + lane;
@@ -284,7 +346,10 @@ __global__ void __launch_bounds__(256) k_lod_update(const uint32_t* __restrict__
                 else vis = out.in_front_segment(cc[u], ll[u], qq[u], sc.lmax[pp[u]]);
             }
             warp_bitmap_set(front, nn[u], vis);
+            in_cut[u] = stay;
+            in_front[u] = vis;
         }
+        warp_tile_count<LOD_UNROLL>(counts, nn, in_cut, in_front);
     }
     // one atomic per warp for the statistics
     uint32_t wsum = __reduce_add_sync(0xFFFFFFFFu, evals);
@@ -301,12 +366,12 @@ __global__ void __launch_bounds__(256) k_lod_level(int level, const uint32_t* __
                                                    uint32_t* __restrict__ fout, uint32_t cap, SceneDev sc,
                                                    const FrameParams* __restrict__ fp,
                                                    uint32_t* __restrict__ bitmap, uint32_t* __restrict__ front,
-                                                   Counters* __restrict__ ctr) {
+                                                   uint32_t* __restrict__ counts, Counters* __restrict__ ctr) {
     pdl_wait();
     const uint32_t n_in = level == 0 ? 1u : min(ctr->frontier_n[level], cap);
     uint32_t* n_out = &ctr->frontier_n[level + 1];
     const float px = fp->pos[0], py = fp->pos[1], pz = fp->pos[2], k = fp->k;
-    const CutOut out = make_cut_out<IP>(fp, sc, bitmap, front);
+    const CutOut out = make_cut_out<IP>(fp, sc, bitmap, front, counts);
     LodFrustum fr;
     if (FR) fr.load(fp, sc.box);
     const uint32_t lane = lane_id();
@@ -334,6 +399,7 @@ __global__ void __launch_bounds__(256) k_lod_level(int level, const uint32_t* __
         // one atomic per bitmap word and warp (a node's siblings are neighbours)
         warp_bitmap_set(bitmap, n, is_cut);
         warp_bitmap_set(front, n, in_front);
+        warp_tile_count<1>(counts, &n, &is_cut, &in_front);
         uint32_t total;
         const uint32_t off = warp_excl_scan(cnt, &total);
         uint32_t basepos = 0;
@@ -350,116 +416,99 @@ __global__ void __launch_bounds__(256) k_lod_level(int level, const uint32_t* __
 }
 
 // Bitmaps -> ascending id lists (the cut, and its in-front part), clearing
-// both bitmaps for the next frame.  Tiles of 256 threads x 4 words; two
-// decoupled look-back chains (warp 0: cut, warp 1: in-front) give each tile
-// its output offsets.  A warp owns 128 contiguous words of the tile and takes
-// them in four rounds of 32 (lane l holds word 32 j + l of round j, so every
-// load is coalesced): a shuffle scan of the words' bit counts places each
-// lane's ids in the warp's staging buffer in shared memory, and the warp then
-// stores the round's ids contiguously (coalesced) -- no serial per-word loop.
+// both bitmaps for the next frame.  The LoD kernels count the bits they set per
+// tile of 256 words, so a tile's place in the lists is the sum of the counts
+// before it: no count is waited for, and the CTAs take tiles in any order.  A
+// warp takes a row of 32 words: a scan of their bit counts gives every word its
+// place, and the warp goes through the words that have bits, lane l storing the
+// id of bit l if it is set (contiguous stores, no barrier, no staging).  Bound by
+// those instructions and, on small scenes, by the kernel's three round trips.
+// Tiles of 1024 words on a look-back chain, their ids unpacked in shared memory
+// bit by bit, took 28 us on the 1M-leaf box (44 tiles for 152 SMs; now 10) and
+// 41 us on the city (26.5M nodes; now 32, while counting adds 10 to the 119 us
+// of its LoD update).
 constexpr int CC_THREADS = 256;
 constexpr int CC_WARPS = CC_THREADS / 32;
-constexpr int CC_WORDS = 4;  // words per lane = rounds per warp
-constexpr int CC_TILE_WORDS = CC_THREADS * CC_WORDS;
+static_assert(CC_TILE_WORDS == CC_THREADS, "one row of 32 words per warp");
 
-// One round of one bitmap: this lane's word `word` (index `wi`), the round's
-// ids staged in `stage` (32 words x 32 bits at most) and stored from `off`.
-__device__ __forceinline__ uint32_t cc_round(uint32_t word, uint32_t wi, uint32_t off, uint32_t* stage,
-                                             uint32_t* out, uint32_t cap) {
-    const uint32_t lane = lane_id();
-    const uint32_t c = __popc(word);
-    uint32_t incl = c;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, d);
-        if ((int)lane >= d) incl += y;
+// Store the ids of a row's set bits (lane l holds word l, first id id0 + 32 l)
+// from out[at] on.
+__device__ __forceinline__ void cc_row(uint32_t word, uint32_t pre, uint32_t id0, uint32_t* __restrict__ out,
+                                       uint32_t cap) {
+    const uint32_t lane = lane_id(), below = lanemask_lt();
+    uint32_t some = __ballot_sync(0xFFFFFFFFu, word != 0u);
+    if (__popc(some) >= 12) {  // most words have bits: all of them, independent of one another
+#pragma unroll 8
+        for (int w = 0; w < 32; ++w) {
+            const uint32_t bits = __shfl_sync(0xFFFFFFFFu, word, w);
+            const uint32_t p = __shfl_sync(0xFFFFFFFFu, pre, w) + __popc(bits & below);
+            if (((bits >> lane) & 1u) && p < cap) out[p] = id0 + 32u * w + lane;
+        }
+        return;
     }
-    const uint32_t n = __shfl_sync(0xFFFFFFFFu, incl, 31);
-    if (n == 0u) return off;
-    uint32_t p = incl - c;
-    while (word) {
-        stage[p++] = wi * 32u + (uint32_t)(__ffs(word) - 1);
-        word &= word - 1u;
+    while (some) {
+        const int w = __ffs(some) - 1;
+        some &= some - 1u;
+        const uint32_t bits = __shfl_sync(0xFFFFFFFFu, word, w);
+        const uint32_t p = __shfl_sync(0xFFFFFFFFu, pre, w) + __popc(bits & below);
+        if (((bits >> lane) & 1u) && p < cap) out[p] = id0 + 32u * w + lane;
     }
-    __syncwarp();
-    for (uint32_t i = lane; i < n; i += 32u)
-        if (off + i < cap) out[off + i] = stage[i];
-    __syncwarp();  // the buffer is read before the next round writes it
-    return off + n;
 }
 
 __global__ void __launch_bounds__(CC_THREADS) k_cut_compact(uint32_t* __restrict__ bitmap, uint32_t* __restrict__ front,
-                                                            uint32_t n_words, uint32_t* __restrict__ cut,
+                                                            const uint32_t* __restrict__ counts, uint32_t n_words,
+                                                            uint32_t* __restrict__ cut,
                                                             uint32_t* __restrict__ front_list, uint32_t cap,
                                                             uint32_t* __restrict__ n_cut_out,
-                                                            unsigned long long* __restrict__ status,
-                                                            unsigned long long* __restrict__ status_front,
-                                                            Counters* __restrict__ ctr,
-                                                            const FrameParams* __restrict__ fp) {
+                                                            Counters* __restrict__ ctr) {
     pdl_wait();
-    __shared__ uint32_t s_stage[CC_WARPS][32 * 32];
-    __shared__ uint32_t s_wtot[CC_WARPS];
-    __shared__ uint32_t s_tile, s_prefix[2];
-    const uint32_t ntiles = (n_words + CC_TILE_WORDS - 1) / CC_TILE_WORDS;
-    const uint32_t epoch = fp->epoch;
-    const uint32_t warp = threadIdx.x >> 5, lane = lane_id();
-    for (;;) {
-        if (threadIdx.x == 0) s_tile = atomicAdd(&ctr->tickets[TK_COMPACT], 1u);
-        __syncthreads();
-        const uint32_t tile = s_tile;
-        if (tile >= ntiles) break;
-        // the bitmaps are padded to a whole number of tiles
-        const uint32_t wbase = tile * CC_TILE_WORDS + warp * (32u * CC_WORDS);
-        uint32_t a[CC_WORDS], b[CC_WORDS];
-#pragma unroll
-        for (int j = 0; j < CC_WORDS; ++j) {
-            a[j] = bitmap[wbase + 32u * j + lane];
-            b[j] = front[wbase + 32u * j + lane];
+    __shared__ uint2 s_sum[2][CC_WARPS];
+    __shared__ uint32_t s_scan[2][CC_WARPS];
+    const uint32_t ntiles = n_words / CC_TILE_WORDS;  // the bitmaps are padded to whole tiles
+    const uint32_t t = threadIdx.x, warp = t >> 5, lane = lane_id();
+    uint32_t oa = 0, ob = 0, seen = 0, flip = 0;  // ids in the tiles before 'seen'
+    for (uint32_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x, flip ^= 1u) {
+        const uint32_t wi = tile * CC_TILE_WORDS + t;
+        const uint32_t a = bitmap[wi], b = front[wi];
+        uint32_t sa = 0, sb = 0;
+        for (uint32_t j = seen + t; j < tile; j += CC_THREADS) {
+            const uint32_t c = counts[j * CC_COUNT_STRIDE];
+            sa += c & 0xFFFFu;
+            sb += c >> 16;
         }
-        uint32_t cnt = 0;  // both counts packed: at most 32768 each per tile
-#pragma unroll
-        for (int j = 0; j < CC_WORDS; ++j) cnt += __popc(a[j]) | (__popc(b[j]) << 16);
-        cnt = __reduce_add_sync(0xFFFFFFFFu, cnt);
-        if (lane == 0) s_wtot[warp] = cnt;
-        __syncthreads();
-        uint32_t wexcl = 0, total = 0;
+        seen = tile;
+        sa = __reduce_add_sync(0xFFFFFFFFu, sa);
+        sb = __reduce_add_sync(0xFFFFFFFFu, sb);
+        if (lane == 0) s_sum[flip][warp] = make_uint2(sa, sb);
+        uint32_t total;  // both counts packed: at most 8192 each
+        const uint32_t pre = block_excl_scan<CC_WARPS>(__popc(a) | (__popc(b) << 16), s_scan[flip], &total);
 #pragma unroll
         for (int w = 0; w < CC_WARPS; ++w) {
-            const uint32_t v = s_wtot[w];
-            wexcl += (uint32_t)w < warp ? v : 0u;
-            total += v;
+            const uint2 c = s_sum[flip][w];
+            oa += c.x;
+            ob += c.y;
         }
-        if (warp < 2) {
-            const uint32_t agg = warp == 0 ? (total & 0xFFFFu) : (total >> 16);
-            const uint32_t pre = lookback_warp(warp == 0 ? status : status_front, 1, tile, agg, epoch, &ctr->flags);
-            if (lane == 0) s_prefix[warp] = pre;
-        }
-        __syncthreads();
-        uint32_t oa = s_prefix[0] + (wexcl & 0xFFFFu), ob = s_prefix[1] + (wexcl >> 16);
-#pragma unroll
-        for (int j = 0; j < CC_WORDS; ++j) {
-            const uint32_t wi = wbase + 32u * j + lane;
-            oa = cc_round(a[j], wi, oa, s_stage[warp], cut, cap);
-            ob = cc_round(b[j], wi, ob, s_stage[warp], front_list, cap);
-            if (a[j]) bitmap[wi] = 0u;
-            if (b[j]) front[wi] = 0u;
-        }
-        if (tile == ntiles - 1 && threadIdx.x == 0) {
-            const uint32_t n = s_prefix[0] + (total & 0xFFFFu);
+        const uint32_t id0 = (tile * CC_TILE_WORDS + 32u * warp) * 32u;
+        cc_row(a, oa + (pre & 0xFFFFu), id0, cut, cap);
+        cc_row(b, ob + (pre >> 16), id0, front_list, cap);
+        if (a) bitmap[wi] = 0u;
+        if (b) front[wi] = 0u;
+        if (tile == ntiles - 1 && t == 0) {
+            const uint32_t n = oa + (total & 0xFFFFu);
             *n_cut_out = n;
-            ctr->n_front = s_prefix[1] + (total >> 16);
+            ctr->n_front = ob + (total >> 16);
             if (n > cap) atomicOr(&ctr->flags, F_OVF_CUT);
         }
-        __syncthreads();
+        // (the shared words of this tile are written again two barriers from here)
     }
 }
 
 // ------------------------------------------------------------ launchers
 void launch_lod_update(const SceneDev& sc, const uint32_t* prev_cut, const uint32_t* n_prev, uint32_t cap_prev,
-                       const FrameParams* fp, uint32_t* bitmap, uint32_t* front, Counters* ctr, int grid,
+                       const FrameParams* fp, uint32_t* bitmap, uint32_t* front, uint32_t* counts, Counters* ctr, int grid,
                        bool frustum, bool interp, cudaStream_t s) {
 #define VGR_LOD_UPDATE(FR, IP) \
-    launch_k(k_lod_update<FR, IP>, grid, 256, s, prev_cut, n_prev, cap_prev, sc, fp, bitmap, front, ctr)
+    launch_k(k_lod_update<FR, IP>, grid, 256, s, prev_cut, n_prev, cap_prev, sc, fp, bitmap, front, counts, ctr)
     if (frustum) {
         if (interp) VGR_LOD_UPDATE(true, true);
         else VGR_LOD_UPDATE(true, false);
@@ -471,10 +520,10 @@ void launch_lod_update(const SceneDev& sc, const uint32_t* prev_cut, const uint3
 }
 
 void launch_lod_level(int level, const SceneDev& sc, const uint32_t* fin, uint32_t* fout, uint32_t cap,
-                      const FrameParams* fp, uint32_t* bitmap, uint32_t* front, Counters* ctr, int grid,
+                      const FrameParams* fp, uint32_t* bitmap, uint32_t* front, uint32_t* counts, Counters* ctr, int grid,
                       bool frustum, bool interp, cudaStream_t s) {
 #define VGR_LOD_LEVEL(FR, IP) \
-    launch_k(k_lod_level<FR, IP>, grid, 256, s, level, fin, fout, cap, sc, fp, bitmap, front, ctr)
+    launch_k(k_lod_level<FR, IP>, grid, 256, s, level, fin, fout, cap, sc, fp, bitmap, front, counts, ctr)
     if (frustum) {
         if (interp) VGR_LOD_LEVEL(true, true);
         else VGR_LOD_LEVEL(true, false);
@@ -485,15 +534,13 @@ void launch_lod_level(int level, const SceneDev& sc, const uint32_t* fin, uint32
 #undef VGR_LOD_LEVEL
 }
 
-void launch_cut_compact(uint32_t* bitmap, uint32_t* front, uint32_t n_words, uint32_t* cut, uint32_t* front_list,
-                        uint32_t cap, uint32_t* n_cut_out, unsigned long long* status,
-                        unsigned long long* status_front, Counters* ctr, const FrameParams* fp, int grid,
+void launch_cut_compact(uint32_t* bitmap, uint32_t* front, const uint32_t* counts, uint32_t n_words, uint32_t* cut,
+                        uint32_t* front_list, uint32_t cap, uint32_t* n_cut_out, Counters* ctr, int grid,
                         cudaStream_t s) {
-    launch_k(k_cut_compact, grid, CC_THREADS, s, bitmap, front, n_words, cut, front_list, cap, n_cut_out, status,
-                                       status_front, ctr, fp);
+    launch_k(k_cut_compact, grid, CC_THREADS, s, bitmap, front, counts, n_words, cut, front_list, cap, n_cut_out, ctr);
 }
 
-uint32_t cut_compact_tiles(uint32_t n_words) { return (n_words + CC_TILE_WORDS - 1) / CC_TILE_WORDS; }
 uint32_t cut_compact_tile_words() { return CC_TILE_WORDS; }
+uint32_t cut_compact_count_words(uint32_t n_words) { return n_words / CC_TILE_WORDS * CC_COUNT_STRIDE; }
 
 }  // namespace vgr

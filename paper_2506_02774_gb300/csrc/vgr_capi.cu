@@ -156,9 +156,11 @@ struct vgr_view {
     // radix passes use its halves as their key buffers
     uint32_t* sort_kv = nullptr;
     uint32_t* sortV[2] = {nullptr, nullptr};  // sortV[1] receives the order
-    uint32_t* depth_bins = nullptr;           // [DEPTH_BINS], after the counters (one clear per frame)
-    unsigned long long* bucket_cursor = nullptr;  // [depth_bucket_cap], after the bins
-    uint32_t* bucket_start = nullptr;
+    // (these three follow the counters in one allocation: one clear per frame)
+    uint32_t* depth_bins = nullptr;               // [DEPTH_BINS]
+    uint32_t* cut_counts = nullptr;               // bits set per bitmap tile: cut | in front << 16
+    unsigned long long* bucket_cursor = nullptr;  // [depth_bucket_cap]
+    uint2* bucket_start = nullptr;  // per bucket its first position and bin
     int radix_frames = 0;  // frames left that order depths by radix passes (a bucket did not fit)
     uint32_t* slot_off = nullptr;  // first pair slot of each visible Gaussian by depth rank (cap_vis + 1)
     uint32_t* slot_owner = nullptr;  // depth rank of the first slot of each emission chunk
@@ -178,7 +180,7 @@ struct vgr_view {
     int img_sel = 0;  // device image the next pipelined frame writes
     float* lut = nullptr;
     unsigned long long* status = nullptr;
-    size_t st_compact = 0, st_front = 0, st_emit = 0, st_depth = 0, st_tile = 0, st_depth_stride = 0,
+    size_t st_emit = 0, st_depth = 0, st_tile = 0, st_depth_stride = 0,
            st_tile_stride = 0, st_words = 0;
     Counters* ctr = nullptr;
     ViewState* vstate = nullptr;
@@ -633,9 +635,7 @@ vgr_status alloc_status(vgr_view* v) {
     drop_graphs(v);
     dfree(v->status);
     const uint32_t RT = radix_tile();
-    v->st_compact = 0;
-    v->st_front = v->st_compact + cut_compact_tiles(v->n_words) + 1;
-    v->st_emit = v->st_front + cut_compact_tiles(v->n_words) + 1;
+    v->st_emit = 0;
     v->st_depth = v->st_emit + ceil_div(v->cap_vis, slot_scan_tile()) + 1;
     v->st_depth_stride = (size_t)(ceil_div(v->cap_vis, RT) + 1) * 256;
     v->st_tile = v->st_depth + 4 * v->st_depth_stride;
@@ -647,11 +647,14 @@ vgr_status alloc_status(vgr_view* v) {
     return s;
 }
 
-// Bytes cleared at the start of a frame: the counters, the depth bins and the
-// cursors of the buckets that cap_vis entries can make.
+// Bytes cleared at the start of a frame: the counters, the depth bins, the bit
+// counts of the bitmaps' tiles and the cursors of the buckets that cap_vis
+// entries can make.
 constexpr size_t CTR_BYTES = (sizeof(Counters) + 15) / 16 * 16;
-size_t cleared_bytes(uint32_t cap_vis) {
-    return CTR_BYTES + DEPTH_BINS * sizeof(uint32_t) +
+constexpr size_t BIN_BYTES = DEPTH_BINS * sizeof(uint32_t);
+size_t cut_count_bytes(uint32_t n_words) { return (size_t)cut_compact_count_words(n_words) * 4; }
+size_t cleared_bytes(uint32_t n_words, uint32_t cap_vis) {
+    return CTR_BYTES + BIN_BYTES + cut_count_bytes(n_words) +
            depth_bucket_cap(std::min(cap_vis, MAX_RANKS)) * sizeof(unsigned long long);
 }
 
@@ -801,12 +804,14 @@ vgr_status vgr_create_view(vgr_hierarchy* h, const vgr_view_opts* opts, vgr_view
     VGR_VTRY(dalloc(&v->front_bm, v->n_words, &v->fixed_bytes));
     VGR_VTRY(dalloc(&v->frontier[0], N, &v->fixed_bytes));
     VGR_VTRY(dalloc(&v->frontier[1], N, &v->fixed_bytes));
-    {  // the counters, the depth bins and the buckets' cursors: cleared together every frame
+    {  // what a frame clears: one allocation, one fill
         unsigned char* z = nullptr;
-        VGR_VTRY(dalloc(&z, cleared_bytes(MAX_RANKS), &v->fixed_bytes));
+        VGR_VTRY(dalloc(&z, cleared_bytes(v->n_words, MAX_RANKS), &v->fixed_bytes));
         v->ctr = reinterpret_cast<Counters*>(z);
         v->depth_bins = reinterpret_cast<uint32_t*>(z + CTR_BYTES);
-        v->bucket_cursor = reinterpret_cast<unsigned long long*>(z + CTR_BYTES + DEPTH_BINS * sizeof(uint32_t));
+        v->cut_counts = reinterpret_cast<uint32_t*>(z + CTR_BYTES + BIN_BYTES);
+        v->bucket_cursor =
+            reinterpret_cast<unsigned long long*>(z + CTR_BYTES + BIN_BYTES + cut_count_bytes(v->n_words));
     }
     VGR_VTRY(dalloc(&v->bucket_start, depth_bucket_cap(MAX_RANKS) + 1, &v->fixed_bytes));
     {
@@ -901,12 +906,12 @@ vgr_status vgr_view_bytes_estimate(const vgr_hierarchy* h, const vgr_view_opts* 
     const uint64_t per_vis = 2 * sizeof(uint32_t) + 3 * sizeof(float4) + sizeof(float) /* visible SoA */ +
                              sizeof(uint32_t) /* slot offsets */ + 4 * sizeof(uint32_t) /* depth sort */;
     const uint64_t RT = radix_tile();
-    const uint64_t status_words = 2 * (cut_compact_tiles((uint32_t)n_words) + 1) + ceil_div(cap_vis, slot_scan_tile()) + 1 +
+    const uint64_t status_words = ceil_div(cap_vis, slot_scan_tile()) + 1 +
                                   4 * (ceil_div(cap_vis, RT) + 1) * 256 + 4 * (ceil_div(cap_pairs, RT) + 1) * 256;
     const uint32_t T = o.tile_size ? o.tile_size : TILE_DEFAULT;
     const uint64_t tiles = (uint64_t)((width + T - 1) / T) * ((height + T - 1) / T);
     uint64_t b = 3 * 4 * cap_cut + per_vis * cap_vis + 4 * 4 * cap_pairs + 4 * emit_owner_cap(cap_pairs) + 2 * 4 * n_words + 2 * 4 * N +
-                 cleared_bytes(MAX_RANKS) + 4 * (depth_bucket_cap(MAX_RANKS) + 1) + sizeof(ViewState) + sizeof(FrameParams) + 260 * 4 + 8 * status_words;
+                 cleared_bytes((uint32_t)n_words, MAX_RANKS) + 8 * (depth_bucket_cap(MAX_RANKS) + 1) + sizeof(ViewState) + sizeof(FrameParams) + 260 * 4 + 8 * status_words;
     b += (uint64_t)width * height * 3 * 4 + tiles * (sizeof(uint2) + 4);
     *bytes = b;
     return VGR_OK;
@@ -964,7 +969,7 @@ uint32_t enqueue_frame(vgr_view* v, bool scratch, bool radix_depth, int tile_pas
     const FrameParams& fh = *v->fp_host;
     const uint32_t n_tiles = fh.tiles_x * fh.tiles_y;
     cudaMemcpyAsync(v->fp_dev, v->fp_host, sizeof(FrameParams), cudaMemcpyHostToDevice, s);
-    cudaMemsetAsync(v->ctr, 0, cleared_bytes(v->cap_vis), s);
+    cudaMemsetAsync(v->ctr, 0, cleared_bytes(v->n_words, v->cap_vis), s);
     cudaMemsetAsync(v->ranges, 0xFF, (size_t)n_tiles * sizeof(uint2), s);  // (start, ~end): both all ones
     // the first kernel waits for the copies above in plain stream order; with
     // stage events between the kernels none of them is launched early
@@ -974,16 +979,15 @@ uint32_t enqueue_frame(vgr_view* v, bool scratch, bool radix_depth, int tile_pas
     if (scratch) {
         for (uint32_t level = 0; level <= v->h->max_depth; ++level)
             launch_lod_level((int)level, sc, v->frontier[level & 1], v->frontier[(level + 1) & 1], v->h->n_nodes,
-                             v->fp_dev, v->bitmap, v->front_bm, v->ctr, v->grid_wide, fh.lod_frustum != 0,
+                             v->fp_dev, v->bitmap, v->front_bm, v->cut_counts, v->ctr, v->grid_wide, fh.lod_frustum != 0,
                              fh.lod_interp != 0, s);
     } else {
         launch_lod_update(sc, v->cut[prev], &v->vstate->n_cut[prev], v->cap_cut, v->fp_dev, v->bitmap, v->front_bm,
-                          v->ctr, v->grid_wide, fh.lod_frustum != 0, fh.lod_interp != 0, s);
+                          v->cut_counts, v->ctr, v->grid_wide, fh.lod_frustum != 0, fh.lod_interp != 0, s);
     }
     mark(VGR_STAGE_COMPACT);
-    launch_cut_compact(v->bitmap, v->front_bm, v->n_words, v->cut[cur], v->front_list, v->cap_cut,
-                       &v->vstate->n_cut[cur], v->status + v->st_compact, v->status + v->st_front, v->ctr, v->fp_dev,
-                       v->grid_scan, s);
+    launch_cut_compact(v->bitmap, v->front_bm, v->cut_counts, v->n_words, v->cut[cur], v->front_list, v->cap_cut,
+                       &v->vstate->n_cut[cur], v->ctr, v->grid_scan, s);
     mark(VGR_STAGE_PREPROCESS);
     launch_preprocess(sc, v->front_list, &v->ctr->n_front, v->cap_cut, v->fp_dev, v->vis, v->ctr, v->depth_bins,
                       fh.lod_interp != 0, std::min(v->grid_wide, 2 * v->h->num_sms), s);

@@ -26,7 +26,7 @@ constexpr uint32_t CHILD_MASK = (1u << CHILD_SHIFT) - 1u;
 constexpr int RADIX_THREADS = 256;            // one radix-sort tile: 256 threads x 15 keys
 constexpr int RADIX_ITEMS = 15;
 constexpr int RADIX_TILE = RADIX_THREADS * RADIX_ITEMS;
-constexpr int DEPTH_BINS = 4096;              // bins of the depth keys' histogram (k_depth.cu)
+constexpr int DEPTH_BINS = 6144;              // bins of the depth keys' histogram (k_depth.cu)
 
 // flags in Counters::flags
 enum : uint32_t {
@@ -51,9 +51,8 @@ constexpr uint32_t EMIT_SLOTS = 1024;  // pair slots per emission chunk
 // depth rank that owns the first slot of that chunk.
 __device__ __forceinline__ void emit_owner(uint32_t* owner, uint32_t cap_owner, uint32_t off, uint32_t c,
                                            uint32_t rank) {
-    const uint64_t end = (uint64_t)off + c;
-    for (uint64_t k = ((uint64_t)off + EMIT_SLOTS - 1u) / EMIT_SLOTS; k * EMIT_SLOTS < end && k < cap_owner; ++k)
-        owner[k] = rank;
+    const uint32_t k1 = min((off + c + EMIT_SLOTS - 1u) / EMIT_SLOTS, cap_owner);
+    for (uint32_t k = (off + EMIT_SLOTS - 1u) / EMIT_SLOTS; k < k1; ++k) owner[k] = rank;
 }
 
 // Candidate tiles of an entry in one word: x0 | y0 << 10 | width << 20 (an
@@ -174,23 +173,19 @@ __device__ __forceinline__ uint32_t warp_excl_scan(uint32_t v, uint32_t* total) 
     return x - v;
 }
 
-// Block-wide exclusive scan (blockDim.x = 32 * NW).  smem: NW + 1 words.
+// Block-wide exclusive scan (blockDim.x = 32 * NW).  smem: NW words, not to be
+// written again before a later barrier.  One barrier: every warp scans the
+// warps' totals for itself.
 template <int NW>
 __device__ __forceinline__ uint32_t block_excl_scan(uint32_t v, uint32_t* smem, uint32_t* total) {
+    static_assert(NW <= 32, "one lane per warp");
     uint32_t wt;
-    uint32_t x = warp_excl_scan(v, &wt);
+    const uint32_t x = warp_excl_scan(v, &wt);
     const uint32_t w = threadIdx.x >> 5;
     if (lane_id() == 31) smem[w] = wt;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        uint32_t run = 0;
-        for (int i = 0; i < NW; ++i) { uint32_t c = smem[i]; smem[i] = run; run += c; }
-        smem[NW] = run;
-    }
-    __syncthreads();
-    uint32_t r = x + smem[w];
-    *total = smem[NW];
-    return r;
+    const uint32_t before = warp_excl_scan(lane_id() < (uint32_t)NW ? smem[lane_id()] : 0u, total);
+    return x + __shfl_sync(0xFFFFFFFFu, before, w);
 }
 
 // ------------------------------------------- decoupled look-back words
@@ -300,10 +295,13 @@ __device__ __forceinline__ float depth_key(float4 m, float R6, float R7, float R
 // The key's bin.  Every step is a correctly rounded monotone operation, so the
 // bin never falls as the key rises; single intrinsics give every kernel the
 // same bin.
-__device__ __forceinline__ uint32_t depth_bin(const DepthMap& m, uint32_t key) {
+__device__ __forceinline__ float depth_coord(const DepthMap& m, uint32_t key) {
     const float a = __fmul_rn(__uint2float_rn(key > m.key_lo ? key - m.key_lo : 0u), m.c_log);
     const float b = __fmul_rn(fmaxf(__fsub_rn(__uint_as_float(key), m.z_lo), 0.f), m.c_lin);
-    return min(__float2uint_rz(__fadd_rn(a, b)), (uint32_t)DEPTH_BINS - 1u);
+    return __fadd_rn(a, b);
+}
+__device__ __forceinline__ uint32_t depth_bin(const DepthMap& m, uint32_t key) {
+    return min(__float2uint_rz(depth_coord(m, key)), (uint32_t)DEPTH_BINS - 1u);
 }
 
 // The granularity test, single-rounded FP32 (no contraction): expand iff
@@ -367,8 +365,6 @@ __device__ __forceinline__ float lod_interp_weight(float an, float ap, float t) 
 __device__ __forceinline__ float lod_lerp_rn(float a, float b, float w) {
     return __fadd_rn(a, __fmul_rn(w, __fsub_rn(b, a)));
 }
-
-__device__ __forceinline__ void bitmap_set(uint32_t* bm, uint32_t n) { atomicOr(&bm[n >> 5], 1u << (n & 31u)); }
 
 // Lanes of the (full) warp holding the same 9-bit value (a radix digit
 // 0..255, or 256 for "no digit"): one ballot per bit.

@@ -60,17 +60,16 @@ struct Counters;
 
 // k_lod.cu
 void launch_lod_update(const SceneDev& sc, const uint32_t* prev_cut, const uint32_t* n_prev, uint32_t cap_prev,
-                       const FrameParams* fp, uint32_t* bitmap, uint32_t* front, Counters* ctr, int grid,
+                       const FrameParams* fp, uint32_t* bitmap, uint32_t* front, uint32_t* counts, Counters* ctr, int grid,
                        bool frustum, bool interp, cudaStream_t s);
 void launch_lod_level(int level, const SceneDev& sc, const uint32_t* fin, uint32_t* fout, uint32_t cap,
-                      const FrameParams* fp, uint32_t* bitmap, uint32_t* front, Counters* ctr, int grid,
+                      const FrameParams* fp, uint32_t* bitmap, uint32_t* front, uint32_t* counts, Counters* ctr, int grid,
                       bool frustum, bool interp, cudaStream_t s);
-void launch_cut_compact(uint32_t* bitmap, uint32_t* front, uint32_t n_words, uint32_t* cut, uint32_t* front_list,
-                        uint32_t cap, uint32_t* n_cut_out, unsigned long long* status,
-                        unsigned long long* status_front, Counters* ctr, const FrameParams* fp, int grid,
+void launch_cut_compact(uint32_t* bitmap, uint32_t* front, const uint32_t* counts, uint32_t n_words, uint32_t* cut,
+                        uint32_t* front_list, uint32_t cap, uint32_t* n_cut_out, Counters* ctr, int grid,
                         cudaStream_t s);
-uint32_t cut_compact_tiles(uint32_t n_words);
 uint32_t cut_compact_tile_words();
+uint32_t cut_compact_count_words(uint32_t n_words);  // words of the tiles' counters
 
 // k_preprocess.cu
 // Per in-front entry i (the entry's node id is the in-front list's entry i)
@@ -98,7 +97,7 @@ void prepare_scene_half(float4* covB, uint32_t n, cudaStream_t s);
 // the in-front index of depth rank r, slot_off[r] its first slot (r <= n_vis).
 uint32_t depth_bucket_cap(uint32_t cap_vis);  // bucket ids a frame of cap_vis entries can have, plus one
 cudaError_t depth_sort_init();                // once per device: the kernels' shared-memory limits
-void launch_depth_sort(const VisBuffers& vis, uint32_t cap_vis, const uint32_t* bins, uint32_t* bstart,
+void launch_depth_sort(const VisBuffers& vis, uint32_t cap_vis, const uint32_t* bins, uint2* bstart,
                        unsigned long long* cursor, uint2* part, uint32_t* order, uint32_t* slot_off,
                        uint32_t* owner, uint64_t cap_pairs, Counters* ctr, const FrameParams* fp, int sms, cudaStream_t s);
 
