@@ -429,12 +429,12 @@ vgr_status vgr_server_client_view(vgr_server* s, uint32_t client, vgr_view** vie
  * the inputs are only read, the outputs receive the sorted pairs, and input
  * and output ranges must not overlap.  Equal keys keep their input order.
  * Runs on 'stream' (a cudaStream_t, NULL for the default stream) and waits
- * for it before returning.  Scratch (histograms, look-back words, the
+ * for it before returning.  Scratch (digit counts of its tiles, the
  * ping-pong buffer of a multi-pass sort) is allocated by the library on
  * first use per device, grown when a larger n arrives and kept until exit;
  * calls on one device are serialised.  1 <= key_bits <= 32, n < 2^32 - 1
  * (n = 0 is a no-op).  Errors: VGR_E_INVALID, VGR_E_NOMEM, VGR_E_CUDA,
- * VGR_E_TIMEOUT (a bounded look-back wait ran out).
+ * VGR_E_TIMEOUT (not returned by the present passes, which wait for nothing).
  */
 vgr_status vgr_sort_pairs(const uint32_t* keys_in, const uint32_t* vals_in, uint32_t* keys_out,
                           uint32_t* vals_out, uint64_t n, uint32_t key_bits, void* stream);
@@ -450,10 +450,10 @@ vgr_status vgr_sort_pairs(const uint32_t* keys_in, const uint32_t* vals_in, uint
  * allowed.  The paper has no counterpart; it is a service of this library.
  *
  * Same arguments, result and errors as vgr_sort_pairs, but it calls no
- * cudaMalloc, cudaFree or other allocating routine: all scratch (look-back
- * epoch, tickets, histograms, look-back words, the ping-pong buffer) lives in
+ * cudaMalloc, cudaFree or other allocating routine: all scratch (the
+ * tiles' digit counts, the ping-pong buffer) lives in
  * one fixed array in device memory that the library declares and that every
- * GPU loading the library holds until the process exits (about 2.7 MB).
+ * GPU loading the library holds until the process exits (about 2.2 MB).
  *   - n is limited to VGR_SORT_NOALLOC_MAX_N (262,144) pairs; larger n
  *     returns VGR_E_INVALID without touching the GPU.
  *   - The first call on a device (with that device current) looks up the

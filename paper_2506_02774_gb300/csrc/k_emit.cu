@@ -17,16 +17,16 @@
 // 1M-leaf box at 1080p (981K slots): 53 -> 21 us, city at 1080p (4.26M slots):
 // 107 -> 61 us.  For each slot the tile-level form of
 // Eq. 4 (paper Sec. 4.2) decides: a kept slot gets key = tile id, a dropped one
-// the sentinel key, which the stable tile sort moves behind every real pair
-// (which stay in depth order within a tile, the sort being stable).  The slot's
+// all ones, which the tile sort's first pass leaves out (the others stay in
+// depth order within a tile, the sort being stable).  The slot's
 // value is the Gaussian's index in the in-front arrays << 8 | its row mask in
 // that tile: bit w is set when the footprint box reaches one of the tile's
 // pixel rows w MR .. w MR + MR - 1, MR = tile / 8 rows (1 for 8-pixel tiles);
 // outside the box the Eq. 4 test fails at every pixel, so the blend reads only
 // the records a strip needs, straight from the in-front arrays.  Indices
 // therefore take 24 bits: a frame with more cut nodes in front of the camera
-// reports an overflow.  The digit histograms of the tile sort are accumulated
-// here as well.
+// reports an overflow.  The digit counts of the tile sort's first pass are
+// written here as well, a row per chunk.
 #include <cuda_fp16.h>
 
 #include "vgr_internal.cuh"
@@ -120,15 +120,14 @@ __global__ void __launch_bounds__(EM_THREADS, 4) k_emit(const uint32_t* __restri
                                                      const uint32_t* __restrict__ slot_off,
                                                      const uint32_t* __restrict__ owner,
                                                      uint32_t* __restrict__ pair_key,
-                                                     uint32_t* __restrict__ pair_val, uint64_t cap, int tile_passes,
-                                                     uint32_t sentinel, Counters* __restrict__ ctr,
+                                                     uint32_t* __restrict__ pair_val, uint64_t cap, int bits,
+                                                     RadixTab tab, Counters* __restrict__ ctr,
                                                      const FrameParams* __restrict__ fp) {
     pdl_wait();
     __shared__ uint2 s_g[EM_GAUSS];   // per Gaussian: index in the in-front arrays, first slot
     __shared__ uint32_t s_bits[32];   // slots at which a Gaussian starts
-    __shared__ uint32_t s_hist[4][256];
-    const uint32_t lane = lane_id(), warp = threadIdx.x >> 5;
-    for (int i = threadIdx.x; i < tile_passes * 256; i += EM_THREADS) (&s_hist[0][0])[i] = 0u;
+    __shared__ uint32_t s_cnt[EM_THREADS];  // the chunk's kept slots by first digit
+    const uint32_t lane = lane_id(), warp = threadIdx.x >> 5, D = 1u << bits;
     const uint32_t n_vis = min(ctr->n_vis, cap_vis);
     const uint64_t cand = ctr->n_cand;
     const uint32_t ns = (uint32_t)(cand < cap ? cand : cap);
@@ -145,6 +144,7 @@ __global__ void __launch_bounds__(EM_THREADS, 4) k_emit(const uint32_t* __restri
         const uint32_t g1 = ck + 1u < nchunks ? owner[ck + 1u] : n_vis - 1u;  // may start past the chunk
         const uint32_t m = min(g1 - g0 + 1u, EM_GAUSS);
         if (threadIdx.x < 32) s_bits[threadIdx.x] = threadIdx.x == 0 ? 1u : 0u;  // the chunk's first slot has an owner
+        s_cnt[threadIdx.x] = 0u;
         __syncthreads();
         for (uint32_t q = threadIdx.x; q < m; q += EM_THREADS) {
             const uint32_t o = slot_off[g0 + q];
@@ -193,22 +193,35 @@ __global__ void __launch_bounds__(EM_THREADS, 4) k_emit(const uint32_t* __restri
                         rows = ((2u << w1) - 1u) & ~((1u << w0) - 1u);
                     }
                 }
-                const uint32_t key = keep ? (uint32_t)ty * TW + (uint32_t)tx : sentinel;
+                const uint32_t key = keep ? (uint32_t)ty * TW + (uint32_t)tx : NONE;
                 kept += keep;
                 pair_key[j] = key;
                 pair_val[j] = (gv.x << 8) | rows;
-                for (int p = 0; p < tile_passes; ++p) atomicAdd(&s_hist[p][(key >> (8 * p)) & 255u], 1u);
+                if (keep) atomicAdd(&s_cnt[key & (D - 1u)], 1u);
             }
         }
         __syncthreads();
+        if (threadIdx.x < D) {
+            const uint32_t c = s_cnt[threadIdx.x];
+            tab.rows[(size_t)ck * D + threadIdx.x] = (uint16_t)c;
+            if (c) atomicAdd(&tab.groups[(size_t)(ck / RADIX_GROUP) * D + threadIdx.x], c);
+        }
     }
     const uint32_t wk = __reduce_add_sync(0xFFFFFFFFu, kept);
     if (lane == 0 && wk) atomicAdd(&ctr->n_pairs, (unsigned long long)wk);
-    __syncthreads();
-    for (int i = threadIdx.x; i < tile_passes * 256; i += EM_THREADS) {
-        const uint32_t c = (&s_hist[0][0])[i];
-        if (c) atomicAdd(&ctr->tile_hist[0][0] + i, c);
+}
+
+// The tile of every sorted pair (the debug view's array), from the ranges.
+__global__ void k_debug_tiles(const uint2* __restrict__ ranges, uint32_t n_tiles, uint32_t* __restrict__ pair_tile,
+                              uint64_t n_pairs) {
+    for (uint32_t t = blockIdx.x; t < n_tiles; t += gridDim.x) {
+        const uint2 r = ranges[t];
+        for (uint64_t i = r.x + threadIdx.x; i < r.y && i < n_pairs; i += blockDim.x) pair_tile[i] = t;
     }
+}
+
+void launch_debug_tiles(const uint2* ranges, uint32_t n_tiles, uint32_t* pair_tile, uint64_t n_pairs, cudaStream_t s) {
+    if (n_pairs) k_debug_tiles<<<1024, 128, 0, s>>>(ranges, n_tiles, pair_tile, n_pairs);
 }
 
 void launch_slot_scan(const uint32_t* order, uint32_t cap_vis, const VisBuffers& vis, uint32_t* slot_off,
@@ -219,10 +232,10 @@ void launch_slot_scan(const uint32_t* order, uint32_t cap_vis, const VisBuffers&
 }
 
 void launch_emit(const uint32_t* order, uint32_t cap_vis, const VisBuffers& vis, const uint32_t* slot_off,
-                 const uint32_t* owner, uint32_t* pair_key, uint32_t* pair_val, uint64_t cap_pairs, int tile_passes,
-                 uint32_t sentinel, Counters* ctr, const FrameParams* fp, int grid, cudaStream_t s) {
+                 const uint32_t* owner, uint32_t* pair_key, uint32_t* pair_val, uint64_t cap_pairs, int bits,
+                 RadixTab tab, Counters* ctr, const FrameParams* fp, int grid, cudaStream_t s) {
     launch_k(k_emit, grid, EM_THREADS, s, order, cap_vis, (const float4*)vis.rec, slot_off, owner, pair_key, pair_val,
-             cap_pairs, tile_passes, sentinel, ctr, fp);
+             cap_pairs, bits, tab, ctr, fp);
 }
 
 // Blend order: tiles by descending pair count (classes of floor(log2(count+1)),

@@ -1,13 +1,25 @@
-// k_sort.cu -- stable LSD radix sort of (u32 key, u32 value) pairs, 8-bit
-// digits, one kernel per digit pass ("onesweep": every tile ranks its keys
-// locally, publishes its per-digit counts and finds its global offsets by a
-// decoupled look-back over earlier tiles), plus an upfront histogram kernel
-// giving each pass its digit totals.
+// k_sort.cu -- stable LSD radix sort of (u32 key, u32 value) pairs, one or two
+// kernels per digit of up to 8 bits: a count of the digits of every tile, and a
+// scatter of the tiles.
 //
-// Used twice per frame (paper Sec. 3.1 'Sorting'): depth keys of the visible
-// Gaussians (4 passes; equal depths keep their ascending node-id order), then
-// tile ids of the kept pairs (2 passes at 1080p), which yields the
-// (tile, depth, node id) order with nothing but stable passes.
+// Sorts the emitted pairs by tile id (paper Sec. 3.1 'Sorting'), stable, so a
+// tile's pairs keep their depth order; the depth keys of frames whose depths
+// are too concentrated for the partition (k_depth.cu); and the pairs of the
+// standalone calls.
+//
+// A pass's tables hold the digit counts of every tile (rows) and of every 32
+// rows (groups).  A tile's base per digit is the sum of the groups and rows
+// before it, which the scatter adds up for itself while the tile's keys are on
+// their way: nothing waits for another tile.  (One kernel per pass whose tiles
+// found their bases by look-back took 18-24 us for up to a million keys whatever
+// the traffic: all the tiles were in flight at once, each digit's chain was as
+// long as their number.)  The rows of the tile sort's first pass are written by
+// the emission, so its count kernel is saved there.  Tile sort of 981K slots
+// (1M-leaf box, 1080p): 47 -> 31 us; of 4.26M (city, 1080p): 85 -> 76; of 235K
+// (320 x 180, one pass): 24 -> 12; the standalone sort of 4M 32-bit keys: 191 ->
+// 171.  Large inputs are bound by the instructions of the ranking (half of the
+// issue slots, the ballots' pipe first); three CTAs an SM at 40 registers were no
+// faster.
 #include "vgr_internal.cuh"
 #include "vgr_launch.h"
 
@@ -15,226 +27,263 @@ namespace vgr {
 
 constexpr int RS_THREADS = RADIX_THREADS;
 constexpr int RS_WARPS = RS_THREADS / 32;
-constexpr int RS_ITEMS = RADIX_ITEMS;
-constexpr int RS_TILE = RADIX_TILE;  // 3840 keys per tile
-constexpr int RS_BINS = 256;
+constexpr int RS_ITEMS = RADIX_TILE / RADIX_THREADS;
+constexpr uint32_t RS_TILE = RADIX_TILE;
+static_assert(RS_TILE <= 0xFFFFu, "a row's counts and a tile's places fit 16 bits");
 
-uint32_t radix_tile() { return RS_TILE; }
+size_t radix_rows(uint64_t n, uint32_t row_len) { return (size_t)((n + row_len - 1) / row_len); }
+size_t radix_groups(uint64_t n, uint32_t row_len) { return (radix_rows(n, row_len) + RADIX_GROUP - 1) / RADIX_GROUP; }
+size_t radix_row_words(uint64_t n, uint32_t row_len, int bits) { return radix_rows(n, row_len) << bits; }
+size_t radix_group_words(uint64_t n, uint32_t row_len, int bits) { return radix_groups(n, row_len) << bits; }
 
-// Digit histograms of up to 4 passes (shift 0, 8, 16, 24): one shared-memory
-// atomic per key and digit (equal digits within a warp are combined by the
-// hardware), then one global atomic per nonzero bin and CTA.
-__global__ void __launch_bounds__(256) k_radix_hist(const uint32_t* __restrict__ keys,
-                                                    const uint32_t* __restrict__ n32,
-                                                    const unsigned long long* __restrict__ n64, uint64_t cap,
-                                                    int passes, uint32_t* __restrict__ hist) {
-    __shared__ uint32_t h[4][RS_BINS];
-    for (int i = threadIdx.x; i < 4 * RS_BINS; i += blockDim.x) (&h[0][0])[i] = 0;
+__device__ __forceinline__ uint32_t radix_n(const uint32_t* n32, const unsigned long long* n64, uint64_t cap) {
+    uint64_t n = n32 ? (uint64_t)*n32 : n64 ? (uint64_t)*n64 : cap;
+    return (uint32_t)(n < cap ? n : cap);
+}
+
+// Digit counts of every tile, and of every group of tiles.
+__global__ void __launch_bounds__(RS_THREADS) k_radix_count(const uint32_t* __restrict__ keys,
+                                                            const uint32_t* __restrict__ n32,
+                                                            const unsigned long long* __restrict__ n64, uint64_t cap,
+                                                            int shift, int bits, RadixTab tab) {
+    pdl_wait();
+    __shared__ uint32_t s_cnt[2][256];
+    const uint32_t n = radix_n(n32, n64, cap);
+    const uint32_t ntiles = (uint32_t)(((uint64_t)n + RS_TILE - 1) / RS_TILE), D = 1u << bits, t = threadIdx.x;
+    if (t < 256) s_cnt[0][t] = s_cnt[1][t] = 0u;
     __syncthreads();
-    uint64_t nv = n32 ? (uint64_t)*n32 : (uint64_t)*n64;
-    if (nv > cap) nv = cap;
-    const uint32_t n = (uint32_t)nv;
-    const uint32_t stride = gridDim.x * blockDim.x;
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-        const uint32_t k = keys[i];
-        for (int p = 0; p < passes; ++p) atomicAdd(&h[p][(k >> (8 * p)) & 255u], 1u);
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < passes * RS_BINS; i += blockDim.x) {
-        const uint32_t c = (&h[0][0])[i];
-        if (c) atomicAdd(&hist[i], c);
+    uint32_t flip = 0;
+    for (uint32_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x, flip ^= 1u) {
+        const uint32_t base = tile * RS_TILE + t;  // n < 2^32, and so is a tile's end
+        uint32_t key[RS_ITEMS];
+#pragma unroll
+        for (int k = 0; k < RS_ITEMS; ++k) {
+            const uint32_t i = base + k * RS_THREADS;
+            key[k] = i < n ? keys[i] : 0u;
+        }
+#pragma unroll
+        for (int k = 0; k < RS_ITEMS; ++k)
+            if (base + k * RS_THREADS < n) atomicAdd(&s_cnt[flip][(key[k] >> shift) & (D - 1u)], 1u);
+        __syncthreads();
+        if (t < D) {
+            const uint32_t c = s_cnt[flip][t];
+            s_cnt[flip][t] = 0u;  // used again after the next tile's barrier
+            tab.rows[(size_t)tile * D + t] = (uint16_t)c;
+            if (c) atomicAdd(&tab.groups[(size_t)(tile / RADIX_GROUP) * D + t], c);
+        }
     }
 }
 
-// One digit pass.  n comes from n32 (if non-null) or n64, clamped to cap.
-// Per tile of RS_TILE keys (warp w owns a contiguous run of 32 * RS_ITEMS):
-//  1. each warp ranks its keys: peers with the same digit come from
-//     the match instruction (last pass) or per-bit ballots; the run leader's shared atomicAdd on the warp's digit
-//     counter returns the count of earlier keys, shuffled to the peers;
-//  2. the tile's digit counts are published to the look-back words at once,
-//     so later tiles rarely wait for this one;
-//  3. keys and values are placed digit-sorted in shared memory (one 8-byte
-//     store per element);
-//  4. the look-back over earlier tiles gives each digit its global start;
-//  5. every thread writes consecutive staged elements, so each digit's run
-//     is stored contiguously (coalesced).
-// The last pass of the tile sort also records each tile's range: a CTA's
-// staged elements are in final key order and each key's run is one
-// contiguous stretch of global positions, so the first and last element of
-// every run it holds give atomicMin / atomicMax updates of [start, end) (the
-// end kept as its complement, so both start from all ones and take a min).
-// Keys >= n_ranges (dropped slots) have no range.
-constexpr int LB_BATCH = 8;  // look-back words read per round trip
-
-template <bool HW_MATCH>
-__global__ void __launch_bounds__(RS_THREADS, 4) k_radix_pass(const uint32_t* __restrict__ keys_in,
-                                                           const uint32_t* __restrict__ vals_in,
-                                                           uint32_t* __restrict__ keys_out,
-                                                           uint32_t* __restrict__ vals_out,
-                                                           const uint32_t* __restrict__ n32,
-                                                           const unsigned long long* __restrict__ n64, uint64_t cap,
-                                                           int shift, const uint32_t* __restrict__ hist,
-                                                           unsigned long long* __restrict__ status,
-                                                           uint32_t* __restrict__ ticket,
-                                                           const FrameParams* __restrict__ fp,
-                                                           Counters* __restrict__ ctr, uint2* __restrict__ ranges,
-                                                           uint32_t n_ranges) {
-    pdl_wait();
-    __shared__ uint32_t s_wc[RS_WARPS][RS_BINS];  // per-warp digit counts, then per-warp run offsets
-    __shared__ uint32_t s_gbase[RS_BINS];         // global start of each digit (all tiles)
-    __shared__ uint32_t s_lstart[RS_BINS];        // start of each digit's run in the staged tile
-    __shared__ uint32_t s_gofs[RS_BINS];          // global index minus staged index, per digit
-    __shared__ uint2 s_kv[RS_TILE];               // the tile staged digit-sorted: (key, value)
-    __shared__ uint32_t s_scan[RS_WARPS + 1];
-    __shared__ uint32_t s_tile;
-    uint64_t n64v = n32 ? (uint64_t)*n32 : (uint64_t)*n64;
-    if (n64v > cap) n64v = cap;
-    const uint32_t n = (uint32_t)n64v;
-    const uint32_t ntiles = (n + RS_TILE - 1) / RS_TILE;
-    const uint32_t epoch = fp->epoch;
-    const uint32_t lane = lane_id(), warp = threadIdx.x >> 5;
-    {
-        uint32_t total;
-        s_gbase[threadIdx.x] = block_excl_scan<RS_WARPS>(hist[threadIdx.x], s_scan, &total);
+// Lanes of the (full) warp with the same digit of BITS bits, among the valid
+// ones; an invalid lane gets the invalid ones.
+template <int BITS, bool ALL>
+__device__ __forceinline__ uint32_t match_digit(uint32_t d, bool valid) {
+    uint32_t m = 0xFFFFFFFFu;
+    if (!ALL) {
+        const uint32_t ok = __ballot_sync(0xFFFFFFFFu, valid);
+        m = valid ? ok : ~ok;
     }
-    for (;;) {
-        if (threadIdx.x == 0) s_tile = atomicAdd(ticket, 1u);
 #pragma unroll
-        for (int w = 0; w < RS_WARPS; ++w) s_wc[w][threadIdx.x] = 0u;
-        __syncthreads();
-        const uint32_t tile = s_tile;
-        if (tile >= ntiles) break;
-        const uint32_t base = tile * RS_TILE + warp * (32 * RS_ITEMS) + lane;
-        uint32_t key[RS_ITEMS], val[RS_ITEMS], rank[RS_ITEMS];
-#pragma unroll
-        for (int it = 0; it < RS_ITEMS; ++it) {
-            const uint32_t idx = base + it * 32;
-            key[it] = idx < n ? keys_in[idx] : 0u;
-            val[it] = idx < n ? (vals_in ? vals_in[idx] : idx) : 0u;
+    for (int b = 0; b < BITS; ++b) {
+        const bool bit = (d >> b) & 1u;
+        const uint32_t vote = __ballot_sync(0xFFFFFFFFu, bit);
+        m &= bit ? vote : ~vote;
+    }
+    return m;
+}
+
+// One digit pass over tiles of RS_TILE pairs (row_tiles rows each):
+//  1. the tile's keys and values are requested; meanwhile the tables' entries
+//     before the tile are added up (two digits per thread and load);
+//  2. each warp ranks its contiguous share: peers by one ballot per digit bit,
+//     the first of them advances the warp's counter of the digit;
+//  3. a thread per digit turns the warps' counts into places in the tile;
+//  4. the pairs are staged digit-sorted in shared memory and
+//  5. stored, each digit's run contiguously.
+// With DROP, pairs whose key is all ones are left out.  keys_out may be null.
+// The last pass of the tile sort also records each tile's range: a CTA's staged
+// elements are in final key order and each key's run is one contiguous stretch
+// of global positions, so the first and last element of every run it holds give
+// atomicMin updates of (start, ~end), from all ones.
+template <int BITS, bool DROP>
+__global__ void __launch_bounds__(RS_THREADS, 2) k_radix_scatter(
+    const uint32_t* __restrict__ keys_in, const uint32_t* __restrict__ vals_in, uint32_t* __restrict__ keys_out,
+    uint32_t* __restrict__ vals_out, const uint32_t* __restrict__ n32, const unsigned long long* __restrict__ n64,
+    uint64_t cap, int shift, RadixTab tab, uint32_t row_tiles, uint2* __restrict__ ranges, uint32_t n_ranges) {
+    pdl_wait();
+    constexpr uint32_t D = 1u << BITS, NQ = 2 * RS_THREADS / D;  // rows read at once, two digits a thread
+    static_assert(D <= RS_THREADS && 2 * RS_THREADS % D == 0 && RS_TILE >= 2 * RS_THREADS, "table layout");
+    __shared__ __align__(16) uint2 s_kv[RS_TILE];   // the tile staged digit-sorted: (key, value)
+    __shared__ __align__(16) uint16_t s_wc[RS_WARPS][D];          // per-warp digit counts, then per-warp places
+    __shared__ uint32_t s_gofs[D];                  // global index minus staged index, per digit
+    __shared__ uint32_t s_scan[2][RS_WARPS];
+    // the tables' partial sums lie under the staging buffer: groups, then rows
+    uint32_t (*s_grp)[D] = reinterpret_cast<uint32_t (*)[D]>(s_kv);
+    uint32_t (*s_row)[D] = reinterpret_cast<uint32_t (*)[D]>(s_kv + RS_THREADS);
+    const uint32_t n = radix_n(n32, n64, cap);
+    const uint32_t ntiles = (uint32_t)(((uint64_t)n + RS_TILE - 1) / RS_TILE);
+    const uint32_t t = threadIdx.x, lane = lane_id(), warp = t >> 5;
+    const uint32_t pair = t % (D / 2), q = t / (D / 2);
+    if (blockIdx.x >= ntiles) return;
+    const uint32_t nrows = row_tiles == 1u ? ntiles
+                                           : (uint32_t)(((uint64_t)n + RS_TILE / row_tiles - 1) / (RS_TILE / row_tiles));
+    const uint32_t ngroups = (nrows + RADIX_GROUP - 1) / RADIX_GROUP;
+    const uint2* groups2 = reinterpret_cast<const uint2*>(tab.groups);
+    const uint32_t* rows2 = reinterpret_cast<const uint32_t*>(tab.rows);
+    uint32_t run = 0;       // thread d: pairs of smaller digits, and of digit d in the groups before 'seen'
+    uint32_t seen = 0;
+    {
+        uint2 tot = make_uint2(0u, 0u);
+        for (uint32_t g = q; g < ngroups; g += NQ) {
+            const uint2 v = groups2[(size_t)g * (D / 2) + pair];
+            tot.x += v.x;
+            tot.y += v.y;
         }
-        // 1. ranks within the warp, in (item, lane) = input order
+        reinterpret_cast<uint2*>(s_grp[q])[pair] = tot;
+        __syncthreads();
+        uint32_t c = 0, total;
+        if (t < D) {
 #pragma unroll
-        for (int it = 0; it < RS_ITEMS; ++it) {
-            const uint32_t idx = base + it * 32;
-            const uint32_t d = idx < n ? ((key[it] >> shift) & 255u) : 256u;
-            // the last pass (the top byte: few distinct digits per warp) by the match
-            // instruction; the lower bytes (many distinct digits) by one ballot per
-            // digit bit, faster there (depth keys and tile ids alike)
-            const uint32_t peers = HW_MATCH ? __match_any_sync(0xFFFFFFFFu, d) : match_digit(d);
+            for (uint32_t k = 0; k < NQ; ++k) c += s_grp[k][t];
+        }
+        run = block_excl_scan<RS_WARPS>(c, s_scan[0], &total);
+        __syncthreads();
+    }
+    for (uint32_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+        const uint32_t base = tile * RS_TILE + warp * (32u * RS_ITEMS) + lane;  // n < 2^32, and so is a tile's end
+        uint32_t key[RS_ITEMS], val[RS_ITEMS], rank[RS_ITEMS];
+        const bool full = n - tile * RS_TILE >= RS_TILE;  // (uniform)
+        if (full) {
+#pragma unroll
+            for (int it = 0; it < RS_ITEMS; ++it) key[it] = keys_in[base + it * 32u];
+#pragma unroll
+            for (int it = 0; it < RS_ITEMS; ++it) val[it] = vals_in ? vals_in[base + it * 32u] : base + it * 32u;
+        } else {
+#pragma unroll
+            for (int it = 0; it < RS_ITEMS; ++it) {
+                const uint32_t idx = base + it * 32u;
+                key[it] = idx < n ? keys_in[idx] : 0u;
+                val[it] = idx < n ? (vals_in ? vals_in[idx] : idx) : 0u;
+            }
+        }
+        const uint32_t r0 = tile * row_tiles, g0 = r0 / RADIX_GROUP;
+        {
+            uint2 a = make_uint2(0u, 0u), b = make_uint2(0u, 0u);
+            for (uint32_t g = seen + q; g < g0; g += NQ) {
+                const uint2 v = groups2[(size_t)g * (D / 2) + pair];
+                a.x += v.x;
+                a.y += v.y;
+            }
+            for (uint32_t r = g0 * RADIX_GROUP + q; r < r0; r += NQ) {
+                const uint32_t v = rows2[(size_t)r * (D / 2) + pair];
+                b.x += v & 0xFFFFu;
+                b.y += v >> 16;
+            }
+            reinterpret_cast<uint2*>(s_grp[q])[pair] = a;
+            reinterpret_cast<uint2*>(s_row[q])[pair] = b;
+        }
+        seen = g0;
+        for (uint32_t i = t; i < RS_WARPS * D / 2; i += RS_THREADS) reinterpret_cast<uint32_t*>(&s_wc[0][0])[i] = 0u;
+        __syncthreads();
+        uint32_t live = 0xFFFFFFFFu;  // bit it: the pair takes part
+        auto rank_item = [&](int it, bool valid, uint32_t peers) {
+            const uint32_t d = (key[it] >> shift) & (D - 1u);
             const int leader = __ffs(peers) - 1;
             uint32_t before = 0;
-            if (d < 256u && (int)lane == leader) before = atomicAdd(&s_wc[warp][d], (uint32_t)__popc(peers));
+            if (valid && (int)lane == leader) {
+                before = s_wc[warp][d];
+                s_wc[warp][d] = (uint16_t)(before + __popc(peers));
+            }
             before = __shfl_sync(0xFFFFFFFFu, before, leader);
             rank[it] = before + __popc(peers & lanemask_lt());
-        }
-        __syncthreads();
-        // 2. digit d (thread d): per-warp run offsets, tile total, early publish
-        const uint32_t d = threadIdx.x;
-        uint32_t run = 0;
+            __syncwarp();  // the counters as the next item's leaders read them
+        };
+        if (full && !DROP) {
 #pragma unroll
-        for (int w = 0; w < RS_WARPS; ++w) {
-            const uint32_t c = s_wc[w][d];
-            s_wc[w][d] = run;
-            run += c;
-        }
-        unsigned long long* my = status + (size_t)tile * RS_BINS + d;
-        if (tile == 0) lb_store(my, lb_pack(epoch, 2u, run));
-        else lb_store(my, lb_pack(epoch, 1u, run));
-        {
-            uint32_t total;
-            s_lstart[d] = block_excl_scan<RS_WARPS>(run, s_scan, &total);
-        }
-        __syncthreads();
-        // 3. stage digit-sorted
+            for (int it = 0; it < RS_ITEMS; ++it)
+                rank_item(it, true, match_digit<BITS, true>((key[it] >> shift) & (D - 1u), true));
+        } else {
+            live = 0u;
 #pragma unroll
-        for (int it = 0; it < RS_ITEMS; ++it) {
-            const uint32_t idx = base + it * 32;
-            if (idx < n) {
-                const uint32_t dd = (key[it] >> shift) & 255u;
-                const uint32_t pos = s_lstart[dd] + s_wc[warp][dd] + rank[it];
-                s_kv[pos] = make_uint2(key[it], val[it]);
+            for (int it = 0; it < RS_ITEMS; ++it) {
+                const bool valid = base + it * 32u < n && !(DROP && key[it] == NONE);
+                live |= (uint32_t)valid << it;
+                rank_item(it, valid, match_digit<BITS, false>((key[it] >> shift) & (D - 1u), valid));
             }
         }
-        // 4. look-back for digit d over earlier tiles (aggregate already
-        // published), LB_BATCH status words per round trip: the words are
-        // read together and consumed in order up to the first inclusive
-        // prefix (done) or the first one not yet published (wait, retry there)
-        uint32_t prefix = 0;
-        if (tile > 0) {
-            const uint32_t ep = epoch & 0x3FFFFFFFu;
-            int64_t j = (int64_t)tile - 1;
-            uint32_t spins = 0;
-            for (;;) {
-                unsigned long long wv[LB_BATCH];
-#pragma unroll
-                for (int q = 0; q < LB_BATCH; ++q)
-                    wv[q] = j - q >= 0 ? lb_load(status + (size_t)(j - q) * RS_BINS + d) : 0ull;
-                uint32_t consumed = 0;
-                int state = 0;  // 0: all consumed, 1: inclusive prefix reached, 2: wait
-#pragma unroll
-                for (int q = 0; q < LB_BATCH; ++q) {
-                    if (state == 0) {
-                        const uint32_t wep = (uint32_t)(wv[q] >> 34), fl = (uint32_t)(wv[q] >> 32) & 3u;
-                        if (wep != ep || fl == 0u) {
-                            state = 2;
-                        } else {
-                            prefix += (uint32_t)wv[q];
-                            ++consumed;
-                            if (fl == 2u) state = 1;
-                        }
-                    }
-                }
-                if (state == 1) break;
-                j -= consumed;  // tile 0 always holds an inclusive prefix, so j stays >= 0
-                if (state == 2) {
-                    if (++spins > SPIN_LIMIT) { atomicOr(&ctr->flags, F_SPIN_TIMEOUT); break; }
-                    __nanosleep(20);
-                }
-            }
-            lb_store(my, lb_pack(epoch, 2u, prefix + run));
-        }
-        s_gofs[d] = s_gbase[d] + prefix - s_lstart[d];
         __syncthreads();
-        // 5. coalesced write of the staged tile
-        const uint32_t tile_n = min((uint32_t)RS_TILE, n - tile * RS_TILE);
-        for (uint32_t j0 = threadIdx.x & ~31u; j0 < tile_n; j0 += RS_THREADS) {  // warp-uniform trips
-            const uint32_t j = j0 + lane;
-            const bool valid = j < tile_n;
-            const uint2 kv = valid ? s_kv[j] : make_uint2(0xFFFFFFFFu, 0u);
-            const uint32_t pos = s_gofs[(kv.x >> shift) & 255u] + j;
-            if (valid && pos < n) {
-                if (keys_out) keys_out[pos] = kv.x;  // null: only the permutation is wanted
+        uint32_t cnt = 0, ofs = 0, tile_n;
+        if (t < D) {
+#pragma unroll
+            for (int w = 0; w < RS_WARPS; ++w) cnt += s_wc[w][t];
+#pragma unroll
+            for (uint32_t k = 0; k < NQ; ++k) {
+                run += s_grp[k][t];
+                ofs += s_row[k][t];
+            }
+        }
+        const uint32_t lstart = block_excl_scan<RS_WARPS>(cnt, s_scan[1], &tile_n);
+        if (t < D) {
+            uint32_t p = lstart;
+#pragma unroll
+            for (int w = 0; w < RS_WARPS; ++w) {
+                const uint32_t c = s_wc[w][t];
+                s_wc[w][t] = (uint16_t)p;
+                p += c;
+            }
+            s_gofs[t] = run + ofs - lstart;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int it = 0; it < RS_ITEMS; ++it)
+            if ((live >> it) & 1u)
+                s_kv[s_wc[warp][(key[it] >> shift) & (D - 1u)] + rank[it]] = make_uint2(key[it], val[it]);
+        __syncthreads();
+        for (uint32_t j = t; j < tile_n; j += RS_THREADS) {
+            const uint2 kv = s_kv[j];
+            const uint32_t pos = s_gofs[(kv.x >> shift) & (D - 1u)] + j;
+            if (pos < n) {
+                if (keys_out) keys_out[pos] = kv.x;
                 vals_out[pos] = kv.y;
-            }
-            if (ranges) {  // neighbours' keys from the adjacent lanes, across warps from shared memory
-                uint32_t kp = __shfl_up_sync(0xFFFFFFFFu, kv.x, 1), kn = __shfl_down_sync(0xFFFFFFFFu, kv.x, 1);
-                if (lane == 0) kp = j > 0 ? s_kv[j - 1].x : ~kv.x;
-                if (lane == 31) kn = j + 1 < tile_n ? s_kv[j + 1].x : ~kv.x;
-                if (valid && pos < n && kv.x < n_ranges) {
+                if (ranges && kv.x < n_ranges) {
+                    const uint32_t kp = j > 0u ? s_kv[j - 1u].x : ~kv.x;
+                    const uint32_t kn = j + 1u < tile_n ? s_kv[j + 1u].x : ~kv.x;
                     if (kp != kv.x) atomicMin(&ranges[kv.x].x, pos);
                     if (kn != kv.x) atomicMin(&ranges[kv.x].y, ~(pos + 1u));
                 }
             }
         }
-        __syncthreads();
+        __syncthreads();  // the partial sums of the next tile go over the staged pairs
     }
 }
 
-void launch_radix_hist(const uint32_t* keys, const uint32_t* n32, const unsigned long long* n64, uint64_t cap,
-                       int passes, uint32_t* hist, int grid, cudaStream_t s) {
-    k_radix_hist<<<grid, 256, 0, s>>>(keys, n32, n64, cap, passes, hist);
+int radix_grid(int sms) { return 2 * sms; }
+
+void launch_radix_count(const uint32_t* keys, const uint32_t* n32, const unsigned long long* n64, uint64_t cap,
+                        int shift, int bits, RadixTab tab, int grid, cudaStream_t s) {
+    launch_k(k_radix_count, grid, RS_THREADS, s, keys, n32, n64, cap, shift, bits, tab);
 }
 
-void launch_radix_pass(const uint32_t* keys_in, const uint32_t* vals_in, uint32_t* keys_out, uint32_t* vals_out,
-                       const uint32_t* n32, const unsigned long long* n64, uint64_t cap, int shift,
-                       const uint32_t* hist, unsigned long long* status, uint32_t* ticket, const FrameParams* fp,
-                       Counters* ctr, int grid, cudaStream_t s, int hw_match, uint2* ranges, uint32_t n_ranges) {
-    if (hw_match)
-        launch_k(k_radix_pass<true>, grid, RS_THREADS, s, keys_in, vals_in, keys_out, vals_out, n32,
-                  n64, cap, shift, hist, status, ticket, fp, ctr, ranges, n_ranges);
-    else
-        launch_k(k_radix_pass<false>, grid, RS_THREADS, s, keys_in, vals_in, keys_out, vals_out, n32,
-                  n64, cap, shift, hist, status, ticket, fp, ctr, ranges, n_ranges);
+void launch_radix_scatter(const uint32_t* keys_in, const uint32_t* vals_in, uint32_t* keys_out, uint32_t* vals_out,
+                          const uint32_t* n32, const unsigned long long* n64, uint64_t cap, int shift, int bits,
+                          RadixTab tab, uint32_t row_len, bool drop, int grid, cudaStream_t s, uint2* ranges,
+                          uint32_t n_ranges) {
+#define VGR_SCATTER_D(B, DR)                                                                                          \
+    launch_k(k_radix_scatter<B, DR>, grid, RS_THREADS, s, keys_in, vals_in, keys_out, vals_out, n32, n64, cap, shift, \
+             tab, RS_TILE / row_len, ranges, n_ranges)
+#define VGR_SCATTER(B)                   \
+    do {                                 \
+        if (drop) VGR_SCATTER_D(B, true); \
+        else VGR_SCATTER_D(B, false);    \
+    } while (0)
+    switch (bits) {
+        case 5: VGR_SCATTER(5); break;
+        case 6: VGR_SCATTER(6); break;
+        case 7: VGR_SCATTER(7); break;
+        default: VGR_SCATTER(8); break;
+    }
+#undef VGR_SCATTER
+#undef VGR_SCATTER_D
 }
 
 }  // namespace vgr

@@ -151,6 +151,7 @@ struct vgr_view {
     VisBuffers vis{};
     // vgr_view_debug's copies of the records, made on its first call
     uint2* dbg_rect = nullptr;
+    uint32_t* dbg_tile = nullptr;
     float4 *dbg_recA = nullptr, *dbg_recB = nullptr, *dbg_rgb = nullptr;
     // depth sort: the partition's (key, value) pairs fill all of sort_kv; the
     // radix passes use its halves as their key buffers
@@ -179,9 +180,10 @@ struct vgr_view {
     bool copy_pending[2] = {false, false};
     int img_sel = 0;  // device image the next pipelined frame writes
     float* lut = nullptr;
-    unsigned long long* status = nullptr;
-    size_t st_emit = 0, st_depth = 0, st_tile = 0, st_depth_stride = 0,
-           st_tile_stride = 0, st_words = 0;
+    unsigned long long* status = nullptr;  // look-back words of the slot scan
+    uint16_t* radix_rows = nullptr;        // digit counts: of the pass under way,
+    uint32_t* tile_groups = nullptr;       // per group of rows: of the tile sort's passes,
+    uint32_t* depth_groups = nullptr;      // and of the four passes of a radix depth order
     Counters* ctr = nullptr;
     ViewState* vstate = nullptr;
     FrameParams* fp_dev = nullptr;
@@ -591,7 +593,7 @@ vgr_status alloc_vis(vgr_view* v, uint32_t cap) {
 void free_pairs(vgr_view* v) {
     drop_graphs(v);
     for (int i = 0; i < 2; ++i) { dfree(v->pairK[i]); dfree(v->pairV[i]); }
-    dfree(v->slot_owner);
+    dfree(v->slot_owner); dfree(v->dbg_tile);
     v->pair_bytes = 0;
 }
 
@@ -630,21 +632,43 @@ vgr_status alloc_cut(vgr_view* v, uint32_t cap) {
     return VGR_OK;
 }
 
-// look-back word regions; sized from the current capacities
+// Digit passes of the tile sort: tile ids 0 .. n_tiles - 1 in digits of 5 to 8
+// bits, the last one no wider than it has to be.
+struct TilePlan {
+    int passes, bits, last_bits;
+};
+TilePlan tile_plan(uint32_t n_tiles) {
+    int need = 1;
+    while (need < 32 && ((uint64_t)1 << need) < n_tiles) ++need;
+    const int passes = (need + 7) / 8;
+    const int bits = std::max(5, (need + passes - 1) / passes);
+    return {passes, bits, std::max(5, need - (passes - 1) * bits)};
+}
+constexpr int TILE_PASSES_MAX = 3;  // at most 2^20 tiles
+
+// Words of the tile sort's group counts: the first pass has a row per emission
+// chunk, the others one per radix tile.
+size_t tile_group_words(uint64_t cap_pairs, int passes, int bits) {
+    return radix_group_words(cap_pairs, EMIT_SLOTS, bits) +
+           (size_t)(passes - 1) * radix_group_words(cap_pairs, RADIX_TILE, bits);
+}
+size_t table_row_words(uint64_t cap_pairs, uint32_t cap_vis) {
+    return std::max(radix_row_words(cap_pairs, EMIT_SLOTS, 8), radix_row_words(cap_vis, RADIX_TILE, 8));
+}
+
+// the sorts' tables and the slot scan's look-back words; sized from the current capacities
 vgr_status alloc_status(vgr_view* v) {
     drop_graphs(v);
-    dfree(v->status);
-    const uint32_t RT = radix_tile();
-    v->st_emit = 0;
-    v->st_depth = v->st_emit + ceil_div(v->cap_vis, slot_scan_tile()) + 1;
-    v->st_depth_stride = (size_t)(ceil_div(v->cap_vis, RT) + 1) * 256;
-    v->st_tile = v->st_depth + 4 * v->st_depth_stride;
-    v->st_tile_stride = (size_t)(ceil_div(v->cap_pairs, RT) + 1) * 256;
-    v->st_words = v->st_tile + 4 * v->st_tile_stride;
+    dfree(v->status); dfree(v->radix_rows); dfree(v->tile_groups); dfree(v->depth_groups);
     uint64_t b = 0;
-    vgr_status s = dalloc(&v->status, v->st_words, &b);
+    vgr_status s;
+    if ((s = dalloc(&v->status, ceil_div(v->cap_vis, slot_scan_tile()) + 1, &b)) ||
+        (s = dalloc(&v->radix_rows, table_row_words(v->cap_pairs, v->cap_vis), &b)) ||
+        (s = dalloc(&v->tile_groups, tile_group_words(v->cap_pairs, TILE_PASSES_MAX, 8), &b)) ||
+        (s = dalloc(&v->depth_groups, 4 * radix_group_words(v->cap_vis, RADIX_TILE, 8), &b)))
+        return s;
     v->status_bytes = b;
-    return s;
+    return VGR_OK;
 }
 
 // Bytes cleared at the start of a frame: the counters, the depth bins, the bit
@@ -718,6 +742,7 @@ void destroy_view(vgr_view* v) {
     free_cut(v);
     dfree(v->bitmap); dfree(v->front_bm); dfree(v->frontier[0]); dfree(v->frontier[1]);
     dfree(v->ranges); dfree(v->tile_order); dfree(v->image); dfree(v->lut); dfree(v->status);
+    dfree(v->radix_rows); dfree(v->tile_groups); dfree(v->depth_groups);
     dfree(v->ctr); dfree(v->bucket_start); dfree(v->vstate); dfree(v->fp_dev);
     if (v->fp_host) cudaFreeHost(v->fp_host);
     if (v->ctr_host) cudaFreeHost(v->ctr_host);
@@ -905,15 +930,16 @@ vgr_status vgr_view_bytes_estimate(const vgr_hierarchy* h, const vgr_view_opts* 
     const uint64_t n_words = ((N + 31) / 32 + TW - 1) / TW * TW;
     const uint64_t per_vis = 2 * sizeof(uint32_t) + 3 * sizeof(float4) + sizeof(float) /* visible SoA */ +
                              sizeof(uint32_t) /* slot offsets */ + 4 * sizeof(uint32_t) /* depth sort */;
-    const uint64_t RT = radix_tile();
-    const uint64_t status_words = ceil_div(cap_vis, slot_scan_tile()) + 1 +
-                                  4 * (ceil_div(cap_vis, RT) + 1) * 256 + 4 * (ceil_div(cap_pairs, RT) + 1) * 256;
+    const uint64_t table_bytes = 8 * (ceil_div(cap_vis, slot_scan_tile()) + 1) +
+                                 2 * table_row_words(cap_pairs, (uint32_t)cap_vis) +
+                                 4 * (tile_group_words(cap_pairs, TILE_PASSES_MAX, 8) +
+                                      4 * radix_group_words(cap_vis, RADIX_TILE, 8));
     const uint32_t T = o.tile_size ? o.tile_size : TILE_DEFAULT;
     const uint64_t tiles = (uint64_t)((width + T - 1) / T) * ((height + T - 1) / T);
     uint64_t b = 3 * 4 * cap_cut + per_vis * cap_vis + 4 * 4 * cap_pairs + 4 * emit_owner_cap(cap_pairs) + 2 * 4 * n_words + 2 * 4 * N +
-                 cleared_bytes((uint32_t)n_words, MAX_RANKS) + 8 * (depth_bucket_cap(MAX_RANKS) + 1) + sizeof(ViewState) + sizeof(FrameParams) + 260 * 4 + 8 * status_words;
+                 cleared_bytes((uint32_t)n_words, MAX_RANKS) + 8 * (depth_bucket_cap(MAX_RANKS) + 1) + sizeof(ViewState) + sizeof(FrameParams) + 260 * 4 + table_bytes;
     b += (uint64_t)width * height * 3 * 4 + tiles * (sizeof(uint2) + 4);
-    *bytes = b;
+    *bytes = (b + (2u << 20) - 1) / (2u << 20) * (2u << 20);  // device memory is handed out in 2 MiB pieces
     return VGR_OK;
 }
 
@@ -927,19 +953,6 @@ vgr_status vgr_view_device_bytes(const vgr_view* v, uint64_t* bytes) {
 
 namespace {
 
-// Digit passes of the tile sort: tile ids 0 .. n_tiles-1 plus the sentinel
-// (all ones in the sorted bits) that marks dropped candidate slots.
-int tile_passes_for(uint32_t n_tiles) {
-    int bits = 0;
-    while (bits < 32 && ((uint64_t)1 << bits) <= n_tiles) ++bits;
-    return std::max(1, (bits + 7) / 8);
-}
-
-// The emission's grid relative to the look-back kernels' (x/4): four CTAs
-// per SM, like the radix passes (with room for 54 registers a thread it ran
-// 0.199 ms on the city against 0.221 at six CTAs per SM and 40 registers).
-constexpr int EMIT_GRID_NUM = 4;
-
 // After a depth bucket did not fit a CTA, this many frames of the view order
 // their depths by radix passes before the partition is tried again.
 constexpr int RADIX_FRAMES = 64;
@@ -947,8 +960,8 @@ constexpr int RADIX_FRAMES = 64;
 uint32_t frame_kernels(const vgr_view* v, bool scratch, bool radix_depth, int tile_passes) {
     const uint32_t lod = scratch ? v->h->max_depth + 1u : 1u;
     return lod + 1u /*compact*/ + 1u /*preprocess, with colour*/ +
-           (radix_depth ? 6u /*histogram, 4 passes, slot scan*/ : 2u /*partition, buckets*/) + 1u /*emit*/ +
-           (uint32_t)tile_passes + 1u /*tile order (finishes the ranges)*/ + 1u /*blend*/;
+           (radix_depth ? 9u /*4 counts, 4 scatters, slot scan*/ : 2u /*partition, buckets*/) + 1u /*emit*/ +
+           2u * (uint32_t)tile_passes - 1u /*counts but the first, scatters*/ + 1u /*tile order (finishes the ranges)*/ + 1u /*blend*/;
 }
 
 // The frame's status block and cut sizes, read back after its last kernel.
@@ -969,7 +982,11 @@ uint32_t enqueue_frame(vgr_view* v, bool scratch, bool radix_depth, int tile_pas
     const FrameParams& fh = *v->fp_host;
     const uint32_t n_tiles = fh.tiles_x * fh.tiles_y;
     cudaMemcpyAsync(v->fp_dev, v->fp_host, sizeof(FrameParams), cudaMemcpyHostToDevice, s);
+    const TilePlan plan = tile_plan(n_tiles);
     cudaMemsetAsync(v->ctr, 0, cleared_bytes(v->n_words, v->cap_vis), s);
+    cudaMemsetAsync(v->tile_groups, 0, tile_group_words(v->cap_pairs, plan.passes, plan.bits) * sizeof(uint32_t), s);
+    if (radix_depth)
+        cudaMemsetAsync(v->depth_groups, 0, 4 * radix_group_words(v->cap_vis, RADIX_TILE, 8) * sizeof(uint32_t), s);
     cudaMemsetAsync(v->ranges, 0xFF, (size_t)n_tiles * sizeof(uint2), s);  // (start, ~end): both all ones
     // the first kernel waits for the copies above in plain stream order; with
     // stage events between the kernels none of them is launched early
@@ -1001,33 +1018,39 @@ uint32_t enqueue_frame(vgr_view* v, bool scratch, bool radix_depth, int tile_pas
         // every potentially visible entry is sorted; culled ones carry the key
         // 0xFFFFFFFF and land last
         uint32_t* const sortK[2] = {v->sort_kv, v->sort_kv + v->cap_vis};
-        launch_radix_hist(v->vis.depth, &v->ctr->n_front, nullptr, v->cap_vis, 4, &v->ctr->depth_hist[0][0],
-                          v->grid_scan, s);
+        const int grid = radix_grid(v->h->num_sms);
         for (int p = 0; p < 4; ++p) {
             const uint32_t* kin = p == 0 ? v->vis.depth : sortK[(p + 1) & 1];
             const uint32_t* vin = p == 0 ? nullptr : v->sortV[(p + 1) & 1];
+            const RadixTab tab{v->radix_rows, v->depth_groups + p * radix_group_words(v->cap_vis, RADIX_TILE, 8)};
+            launch_radix_count(kin, &v->ctr->n_front, nullptr, v->cap_vis, 8 * p, 8, tab, grid, s);
             // the last pass writes only the permutation (the sorted keys are not read)
-            launch_radix_pass(kin, vin, p == 3 ? nullptr : sortK[p & 1], v->sortV[p & 1], &v->ctr->n_front, nullptr,
-                              v->cap_vis, 8 * p,
-                              v->ctr->depth_hist[p], v->status + v->st_depth + p * v->st_depth_stride,
-                              &v->ctr->tickets[TK_SORT0 + p], v->fp_dev, v->ctr, v->grid_scan, s, p == 3 ? 1 : 0);
+            launch_radix_scatter(kin, vin, p == 3 ? nullptr : sortK[p & 1], v->sortV[p & 1], &v->ctr->n_front,
+                                 nullptr, v->cap_vis, 8 * p, 8, tab, RADIX_TILE, false, grid, s);
         }
-        launch_slot_scan(order, v->cap_vis, v->vis, v->slot_off, v->slot_owner, v->cap_pairs, v->status + v->st_emit,
+        launch_slot_scan(order, v->cap_vis, v->vis, v->slot_off, v->slot_owner, v->cap_pairs, v->status,
                          v->ctr, v->fp_dev, v->grid_scan, s);
     }
     mark(VGR_STAGE_COLOR);  // (evaluated in preprocess: the stage is empty)
     mark(VGR_STAGE_EMIT);
-    const uint32_t sentinel = (uint32_t)((1ull << (8 * tile_passes)) - 1ull);
-    launch_emit(order, v->cap_vis, v->vis, v->slot_off, v->slot_owner, v->pairK[0], v->pairV[0], v->cap_pairs, tile_passes, sentinel,
-                v->ctr, v->fp_dev, v->grid_scan * EMIT_GRID_NUM / 4, s);
+    RadixTab tab{v->radix_rows, v->tile_groups};
+    launch_emit(order, v->cap_vis, v->vis, v->slot_off, v->slot_owner, v->pairK[0], v->pairV[0], v->cap_pairs,
+                plan.passes == 1 ? plan.last_bits : plan.bits, tab, v->ctr, v->fp_dev, v->grid_scan, s);
     mark(VGR_STAGE_TILE_SORT);
-    // (the last pass also records each tile's range)
-    for (int p = 0; p < tile_passes; ++p) {
-        const bool last = p + 1 == tile_passes;
-        launch_radix_pass(v->pairK[p & 1], v->pairV[p & 1], v->pairK[(p + 1) & 1], v->pairV[(p + 1) & 1], nullptr,
-                          &v->ctr->n_cand, v->cap_pairs, 8 * p, v->ctr->tile_hist[p],
-                          v->status + v->st_tile + p * v->st_tile_stride, &v->ctr->tickets[TK_SORT0 + 4 + p],
-                          v->fp_dev, v->ctr, v->grid_scan, s, last ? 1 : 0, last ? v->ranges : nullptr, n_tiles);
+    // the first pass drops the slots that failed the tile test; the last records
+    // each tile's range, and nothing reads its keys
+    for (int p = 0; p < plan.passes; ++p) {
+        const int bits = p + 1 == plan.passes ? plan.last_bits : plan.bits, shift = plan.bits * p;
+        const bool last = p + 1 == plan.passes;
+        const unsigned long long* n = p == 0 ? &v->ctr->n_cand : &v->ctr->n_pairs;
+        const int grid = radix_grid(v->h->num_sms);
+        if (p > 0) {
+            tab.groups = v->tile_groups + tile_group_words(v->cap_pairs, p, plan.bits);
+            launch_radix_count(v->pairK[p & 1], nullptr, n, v->cap_pairs, shift, bits, tab, grid, s);
+        }
+        launch_radix_scatter(v->pairK[p & 1], v->pairV[p & 1], last ? nullptr : v->pairK[(p + 1) & 1],
+                             v->pairV[(p + 1) & 1], nullptr, n, v->cap_pairs, shift, bits, tab,
+                             p == 0 ? EMIT_SLOTS : RADIX_TILE, p == 0, grid, s, last ? v->ranges : nullptr, n_tiles);
     }
     v->last_tile_buf = tile_passes & 1;
     mark(VGR_STAGE_RANGES);
@@ -1241,7 +1264,7 @@ vgr_status prepare_frame(vgr_view* v, const vgr_camera* cam, float tau, float* h
     q.cam = *cam;
     q.tau = tau;
     q.host = host_rgb;
-    q.tile_passes = tile_passes_for(TW * TH);
+    q.tile_passes = tile_plan(TW * TH).passes;
     volatile float f = std::max(cam->fx, cam->fy);
     volatile float t = tau / f;
     volatile float k = t * t;
@@ -1706,6 +1729,8 @@ vgr_status vgr_view_debug(vgr_view* v, vgr_debug_buffers* o) {
         dfree(v->dbg_rect); dfree(v->dbg_recA); dfree(v->dbg_recB); dfree(v->dbg_rgb);
         return s;
     }
+    if (!v->dbg_tile && (s = dalloc(&v->dbg_tile, v->cap_pairs, nullptr))) return s;
+    launch_debug_tiles(v->ranges, v->last_tw * v->last_th, v->dbg_tile, v->last_n_pairs, v->stream);
     launch_debug_records(v->vis, std::min(v->last_n_front, v->cap_vis), v->dbg_rect, v->dbg_recA, v->dbg_recB,
                          v->dbg_rgb, v->stream);
     VGR_CK(cudaGetLastError());
@@ -1715,7 +1740,7 @@ vgr_status vgr_view_debug(vgr_view* v, vgr_debug_buffers* o) {
     o->vis_recB = reinterpret_cast<const float*>(v->dbg_recB);
     o->vis_rgb = reinterpret_cast<const float*>(v->dbg_rgb);
     o->depth_order = v->sortV[1];
-    o->pair_tile = v->pairK[v->last_tile_buf];
+    o->pair_tile = v->dbg_tile;
     o->pair_val = v->pairV[v->last_tile_buf];
     o->tile_range = reinterpret_cast<const uint32_t*>(v->ranges);
     o->tile_size = tile_of(v);

@@ -23,9 +23,9 @@ constexpr int MAX_TREE_DEPTH = 64;
 constexpr uint32_t SPIN_LIMIT = 1u << 22;     // bounded waits in look-back scans
 constexpr uint32_t CHILD_SHIFT = 28;          // child word: first_child | n_child << 28
 constexpr uint32_t CHILD_MASK = (1u << CHILD_SHIFT) - 1u;
-constexpr int RADIX_THREADS = 256;            // one radix-sort tile: 256 threads x 15 keys
-constexpr int RADIX_ITEMS = 15;
-constexpr int RADIX_TILE = RADIX_THREADS * RADIX_ITEMS;
+constexpr int RADIX_THREADS = 512;            // one radix-sort tile: 512 threads x 8 keys
+constexpr uint32_t RADIX_TILE = RADIX_THREADS * 8;
+constexpr uint32_t RADIX_GROUP = 32;          // rows of digit counts per group
 constexpr int DEPTH_BINS = 6144;              // bins of the depth keys' histogram (k_depth.cu)
 
 // flags in Counters::flags
@@ -40,8 +40,8 @@ enum : uint32_t {
     F_SORT_SKEW = 128u,    // a depth bucket too large for one CTA: redo the frame with the radix passes
 };
 
-// ticket slots (dynamic tile order for the chained scans)
-enum : int { TK_COMPACT = 0, TK_PRE = 1, TK_EMIT = 2, TK_SORT0 = 3 /* .. TK_SORT0 + 7 */, TK_COUNT = 12 };
+// ticket slots (dynamic tile order for the chained scan)
+enum : int { TK_EMIT = 0, TK_COUNT = 1 };
 
 struct Counters;
 
@@ -119,8 +119,6 @@ struct Counters {
     unsigned long long pix_contribs;
     uint32_t tickets[TK_COUNT];
     uint32_t frontier_n[MAX_TREE_DEPTH + 2];
-    uint32_t depth_hist[4][256];
-    uint32_t tile_hist[4][256];
     uint32_t tile_buckets[33];  // tiles per log2(pairs + 1) class (the blend order)
     uint32_t blend_next;        // the blend's next tile in its work list
 };
@@ -203,42 +201,12 @@ __device__ __forceinline__ unsigned long long lb_load(unsigned long long* p) {
     return a.load(cuda::memory_order_relaxed);
 }
 
-// Publish this tile's aggregate, walk back to an inclusive prefix, publish
-// the inclusive value; returns the exclusive prefix.  'status' points at
-// this scan's word array with 'stride' words between consecutive tiles.
-// Tiles are handed out in ticket order, so every predecessor is running or
-// done; the wait is still bounded and reports F_SPIN_TIMEOUT.
-__device__ __forceinline__ uint32_t lookback(unsigned long long* status, uint32_t stride, uint32_t tile,
-                                             uint32_t agg, uint32_t epoch, uint32_t* flags) {
-    const uint32_t ep = epoch & 0x3FFFFFFFu;
-    if (tile == 0) {
-        lb_store(status, lb_pack(epoch, 2u, agg));
-        return 0;
-    }
-    lb_store(status + (size_t)tile * stride, lb_pack(epoch, 1u, agg));
-    uint32_t prefix = 0;
-    int64_t j = (int64_t)tile - 1;
-    uint32_t spins = 0;
-    while (j >= 0) {
-        unsigned long long w = lb_load(status + (size_t)j * stride);
-        uint32_t wep = (uint32_t)(w >> 34), fl = (uint32_t)(w >> 32) & 3u;
-        if (wep != ep || fl == 0u) {
-            if (++spins > SPIN_LIMIT) { atomicOr(flags, F_SPIN_TIMEOUT); break; }
-            __nanosleep(20);
-            continue;
-        }
-        prefix += (uint32_t)w;
-        if (fl == 2u) break;
-        --j;
-    }
-    lb_store(status + (size_t)tile * stride, lb_pack(epoch, 2u, prefix + agg));
-    return prefix;
-}
-
-// Warp-wide variant (all 32 lanes of one warp call it): each step reads 32
-// predecessor words at once, so the prefix is usually found after one L2
-// round trip instead of one per predecessor.  Same words and result as
-// lookback(); every lane returns the exclusive prefix.
+// Publish this tile's aggregate, look back to an inclusive prefix, publish the
+// inclusive value; returns the exclusive prefix in every lane (all 32 lanes of
+// one warp call it).  'status' points at the scan's word array with 'stride'
+// words between consecutive tiles.  Each step reads 32 predecessor words at
+// once.  Tiles are handed out in ticket order, so every predecessor is running
+// or done; the wait is still bounded and reports F_SPIN_TIMEOUT.
 __device__ __forceinline__ uint32_t lookback_warp(unsigned long long* status, uint32_t stride, uint32_t tile,
                                                   uint32_t agg, uint32_t epoch, uint32_t* flags) {
     const uint32_t lane = lane_id();
@@ -364,19 +332,6 @@ __device__ __forceinline__ float lod_interp_weight(float an, float ap, float t) 
 // The interpolated mean, single-rounded per component: mn + w (mp - mn).
 __device__ __forceinline__ float lod_lerp_rn(float a, float b, float w) {
     return __fadd_rn(a, __fmul_rn(w, __fsub_rn(b, a)));
-}
-
-// Lanes of the (full) warp holding the same 9-bit value (a radix digit
-// 0..255, or 256 for "no digit"): one ballot per bit.
-__device__ __forceinline__ uint32_t match_digit(uint32_t d) {
-    uint32_t m = 0xFFFFFFFFu;
-#pragma unroll
-    for (int b = 0; b < 9; ++b) {
-        const bool bit = (d >> b) & 1u;
-        const uint32_t vote = __ballot_sync(0xFFFFFFFFu, bit);
-        m &= bit ? vote : ~vote;
-    }
-    return m;
 }
 
 }  // namespace vgr

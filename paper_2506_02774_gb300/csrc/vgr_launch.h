@@ -102,14 +102,24 @@ void launch_depth_sort(const VisBuffers& vis, uint32_t cap_vis, const uint32_t* 
                        uint32_t* owner, uint64_t cap_pairs, Counters* ctr, const FrameParams* fp, int sms, cudaStream_t s);
 
 // k_sort.cu
-uint32_t radix_tile();
-void launch_radix_hist(const uint32_t* keys, const uint32_t* n32, const unsigned long long* n64, uint64_t cap,
-                       int passes, uint32_t* hist /*[4][256]*/, int grid, cudaStream_t s);
-void launch_radix_pass(const uint32_t* keys_in, const uint32_t* vals_in, uint32_t* keys_out, uint32_t* vals_out,
-                       const uint32_t* n32, const unsigned long long* n64, uint64_t cap, int shift,
-                       const uint32_t* hist, unsigned long long* status, uint32_t* ticket, const FrameParams* fp,
-                       Counters* ctr, int grid, cudaStream_t s, int hw_match = 0, uint2* ranges = nullptr,
-                       uint32_t n_ranges = 0);
+// Tables of one digit pass: digit counts per row (a tile's keys, or a part of
+// it) and per RADIX_GROUP rows; the groups are cleared before they are counted.
+struct RadixTab {
+    uint16_t* rows;
+    uint32_t* groups;
+};
+size_t radix_row_words(uint64_t n, uint32_t row_len, int bits);    // 16-bit words of the rows
+size_t radix_group_words(uint64_t n, uint32_t row_len, int bits);  // 32-bit words of the groups
+int radix_grid(int sms);
+// rows of RADIX_TILE keys
+void launch_radix_count(const uint32_t* keys, const uint32_t* n32, const unsigned long long* n64, uint64_t cap,
+                        int shift, int bits, RadixTab tab, int grid, cudaStream_t s);
+// bits: 5 to 8; row_len: keys per row of the tables, RADIX_TILE or a divisor of it; the element count is *n32, *n64
+// or (both null) cap, and at most cap
+void launch_radix_scatter(const uint32_t* keys_in, const uint32_t* vals_in, uint32_t* keys_out, uint32_t* vals_out,
+                          const uint32_t* n32, const unsigned long long* n64, uint64_t cap, int shift, int bits,
+                          RadixTab tab, uint32_t row_len, bool drop, int grid, cudaStream_t s, uint2* ranges = nullptr,
+                          uint32_t n_ranges = 0);
 
 // k_emit.cu
 // slot offsets in depth order, into slot_off[cap_vis + 1], after a radix depth sort
@@ -117,9 +127,13 @@ void launch_slot_scan(const uint32_t* order, uint32_t cap_vis, const VisBuffers&
                       uint32_t* owner, uint64_t cap_pairs, unsigned long long* status, Counters* ctr, const FrameParams* fp, int grid,
                       cudaStream_t s);
 uint32_t emit_owner_cap(uint64_t cap_pairs);  // entries of the owner table (first rank of each emission chunk)
+// 'tab' receives the counts of the keys' low 'bits' bits, one row per EMIT_SLOTS slots; dropped slots (key all ones)
+// are not counted
 void launch_emit(const uint32_t* order, uint32_t cap_vis, const VisBuffers& vis, const uint32_t* slot_off,
-                 const uint32_t* owner, uint32_t* pair_key, uint32_t* pair_val, uint64_t cap_pairs, int tile_passes,
-                 uint32_t sentinel, Counters* ctr, const FrameParams* fp, int grid, cudaStream_t s);
+                 const uint32_t* owner, uint32_t* pair_key, uint32_t* pair_val, uint64_t cap_pairs, int bits,
+                 RadixTab tab, Counters* ctr, const FrameParams* fp, int grid, cudaStream_t s);
+// the tile of every sorted pair, from the ranges
+void launch_debug_tiles(const uint2* ranges, uint32_t n_tiles, uint32_t* pair_tile, uint64_t n_pairs, cudaStream_t s);
 uint32_t slot_scan_tile();
 void launch_tile_order(uint2* ranges, uint32_t n_tiles, uint32_t* order, Counters* ctr, cudaStream_t s);
 constexpr uint32_t BATCH_VIEWS_MAX = 1024;  // views of one batch blend (k_batch_offsets: one thread each)
@@ -140,12 +154,12 @@ void launch_batch_order(const FrameParams* const* fps, uint32_t n_views, const u
                         int grid, cudaStream_t s);
 
 // vgr_sort_api.cu: enqueue a standalone pair sort on caller-provided scratch
-size_t sort_status_words(uint64_t n, int passes);
+size_t sort_row_words(uint64_t n);                  // 16-bit words
+size_t sort_group_words(uint64_t n, int passes);    // 32-bit words
 int sort_passes(uint32_t key_bits);
 cudaError_t sort_pairs_enqueue(const uint32_t* keys_in, const uint32_t* vals_in, uint32_t* keys_out,
-                               uint32_t* vals_out, uint64_t n, uint32_t key_bits, FrameParams* fp, Counters* ctr,
-                               unsigned long long* status, uint32_t* tmp_keys, uint32_t* tmp_vals, int grid,
-                               cudaStream_t s);
+                               uint32_t* vals_out, uint64_t n, int passes, uint16_t* rows, uint32_t* groups,
+                               uint32_t* tmp_keys, uint32_t* tmp_vals, int sms, cudaStream_t s);
 
 // k_store.cu
 void convert_sh_half(const float* src, uint32_t n, uint32_t k3, void* dst, uint32_t stride, cudaStream_t s);

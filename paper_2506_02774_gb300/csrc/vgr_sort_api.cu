@@ -1,9 +1,8 @@
 // vgr_sort_api.cu -- the pair sort of the frame path (paper Sec. 3.1
 // 'Sorting') as a standalone C-ABI call: stable LSD radix sort of u32
-// (key, value) pairs on the device, 8-bit digits, one onesweep pass per digit
-// (k_sort.cu).  Scratch (digit histograms, look-back words, the ping-pong
-// buffer of multi-pass sorts) comes from a per-device cache owned by the
-// library.
+// (key, value) pairs on the device, 8-bit digits, a count and a scatter kernel
+// per digit (k_sort.cu).  Scratch (digit counts, the ping-pong buffer of
+// multi-pass sorts) comes from a per-device cache owned by the library.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -18,37 +17,19 @@
 
 namespace vgr {
 
-// Start of a sort: new look-back epoch, element count, zeroed tickets,
-// histograms and flags.
-__global__ void k_sort_setup(FrameParams* fp, Counters* ctr, unsigned long long n) {
-    uint32_t* t = ctr->tickets;
-    for (int i = threadIdx.x; i < TK_COUNT; i += blockDim.x) t[i] = 0u;
-    uint32_t* h = &ctr->depth_hist[0][0];
-    for (int i = threadIdx.x; i < 4 * 256; i += blockDim.x) h[i] = 0u;
-    if (threadIdx.x == 0) {
-        uint32_t e = fp->epoch + 1u;
-        if ((e & 0x3FFFFFFFu) == 0u) ++e;
-        fp->epoch = e;
-        ctr->flags = 0u;
-        ctr->n_pairs = n;
-    }
-}
-
-size_t sort_status_words(uint64_t n, int passes) {
-    return (size_t)passes * ((n + radix_tile() - 1) / radix_tile() + 1) * 256;
-}
+size_t sort_row_words(uint64_t n) { return radix_row_words(n, RADIX_TILE, 8); }
+size_t sort_group_words(uint64_t n, int passes) { return (size_t)passes * radix_group_words(n, RADIX_TILE, 8); }
 
 int sort_passes(uint32_t key_bits) { return (int)((key_bits + 7u) / 8u); }
 
 // Enqueue a sort on 's' with the given scratch; returns a CUDA error code.
 cudaError_t sort_pairs_enqueue(const uint32_t* keys_in, const uint32_t* vals_in, uint32_t* keys_out,
-                               uint32_t* vals_out, uint64_t n, uint32_t key_bits, FrameParams* fp, Counters* ctr,
-                               unsigned long long* status, uint32_t* tmp_keys, uint32_t* tmp_vals, int grid,
-                               cudaStream_t s) {
-    const int passes = sort_passes(key_bits);
-    k_sort_setup<<<1, 256, 0, s>>>(fp, ctr, (unsigned long long)n);
-    launch_radix_hist(keys_in, nullptr, &ctr->n_pairs, n, passes, &ctr->depth_hist[0][0], grid, s);
-    const size_t stride = sort_status_words(n, 1);
+                               uint32_t* vals_out, uint64_t n, int passes, uint16_t* rows, uint32_t* groups,
+                               uint32_t* tmp_keys, uint32_t* tmp_vals, int sms, cudaStream_t s) {
+    cudaError_t e = cudaMemsetAsync(groups, 0, sort_group_words(n, passes) * sizeof(uint32_t), s);
+    if (e != cudaSuccess) return e;
+    const int grid = (int)std::min<uint64_t>(radix_grid(sms), (n + RADIX_TILE - 1) / RADIX_TILE);
+    PdlScope pdl(true);  // the first kernel follows the clear in plain stream order
     // the last pass writes the output; earlier passes alternate backwards
     const uint32_t* kin = keys_in;
     const uint32_t* vin = vals_in;
@@ -56,9 +37,9 @@ cudaError_t sort_pairs_enqueue(const uint32_t* keys_in, const uint32_t* vals_in,
         const bool to_out = ((passes - 1 - p) & 1) == 0;
         uint32_t* ko = to_out ? keys_out : tmp_keys;
         uint32_t* vo = to_out ? vals_out : tmp_vals;
-        launch_radix_pass(kin, vin, ko, vo, nullptr, &ctr->n_pairs, n, 8 * p, ctr->depth_hist[p],
-                          status + (size_t)p * stride, &ctr->tickets[TK_SORT0 + p], fp, ctr, grid, s,
-                          p == passes - 1 ? 1 : 0);
+        const RadixTab tab{rows, groups + sort_group_words(n, p)};
+        launch_radix_count(kin, nullptr, nullptr, n, 8 * p, 8, tab, grid, s);
+        launch_radix_scatter(kin, vin, ko, vo, nullptr, nullptr, n, 8 * p, 8, tab, RADIX_TILE, false, grid, s);
         kin = ko;
         vin = vo;
     }
@@ -73,14 +54,27 @@ namespace {
 
 struct SortCache {
     std::mutex mu;
-    FrameParams* fp = nullptr;
-    Counters* ctr = nullptr;
-    unsigned long long* status = nullptr;
-    size_t status_words = 0;
+    uint16_t* rows = nullptr;
+    size_t row_words = 0;
+    uint32_t* groups = nullptr;
+    size_t group_words = 0;
     uint32_t* tmp = nullptr;
     uint64_t tmp_n = 0;
-    int grid = 0;
+    int sms = 0;
 };
+
+// Room for 'words' elements at p, growing it if there is less.
+template <typename T>
+cudaError_t sort_room(T*& p, size_t& have, size_t words) {
+    if (words <= have) return cudaSuccess;
+    if (p) cudaFree(p);
+    p = nullptr;
+    have = 0;
+    const cudaError_t e = cudaMalloc(&p, words * sizeof(T));
+    if (e == cudaSuccess) have = words;
+    else p = nullptr;
+    return e;
+}
 
 SortCache g_cache[64];
 
@@ -104,29 +98,15 @@ extern "C" vgr_status vgr_sort_pairs(const uint32_t* keys_in, const uint32_t* va
     if (e != cudaSuccess || dev < 0 || dev >= 64) return sort_fail(VGR_E_CUDA, "cudaGetDevice", e);
     SortCache& c = g_cache[dev];
     std::lock_guard<std::mutex> lock(c.mu);
-    if (!c.fp) {
-        if ((e = cudaMalloc(&c.fp, sizeof(FrameParams))) != cudaSuccess ||
-            (e = cudaMemset(c.fp, 0, sizeof(FrameParams))) != cudaSuccess ||
-            (e = cudaMalloc(&c.ctr, sizeof(Counters))) != cudaSuccess ||
-            (e = cudaMemset(c.ctr, 0, sizeof(Counters))) != cudaSuccess ||
-            (e = cudaStreamSynchronize(cudaStreamLegacy)) != cudaSuccess)  // the fills before any use on 's'
-            return sort_fail(VGR_E_NOMEM, "sort scratch", e);
+    if (!c.sms) {
         int sms = 0;
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        c.grid = std::max(1, sms * 4);
+        c.sms = std::max(1, sms);
     }
     const int passes = sort_passes(key_bits);
-    const size_t words = sort_status_words(n, passes);
-    if (words > c.status_words) {
-        if (c.status) cudaFree(c.status);
-        c.status = nullptr;
-        c.status_words = 0;
-        if ((e = cudaMalloc(&c.status, words * sizeof(unsigned long long))) != cudaSuccess ||
-            (e = cudaMemset(c.status, 0, words * sizeof(unsigned long long))) != cudaSuccess ||
-            (e = cudaStreamSynchronize(cudaStreamLegacy)) != cudaSuccess)
-            return sort_fail(VGR_E_NOMEM, "sort look-back words", e);
-        c.status_words = words;
-    }
+    if ((e = sort_room(c.rows, c.row_words, sort_row_words(n))) != cudaSuccess ||
+        (e = sort_room(c.groups, c.group_words, sort_group_words(n, passes))) != cudaSuccess)
+        return sort_fail(VGR_E_NOMEM, "sort digit counts", e);
     if (passes > 1 && n > c.tmp_n) {
         if (c.tmp) cudaFree(c.tmp);
         c.tmp = nullptr;
@@ -137,13 +117,9 @@ extern "C" vgr_status vgr_sort_pairs(const uint32_t* keys_in, const uint32_t* va
         c.tmp_n = n_al;
     }
     cudaStream_t s = (cudaStream_t)stream;
-    e = sort_pairs_enqueue(keys_in, vals_in, keys_out, vals_out, n, key_bits, c.fp, c.ctr, c.status, c.tmp,
-                           c.tmp ? c.tmp + c.tmp_n : nullptr, c.grid, s);
+    e = sort_pairs_enqueue(keys_in, vals_in, keys_out, vals_out, n, passes, c.rows, c.groups, c.tmp,
+                           c.tmp ? c.tmp + c.tmp_n : nullptr, c.sms, s);
     if (e != cudaSuccess) return sort_fail(VGR_E_CUDA, "sort launch", e);
-    uint32_t flags = 0;
-    if ((e = cudaMemcpyAsync(&flags, &c.ctr->flags, sizeof(flags), cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
-        (e = cudaStreamSynchronize(s)) != cudaSuccess)
-        return sort_fail(VGR_E_CUDA, "sort", e);
-    if (flags & F_SPIN_TIMEOUT) return sort_fail(VGR_E_TIMEOUT, "a look-back wait of the sort timed out");
+    if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return sort_fail(VGR_E_CUDA, "sort", e);
     return VGR_OK;
 }

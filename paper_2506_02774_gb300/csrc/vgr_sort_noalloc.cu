@@ -18,18 +18,16 @@ namespace {
 constexpr uint64_t NA_MAX_N = VGR_SORT_NOALLOC_MAX_N;
 constexpr int NA_MAX_PASSES = 4;
 constexpr size_t na_round(size_t x) { return (x + 255) / 256 * 256; }
-// layout of the static scratch: frame params (look-back epoch) | counters
-// (tickets, histograms, flags) | look-back words | ping-pong keys | ping-pong values
-constexpr size_t NA_OFF_FP = 0;
-constexpr size_t NA_OFF_CTR = na_round(sizeof(FrameParams));
-constexpr size_t NA_OFF_STATUS = NA_OFF_CTR + na_round(sizeof(Counters));
-constexpr size_t NA_STATUS_WORDS = (size_t)NA_MAX_PASSES * ((NA_MAX_N + RADIX_TILE - 1) / RADIX_TILE + 1) * 256;
-constexpr size_t NA_OFF_TMP = NA_OFF_STATUS + na_round(NA_STATUS_WORDS * sizeof(unsigned long long));
+// layout of the static scratch: digit counts of the tiles | of the groups, per pass | ping-pong keys | ping-pong values
+constexpr size_t NA_TILES = (NA_MAX_N + RADIX_TILE - 1) / RADIX_TILE;
+constexpr size_t NA_GROUPS = (NA_TILES + RADIX_GROUP - 1) / RADIX_GROUP;
+constexpr size_t NA_OFF_GROUPS = na_round(NA_TILES * 256 * sizeof(uint16_t));
+constexpr size_t NA_OFF_TMP = NA_OFF_GROUPS + na_round(NA_MAX_PASSES * NA_GROUPS * 256 * sizeof(uint32_t));
 constexpr size_t NA_BYTES = NA_OFF_TMP + 2 * NA_MAX_N * sizeof(uint32_t);
 
 struct NaDevice {
     unsigned char* base = nullptr;  // device address of the scratch array on this device
-    int grid = 0;
+    int sms = 0;
 };
 std::mutex g_na_mu;
 NaDevice g_na_dev[64];
@@ -64,13 +62,13 @@ extern "C" vgr_status vgr_sort_pairs_noalloc(const uint32_t* keys_in, const uint
     if (e != cudaSuccess || dev < 0 || dev >= 64) return na_fail(VGR_E_CUDA, "cudaGetDevice", e);
     cudaStream_t s = (cudaStream_t)stream;
     unsigned char* base = nullptr;
-    int grid = 0;
+    int sms = 0;
     {
         std::lock_guard<std::mutex> lock(g_na_mu);
         NaDevice& d = g_na_dev[dev];
         if (!d.base) {
             // first call on this device, with it current: resolve the array's
-            // device address and clear it (epoch and look-back words start at 0)
+            // device address and clear it
             void* p = nullptr;
             if ((e = cudaGetSymbolAddress(&p, g_sort_scratch)) != cudaSuccess)
                 return na_fail(VGR_E_CUDA, "cudaGetSymbolAddress of the sort scratch", e);
@@ -78,25 +76,20 @@ extern "C" vgr_status vgr_sort_pairs_noalloc(const uint32_t* keys_in, const uint
             // other stream is ordered after it
             if ((e = cudaMemsetAsync(p, 0, NA_BYTES, s)) != cudaSuccess || (e = cudaStreamSynchronize(s)) != cudaSuccess)
                 return na_fail(VGR_E_CUDA, "clearing the sort scratch", e);
-            int sms = 0;
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-            d.grid = std::max(1, sms * 4);
+            int count = 0;
+            cudaDeviceGetAttribute(&count, cudaDevAttrMultiProcessorCount, dev);
+            d.sms = std::max(1, count);
             d.base = static_cast<unsigned char*>(p);
         }
         base = d.base;
-        grid = d.grid;
+        sms = d.sms;
     }
-    FrameParams* fp = reinterpret_cast<FrameParams*>(base + NA_OFF_FP);
-    Counters* ctr = reinterpret_cast<Counters*>(base + NA_OFF_CTR);
-    unsigned long long* status = reinterpret_cast<unsigned long long*>(base + NA_OFF_STATUS);
+    uint16_t* rows = reinterpret_cast<uint16_t*>(base);
+    uint32_t* groups = reinterpret_cast<uint32_t*>(base + NA_OFF_GROUPS);
     uint32_t* tmp = reinterpret_cast<uint32_t*>(base + NA_OFF_TMP);
-    e = sort_pairs_enqueue(keys_in, vals_in, keys_out, vals_out, n, key_bits, fp, ctr, status, tmp, tmp + NA_MAX_N,
-                           grid, s);
+    e = sort_pairs_enqueue(keys_in, vals_in, keys_out, vals_out, n, sort_passes(key_bits), rows, groups, tmp,
+                           tmp + NA_MAX_N, sms, s);
     if (e != cudaSuccess) return na_fail(VGR_E_CUDA, "sort launch", e);
-    uint32_t flags = 0;
-    if ((e = cudaMemcpyAsync(&flags, &ctr->flags, sizeof(flags), cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
-        (e = cudaStreamSynchronize(s)) != cudaSuccess)
-        return na_fail(VGR_E_CUDA, "sort", e);
-    if (flags & F_SPIN_TIMEOUT) return na_fail(VGR_E_TIMEOUT, "a look-back wait of the sort timed out");
+    if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return na_fail(VGR_E_CUDA, "sort", e);
     return VGR_OK;
 }

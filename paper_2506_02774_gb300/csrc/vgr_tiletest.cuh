@@ -1,7 +1,5 @@
 // vgr_tiletest.cuh -- tile-level preemptive alpha test (paper Sec. 4.2,
-// Eq. 4, moved to binning).  Used by the counting pass (preprocess) and by
-// the emission pass; every operation is an explicitly rounded intrinsic so
-// both passes take bit-identical decisions.
+// Eq. 4, moved to binning), in explicitly rounded operations.
 #pragma once
 
 #include "vgr_internal.cuh"
@@ -20,10 +18,12 @@ __device__ __forceinline__ float clampf(float x, float lo, float hi) { return fm
 
 // Keep the pair when the maximum of rho over the rectangle spanned by the
 // tile's pixel centres reaches thre (= ln alpha* - ln theta - slack).  The
-// maximum is 0 when the mean lies inside; otherwise it is on an edge, where
-// rho is a concave quadratic in the free coordinate: on the edges x = x0, x1
-// its optimum is dy* = (-b/c) dx = ry dx, on y = y0, y1 it is
-// dx* = (-b/a) dy = rx dy, each clamped to the edge.
+// maximum is 0 when the mean lies inside; otherwise it is on an edge that faces
+// the mean (rho rises on the way from any point towards the mean, which leaves
+// the rectangle through one), where rho is a concave quadratic in the free
+// coordinate: on x = x0 or x1 its optimum is dy* = (-b/c) dx = ry dx, on y = y0 or
+// y1 it is dx* = (-b/a) dy = rx dy, each clamped to the edge.  At most one edge
+// of each pair faces the mean.
 // T is the tile side in pixels (8, 16 or 32): every coordinate below is exact in FP32.
 __device__ __forceinline__ bool tile_keep(float u, float v, float a, float b, float c, float rx, float ry, float thre,
                                           int tx, int ty, float W, float H, int T) {
@@ -34,11 +34,10 @@ __device__ __forceinline__ bool tile_keep(float u, float v, float a, float b, fl
     if (u >= x0 && u <= x1 && v >= y0 && v <= y1) return thre <= 0.f;
     const float dy_lo = __fsub_rn(y0, v), dy_hi = __fsub_rn(y1, v);
     const float dx_lo = __fsub_rn(x0, u), dx_hi = __fsub_rn(x1, u);
-    float best = rho_rn(a, b, c, dx_lo, clampf(__fmul_rn(ry, dx_lo), dy_lo, dy_hi));
-    best = fmaxf(best, rho_rn(a, b, c, dx_hi, clampf(__fmul_rn(ry, dx_hi), dy_lo, dy_hi)));
-    best = fmaxf(best, rho_rn(a, b, c, clampf(__fmul_rn(rx, dy_lo), dx_lo, dx_hi), dy_lo));
-    best = fmaxf(best, rho_rn(a, b, c, clampf(__fmul_rn(rx, dy_hi), dx_lo, dx_hi), dy_hi));
-    return best >= thre;
+    const float dx = u < x0 ? dx_lo : dx_hi, dy = v < y0 ? dy_lo : dy_hi;
+    const float rx_best = rho_rn(a, b, c, dx, clampf(__fmul_rn(ry, dx), dy_lo, dy_hi));
+    const float ry_best = rho_rn(a, b, c, clampf(__fmul_rn(rx, dy), dx_lo, dx_hi), dy);
+    return ((u < x0 || u > x1) && rx_best >= thre) || ((v < y0 || v > y1) && ry_best >= thre);
 }
 
 }  // namespace vgr
