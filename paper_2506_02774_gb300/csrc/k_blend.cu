@@ -4,9 +4,11 @@
 //
 // A tile of T x T pixels (T = 8, 16 or 32, a tuning knob) is T T / 32
 // strips of 32 / T rows x T columns; one warp shades one strip, one pixel per
-// lane.  The kernel is persistent: its CTAs (a few per SM) take tiles one at a
-// time from a work list ordered heaviest first -- the tiles of one view, or
-// of every view of a batch -- through a global counter, and the CTA's warps
+// lane (k_blend), or half as many strips with two pixels per lane (k_blend_wide,
+// for launches with many strips).  The kernels are persistent: their CTAs (a few
+// per SM) take tiles one at a time from a work list ordered heaviest first --
+// the tiles of one view, or of every view of a batch -- their first by block
+// index, then through a global counter, and the CTA's warps
 // claim the strips of the CTA's tiles from a shared counter, so a warp that
 // finishes a light strip moves on to the next strip at once instead of idling
 // until its tile's heaviest strip is done, and the strips of a tile run on
@@ -21,8 +23,9 @@
 // bit in a ring, and copies the 48-byte records (mean, conic, threshold,
 // opacity, colour) of DEPTH queued hits at a time with cp.async into its own
 // double-buffered slice of shared memory; the copies of the next chunk are in
-// flight while the current one is walked, two records at a time for
-// instruction-level parallelism.  Before the walk each lane rewrites its
+// flight while the current one is walked, four records at a time: their reads
+// and exponentials are independent, and only the transmittance runs through them
+// in order.  Before the walk each lane rewrites its
 // staged records for the strip's rows (the row offsets of the mean folded
 // into the conic terms), so a pixel evaluates rho with one subtraction and
 // two FMAs.  Records are read only for the pairs a strip needs, and the warps
@@ -42,6 +45,14 @@
 // the filtered-vs-unfiltered comparison; its row masks are all ones) and the
 // Eq. 5 lookup table for e^rho.  DEPTH (hits staged per chunk: 16, 32 or 48)
 // and T are tuning knobs; the image does not depend on them.
+//
+// What bounds it: large images by their instructions (issue slots 75 % busy),
+// small ones by the chunks of the longest strips (a horizon tile's 2000 to 3500
+// hits).  Groups of four records, first tiles dealt out, two pixels per lane and
+// parts of 32-pixel tiles as items of their own took the blend from 110 to 80 us
+// (1M-leaf box, 1080p), 184 to 161 (city, 1080p), 347 to 162 (1440p, 32-pixel
+// tiles), 81 to 48 and 56 (640 x 360 and 320 x 180 city views), 312 to 208
+// (canonical mode, 960 x 540).
 #include "vgr_internal.cuh"
 #include "vgr_launch.h"
 
@@ -50,7 +61,13 @@ namespace vgr {
 constexpr int BL_THREADS = 256;          // 8 warps: a warp shades one strip of 32 pixels at a time
 constexpr int BL_WARPS = BL_THREADS / 32;
 constexpr int BL_SCAN = 128;   // pair values scanned per batch (4 per lane, loaded one batch ahead)
+constexpr int BL_RING = 256;   // a warp's queue of pair values
+constexpr int BL_GROUP = 4;    // records a pixel evaluates at a time
 constexpr int BL_MIN_CTAS = 4; // resident CTAs per SM the register budget is set for (up to 64 registers)
+// resident CTAs per SM of k_blend by tile side: with three (80 registers) a group's
+// reads and the next group's slots are in flight together; strips of 4 rows read
+// two words per record and are better off with four CTAs and neither
+constexpr int bl_narrow_ctas(int tile) { return tile == 8 ? 4 : 3; }
 constexpr uint32_t FULL = 0xFFFFFFFFu;
 constexpr uint32_t WORK_TILE_BITS = 20;  // work item = view << 20 | tile
 constexpr uint32_t WORK_TILE_MASK = (1u << WORK_TILE_BITS) - 1u;
@@ -91,15 +108,14 @@ __device__ __forceinline__ uint32_t blend_prepare(float4& a, float4& b, float4& 
         const uint32_t hw = __float_as_uint(b.w);
         const float by = __half2float(__ushort_as_half((unsigned short)(hw & 0xFFFFu))) + 0.01f;
         const float bx = __half2float(__ushort_as_half((unsigned short)(hw >> 16))) + 0.01f;
-        const float cl = ceilf(a.x - bx - col0), ch = floorf(a.x + bx - col0);  // columns c: |col0 + c - u| <= bx
-        const float rl = ceilf(a.y - by - row0), rh = floorf(a.y + by - row0);  // rows of the strip likewise
+        // columns c with |col0 + c - u| <= bx, and rows of the strip likewise (conversions round and saturate)
+        const int c0 = max(__float2int_ru(a.x - bx - col0), 0), c1 = min(__float2int_rd(a.x + bx - col0), T - 1);
+        const int r0 = max(__float2int_ru(a.y - by - row0), 0), r1 = min(__float2int_rd(a.y + by - row0), SR - 1);
         pmask = 0u;
-        if (cl <= ch && rl <= rh && ch >= 0.f && cl <= (float)(T - 1) && rh >= 0.f && rl <= (float)(SR - 1)) {
-            const uint32_t c0 = (uint32_t)fmaxf(cl, 0.f), c1 = (uint32_t)fminf(ch, (float)(T - 1));
-            const uint32_t r0 = (uint32_t)fmaxf(rl, 0.f), r1 = (uint32_t)fminf(rh, (float)(SR - 1));
-            const uint32_t cols = ((2u << c1) - 1u) & ~((1u << c0) - 1u);
+        if (c0 <= c1) {
+            const uint32_t cols = (0xFFFFFFFFu >> (31 - c1)) & (0xFFFFFFFFu << c0);
 #pragma unroll
-            for (uint32_t r = 0; r < (uint32_t)SR; ++r)
+            for (int r = 0; r < SR; ++r)
                 if (r >= r0 && r <= r1) pmask |= cols << (r * T);
         }
     }
@@ -137,18 +153,32 @@ __device__ __forceinline__ uint32_t blend_prepare(float4& a, float4& b, float4& 
 // Transpose of the 32 x 32 bit matrix held by a warp, lane l holding row l:
 // afterwards lane q holds column q (bit l = bit q of lane l's row).  Five
 // exchange steps, each swapping the off-diagonal blocks of half the size.
+// The two larger ones move whole bytes.
 template <uint32_t J, uint32_t M>
 __device__ __forceinline__ uint32_t transpose_step(uint32_t x, uint32_t lane) {
     const uint32_t y = __shfl_xor_sync(0xFFFFFFFFu, x, J);
-    return (lane & J) ? ((x & ~M) | ((y & ~M) >> J)) : ((x & M) | ((y & M) << J));
+    const uint32_t up = lane & J;                      // 0: keep M and take the partner's M shifted up; J: the others
+    const uint32_t m = __funnelshift_l(M, M, up);      // M, or ~M
+    return (x & m) | (__funnelshift_l(y, y, J - 2u * up) & ~m);
 }
 __device__ __forceinline__ uint32_t warp_transpose32(uint32_t x) {
     const uint32_t lane = lane_id();
-    x = transpose_step<16, 0x0000FFFFu>(x, lane);
-    x = transpose_step<8, 0x00FF00FFu>(x, lane);
+    x = __byte_perm(x, __shfl_xor_sync(0xFFFFFFFFu, x, 16), (lane & 16u) ? 0x3276u : 0x5410u);
+    x = __byte_perm(x, __shfl_xor_sync(0xFFFFFFFFu, x, 8), (lane & 8u) ? 0x3715u : 0x6240u);
     x = transpose_step<4, 0x0F0F0F0Fu>(x, lane);
     x = transpose_step<2, 0x33333333u>(x, lane);
     return transpose_step<1, 0x55555555u>(x, lane);
+}
+
+// The staged slot of the foremost record in mm (bit 31 - l: slot 32 q + l), which
+// leaves mm; slot DEPTH when there is none: a record that no pixel takes
+// (dummy_part), so that a group of records needs no flags.
+template <int DEPTH>
+__device__ __forceinline__ uint32_t next_slot(uint32_t& mm, int q) {
+    const uint32_t c = __clz(mm);
+    mm &= ~(0x80000000u >> (c & 31u));
+    if (DEPTH == 32) return c;
+    return c < 32u ? 32u * q + c : (uint32_t)DEPTH;
 }
 
 __device__ __forceinline__ float ex2_approx(float x) {
@@ -157,33 +187,23 @@ __device__ __forceinline__ float ex2_approx(float x) {
     return y;
 }
 
-// One record at one pixel; returns false once the pixel has stopped.
+// Opacity of a record at a pixel (Eq. 3), and whether it takes part (Eq. 4, or
+// the alpha* test of the canonical mode).
 template <int MODE>
-__device__ __forceinline__ bool blend_step(BlendPixel& p, const float4& X, const float4* __restrict__ sC, uint32_t k,
-                                           float rho, const float* s_lut, uint32_t m, float lut_scale) {
-    float alpha;
+__device__ __forceinline__ bool blend_alpha(const float4& X, float rho, const float* s_lut, uint32_t m, float lut_scale,
+                                            float& alpha) {
     if (MODE == 0) {  // base 2, opacity folded in (see blend_prepare)
-        if (rho < LOG2_ALPHA_MIN) return true;
         alpha = fminf(ALPHA_MAX, ex2_approx(rho));
+        return !(rho < LOG2_ALPHA_MIN);
     } else if (MODE == 1) {  // canonical: Eq. 3, then the alpha* test
         alpha = fminf(ALPHA_MAX, X.w * __expf(rho));
-        if (alpha < ALPHA_MIN) return true;
+        return !(alpha < ALPHA_MIN);
     } else {
-        if (rho < X.z) return true;  // Eq. 4 before Eq. 3
-        // Eq. 5: nearest of m intervals over [-5.55, 0]
+        // Eq. 5: nearest of m intervals over [-5.55, 0] (the index is clamped for records that fail Eq. 4 too)
         const uint32_t idx = min(m, (uint32_t)__float2int_rn(rho * lut_scale));
         alpha = fminf(ALPHA_MAX, X.w * s_lut[idx]);
+        return !(rho < X.z);
     }
-    const float Tn = p.T * (1.f - alpha);
-    if (Tn < T_MIN) { p.done = true; return false; }
-    const float w = alpha * p.T;
-    const float4 C4 = sC[k];
-    p.cr = fmaf(w, C4.x, p.cr);
-    p.cg = fmaf(w, C4.y, p.cg);
-    p.cb = fmaf(w, C4.z, p.cb);
-    p.T = Tn;
-    ++p.contribs;
-    return true;
 }
 
 // The staged X of slot i: only (u, A') in the exact mode.
@@ -227,6 +247,122 @@ struct WarpItem {
     uint32_t view;
 };
 
+// A CTA's claims: its warps take (slot, strip) items in order, a slot being a
+// tile of the work list, or a part of one of at most BL_WARPS strips (so that a
+// heavy tile of 32 x 32 pixels is not left to one CTA), claimed from the global
+// counter and published in a ring of 4 entries.
+constexpr int slot_strips(int ns) { return ns < BL_WARPS ? ns : BL_WARPS; }
+struct ClaimRing {
+    uint32_t claim;                        // next (slot, strip) item
+    uint32_t tile[4], tag[4], read[4];     // per entry: the slot's global number, slot + 1, strips that have read it
+    template <int TILE_STRIPS>
+    __device__ __forceinline__ void init() {
+        if (threadIdx.x == 0) claim = 0u;
+        if (threadIdx.x < 4) {
+            tag[threadIdx.x] = 0u;
+            read[threadIdx.x] = slot_strips(TILE_STRIPS) - 1;
+        }
+    }
+};
+
+// The next (tile, strip) item of this warp's CTA: idx is the tile's place in the
+// work list.  The CTA's first slot is number 'first' (NONE: a claimed one), later
+// ones are base + the global counter *next.  The warp that takes strip 0 of a
+// slot claims and publishes it; the other strips' warps wait for it.  False: a
+// wait ran out (F_SPIN_TIMEOUT).
+// First slots by block index deal the heaviest tiles out to the SMs one by one
+// (blocks go to the SMs in turn); claimed, they went to whichever CTAs came first,
+// and the SMs that got several finished last (240 tiles of a 320 x 180 view:
+// 82 us, dealt out 62).
+template <int TILE_STRIPS>
+__device__ __forceinline__ bool claim_item(ClaimRing& ring, uint32_t* next, uint32_t first, uint32_t base,
+                                           const FrameParams* fp0, uint32_t& idx_out, uint32_t& strip_out) {
+    constexpr uint32_t NS = slot_strips(TILE_STRIPS), PARTS = TILE_STRIPS / NS;
+    volatile uint32_t* slot_tile = ring.tile;
+    volatile uint32_t* slot_tag = ring.tag;
+    volatile uint32_t* slot_read = ring.read;
+    uint32_t idx = 0, strip = 0;
+    bool timed_out = false;
+    if (lane_id() == 0) {
+        const uint32_t k = atomicAdd(&ring.claim, 1u);
+        const uint32_t slot = k / NS, e = slot & 3u;
+        strip = k % NS;
+        uint32_t spins = 0;
+        if (strip == 0) {
+            while (slot_read[e] < NS - 1) {  // the entry's last readers
+                if (++spins > SPIN_LIMIT) { timed_out = true; break; }
+                __nanosleep(32);
+            }
+            idx = slot == 0u && first != NONE ? first : base + atomicAdd(next, 1u);
+            slot_read[e] = 0u;
+            slot_tile[e] = idx;
+            __threadfence_block();
+            slot_tag[e] = slot + 1u;
+        } else {
+            while (slot_tag[e] != slot + 1u) {
+                if (++spins > SPIN_LIMIT) { timed_out = true; break; }
+                __nanosleep(32);
+            }
+            __threadfence_block();
+            idx = slot_tile[e];
+            atomicAdd(&ring.read[e], 1u);
+        }
+        if (timed_out) atomicOr(&fp0->bl_ctr->flags, F_SPIN_TIMEOUT);
+    }
+    idx = __shfl_sync(FULL, idx, 0);
+    idx_out = idx / PARTS;
+    strip_out = __shfl_sync(FULL, strip, 0) + idx % PARTS * NS;
+    return !__shfl_sync(FULL, (uint32_t)timed_out, 0);
+}
+
+// The record in slot DEPTH of every staged part: at any pixel rho is far below
+// every threshold (and theta 0), in the layout that blend_prepare leaves.
+template <int MODE, int SR>
+__device__ __forceinline__ float4 dummy_part(int part) {
+    constexpr float LOW = -1e30f;
+    if (MODE == 0 && SR <= 2) return make_float4(0.f, 0.f, 0.f, LOW);
+    return part == 0 ? make_float4(0.f, 0.f, 0.f, 0.f) : make_float4(0.f, LOW, 0.f, LOW);
+}
+
+__device__ __forceinline__ void init_item(WarpItem& it) {
+    it.ctr = nullptr;
+    it.evals = it.contribs = 0ull;
+    it.view = 0xFFFFFFFFu;
+}
+
+// Lane 0: the statistics of the warp's last view.
+__device__ __forceinline__ void flush_item(volatile WarpItem& it) {
+    if (it.ctr && it.evals) {
+        atomicAdd(&it.ctr->pix_evals, (unsigned long long)it.evals);
+        atomicAdd(&it.ctr->pix_contribs, (unsigned long long)it.contribs);
+    }
+    it.evals = it.contribs = 0ull;
+}
+
+// Lane 0: the warp's item, a strip of nrows rows of T columns at (x0, y0) of the view.
+__device__ __forceinline__ void fill_item(volatile WarpItem& it, const FrameParams* fp, uint32_t view, uint32_t x0,
+                                          uint32_t y0, uint32_t T, uint32_t nrows) {
+    if (view != it.view) {
+        flush_item(it);
+        it.view = view;
+        it.ctr = fp->bl_ctr;
+    }
+    it.pair_val = fp->bl_pair_val;
+    it.rec = fp->bl_rec;
+    it.rgb = fp->bl_rgb;
+    it.image = fp->bl_image;
+    it.host_image = fp->host_image;
+    it.at = y0 * fp->width + x0;
+    it.width = fp->width;
+    it.nx = min(T, fp->width - x0);
+    it.ny = y0 < fp->height ? min(nrows, fp->height - y0) : 0u;
+}
+
+// Bits p0 .. p1 (0 <= p0, p1 < 32; none if p1 < p0)
+__device__ __forceinline__ uint32_t pair_range(int p0, int p1) {
+    return p1 < p0 ? 0u : (0xFFFFFFFFu >> (31 - p1)) & (0xFFFFFFFFu << p0);
+}
+
 // The blend, for tiles of T x T pixels.  A strip is SR = 32 / T rows of T
 // columns (one warp, one pixel per lane); a tile has NS = T T / 32 strips.  A
 // pair's 8-bit row mask has one bit per MR = max(1, T / 8) rows, and strip s
@@ -238,96 +374,33 @@ struct WarpItem {
 // reuses an entry the publishing warp waits until the entry's previous readers
 // have read it.  Every wait is on a claim made earlier in the CTA's order, so
 // none can close a cycle; each is still bounded and reports F_SPIN_TIMEOUT.
+//
+// The strips of one warp, tiles from place 0 up to n_work of the work list.
+// sbuf: staged records, [buffer][part: 0 = record A / X, 1 = colour, 2.. = record
+// B / row terms][warp][slot]; ring: the warp's queue of hit pair values (at a
+// strip's end its pixels); pm: the staged records' pixel masks.
 template <int MODE, int DEPTH, int T>
-__global__ void __launch_bounds__(BL_THREADS, BL_MIN_CTAS) k_blend(const FrameParams* __restrict__ fp0,
-                                                                   const FrameParams* const* __restrict__ fps,
-                                                                   const uint32_t* __restrict__ work,
-                                                                   uint32_t n_work, uint32_t* __restrict__ next) {
+__device__ __forceinline__ void blend_strips(float4 (*sbuf)[2 + (32 / T > 2 ? 2 : 1)][BL_WARPS][DEPTH + 1], uint32_t* ring,
+                                             uint32_t* pm, volatile WarpItem& it, ClaimRing& claims,
+                                             const FrameParams* __restrict__ fp0,
+                                             const FrameParams* const* __restrict__ fps,
+                                             const uint32_t* __restrict__ work, uint32_t n_work, uint32_t* next,
+                                             uint32_t first, uint32_t base, const float* s_lut, uint32_t m, float lut_scale, bool full_walk) {
     constexpr int SR = 32 / T;                    // rows per strip
     constexpr int NS = T * T / 32;                // strips per tile
     constexpr int MR = T >= 8 ? T / 8 : 1;        // rows per mask bit
     constexpr int SB = SR >= MR ? SR / MR : 1;    // mask bits of one strip
-    constexpr int RV = SR > 2 ? 2 : 1;            // float4 parts of the rewritten row terms
-    constexpr int NP = 2 + RV;                    // staged parts: X, colour, row terms
-    constexpr int RING = 256;                     // < DEPTH queued + BL_SCAN appended never exceeds it
+    constexpr int NP = 2 + (SR > 2 ? 2 : 1);      // staged parts: X, colour, row terms
+    constexpr bool AHEAD = SR <= 2;               // the next group's slots are found while one is evaluated
+    constexpr int RING = BL_RING;                 // < DEPTH queued + BL_SCAN appended never exceeds it
     static_assert(T == 8 || T == 16 || T == 32, "tile size 8, 16 or 32");
     static_assert(DEPTH % 16 == 0 && DEPTH <= 48, "staging depth: 16, 32 or 48 hits");
     static_assert(DEPTH + BL_SCAN <= RING, "ring too small");
-    pdl_wait();
-    // [buffer][part: 0 = record A / X, 1 = colour, 2.. = record B / row terms][warp][slot]
-    __shared__ __align__(16) float4 sbuf[2][NP][BL_WARPS][DEPTH];
-    __shared__ uint32_t s_ring[BL_WARPS][RING];  // per-warp queue of hit pair values
-    __shared__ float s_lut[MODE == 2 ? 260 : 1];
-    __shared__ WarpItem s_item[BL_WARPS];
-    __shared__ uint32_t s_pm[BL_WARPS][DEPTH];   // staged records' pixel masks
-    __shared__ __align__(16) float s_px[BL_WARPS][96];  // a finished strip's pixels, RGB
-    __shared__ uint32_t s_claim;                 // next (slot, strip) item of this CTA
-    __shared__ uint32_t s_slot_tile[4], s_slot_tag[4], s_slot_read[4];
     const uint32_t lane = lane_id(), warp = threadIdx.x >> 5;
-    uint32_t m = 0;
-    float lut_scale = 0.f;
-    if (threadIdx.x == 0) s_claim = 0u;
-    if (threadIdx.x < 4) {
-        s_slot_tag[threadIdx.x] = 0u;
-        s_slot_read[threadIdx.x] = NS - 1;
-    }
-    if (lane == 0) {
-        s_item[warp].ctr = nullptr;
-        s_item[warp].evals = s_item[warp].contribs = 0ull;
-        s_item[warp].view = 0xFFFFFFFFu;
-    }
-    if (MODE == 2) {  // the table mode runs on one view at a time
-        m = fp0->lut_size;
-        lut_scale = -(float)m / 5.55f;
-        for (uint32_t i = threadIdx.x; i <= m; i += BL_THREADS) s_lut[i] = fp0->bl_lut[i];
-    }
-    __syncthreads();
-    uint32_t* ring = s_ring[warp];
-    volatile WarpItem& it = s_item[warp];
-    const bool full_walk = (fp0->test_hooks & VGR_HOOK_FULL_STRIP_WALK) != 0u;
-    volatile uint32_t* slot_tile = s_slot_tile;
-    volatile uint32_t* slot_tag = s_slot_tag;
-    volatile uint32_t* slot_read = s_slot_read;
-    auto flush = [&]() {  // lane 0: the statistics of the warp's last view
-        if (it.ctr && it.evals) {
-            atomicAdd(&it.ctr->pix_evals, (unsigned long long)it.evals);
-            atomicAdd(&it.ctr->pix_contribs, (unsigned long long)it.contribs);
-        }
-        it.evals = it.contribs = 0ull;
-    };
     for (;;) {
-        // ---- claim a (tile, strip) item
-        uint32_t idx = 0, strip = 0;
-        bool timed_out = false;
-        if (lane == 0) {
-            const uint32_t k = atomicAdd(&s_claim, 1u);
-            const uint32_t slot = k / NS, e = slot & 3u;
-            strip = k % NS;
-            uint32_t spins = 0;
-            if (strip == 0) {
-                while (slot_read[e] < NS - 1) {  // the entry's last readers
-                    if (++spins > SPIN_LIMIT) { timed_out = true; break; }
-                    __nanosleep(32);
-                }
-                idx = atomicAdd(next, 1u);
-                slot_read[e] = 0u;
-                slot_tile[e] = idx;
-                __threadfence_block();
-                slot_tag[e] = slot + 1u;
-            } else {
-                while (slot_tag[e] != slot + 1u) {
-                    if (++spins > SPIN_LIMIT) { timed_out = true; break; }
-                    __nanosleep(32);
-                }
-                __threadfence_block();
-                idx = slot_tile[e];
-                atomicAdd(&s_slot_read[e], 1u);
-            }
-            if (timed_out) atomicOr(&fp0->bl_ctr->flags, F_SPIN_TIMEOUT);
-        }
-        idx = __shfl_sync(FULL, idx, 0);
-        strip = __shfl_sync(FULL, strip, 0);
-        if (__shfl_sync(FULL, (uint32_t)timed_out, 0) || idx >= n_work) break;
+        uint32_t idx, strip;
+        if (!claim_item<NS>(claims, next, first, base, fp0, idx, strip) || idx >= n_work)
+            break;
         uint2 rg;
         float rlo, clo;
         uint32_t wbits;
@@ -338,22 +411,7 @@ __global__ void __launch_bounds__(BL_THREADS, BL_MIN_CTAS) k_blend(const FramePa
             const FrameParams* fp = fps ? fps[view] : fp0;
             const uint32_t W = fp->width, H = fp->height, TW = fp->tiles_x;
             const uint32_t x0 = (tile % TW) * T, y0 = (tile / TW) * T + SR * strip;
-            if (lane == 0) {
-                if (view != it.view) {
-                    flush();
-                    it.view = view;
-                    it.ctr = fp->bl_ctr;
-                }
-                it.pair_val = fp->bl_pair_val;
-                it.rec = fp->bl_rec;
-                it.rgb = fp->bl_rgb;
-                it.image = fp->bl_image;
-                it.host_image = fp->host_image;
-                it.at = y0 * W + x0;
-                it.width = W;
-                it.nx = min((uint32_t)T, W - x0);
-                it.ny = y0 < H ? min((uint32_t)SR, H - y0) : 0u;
-            }
+            if (lane == 0) fill_item(it, fp, view, x0, y0, (uint32_t)T, (uint32_t)SR);
             rg = fp->bl_ranges[tile];
             inside = x0 + lane % T < W && y0 + lane / T < H;
             wbits = ((1u << SB) - 1u) << (SR * strip / MR);
@@ -440,7 +498,7 @@ __global__ void __launch_bounds__(BL_THREADS, BL_MIN_CTAS) k_blend(const FramePa
             for (int q = 0; q < (DEPTH + 31) / 32; ++q) {
                 const uint32_t sl = 32u * q + lane;
                 if (sl < (uint32_t)DEPTH)  // each lane its own slots; empty slots reach no pixel
-                    s_pm[warp][sl] = sl < nh ? blend_prepare<MODE, SR, T>(wA[sl], sbuf[buf][2][warp][sl],
+                    pm[sl] = sl < nh ? blend_prepare<MODE, SR, T>(wA[sl], sbuf[buf][2][warp][sl],
                                                                            sbuf[buf][NP - 1][warp][sl],
                                                                            MODE != 0 ? wC[sl].w : 0.f, rlo, clo,
                                                                            full_walk)
@@ -448,12 +506,12 @@ __global__ void __launch_bounds__(BL_THREADS, BL_MIN_CTAS) k_blend(const FramePa
             }
             __syncwarp();
             // the records that can reach this lane's pixel, as slot bits in
-            // depth order: the transpose of the records' pixel masks
+            // depth order from bit 31 down: the transpose of the records' pixel masks
             uint32_t reach[(DEPTH + 31) / 32];
 #pragma unroll
             for (int q = 0; q < (DEPTH + 31) / 32; ++q) {
-                const uint32_t sl = 32u * q + lane;
-                reach[q] = warp_transpose32(sl < (uint32_t)DEPTH ? s_pm[warp][sl] : 0u);
+                const uint32_t sl = 32u * q + 31u - lane;
+                reach[q] = warp_transpose32(sl < (uint32_t)DEPTH ? pm[sl] : 0u);
             }
             if (!p.done) {
                 // this lane's row r = lane / T.  Exact mode with strips of one or two
@@ -463,33 +521,105 @@ __global__ void __launch_bounds__(BL_THREADS, BL_MIN_CTAS) k_blend(const FramePa
                 const uint32_t r = lane / T;
                 const float4* wY = sbuf[buf][r == 0 ? 0 : 2][warp];
                 const float2* wR = reinterpret_cast<const float2*>(sbuf[buf][2 + r / 2][warp]) + (r & 1u);
-                auto eval = [&](uint32_t i, float4& X) -> float {
+                auto load = [&](uint32_t i, float4& X, float2& R) {
                     if constexpr (MODE == 0 && SR <= 2) {
                         X = wY[i];
+                    } else {
+                        X = load_x<MODE>(wA, i);
+                        R = wR[2 * i];
+                    }
+                };
+                auto rho_of = [&](const float4& X, const float2& R) -> float {
+                    if constexpr (MODE == 0 && SR <= 2) {
                         const float dx = X.x - p.fxp;
                         return fmaf(fmaf(X.y, dx, X.z), dx, X.w);
                     } else {
-                        X = load_x<MODE>(wA, i);
-                        return blend_rho(p, X, wR[2 * i]);
+                        return blend_rho(p, X, R);
                     }
                 };
 #pragma unroll
                 for (int q = 0; q < (DEPTH + 31) / 32; ++q) {
-                    uint32_t mm = reach[q];
-                    while (mm != 0u) {  // two records at a time for instruction-level parallelism
-                        const uint32_t i0 = 32u * q + __ffs(mm) - 1u;
-                        mm &= mm - 1u;
-                        const bool two = mm != 0u;
-                        const uint32_t i1 = two ? 32u * q + __ffs(mm) - 1u : i0;
-                        mm &= mm - 1u;
-                        float4 X0, X1;
-                        const float r0 = eval(i0, X0), r1 = eval(i1, X1);
-                        ++evals;
-                        if (!blend_step<MODE>(p, X0, wC, i0, r0, s_lut, m, lut_scale)) break;
-                        if (two) {
-                            ++evals;
-                            if (!blend_step<MODE>(p, X1, wC, i1, r1, s_lut, m, lut_scale)) break;
+                    uint32_t mm = reach[q];  // bit 31 - l: slot 32 q + l
+                    // BL_GROUP records at a time: their reads, rho and exponentials are
+                    // independent of one another and go out together; only the
+                    // transmittance runs through them in order
+                    evals += __popc(mm);
+                    uint32_t at[BL_GROUP], nat[BL_GROUP];
+                    auto take = [&](uint32_t* slots) {
+#pragma unroll
+                        for (int g = 0; g < BL_GROUP; ++g) slots[g] = next_slot<DEPTH>(mm, q);
+                    };
+                    auto advance = [&]() {
+                        if constexpr (AHEAD) {
+#pragma unroll
+                            for (int g = 0; g < BL_GROUP; ++g) at[g] = nat[g];
+                        } else {
+                            take(at);
                         }
+                    };
+                    take(at);
+                    while (at[0] != (uint32_t)DEPTH) {
+                        float alpha[BL_GROUP], Tg[BL_GROUP];
+                        bool use[BL_GROUP];
+                        const uint32_t left = mm;  // behind this group
+                        if constexpr (AHEAD) {
+                            float4 X[BL_GROUP];
+                            float2 R[BL_GROUP];
+#pragma unroll
+                            for (int g = 0; g < BL_GROUP; ++g) load(at[g], X[g], R[g]);
+                            take(nat);
+#pragma unroll
+                            for (int g = 0; g < BL_GROUP; ++g)
+                                use[g] = blend_alpha<MODE>(X[g], rho_of(X[g], R[g]), s_lut, m, lut_scale, alpha[g]);
+                        } else {
+#pragma unroll
+                            for (int g = 0; g < BL_GROUP; ++g) {
+                                float4 X;
+                                float2 R;
+                                load(at[g], X, R);
+                                use[g] = blend_alpha<MODE>(X, rho_of(X, R), s_lut, m, lut_scale, alpha[g]);
+                            }
+                        }
+                        if (MODE == 1 && !(use[0] || use[1] || use[2] || use[3])) {  // most fail there
+                            advance();
+                            continue;
+                        }
+                        float Tr = p.T;
+#pragma unroll
+                        for (int g = 0; g < BL_GROUP; ++g) {
+                            Tg[g] = Tr;
+                            if (use[g]) Tr = Tr * (1.f - alpha[g]);
+                        }
+                        // T never rises, so a group that ends at or above T_MIN stops nowhere
+                        int last = BL_GROUP;  // records of the group before the pixel stops
+                        if (Tr < T_MIN) {
+#pragma unroll
+                            for (int g = BL_GROUP - 1; g >= 0; --g)  // the first whose T falls below
+                                if (use[g] && Tg[g] * (1.f - alpha[g]) < T_MIN) last = g;
+                            p.done = true;
+                            // not evaluated: what is left of this word, and the group's after the stop
+                            evals -= __popc(left);
+#pragma unroll
+                            for (int g = 0; g < BL_GROUP; ++g) {
+                                if (g > last && at[g] != (uint32_t)DEPTH) --evals;
+                                if (g >= last) use[g] = false;
+                                if (g == last) Tr = Tg[g];
+                            }
+                        }
+#pragma unroll
+                        for (int g = 0; g < BL_GROUP; ++g) {
+                            const float4 C4 = wC[at[g]];
+                            if (use[g]) {
+                                const float w = alpha[g] * Tg[g];
+                                p.cr = fmaf(w, C4.x, p.cr);
+                                p.cg = fmaf(w, C4.y, p.cg);
+                                p.cb = fmaf(w, C4.z, p.cb);
+                                ++p.contribs;
+                            }
+                        }
+                        p.T = Tr;
+                        if (p.done) break;
+                        advance();
                     }
                     if (p.done) break;
                 }
@@ -507,7 +637,7 @@ __global__ void __launch_bounds__(BL_THREADS, BL_MIN_CTAS) k_blend(const FramePa
         const bool whole = it.nx == (uint32_t)T && it.ny == (uint32_t)SR && (it.width & 3u) == 0u &&
                            ((reinterpret_cast<uintptr_t>(host_image) & 15u) == 0u);
         if (whole) {
-            float* s = s_px[warp];
+            float* s = reinterpret_cast<float*>(ring);  // 96 of its words
             s[3 * lane + 0] = p.cr;
             s[3 * lane + 1] = p.cg;
             s[3 * lane + 2] = p.cb;
@@ -541,13 +671,389 @@ __global__ void __launch_bounds__(BL_THREADS, BL_MIN_CTAS) k_blend(const FramePa
         }
         __syncwarp();  // every lane is done with the item before lane 0 rewrites it
     }
-    if (lane == 0) flush();
+}
+
+template <int MODE, int DEPTH, int T>
+__global__ void __launch_bounds__(BL_THREADS, bl_narrow_ctas(T)) k_blend(const FrameParams* __restrict__ fp0,
+                                                                   const FrameParams* const* __restrict__ fps,
+                                                                   const uint32_t* __restrict__ work,
+                                                                   uint32_t n_work, uint32_t* __restrict__ next) {
+    pdl_wait();
+    __shared__ __align__(16) float4 sbuf[2][2 + (32 / T > 2 ? 2 : 1)][BL_WARPS][DEPTH + 1];
+    __shared__ __align__(16) uint32_t s_ring[BL_WARPS][BL_RING];
+    __shared__ uint32_t s_pm[BL_WARPS][DEPTH];
+    __shared__ float s_lut[MODE == 2 ? 260 : 1];
+    __shared__ WarpItem s_item[BL_WARPS];
+    __shared__ ClaimRing s_claims;
+    const uint32_t lane = lane_id(), warp = threadIdx.x >> 5;
+    uint32_t m = 0;
+    float lut_scale = 0.f;
+    s_claims.init<T * T / 32>();
+    if (lane == 0) init_item(s_item[warp]);
+    constexpr int NP = 2 + (32 / T > 2 ? 2 : 1);
+    if (lane < 2 * NP) sbuf[lane / NP][lane % NP][warp][DEPTH] = dummy_part<MODE, 32 / T>(lane % NP);
+    if (MODE == 2) {  // the table mode runs on one view at a time
+        m = fp0->lut_size;
+        lut_scale = -(float)m / 5.55f;
+        for (uint32_t i = threadIdx.x; i <= m; i += BL_THREADS) s_lut[i] = fp0->bl_lut[i];
+    }
+    __syncthreads();
+    blend_strips<MODE, DEPTH, T>(sbuf, s_ring[warp], s_pm[warp], s_item[warp], s_claims, fp0, fps, work, n_work, next,
+                                 blockIdx.x, gridDim.x, s_lut, m, lut_scale, (fp0->test_hooks & VGR_HOOK_FULL_STRIP_WALK) != 0u);
+    if (lane == 0) flush_item(s_item[warp]);
+}
+
+// The same blend for launches with many strips: tiles with few pairs take strips
+// of 64 pixels (64 / T rows), two neighbours of one row per lane, and a record
+// read for the lane serves both.  The arithmetic of a pixel is that of k_blend,
+// so the image is the same bit for bit.  Exact exponential, tiles of 16 or 32
+// pixels.  What it saves is the work per strip that does not depend on its pixels
+// (claim, parameters, ranges, queue, copies, store: 47 of 114 us on the 1M-leaf
+// box at 1080p with 32-pixel strips) and a part of the records' preparation; what
+// it costs is the length of a heavy tile's strips, so with 16-pixel tiles the
+// first *n_heavy tiles of the work list (BL_HEAVY_CLASS and up) keep strips of 32
+// pixels, claimed first.
+// next[0] counts those, next[1] the others.
+template <int DEPTH, int T>
+__global__ void __launch_bounds__(BL_THREADS, BL_MIN_CTAS) k_blend_wide(const FrameParams* __restrict__ fp0,
+                                                                        const FrameParams* const* __restrict__ fps,
+                                                                        const uint32_t* __restrict__ work,
+                                                                        uint32_t n_work,
+                                                                        const uint32_t* __restrict__ n_heavy,
+                                                                        uint32_t* __restrict__ next) {
+    constexpr int SR = 64 / T;                    // rows per strip
+    constexpr int NS = T * T / 64;                // strips per tile
+    constexpr int MR = T / 8;                     // rows per mask bit
+    constexpr int SB = SR >= MR ? SR / MR : 1;    // mask bits of one strip
+    constexpr int HP = T / 2;                     // lanes (pixel pairs) per row
+    constexpr int XR = SR > 2 ? SR - 2 : 0;       // row terms kept beside the raw records' slots
+    constexpr int RING = BL_RING;
+    constexpr int G = 2;                          // records a lane evaluates at a time, each at both pixels
+    static_assert(T == 16 || T == 32, "tile size 16 or 32");
+    static_assert(DEPTH % 16 == 0 && DEPTH <= 32, "staging depth: 16 or 32 hits");
+    static_assert(DEPTH + BL_SCAN <= RING && RING >= 64 * 3, "ring too small");
+    pdl_wait();
+    // [buffer][part: 0 = record's first half / row 0, 1 = colour, 2 = second half / row 1][warp][slot]
+    __shared__ __align__(16) float4 sbuf[2][3][BL_WARPS][DEPTH + 1];
+    __shared__ __align__(16) float4 s_row[XR > 0 ? XR : 1][BL_WARPS][XR > 0 ? DEPTH + 1 : 1];  // rows 2 and 3
+    __shared__ __align__(16) uint32_t s_ring[BL_WARPS][RING];  // queue of hit pair values; at the end the strip's pixels
+    __shared__ WarpItem s_item[BL_WARPS];
+    __shared__ uint2 s_pm[BL_WARPS][DEPTH];      // staged records' pixel masks: even and odd columns
+    __shared__ ClaimRing s_heavy, s_light;
+    const uint32_t lane = lane_id(), warp = threadIdx.x >> 5;
+    s_heavy.init<T * T / 32>();
+    s_light.init<NS>();
+    if (lane == 0) init_item(s_item[warp]);
+    if (lane < 6) sbuf[lane / 3][lane % 3][warp][DEPTH] = dummy_part<0, 2>(lane % 3);
+    if (XR > 0 && lane < XR) s_row[lane][warp][XR > 0 ? DEPTH : 0] = dummy_part<0, 2>(0);
+    __syncthreads();
+    uint32_t* ring = s_ring[warp];
+    volatile WarpItem& it = s_item[warp];
+    const bool full_walk = (fp0->test_hooks & VGR_HOOK_FULL_STRIP_WALK) != 0u;
+    // (strips of one row of a 32-pixel tile would all look at a mask bit's four rows)
+    const uint32_t heavy = T == 16 ? min(*n_heavy, n_work) : 0u;
+    // the first slots are dealt out over the whole list (heavy ones, then the
+    // others), the rest of the heavy ones and the rest of the others are claimed
+    constexpr uint32_t PARTS = NS / slot_strips(NS);  // slots of a tile (one for a heavy tile of 16 x 16)
+    const uint32_t dealt = gridDim.x, mine = blockIdx.x;
+    if (T == 16 && heavy > 0u)
+        blend_strips<0, DEPTH, T>(sbuf, ring, reinterpret_cast<uint32_t*>(s_pm[warp]), it, s_heavy, fp0, fps, work,
+                                  heavy, next, mine < heavy ? mine : NONE, dealt, nullptr, 0u, 0.f, full_walk);
+    const uint32_t light0 = T == 16 && mine < heavy ? NONE : mine, light_base = max(dealt, heavy);
+    static_assert(T == 32 || PARTS == 1, "slots count tiles where some of them are heavy");
+    const uint32_t row = lane / HP, col = 2u * (lane % HP);  // this lane's first pixel in the strip
+    for (;;) {
+        uint32_t idx, strip;
+        if (!claim_item<NS>(s_light, next + 1, light0, light_base, fp0, idx, strip) || idx >= n_work) break;
+        uint2 rg;
+        float rlo, clo, fxa;
+        uint32_t wbits;
+        bool in_a, in_b;
+        {
+            const uint32_t item = work[idx];
+            const uint32_t view = item >> WORK_TILE_BITS, tile = item & WORK_TILE_MASK;
+            const FrameParams* fp = fps ? fps[view] : fp0;
+            const uint32_t W = fp->width, H = fp->height, TW = fp->tiles_x;
+            const uint32_t x0 = (tile % TW) * T, y0 = (tile / TW) * T + SR * strip;
+            if (lane == 0) fill_item(it, fp, view, x0, y0, (uint32_t)T, (uint32_t)SR);
+            rg = fp->bl_ranges[tile];
+            in_a = x0 + col < W && y0 + row < H;
+            in_b = x0 + col + 1u < W && y0 + row < H;
+            wbits = ((1u << SB) - 1u) << (SR * strip / MR);
+            rlo = (float)y0 + 0.5f;  // centre of the strip's first row
+            clo = (float)x0 + 0.5f;  // and column
+            fxa = (float)(col + x0) + 0.5f;
+            __syncwarp();
+        }
+        const float fxb = fxa + 1.0f;  // exact
+        float Ta = 1.f, ra = 0.f, ga = 0.f, ba = 0.f, Tb = 1.f, rb = 0.f, gb = 0.f, bb = 0.f;
+        bool done_a = !in_a, done_b = !in_b;
+        uint32_t evals = 0, contribs = 0;
+        uint32_t head = 0, tail = 0;
+        uint32_t bp = rg.x;  // first pair value of the pending batch
+        uint32_t pend[BL_SCAN / 32];
+        {
+            const uint32_t* pv = it.pair_val;
+#pragma unroll
+            for (int g = 0; g < BL_SCAN / 32; ++g) {
+                const uint32_t j = bp + 32u * g + lane;
+                pend[g] = j < rg.y ? pv[j] : 0u;
+            }
+        }
+        auto refill = [&]() {
+            while (tail - head < (uint32_t)DEPTH && bp < rg.y) {
+#pragma unroll
+                for (int g = 0; g < BL_SCAN / 32; ++g) {
+                    const uint32_t v = pend[g];
+                    const bool hit = (v & wbits) != 0u;  // entries past the range hold 0
+                    const uint32_t hits = __ballot_sync(FULL, hit);
+                    if (hit) ring[(tail + __popc(hits & lanemask_lt())) & (RING - 1)] = v;
+                    tail += __popc(hits);
+                }
+                bp += BL_SCAN;
+                const uint32_t* pv = it.pair_val;
+#pragma unroll
+                for (int g = 0; g < BL_SCAN / 32; ++g) {
+                    const uint32_t j = bp + 32u * g + lane;
+                    pend[g] = j < rg.y ? pv[j] : 0u;
+                }
+            }
+            __syncwarp();
+        };
+        uint32_t rows_next = 0;  // row-mask bits of the pair staged in this lane's slot
+        auto issue = [&](int buf) -> uint32_t {
+            const uint32_t nh = min((uint32_t)DEPTH, tail - head);
+            if (lane < nh) {
+                const float4* rR = it.rec;
+                const float4* rC = it.rgb;
+                const uint32_t v = ring[(head + lane) & (RING - 1)], gi = v >> 8;
+                rows_next = v & wbits;
+                cp_async16(&sbuf[buf][0][warp][lane], rR + 2 * (size_t)gi);
+                cp_async16(&sbuf[buf][2][warp][lane], rR + 2 * (size_t)gi + 1);
+                cp_async16(&sbuf[buf][1][warp][lane], rC + gi);
+            }
+            cp_async_commit();
+            head += nh;
+            return nh;
+        };
+        refill();
+        uint32_t nh_cur = issue(0);
+        int buf = 0;
+        while (nh_cur > 0) {
+            if (__all_sync(FULL, done_a && done_b)) break;
+            const uint32_t rows = rows_next;
+            refill();
+            const uint32_t nh_next = issue(buf ^ 1);  // the next chunk in flight during this walk
+            cp_async_wait<1>();  // this chunk's copies (all but the newest group)
+            __syncwarp();
+            if (lane < (uint32_t)DEPTH) {  // each lane its own slot; empty slots reach no pixel
+                uint2 pm = make_uint2(0u, 0u);
+                if (lane < nh_cur) {
+                    const float4 a = sbuf[buf][0][warp][lane], b = sbuf[buf][2][warp][lane];
+                    pm = make_uint2(0xFFFFFFFFu, 0xFFFFFFFFu);
+                    if (!full_walk) {
+                        const uint32_t hw = __float_as_uint(b.w);
+                        const float by = __half2float(__ushort_as_half((unsigned short)(hw & 0xFFFFu))) + 0.01f;
+                        const float bx = __half2float(__ushort_as_half((unsigned short)(hw >> 16))) + 0.01f;
+                        const int c0 = max(__float2int_ru(a.x - bx - clo), 0), c1 = min(__float2int_rd(a.x + bx - clo), T - 1);
+                        int r0 = max(__float2int_ru(a.y - by - rlo), 0), r1 = min(__float2int_rd(a.y + by - rlo), SR - 1);
+                        if (SB == 2) {  // rows whose mask bit is clear are out of reach
+                            if (!(rows & (1u << (SR * strip / MR)))) r0 = max(r0, MR);
+                            if (!(rows & (2u << (SR * strip / MR)))) r1 = min(r1, MR - 1);
+                        }
+                        // pairs p with c0 <= 2 p <= c1, and with c0 <= 2 p + 1 <= c1
+                        const uint32_t ma = pair_range((c0 + 1) >> 1, c1 >> 1), mb = pair_range(c0 >> 1, (c1 - 1) >> 1);
+                        pm = make_uint2(0u, 0u);
+#pragma unroll
+                        for (int r = 0; r < SR; ++r)
+                            if (r >= r0 && r <= r1) {
+                                pm.x |= ma << (r * HP);
+                                pm.y |= mb << (r * HP);
+                            }
+                    }
+                    // per row (u, A', B' dy_r, C' dy_r^2 + log2 theta), as blend_prepare computes them
+                    const float Bc = a.w * LOG2E, Cc = b.x * LOG2E, add = (LN_ALPHA_MIN - b.y) * LOG2E;
+                    const float Ap = a.z * LOG2E;
+#pragma unroll
+                    for (int r = 0; r < SR; ++r) {
+                        const float dy = a.y - (rlo + (float)r);
+                        const float4 Y = make_float4(a.x, Ap, Bc * dy, fmaf(Cc * dy, dy, add));
+                        if (r == 0) sbuf[buf][0][warp][lane] = Y;
+                        else if (r == 1) sbuf[buf][2][warp][lane] = Y;
+                        else s_row[XR > 0 ? r - 2 : 0][warp][XR > 0 ? lane : 0] = Y;
+                    }
+                }
+                s_pm[warp][lane] = pm;
+            }
+            __syncwarp();
+            // the records that can reach this lane's pixels, as slot bits in depth
+            // order from bit 31 down: the transposes of the records' pixel masks
+            uint32_t reach_a, reach_b;
+            {
+                const uint32_t sl = 31u - lane;
+                const uint2 pm = sl < (uint32_t)DEPTH ? s_pm[warp][sl] : make_uint2(0u, 0u);
+                reach_a = warp_transpose32(pm.x);
+                reach_b = warp_transpose32(pm.y);
+            }
+            if (done_a) reach_a = 0u;
+            if (done_b) reach_b = 0u;
+            evals += __popc(reach_a) + __popc(reach_b);
+            uint32_t mm = reach_a | reach_b;
+            const float4* wY = row == 0u ? sbuf[buf][0][warp] : row == 1u ? sbuf[buf][2][warp]
+                                                                          : s_row[XR > 1 ? row - 2u : 0u][warp];
+            const float4* wC = sbuf[buf][1][warp];
+            while (mm != 0u) {
+                uint32_t at[G];
+                bool ua[G], ub[G];
+                float aa[G], ab[G];
+#pragma unroll
+                for (int g = 0; g < G; ++g) at[g] = next_slot<DEPTH>(mm, 0);
+                // a pixel outside a record's box fails Eq. 4, so both pixels look at the record
+#pragma unroll
+                for (int g = 0; g < G; ++g) {
+                    const float4 X = wY[at[g]];
+                    const float da = X.x - fxa, db = X.x - fxb;
+                    const float rho_a = fmaf(fmaf(X.y, da, X.z), da, X.w), rho_b = fmaf(fmaf(X.y, db, X.z), db, X.w);
+                    aa[g] = fminf(ALPHA_MAX, ex2_approx(rho_a));
+                    ab[g] = fminf(ALPHA_MAX, ex2_approx(rho_b));
+                    ua[g] = !(rho_a < LOG2_ALPHA_MIN) && !done_a;
+                    ub[g] = !(rho_b < LOG2_ALPHA_MIN) && !done_b;
+                }
+                float ta[G], tb[G], Na = Ta, Nb = Tb;
+#pragma unroll
+                for (int g = 0; g < G; ++g) {
+                    ta[g] = Na;
+                    tb[g] = Nb;
+                    if (ua[g]) Na = Na * (1.f - aa[g]);
+                    if (ub[g]) Nb = Nb * (1.f - ab[g]);
+                }
+                // T never rises, so a group that ends at or above T_MIN stops nowhere
+                if (Na < T_MIN) {
+                    uint32_t after = 0;  // slots behind the stop, which are not evaluated
+                    bool go = true;
+#pragma unroll
+                    for (int g = 0; g < G; ++g) {
+                        if (go && ua[g] && ta[g] * (1.f - aa[g]) < T_MIN) {
+                            go = false;
+                            Na = ta[g];
+                            after = 0x7FFFFFFFu >> at[g];
+                        }
+                        if (!go) ua[g] = false;
+                    }
+                    done_a = true;
+                    evals -= __popc(reach_a & after);
+                    reach_a = 0u;
+                }
+                if (Nb < T_MIN) {
+                    uint32_t after = 0;
+                    bool go = true;
+#pragma unroll
+                    for (int g = 0; g < G; ++g) {
+                        if (go && ub[g] && tb[g] * (1.f - ab[g]) < T_MIN) {
+                            go = false;
+                            Nb = tb[g];
+                            after = 0x7FFFFFFFu >> at[g];
+                        }
+                        if (!go) ub[g] = false;
+                    }
+                    done_b = true;
+                    evals -= __popc(reach_b & after);
+                    reach_b = 0u;
+                }
+#pragma unroll
+                for (int g = 0; g < G; ++g) {
+                    const float4 C4 = wC[at[g]];
+                    if (ua[g]) {
+                        const float w = aa[g] * ta[g];
+                        ra = fmaf(w, C4.x, ra);
+                        ga = fmaf(w, C4.y, ga);
+                        ba = fmaf(w, C4.z, ba);
+                        ++contribs;
+                    }
+                    if (ub[g]) {
+                        const float w = ab[g] * tb[g];
+                        rb = fmaf(w, C4.x, rb);
+                        gb = fmaf(w, C4.y, gb);
+                        bb = fmaf(w, C4.z, bb);
+                        ++contribs;
+                    }
+                }
+                Ta = Na;
+                Tb = Nb;
+                mm &= reach_a | reach_b;
+            }
+            __syncwarp();  // the walk is done with this buffer before it is refilled
+            buf ^= 1;
+            nh_cur = nh_next;
+        }
+        cp_async_wait<0>();  // the chunk staged ahead, if the strip stopped early
+        float* const host_image = it.host_image;
+        // a whole strip whose rows start 16-byte aligned: its pixels through shared
+        // memory, SR rows of 3T/4 float4 (long aligned bursts over the host link)
+        const bool whole = it.nx == (uint32_t)T && it.ny == (uint32_t)SR && (it.width & 3u) == 0u &&
+                           ((reinterpret_cast<uintptr_t>(host_image) & 15u) == 0u);
+        if (whole) {
+            float2* s = reinterpret_cast<float2*>(ring) + 3u * lane;
+            s[0] = make_float2(ra, ga);
+            s[1] = make_float2(ba, rb);
+            s[2] = make_float2(gb, bb);
+            __syncwarp();
+            constexpr uint32_t F4_ROW = 3 * T / 4;
+            for (uint32_t i = lane; i < 48u; i += 32u) {  // 192 floats
+                const float4 val = reinterpret_cast<const float4*>(ring)[i];
+                const size_t at4 = ((size_t)it.at + (size_t)(i / F4_ROW) * it.width) * 3 + 4u * (i % F4_ROW);
+                *reinterpret_cast<float4*>(it.image + at4) = val;
+                if (host_image) *reinterpret_cast<float4*>(host_image + at4) = val;  // pinned host buffer
+            }
+            __syncwarp();
+        } else if (in_a) {
+            const size_t at = ((size_t)it.at + (size_t)row * it.width + col) * 3;
+            const float px[6] = {ra, ga, ba, rb, gb, bb};
+            const int n = in_b ? 6 : 3;
+            for (int k = 0; k < n; ++k) {
+                it.image[at + k] = px[k];
+                if (host_image) host_image[at + k] = px[k];  // the caller's pinned host buffer, over the host link
+            }
+        }
+        const uint32_t ev_w = __reduce_add_sync(FULL, evals), co_w = __reduce_add_sync(FULL, contribs);
+        if (lane == 0) {
+            it.evals = it.evals + ev_w;
+            it.contribs = it.contribs + co_w;
+        }
+        __syncwarp();  // every lane is done with the item before lane 0 rewrites it
+    }
+    if (lane == 0) flush_item(it);
 }
 
 template <int MODE, int DEPTH, int T>
 void launch_blend_t(const FrameParams* fp0, const FrameParams* const* fps, const uint32_t* work, uint32_t n_work,
                     uint32_t* next, int grid, cudaStream_t s) {
     launch_k(k_blend<MODE, DEPTH, T>, grid, BL_THREADS, s, fp0, fps, work, n_work, next);
+}
+
+// Two pixels per lane when the launch has 32-pixel strips for every resident warp
+// BL_WIDE_ROUNDS times over; with fewer, the longest strips decide.  Blend with
+// and without: 801 x 603 (15.5K strips, 3.2 rounds) 21.7 and 26.4 us, 640 x 360
+// (7.4K, 1.5 rounds; long horizon tiles) 49.5 and 47.6, 320 x 180 (1.9K) 58.2 and
+// 55.7.  Tiles of 32 pixels always: a strip of one row would stage the hits of
+// the four rows of its mask bit (1440p: 162 us, 347 before).
+constexpr uint32_t BL_WIDE_ROUNDS = 2;
+
+bool blend_wide(uint32_t filter, uint32_t exp_mode, uint32_t depth, uint32_t tile, uint32_t n_work, int sms) {
+    return filter == VGR_FILTER_PREEMPTIVE && exp_mode == VGR_EXP_EXACT && depth <= 32 && tile >= 16 &&
+           (tile == 32 || (uint64_t)n_work * (tile * tile / 32) >= (uint64_t)BL_WIDE_ROUNDS * sms * BL_MIN_CTAS * BL_WARPS);
+}
+
+template <int DEPTH, int T>
+void launch_blend_wide(const FrameParams* fp0, const FrameParams* const* fps, const uint32_t* work, uint32_t n_work,
+                       const uint32_t* n_heavy, uint32_t* next, int sms, cudaStream_t s) {
+    static int ctas = 0;  // resident CTAs per SM, queried once
+    if (!ctas) {
+        int n = 0;
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_blend_wide<DEPTH, T>, BL_THREADS, 0);
+        ctas = n > 0 ? n : 1;
+    }
+    launch_k(k_blend_wide<DEPTH, T>, sms * ctas, BL_THREADS, s, fp0, fps, work, n_work, n_heavy, next);
 }
 
 // The default mode at every (depth, tile) of the tuner; the canonical and
@@ -569,7 +1075,7 @@ int occupancy() {
     return n > 0 ? n : 1;
 }
 
-int blend_ctas_per_sm(uint32_t filter, uint32_t exp_mode, uint32_t depth, uint32_t tile) {
+static int blend_ctas_per_sm(uint32_t filter, uint32_t exp_mode, uint32_t depth, uint32_t tile) {
     // [mode][depth][tile], queried once each
     static int cache[3][3][3] = {};
     const int md = filter == VGR_FILTER_CANONICAL ? 1 : exp_mode == VGR_EXP_LUT ? 2 : 0;
@@ -599,8 +1105,16 @@ int blend_ctas_per_sm(uint32_t filter, uint32_t exp_mode, uint32_t depth, uint32
 }
 
 void launch_blend(const FrameParams* fp0, const FrameParams* const* fps, const uint32_t* work, uint32_t n_work,
-                  uint32_t* next, int grid, uint32_t filter, uint32_t exp_mode, uint32_t depth, uint32_t tile,
+                  const uint32_t* n_heavy, uint32_t* next, int sms, uint32_t filter, uint32_t exp_mode, uint32_t depth, uint32_t tile,
                   cudaStream_t s) {
+    if (blend_wide(filter, exp_mode, depth, tile, n_work, sms)) {
+        if (tile == 32 && depth == 16) launch_blend_wide<16, 32>(fp0, fps, work, n_work, n_heavy, next, sms, s);
+        else if (tile == 32) launch_blend_wide<32, 32>(fp0, fps, work, n_work, n_heavy, next, sms, s);
+        else if (depth == 16) launch_blend_wide<16, 16>(fp0, fps, work, n_work, n_heavy, next, sms, s);
+        else launch_blend_wide<32, 16>(fp0, fps, work, n_work, n_heavy, next, sms, s);
+        return;
+    }
+    const int grid = sms * blend_ctas_per_sm(filter, exp_mode, depth, tile);
     if (tile == 8) launch_blend_tile<8>(fp0, fps, work, n_work, next, grid, filter, exp_mode, depth, s);
     else if (tile == 32) launch_blend_tile<32>(fp0, fps, work, n_work, next, grid, filter, exp_mode, depth, s);
     else launch_blend_tile<16>(fp0, fps, work, n_work, next, grid, filter, exp_mode, depth, s);

@@ -301,7 +301,11 @@ __global__ void __cluster_dims__(TO_CTAS, 1, 1) __launch_bounds__(1024)
         }
         uint32_t total;
         s_start[b] = warp_excl_scan(all, &total) + before;
-        if (rank == 0) ctr->tile_buckets[b] = all;
+        const uint32_t heavy = __reduce_add_sync(0xFFFFFFFFu, b >= BL_HEAVY_CLASS ? all : 0u);
+        if (rank == 0) {
+            ctr->tile_buckets[b] = all;
+            if (lane == 0) ctr->n_heavy = heavy;
+        }
     }
     cluster_sync();  // the counts have been read, the starts are there
     for (uint32_t t0 = first; t0 < n_tiles; t0 += stride) {
@@ -334,7 +338,8 @@ void launch_tile_order(uint2* ranges, uint32_t n_tiles, uint32_t* order, Counter
 constexpr uint32_t BATCH_MAX_VIEWS = 1024;
 
 __global__ void __launch_bounds__(1024) k_batch_offsets(const FrameParams* const* __restrict__ fps, uint32_t n_views,
-                                                        uint32_t* __restrict__ delta) {
+                                                        uint32_t* __restrict__ delta,
+                                                        uint32_t* __restrict__ n_heavy) {
     pdl_wait();
     __shared__ uint32_t s_scan[33];
     const uint32_t v = threadIdx.x;
@@ -347,6 +352,7 @@ __global__ void __launch_bounds__(1024) k_batch_offsets(const FrameParams* const
         if (c) delta[(size_t)b * n_views + v] = run + pre - vstart;
         vstart += cnt;
         run += total;
+        if (v == 0u && b == (int)BL_HEAVY_CLASS) *n_heavy = run;
         __syncthreads();  // s_scan is reused by the next class
     }
 }
@@ -371,9 +377,9 @@ __global__ void __launch_bounds__(256) k_batch_scatter(const FrameParams* const*
 }
 
 void launch_batch_order(const FrameParams* const* fps, uint32_t n_views, const uint32_t* const* orders,
-                        const uint32_t* tile_base, uint32_t total_tiles, uint32_t* delta, uint32_t* work, int grid,
-                        cudaStream_t s) {
-    launch_k(k_batch_offsets, 1, BATCH_MAX_VIEWS, s, fps, n_views, delta);
+                        const uint32_t* tile_base, uint32_t total_tiles, uint32_t* delta, uint32_t* work,
+                        uint32_t* n_heavy, int grid, cudaStream_t s) {
+    launch_k(k_batch_offsets, 1, BATCH_MAX_VIEWS, s, fps, n_views, delta, n_heavy);
     launch_k(k_batch_scatter, grid, 256, s, fps, n_views, orders, tile_base, total_tiles, (const uint32_t*)delta, work);
 }
 

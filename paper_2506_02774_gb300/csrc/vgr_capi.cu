@@ -1057,9 +1057,8 @@ uint32_t enqueue_frame(vgr_view* v, bool scratch, bool radix_depth, int tile_pas
     launch_tile_order(v->ranges, n_tiles, v->tile_order, v->ctr, s);
     if (!own_blend) return frame_kernels(v, scratch, radix_depth, tile_passes) - 1u;  // a batch blend follows
     mark(VGR_STAGE_BLEND);
-    launch_blend(v->fp_dev, nullptr, v->tile_order, n_tiles, &v->ctr->blend_next,
-                 v->h->num_sms * blend_ctas_per_sm(v->opts.filter, v->opts.exp_mode, v->opts.blend_depth, fh.tile),
-                 v->opts.filter, v->opts.exp_mode, v->opts.blend_depth, fh.tile, s);
+    launch_blend(v->fp_dev, nullptr, v->tile_order, n_tiles, &v->ctr->n_heavy, v->ctr->blend_next,
+                 v->h->num_sms, v->opts.filter, v->opts.exp_mode, v->opts.blend_depth, fh.tile, s);
     mark(VGR_N_STAGES);
     frame_readback(v, s);
     return frame_kernels(v, scratch, radix_depth, tile_passes);
@@ -1438,11 +1437,10 @@ vgr_status launch_batch_graph(vgr_view* const* views, uint32_t n) {
             auto* next_d = reinterpret_cast<uint32_t*>((char*)devbuf + off_next);
             const vgr_view* v0 = views[sh[0]];
             const uint32_t d = v0->opts.blend_depth, t = v0->opts.tile_size;
-            e = cudaMemsetAsync(next_d, 0, sizeof(uint32_t), bs.s);  // the blend's tile counter
-            launch_batch_order(fps_d, ns, orders_d, base_d, total, delta_d, work_d, v0->h->num_sms * 4, bs.s);
-            launch_blend(v0->fp_dev, fps_d, work_d, total, next_d,
-                         v0->h->num_sms * blend_ctas_per_sm(VGR_FILTER_PREEMPTIVE, VGR_EXP_EXACT, d, t),
-                         VGR_FILTER_PREEMPTIVE, VGR_EXP_EXACT, d, t, bs.s);
+            e = cudaMemsetAsync(next_d, 0, 2 * sizeof(uint32_t), bs.s);  // the blend's tile counters
+            launch_batch_order(fps_d, ns, orders_d, base_d, total, delta_d, work_d, next_d + 2, v0->h->num_sms * 4, bs.s);
+            launch_blend(v0->fp_dev, fps_d, work_d, total, next_d + 2, next_d,
+                         v0->h->num_sms, VGR_FILTER_PREEMPTIVE, VGR_EXP_EXACT, d, t, bs.s);
             for (uint32_t j = 0; j < ns; ++j) frame_readback(views[sh[j]], bs.s);
         }
         cudaGraph_t g = nullptr;

@@ -120,7 +120,8 @@ struct Counters {
     uint32_t tickets[TK_COUNT];
     uint32_t frontier_n[MAX_TREE_DEPTH + 2];
     uint32_t tile_buckets[33];  // tiles per log2(pairs + 1) class (the blend order)
-    uint32_t blend_next;        // the blend's next tile in its work list
+    uint32_t n_heavy;           // tiles of the blend order's heavy classes (BL_HEAVY_CLASS and above)
+    uint32_t blend_next[2];     // the blend's next tile in its work list: heavy ones, others
 };
 constexpr size_t COUNTERS_HEAD = 56;  // bytes read back per frame (n_vis .. pix_contribs)
 

@@ -139,19 +139,19 @@ void launch_tile_order(uint2* ranges, uint32_t n_tiles, uint32_t* order, Counter
 constexpr uint32_t BATCH_VIEWS_MAX = 1024;  // views of one batch blend (k_batch_offsets: one thread each)
 
 // k_blend.cu: the persistent blend over a work list of (view << 20 | tile)
-// items in blend order; fps == null: every item is of the view of fp0.  'next'
-// (zero before the launch) hands out the list's tiles.  grid = SMs x
-// blend_ctas_per_sm(...); depth: hits staged per chunk (16, 32, 48; 48 needs
-// tiles of 16 or 32); tile: 8, 16 or 32 pixels.
+// items in blend order; fps == null: every item is of the view of fp0.  next[0..1]
+// (zero before the launch) hand out the list's tiles; *n_heavy: how many of
+// them, from the start, are of BL_HEAVY_CLASS or above.  depth: hits staged per
+// chunk (16, 32, 48; 48 needs tiles of 16 or 32); tile: 8, 16 or 32 pixels.
+constexpr uint32_t BL_HEAVY_CLASS = 11;  // class floor(log2(pairs + 1)) + 1: 1023 pairs and more
 void launch_blend(const FrameParams* fp0, const FrameParams* const* fps, const uint32_t* work, uint32_t n_work,
-                  uint32_t* next, int grid, uint32_t filter, uint32_t exp_mode, uint32_t depth, uint32_t tile,
-                  cudaStream_t s);
-int blend_ctas_per_sm(uint32_t filter, uint32_t exp_mode, uint32_t depth, uint32_t tile);
+                  const uint32_t* n_heavy, uint32_t* next, int sms, uint32_t filter, uint32_t exp_mode, uint32_t depth,
+                  uint32_t tile, cudaStream_t s);
 // k_emit.cu: the order of a batch's tiles over all its views (heaviest class
 // first), from each view's tile order and class counts
 void launch_batch_order(const FrameParams* const* fps, uint32_t n_views, const uint32_t* const* orders,
                         const uint32_t* tile_base, uint32_t total_tiles, uint32_t* delta, uint32_t* work,
-                        int grid, cudaStream_t s);
+                        uint32_t* n_heavy, int grid, cudaStream_t s);
 
 // vgr_sort_api.cu: enqueue a standalone pair sort on caller-provided scratch
 size_t sort_row_words(uint64_t n);                  // 16-bit words
