@@ -139,6 +139,8 @@ typedef struct {
 } vgr_view_opts;
 
 enum { VGR_HOOK_WITHHOLD_LOOKBACK = 1,
+       VGR_HOOK_LOD_LEVELS = 8,      /* a cut without a previous one is found level by level, as in trees too
+                                        large for one pass over the nodes (same cut) */
        VGR_HOOK_RADIX_DEPTH = 4,     /* order the depths by radix passes, as a frame does whose depths are too
                                         concentrated for the partition (same order) */
        VGR_HOOK_FULL_STRIP_WALK = 2  /* the blend walks every record of a strip at every pixel instead of only

@@ -339,6 +339,29 @@ __device__ __forceinline__ void flush_item(volatile WarpItem& it) {
     it.evals = it.contribs = 0ull;
 }
 
+// The launch's last CTA to finish (every CTA calls this at its end) writes the
+// status of the launch's views -- the head of their counters and their cut sizes
+// -- to pinned host memory, where the host reads it once the launch has completed.
+__device__ __forceinline__ void finish_blend(uint32_t* done, const FrameParams* fp0, const FrameParams* const* fps,
+                                             uint32_t n_views) {
+    __shared__ bool s_last;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();  // this CTA's statistics and flags before its count
+        s_last = atomicAdd(done, 1u) == gridDim.x - 1u;
+        __threadfence();
+    }
+    __syncthreads();
+    if (!s_last) return;
+    constexpr uint32_t HEAD = COUNTERS_HEAD / 4, W = HEAD + 2;
+    for (uint32_t i = threadIdx.x; i < W * (fps ? n_views : 1u); i += BL_THREADS) {
+        const FrameParams* fp = fps ? fps[i / W] : fp0;
+        const uint32_t w = i % W;
+        if (w < HEAD) fp->host_status[w] = __ldcg(reinterpret_cast<const uint32_t*>(fp->bl_ctr) + w);
+        else fp->host_n_cut[w - HEAD] = __ldcg(fp->n_cut + (w - HEAD));
+    }
+}
+
 // Lane 0: the warp's item, a strip of nrows rows of T columns at (x0, y0) of the view.
 __device__ __forceinline__ void fill_item(volatile WarpItem& it, const FrameParams* fp, uint32_t view, uint32_t x0,
                                           uint32_t y0, uint32_t T, uint32_t nrows) {
@@ -677,7 +700,8 @@ template <int MODE, int DEPTH, int T>
 __global__ void __launch_bounds__(BL_THREADS, bl_narrow_ctas(T)) k_blend(const FrameParams* __restrict__ fp0,
                                                                    const FrameParams* const* __restrict__ fps,
                                                                    const uint32_t* __restrict__ work,
-                                                                   uint32_t n_work, uint32_t* __restrict__ next) {
+                                                                   uint32_t n_work, uint32_t* __restrict__ next,
+                                                                   uint32_t* __restrict__ done, uint32_t n_views) {
     pdl_wait();
     __shared__ __align__(16) float4 sbuf[2][2 + (32 / T > 2 ? 2 : 1)][BL_WARPS][DEPTH + 1];
     __shared__ __align__(16) uint32_t s_ring[BL_WARPS][BL_RING];
@@ -701,6 +725,7 @@ __global__ void __launch_bounds__(BL_THREADS, bl_narrow_ctas(T)) k_blend(const F
     blend_strips<MODE, DEPTH, T>(sbuf, s_ring[warp], s_pm[warp], s_item[warp], s_claims, fp0, fps, work, n_work, next,
                                  blockIdx.x, gridDim.x, s_lut, m, lut_scale, (fp0->test_hooks & VGR_HOOK_FULL_STRIP_WALK) != 0u);
     if (lane == 0) flush_item(s_item[warp]);
+    finish_blend(done, fp0, fps, n_views);
 }
 
 // The same blend for launches with many strips: tiles with few pairs take strips
@@ -720,7 +745,9 @@ __global__ void __launch_bounds__(BL_THREADS, BL_MIN_CTAS) k_blend_wide(const Fr
                                                                         const uint32_t* __restrict__ work,
                                                                         uint32_t n_work,
                                                                         const uint32_t* __restrict__ n_heavy,
-                                                                        uint32_t* __restrict__ next) {
+                                                                        uint32_t* __restrict__ next,
+                                                                        uint32_t* __restrict__ done,
+                                                                        uint32_t n_views) {
     constexpr int SR = 64 / T;                    // rows per strip
     constexpr int NS = T * T / 64;                // strips per tile
     constexpr int MR = T / 8;                     // rows per mask bit
@@ -1023,12 +1050,13 @@ __global__ void __launch_bounds__(BL_THREADS, BL_MIN_CTAS) k_blend_wide(const Fr
         __syncwarp();  // every lane is done with the item before lane 0 rewrites it
     }
     if (lane == 0) flush_item(it);
+    finish_blend(done, fp0, fps, n_views);
 }
 
 template <int MODE, int DEPTH, int T>
 void launch_blend_t(const FrameParams* fp0, const FrameParams* const* fps, const uint32_t* work, uint32_t n_work,
-                    uint32_t* next, int grid, cudaStream_t s) {
-    launch_k(k_blend<MODE, DEPTH, T>, grid, BL_THREADS, s, fp0, fps, work, n_work, next);
+                    uint32_t* next, uint32_t* done, uint32_t n_views, int grid, cudaStream_t s) {
+    launch_k(k_blend<MODE, DEPTH, T>, grid, BL_THREADS, s, fp0, fps, work, n_work, next, done, n_views);
 }
 
 // Two pixels per lane when the launch has 32-pixel strips for every resident warp
@@ -1046,26 +1074,26 @@ bool blend_wide(uint32_t filter, uint32_t exp_mode, uint32_t depth, uint32_t til
 
 template <int DEPTH, int T>
 void launch_blend_wide(const FrameParams* fp0, const FrameParams* const* fps, const uint32_t* work, uint32_t n_work,
-                       const uint32_t* n_heavy, uint32_t* next, int sms, cudaStream_t s) {
+                       const uint32_t* n_heavy, uint32_t* next, uint32_t* done, uint32_t n_views, int sms, cudaStream_t s) {
     static int ctas = 0;  // resident CTAs per SM, queried once
     if (!ctas) {
         int n = 0;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_blend_wide<DEPTH, T>, BL_THREADS, 0);
         ctas = n > 0 ? n : 1;
     }
-    launch_k(k_blend_wide<DEPTH, T>, sms * ctas, BL_THREADS, s, fp0, fps, work, n_work, n_heavy, next);
+    launch_k(k_blend_wide<DEPTH, T>, sms * ctas, BL_THREADS, s, fp0, fps, work, n_work, n_heavy, next, done, n_views);
 }
 
 // The default mode at every (depth, tile) of the tuner; the canonical and
 // table modes at depth 32.
 template <int T>
 void launch_blend_tile(const FrameParams* fp0, const FrameParams* const* fps, const uint32_t* work, uint32_t n_work,
-                       uint32_t* next, int grid, uint32_t filter, uint32_t exp_mode, uint32_t depth, cudaStream_t s) {
-    if (filter == VGR_FILTER_CANONICAL) launch_blend_t<1, 32, T>(fp0, fps, work, n_work, next, grid, s);
-    else if (exp_mode == VGR_EXP_LUT) launch_blend_t<2, 32, T>(fp0, fps, work, n_work, next, grid, s);
-    else if (depth == 16) launch_blend_t<0, 16, T>(fp0, fps, work, n_work, next, grid, s);
-    else if (depth == 48 && T != 8) launch_blend_t<0, (T != 8 ? 48 : 32), T>(fp0, fps, work, n_work, next, grid, s);
-    else launch_blend_t<0, 32, T>(fp0, fps, work, n_work, next, grid, s);
+                       uint32_t* next, uint32_t* done, uint32_t n_views, int grid, uint32_t filter, uint32_t exp_mode, uint32_t depth, cudaStream_t s) {
+    if (filter == VGR_FILTER_CANONICAL) launch_blend_t<1, 32, T>(fp0, fps, work, n_work, next, done, n_views, grid, s);
+    else if (exp_mode == VGR_EXP_LUT) launch_blend_t<2, 32, T>(fp0, fps, work, n_work, next, done, n_views, grid, s);
+    else if (depth == 16) launch_blend_t<0, 16, T>(fp0, fps, work, n_work, next, done, n_views, grid, s);
+    else if (depth == 48 && T != 8) launch_blend_t<0, (T != 8 ? 48 : 32), T>(fp0, fps, work, n_work, next, done, n_views, grid, s);
+    else launch_blend_t<0, 32, T>(fp0, fps, work, n_work, next, done, n_views, grid, s);
 }
 
 template <int MODE, int DEPTH, int T>
@@ -1105,19 +1133,19 @@ static int blend_ctas_per_sm(uint32_t filter, uint32_t exp_mode, uint32_t depth,
 }
 
 void launch_blend(const FrameParams* fp0, const FrameParams* const* fps, const uint32_t* work, uint32_t n_work,
-                  const uint32_t* n_heavy, uint32_t* next, int sms, uint32_t filter, uint32_t exp_mode, uint32_t depth, uint32_t tile,
+                  const uint32_t* n_heavy, uint32_t* next, uint32_t* done, uint32_t n_views, int sms, uint32_t filter, uint32_t exp_mode, uint32_t depth, uint32_t tile,
                   cudaStream_t s) {
     if (blend_wide(filter, exp_mode, depth, tile, n_work, sms)) {
-        if (tile == 32 && depth == 16) launch_blend_wide<16, 32>(fp0, fps, work, n_work, n_heavy, next, sms, s);
-        else if (tile == 32) launch_blend_wide<32, 32>(fp0, fps, work, n_work, n_heavy, next, sms, s);
-        else if (depth == 16) launch_blend_wide<16, 16>(fp0, fps, work, n_work, n_heavy, next, sms, s);
-        else launch_blend_wide<32, 16>(fp0, fps, work, n_work, n_heavy, next, sms, s);
+        if (tile == 32 && depth == 16) launch_blend_wide<16, 32>(fp0, fps, work, n_work, n_heavy, next, done, n_views, sms, s);
+        else if (tile == 32) launch_blend_wide<32, 32>(fp0, fps, work, n_work, n_heavy, next, done, n_views, sms, s);
+        else if (depth == 16) launch_blend_wide<16, 16>(fp0, fps, work, n_work, n_heavy, next, done, n_views, sms, s);
+        else launch_blend_wide<32, 16>(fp0, fps, work, n_work, n_heavy, next, done, n_views, sms, s);
         return;
     }
     const int grid = sms * blend_ctas_per_sm(filter, exp_mode, depth, tile);
-    if (tile == 8) launch_blend_tile<8>(fp0, fps, work, n_work, next, grid, filter, exp_mode, depth, s);
-    else if (tile == 32) launch_blend_tile<32>(fp0, fps, work, n_work, next, grid, filter, exp_mode, depth, s);
-    else launch_blend_tile<16>(fp0, fps, work, n_work, next, grid, filter, exp_mode, depth, s);
+    if (tile == 8) launch_blend_tile<8>(fp0, fps, work, n_work, next, done, n_views, grid, filter, exp_mode, depth, s);
+    else if (tile == 32) launch_blend_tile<32>(fp0, fps, work, n_work, next, done, n_views, grid, filter, exp_mode, depth, s);
+    else launch_blend_tile<16>(fp0, fps, work, n_work, next, done, n_views, grid, filter, exp_mode, depth, s);
 }
 
 }  // namespace vgr

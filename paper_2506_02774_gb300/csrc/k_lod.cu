@@ -21,9 +21,12 @@
 //    stored together in one 32-byte record per node (built at load), so a
 //    cut node costs one sector and one round instead of waiting for the
 //    parent's id first; the id itself is read only when the node collapses.
-//  * k_lod_level: one level of the from-scratch, top-down traversal (frame 0,
-//    tau change, reset, fallback); frontiers are appended with one atomic per
-//    warp after a warp scan of the child counts.
+//  * k_lod_dense: the cut without a previous one (frame 0, tau change, reset,
+//    fallback), in one pass over the nodes of trees that are not too large
+//    for it (DENSE_MAX_NODES in vgr_capi.cu).
+//  * k_lod_level: one level of the from-scratch, top-down traversal, for larger
+//    trees and for views whose test turned out not monotone; frontiers are
+//    appended with one atomic per warp after a warp scan of the child counts.
 #include "vgr_internal.cuh"
 #include "vgr_launch.h"
 
@@ -49,6 +52,13 @@ constexpr int CC_COUNT_STRIDE = 32;
 // a Gaussian with u + Bx < 0.5 or u - Bx > T tiles_x - 0.5 (or likewise in
 // v) has no candidate tile in preprocess and can be left out here.  The
 // canonical mode's 3-sigma box is bounded the same way.
+// Node n's record in one 32-byte load: its (mean, radius^2) entry and its parent's.
+__device__ __forceinline__ void load_lodr(const float4* __restrict__ lodr, uint32_t n, float4& c, float4& p) {
+    asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n"
+        : "=f"(c.x), "=f"(c.y), "=f"(c.z), "=f"(c.w), "=f"(p.x), "=f"(p.y), "=f"(p.z), "=f"(p.w)
+        : "l"(lodr + 2 * (size_t)n));
+}
+
 // Set bit n of bm in the lanes where pred holds, one atomic per word: the
 // lanes that hit the same word (the match instruction; a warp's nodes are
 // few words) OR their bits together and the lowest of them stores them.
@@ -331,8 +341,7 @@ __global__ void __launch_bounds__(256) k_lod_update(const uint32_t* __restrict__
         }
 #pragma unroll
         for (int u = 0; u < LOD_UNROLL; ++u) {
-            cc[u] = sc.lodr[2 * (size_t)nn[u]];
-            qq[u] = sc.lodr[2 * (size_t)nn[u] + 1];  // the parent's entry, same sector
+            load_lodr(sc.lodr, nn[u], cc[u], qq[u]);  // its entry and the parent's
             ll[u] = sc.lmax[nn[u]];
             pp[u] = WITH_P ? sc.parent[nn[u]] : NONE;
         }
@@ -357,6 +366,89 @@ __global__ void __launch_bounds__(256) k_lod_update(const uint32_t* __restrict__
     if (lane_id() == 0) {
         if (wsum) atomicAdd(&ctr->nodes_eval, (unsigned long long)wsum);
         if (wflags) atomicOr(&ctr->flags, wflags);
+    }
+}
+
+// The cut without a previous one, in a single pass over all the nodes: where
+// the test is monotone (a child expands only if its parent does), a node is
+// reached exactly when its parent expands, so it is in the cut when its parent
+// expands and it does not, and no level waits for the one above.  A node that
+// expands under a parent that does not raises F_NONMONOTONE, and the host redoes
+// the frame with k_lod_level.  A warp takes runs of 4 bitmap words and stores each
+// from a ballot, with no atomics but one count per run.  Bound by HBM (the 32-byte node-and-parent records in order, 5.6 TB/s of them):
+// 23 us on the 1M-leaf box against 130 for 12 level kernels, 181 us on the city
+// at tau = 3 against 550 for 16 (tau = 24: 153 and 141, 48: 148 and 106).
+constexpr int LOD_DENSE_UNROLL = 4;
+constexpr uint32_t LOD_DENSE_RUN = 4;  // words
+
+template <bool FR, bool IP>
+__global__ void __launch_bounds__(256, FR || IP ? 2 : 4) k_lod_dense(SceneDev sc, const FrameParams* __restrict__ fp,
+                                                   uint32_t* __restrict__ bitmap, uint32_t* __restrict__ front,
+                                                   uint32_t* __restrict__ counts, Counters* __restrict__ ctr) {
+    pdl_wait();
+    const uint32_t N = sc.n_nodes;
+    const float px = fp->pos[0], py = fp->pos[1], pz = fp->pos[2], k = fp->k;
+    const CutOut out = make_cut_out<IP>(fp, sc, bitmap, front, counts);
+    LodFrustum fr;
+    if (FR) fr.load(fp, sc.box);
+    constexpr bool WITH_P = FR || IP;
+    constexpr int U = LOD_DENSE_UNROLL;
+    constexpr uint32_t RUN = LOD_DENSE_RUN;
+    static_assert(RUN % U == 0 && CC_TILE_WORDS % RUN == 0, "a run lies in one tile");
+    const uint32_t lane = lane_id();
+    const uint32_t nruns = (N + 32u * RUN - 1u) / (32u * RUN), nwarps = (gridDim.x * blockDim.x) >> 5;
+    uint32_t evals = 0;
+    bool bad = false;
+    for (uint32_t r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < nruns; r += nwarps) {
+        uint32_t total = 0;  // of the run: cut | in front << 16
+        for (uint32_t w0 = r * RUN; w0 < (r + 1u) * RUN; w0 += U) {
+            float4 c[U], q[U];
+            uint32_t p[U];
+            bool ok[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const uint32_t n = 32u * (w0 + u) + lane, at = min(n, N - 1u);
+                ok[u] = n < N;
+                load_lodr(sc.lodr, at, c[u], q[u]);
+                p[u] = WITH_P ? sc.parent[at] : NONE;
+            }
+            bool in_cut[U];
+            float lm[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const uint32_t n = 32u * (w0 + u) + lane;
+                bool en = ok[u] && lod_expand(c[u], px, py, pz, k);
+                bool ep = ok[u] && (q[u].w == INFINITY || lod_expand(q[u], px, py, pz, k));
+                if constexpr (FR) {
+                    if (en) en = fr.meets(n);
+                    if (ep && p[u] != NONE) ep = fr.meets(p[u]);
+                }
+                evals += ep;
+                bad = bad || (en && !ep);
+                in_cut[u] = ep && !en;
+                lm[u] = in_cut[u] ? sc.lmax[n] : 0.f;
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                bool vis = false;
+                if (in_cut[u]) {
+                    if (!IP || p[u] == NONE) vis = out.in_front(c[u], lm[u]);
+                    else vis = out.in_front_segment(c[u], lm[u], q[u], sc.lmax[p[u]]);
+                }
+                const uint32_t cw = __ballot_sync(0xFFFFFFFFu, in_cut[u]), fw = __ballot_sync(0xFFFFFFFFu, vis);
+                total += (uint32_t)__popc(cw) | ((uint32_t)__popc(fw) << 16);
+                // (words without bits are zero already)
+                if (lane == 0 && cw) bitmap[w0 + u] = cw;
+                if (lane == 1 && fw) front[w0 + u] = fw;
+            }
+        }
+        if (lane == 0 && total) atomicAdd(&counts[r * RUN / CC_TILE_WORDS * CC_COUNT_STRIDE], total);
+    }
+    const uint32_t wsum = __reduce_add_sync(0xFFFFFFFFu, evals);
+    const bool wbad = __any_sync(0xFFFFFFFFu, bad);
+    if (lane == 0) {
+        if (wsum) atomicAdd(&ctr->nodes_eval, (unsigned long long)wsum);
+        if (wbad) atomicOr(&ctr->flags, F_NONMONOTONE);
     }
 }
 
@@ -517,6 +609,19 @@ void launch_lod_update(const SceneDev& sc, const uint32_t* prev_cut, const uint3
         else VGR_LOD_UPDATE(false, false);
     }
 #undef VGR_LOD_UPDATE
+}
+
+void launch_lod_dense(const SceneDev& sc, const FrameParams* fp, uint32_t* bitmap, uint32_t* front, uint32_t* counts,
+                      Counters* ctr, int grid, bool frustum, bool interp, cudaStream_t s) {
+#define VGR_LOD_DENSE(FR, IP) launch_k(k_lod_dense<FR, IP>, grid, 256, s, sc, fp, bitmap, front, counts, ctr)
+    if (frustum) {
+        if (interp) VGR_LOD_DENSE(true, true);
+        else VGR_LOD_DENSE(true, false);
+    } else {
+        if (interp) VGR_LOD_DENSE(false, true);
+        else VGR_LOD_DENSE(false, false);
+    }
+#undef VGR_LOD_DENSE
 }
 
 void launch_lod_level(int level, const SceneDev& sc, const uint32_t* fin, uint32_t* fout, uint32_t cap,

@@ -1,13 +1,14 @@
 // vgr_capi.cu -- the C ABI (include/vgr.h): hierarchy upload and validation,
 // per-view buffers, and the per-frame launch sequence
-//   LoD (temporal update or top-down levels) -> cut compaction ->
+//   begin (parameters, clears) -> LoD (temporal update, or from scratch) -> cut compaction ->
 //   preprocess (with colour) -> depth partition and buckets (or radix passes
 //   when a bucket would not fit) -> emission -> tile sort (its last
 //   pass records the tile ranges) -> blend order -> blend
 // all enqueued on the view's stream (or replayed as one captured graph).
 // Counts stay on the device (every kernel reads its element count from
-// device memory), so a frame needs no host round trip until its end, where
-// a 56-byte status block and the cut sizes are read back: buffer overflows
+// device memory), so a frame needs no host round trip until its end, when
+// a 56-byte status block and the cut sizes are in pinned host memory (its first
+// kernel reads the parameters there, its last CTA writes these): buffer overflows
 // are handled by growing the buffer and replaying the frame, a temporal
 // update that ran past its budget by replaying the frame with the top-down
 // cut.
@@ -191,9 +192,13 @@ struct vgr_view {
     FrameParams* fp_host = nullptr;
     unsigned char* ctr_host = nullptr;
     ViewState* vstate_host = nullptr;
+    // and as the device sees them
+    const FrameParams* fp_host_dev = nullptr;
+    uint32_t *status_dev = nullptr, *n_cut_dev = nullptr;
     cudaEvent_t ev[VGR_N_STAGES + 1] = {};
     // temporal state
     bool has_prev = false;
+    bool lod_levels = false;  // cuts without a previous one go level by level: the test was not monotone
     int parity = 0;  // buffer index holding the previous cut
     float prev_tau = -1.f, prev_f = -1.f;
     uint32_t epoch = 0;
@@ -205,9 +210,9 @@ struct vgr_view {
     // captured frames, one per (top-down cut?, buffer parity); every kernel
     // argument they hold is a buffer address or a size fixed by the tile
     // grid, and the per-frame values travel through fp_host (read by the
-    // captured host-to-device copy at replay), so a graph stays valid until a
+    // frame's first kernel at replay), so a graph stays valid until a
     // buffer is reallocated or the tile grid changes
-    cudaGraphExec_t graph[2][2][2] = {};  // [radix depth order?][top-down cut?][buffer parity]
+    cudaGraphExec_t graph[2][3][2] = {};  // [radix depth order?][how the cut is found][buffer parity]
     uint32_t graph_tiles = 0;
     // frame in flight between submit and finish
     bool pending = false;
@@ -847,12 +852,22 @@ vgr_status vgr_create_view(vgr_hierarchy* h, const vgr_view_opts* opts, vgr_view
     VGR_VTRY(dalloc(&v->fp_dev, 1, &v->fixed_bytes));
     VGR_VTRY(dalloc(&v->lut, 260, &v->fixed_bytes));
     VGR_VTRY(alloc_status(v));
-    if (cudaMallocHost((void**)&v->fp_host, sizeof(FrameParams)) != cudaSuccess ||
-        cudaMallocHost((void**)&v->ctr_host, sizeof(Counters)) != cudaSuccess ||
-        cudaMallocHost((void**)&v->vstate_host, sizeof(ViewState)) != cudaSuccess) {
+    if (cudaHostAlloc((void**)&v->fp_host, sizeof(FrameParams), cudaHostAllocMapped) != cudaSuccess ||
+        cudaHostAlloc((void**)&v->ctr_host, sizeof(Counters), cudaHostAllocMapped) != cudaSuccess ||
+        cudaHostAlloc((void**)&v->vstate_host, sizeof(ViewState), cudaHostAllocMapped) != cudaSuccess) {
         cudaGetLastError();
         destroy_view(v);
         return fail(VGR_E_NOMEM, "pinned host buffers");
+    }
+    {
+        void *fp = nullptr, *st = nullptr, *nc = nullptr;
+        cudaError_t ce = cudaHostGetDevicePointer(&fp, v->fp_host, 0);
+        if (ce == cudaSuccess) ce = cudaHostGetDevicePointer(&st, v->ctr_host, 0);
+        if (ce == cudaSuccess) ce = cudaHostGetDevicePointer(&nc, v->vstate_host, 0);
+        if (ce != cudaSuccess) { destroy_view(v); return fail(VGR_E_CUDA, "mapped host: %s", cudaGetErrorString(ce)); }
+        v->fp_host_dev = static_cast<const FrameParams*>(fp);
+        v->status_dev = static_cast<uint32_t*>(st);
+        v->n_cut_dev = reinterpret_cast<uint32_t*>(static_cast<ViewState*>(nc)->n_cut);
     }
     memset(v->fp_host, 0, sizeof(FrameParams));
     memset(v->ctr_host, 0, sizeof(Counters));
@@ -957,43 +972,63 @@ namespace {
 // their depths by radix passes before the partition is tried again.
 constexpr int RADIX_FRAMES = 64;
 
-uint32_t frame_kernels(const vgr_view* v, bool scratch, bool radix_depth, int tile_passes) {
-    const uint32_t lod = scratch ? v->h->max_depth + 1u : 1u;
-    return lod + 1u /*compact*/ + 1u /*preprocess, with colour*/ +
+// How a frame finds its cut: from the previous one, in one pass over the nodes,
+// or level by level.
+enum { LOD_UPDATE = 0, LOD_DENSE = 1, LOD_LEVELS = 2 };
+// A cut without a previous one: the pass costs about 6 us per million nodes
+// whatever the cut, the levels at least 100 us on a deep tree and more with the
+// cut, so they are better only on large trees for cuts of a few percent of the
+// nodes -- which the view's last cut tells, if tau has not fallen much since.
+constexpr uint32_t DENSE_ANY_NODES = 1u << 24;
+int lod_from_scratch(const vgr_view* v, float tau) {
+    const uint32_t N = v->h->n_nodes;
+    if (v->lod_levels || (v->opts.test_hooks & VGR_HOOK_LOD_LEVELS)) return LOD_LEVELS;
+    const bool coarse = v->last_n_cut > 0 && v->last_n_cut < N / 32 && tau >= 0.5f * v->prev_tau;
+    return N > DENSE_ANY_NODES && coarse ? LOD_LEVELS : LOD_DENSE;
+}
+
+int frame_lod(const vgr_view* v, const PendingFrame& q) {
+    return q.scratch ? lod_from_scratch(v, q.tau) : LOD_UPDATE;
+}
+
+uint32_t frame_kernels(const vgr_view* v, int lod, bool radix_depth, int tile_passes) {
+    return (lod == LOD_LEVELS ? v->h->max_depth + 1u : 1u) + 1u /*compact*/ + 1u /*preprocess, with colour*/ +
            (radix_depth ? 9u /*4 counts, 4 scatters, slot scan*/ : 2u /*partition, buckets*/) + 1u /*emit*/ +
-           2u * (uint32_t)tile_passes - 1u /*counts but the first, scatters*/ + 1u /*tile order (finishes the ranges)*/ + 1u /*blend*/;
+           2u * (uint32_t)tile_passes - 1u /*counts but the first, scatters*/ + 1u /*begin*/ + 1u /*tile order (finishes the ranges)*/ + 1u /*blend*/;
 }
 
-// The frame's status block and cut sizes, read back after its last kernel.
-void frame_readback(vgr_view* v, cudaStream_t s) {
-    cudaMemcpyAsync(v->ctr_host, v->ctr, COUNTERS_HEAD, cudaMemcpyDeviceToHost, s);
-    cudaMemcpyAsync(v->vstate_host, v->vstate, sizeof(ViewState), cudaMemcpyDeviceToHost, s);
-}
-
-// Enqueue one frame.  'scratch' selects the top-down cut.  'own_blend' false:
-// the frame stops before the blend, which a batch runs over all its views
-// (frame_readback then follows that blend).  Returns the number of kernels
+// Enqueue one frame.  'lod' selects how its cut is found.  'own_blend' false:
+// the frame stops before the blend, which a batch runs over all its views.
+// Returns the number of kernels
 // launched.
-uint32_t enqueue_frame(vgr_view* v, bool scratch, bool radix_depth, int tile_passes, bool own_blend = true) {
+uint32_t enqueue_frame(vgr_view* v, int lod, bool radix_depth, int tile_passes, bool own_blend = true) {
     const SceneDev& sc = v->h->dev;
     cudaStream_t s = v->stream;
     const bool timing = v->opts.timing != 0;
     auto mark = [&](int i) { if (timing) cudaEventRecord(v->ev[i], s); };
     const FrameParams& fh = *v->fp_host;
     const uint32_t n_tiles = fh.tiles_x * fh.tiles_y;
-    cudaMemcpyAsync(v->fp_dev, v->fp_host, sizeof(FrameParams), cudaMemcpyHostToDevice, s);
     const TilePlan plan = tile_plan(n_tiles);
-    cudaMemsetAsync(v->ctr, 0, cleared_bytes(v->n_words, v->cap_vis), s);
-    cudaMemsetAsync(v->tile_groups, 0, tile_group_words(v->cap_pairs, plan.passes, plan.bits) * sizeof(uint32_t), s);
-    if (radix_depth)
-        cudaMemsetAsync(v->depth_groups, 0, 4 * radix_group_words(v->cap_vis, RADIX_TILE, 8) * sizeof(uint32_t), s);
-    cudaMemsetAsync(v->ranges, 0xFF, (size_t)n_tiles * sizeof(uint2), s);  // (start, ~end): both all ones
-    // the first kernel waits for the copies above in plain stream order; with
-    // stage events between the kernels none of them is launched early
+    // with stage events between the kernels none of them is launched early
     PdlScope pdl(!timing);
+    FrameClear clear{};
+    auto zero = [&](int i, void* p, size_t bytes) {
+        clear.zero[i] = static_cast<uint4*>(p);
+        clear.zero16[i] = (bytes + 15) / 16;
+    };
+    zero(0, v->ctr, cleared_bytes(v->n_words, v->cap_vis));
+    zero(1, v->tile_groups, tile_group_words(v->cap_pairs, plan.passes, plan.bits) * sizeof(uint32_t));
+    zero(2, v->depth_groups, radix_depth ? 4 * radix_group_words(v->cap_vis, RADIX_TILE, 8) * sizeof(uint32_t) : 0);
+    clear.ranges = v->ranges;
+    clear.n_ranges = n_tiles;
+    launch_frame_begin(v->fp_host_dev, v->fp_dev, clear, v->h->num_sms, s);
     const int prev = v->parity, cur = v->parity ^ 1;
     mark(VGR_STAGE_LOD);
-    if (scratch) {
+    if (lod == LOD_DENSE) {
+        launch_lod_dense(sc, v->fp_dev, v->bitmap, v->front_bm, v->cut_counts, v->ctr,
+                         std::min(v->grid_wide, 4 * v->h->num_sms),
+                         fh.lod_frustum != 0, fh.lod_interp != 0, s);
+    } else if (lod == LOD_LEVELS) {
         for (uint32_t level = 0; level <= v->h->max_depth; ++level)
             launch_lod_level((int)level, sc, v->frontier[level & 1], v->frontier[(level + 1) & 1], v->h->n_nodes,
                              v->fp_dev, v->bitmap, v->front_bm, v->cut_counts, v->ctr, v->grid_wide, fh.lod_frustum != 0,
@@ -1055,22 +1090,21 @@ uint32_t enqueue_frame(vgr_view* v, bool scratch, bool radix_depth, int tile_pas
     v->last_tile_buf = tile_passes & 1;
     mark(VGR_STAGE_RANGES);
     launch_tile_order(v->ranges, n_tiles, v->tile_order, v->ctr, s);
-    if (!own_blend) return frame_kernels(v, scratch, radix_depth, tile_passes) - 1u;  // a batch blend follows
+    if (!own_blend) return frame_kernels(v, lod, radix_depth, tile_passes) - 1u;  // a batch blend follows
     mark(VGR_STAGE_BLEND);
     launch_blend(v->fp_dev, nullptr, v->tile_order, n_tiles, &v->ctr->n_heavy, v->ctr->blend_next,
-                 v->h->num_sms, v->opts.filter, v->opts.exp_mode, v->opts.blend_depth, fh.tile, s);
+                 &v->ctr->blend_done, 1, v->h->num_sms, v->opts.filter, v->opts.exp_mode, v->opts.blend_depth, fh.tile, s);
     mark(VGR_N_STAGES);
-    frame_readback(v, s);
-    return frame_kernels(v, scratch, radix_depth, tile_passes);
+    return frame_kernels(v, lod, radix_depth, tile_passes);
 }
 
 // One frame on the view's stream: the plain launch sequence, or (use_graph,
 // no stage timing) the replay of the captured sequence for this
 // (top-down?, parity) pair, captured on first use.
-vgr_status run_frame(vgr_view* v, bool scratch, bool radix_depth, int tile_passes, uint32_t n_tiles,
+vgr_status run_frame(vgr_view* v, int lod, bool radix_depth, int tile_passes, uint32_t n_tiles,
                      uint32_t* kernels) {
     if (!v->opts.use_graph || v->opts.timing) {
-        *kernels += enqueue_frame(v, scratch, radix_depth, tile_passes);
+        *kernels += enqueue_frame(v, lod, radix_depth, tile_passes);
         VGR_CK(cudaGetLastError());
         return VGR_OK;
     }
@@ -1078,10 +1112,10 @@ vgr_status run_frame(vgr_view* v, bool scratch, bool radix_depth, int tile_passe
         drop_graphs(v);
         v->graph_tiles = n_tiles;
     }
-    cudaGraphExec_t& ge = v->graph[radix_depth ? 1 : 0][scratch ? 1 : 0][v->parity];
+    cudaGraphExec_t& ge = v->graph[radix_depth ? 1 : 0][lod][v->parity];
     if (!ge) {
         VGR_CK(cudaStreamBeginCapture(v->stream, cudaStreamCaptureModeThreadLocal));
-        enqueue_frame(v, scratch, radix_depth, tile_passes);
+        enqueue_frame(v, lod, radix_depth, tile_passes);
         cudaGraph_t g = nullptr;
         cudaError_t e = cudaStreamEndCapture(v->stream, &g);
         if (e == cudaSuccess) e = cudaGetLastError();
@@ -1095,7 +1129,7 @@ vgr_status run_frame(vgr_view* v, bool scratch, bool radix_depth, int tile_passe
     }
     v->last_tile_buf = tile_passes & 1;
     VGR_CK(cudaGraphLaunch(ge, v->stream));
-    *kernels += frame_kernels(v, scratch, radix_depth, tile_passes);
+    *kernels += frame_kernels(v, lod, radix_depth, tile_passes);
     return VGR_OK;
 }
 
@@ -1215,6 +1249,9 @@ void fill_params(vgr_view* v, const vgr_camera* cam, float t, float k, float* ho
     p.lod_t = t;
     p.depth = depth_map(v->h, cam);
     if (p.lod_frustum) frustum_planes(cam, v->opts.lod_frustum_guard, p.frustum);
+    p.n_cut = v->vstate->n_cut;
+    p.host_status = v->status_dev;
+    p.host_n_cut = v->n_cut_dev;
     // the blend's buffers: the tile sort's last pass leaves the pairs in
     // buffer (passes & 1)
     p.bl_ranges = v->ranges;
@@ -1301,7 +1338,7 @@ vgr_status submit_impl(vgr_view* v, const vgr_camera* cam, float tau, float* hos
     vgr_status s = prepare_frame(v, cam, tau, host_rgb, pipe);
     if (s != VGR_OK) return s;
     PendingFrame& q = v->pend;
-    if ((s = run_frame(v, q.scratch, q.radix_depth, q.tile_passes, tiles_for(q.cam.width, q.cam.height, tile_of(v)),
+    if ((s = run_frame(v, frame_lod(v, q), q.radix_depth, q.tile_passes, tiles_for(q.cam.width, q.cam.height, tile_of(v)),
                        &q.kernels)) != VGR_OK)
         return s;
     return close_frame(v, v->stream);
@@ -1372,7 +1409,7 @@ vgr_status launch_batch_graph(vgr_view* const* views, uint32_t n) {
         const vgr_view* v = views[i];
         const PendingFrame& q = v->pend;
         const uint64_t tiles = tiles_for(q.cam.width, q.cam.height, tile_of(v));
-        key.insert(key.end(), {v->uid, v->gen, (uint64_t)q.scratch, (uint64_t)q.radix_depth, (uint64_t)v->parity,
+        key.insert(key.end(), {v->uid, v->gen, (uint64_t)frame_lod(v, q), (uint64_t)q.radix_depth, (uint64_t)v->parity,
                                tiles, (uint64_t)q.tile_passes});
     }
     const std::vector<uint32_t> sh = batch_blend_views(views, n);
@@ -1423,7 +1460,7 @@ vgr_status launch_batch_graph(vgr_view* const* views, uint32_t n) {
             vgr_view* v = views[i];
             e = cudaStreamWaitEvent(v->stream, prev[i] < 0 ? bs.fork : views[prev[i]]->join_ev, 0);
             if (e != cudaSuccess) break;
-            enqueue_frame(v, v->pend.scratch, v->pend.radix_depth, v->pend.tile_passes, !shared[i]);
+            enqueue_frame(v, frame_lod(v, v->pend), v->pend.radix_depth, v->pend.tile_passes, !shared[i]);
             e = cudaEventRecord(v->join_ev, v->stream);
             if (e == cudaSuccess && tail[i]) e = cudaStreamWaitEvent(bs.s, v->join_ev, 0);
         }
@@ -1437,11 +1474,10 @@ vgr_status launch_batch_graph(vgr_view* const* views, uint32_t n) {
             auto* next_d = reinterpret_cast<uint32_t*>((char*)devbuf + off_next);
             const vgr_view* v0 = views[sh[0]];
             const uint32_t d = v0->opts.blend_depth, t = v0->opts.tile_size;
-            e = cudaMemsetAsync(next_d, 0, 2 * sizeof(uint32_t), bs.s);  // the blend's tile counters
+            e = cudaMemsetAsync(next_d, 0, 4 * sizeof(uint32_t), bs.s);  // the blend's counters: tiles, -, CTAs done
             launch_batch_order(fps_d, ns, orders_d, base_d, total, delta_d, work_d, next_d + 2, v0->h->num_sms * 4, bs.s);
-            launch_blend(v0->fp_dev, fps_d, work_d, total, next_d + 2, next_d,
+            launch_blend(v0->fp_dev, fps_d, work_d, total, next_d + 2, next_d, next_d + 3, ns,
                          v0->h->num_sms, VGR_FILTER_PREEMPTIVE, VGR_EXP_EXACT, d, t, bs.s);
-            for (uint32_t j = 0; j < ns; ++j) frame_readback(views[sh[j]], bs.s);
         }
         cudaGraph_t g = nullptr;
         const cudaError_t e2 = cudaStreamEndCapture(bs.s, &g);
@@ -1470,7 +1506,7 @@ vgr_status launch_batch_graph(vgr_view* const* views, uint32_t n) {
     for (uint32_t i = 0; i < n; ++i) {
         vgr_view* v = views[i];
         v->last_tile_buf = v->pend.tile_passes & 1;
-        v->pend.kernels += frame_kernels(v, v->pend.scratch, v->pend.radix_depth, v->pend.tile_passes) -
+        v->pend.kernels += frame_kernels(v, frame_lod(v, v->pend), v->pend.radix_depth, v->pend.tile_passes) -
                            (shared[i] ? 1u : 0u);
         if (!sh.empty() && i == sh[0]) v->pend.kernels += 3u;  // class offsets, tile placement, the batch blend
         vgr_status s = close_frame(v, bs.s);
@@ -1501,12 +1537,16 @@ vgr_status finish_impl(vgr_view* v, vgr_frame* out) {
         const int cur = v->parity ^ 1;
         const uint32_t n_cut = v->vstate_host->n_cut[cur];
         if (flags & F_SPIN_TIMEOUT) return fail(VGR_E_TIMEOUT, "a look-back wait timed out");
-        if (flags & F_NONMONOTONE)
+        const bool by_level = q.scratch && (flags & F_NONMONOTONE) && frame_lod(v, q) == LOD_DENSE;
+        if ((flags & F_NONMONOTONE) && !by_level)
             return fail(VGR_E_NONMONOTONE, "granularity test not monotone: a child expands while its parent does not");
         if (flags & F_OVF_FRONTIER) return fail(VGR_E_OVERFLOW, "frontier overflow");
         if (flags & F_OVF_VIS) return fail(VGR_E_OVERFLOW, "more than 2^24 cut nodes in front of the camera in one frame");
         bool again = false;
-        if ((flags & F_LOD_FALLBACK) && !q.scratch) {
+        if (by_level) {
+            v->lod_levels = true;
+            again = true;
+        } else if ((flags & F_LOD_FALLBACK) && !q.scratch) {
             q.scratch = true;
             again = true;
         } else if (flags & F_LOD_FALLBACK) {
@@ -1536,7 +1576,7 @@ vgr_status finish_impl(vgr_view* v, vgr_frame* out) {
         if (attempt >= 12) return fail(VGR_E_OVERFLOW, "frame did not settle after %d replays", attempt + 1);
         ++replays;
         fill_params(v, &q.cam, q.t, q.k, q.host_dev, q.tile_passes);
-        if ((s = run_frame(v, q.scratch, q.radix_depth, q.tile_passes, TW * TH, &q.kernels)) != VGR_OK) return s;
+        if ((s = run_frame(v, frame_lod(v, q), q.radix_depth, q.tile_passes, TW * TH, &q.kernels)) != VGR_OK) return s;
         if (q.host && !q.host_dev && !q.pipe)
             VGR_CK(cudaMemcpyAsync(q.host, v->cur_image, (size_t)W * H * 3 * sizeof(float), cudaMemcpyDeviceToHost,
                                    v->stream));

@@ -103,6 +103,10 @@ struct FrameParams {
     const float* bl_lut;         // Eq. 5 table (m + 1 entries)
     float* bl_image;             // H x W x 3
     Counters* bl_ctr;
+    // the frame's status, which the blend's last CTA writes to pinned host memory
+    const uint32_t* n_cut;       // ViewState::n_cut
+    uint32_t* host_status;       // the head of Counters
+    uint32_t* host_n_cut;
 };
 
 // Zeroed at the start of every frame.  Scalars first: the host reads back
@@ -122,6 +126,7 @@ struct Counters {
     uint32_t tile_buckets[33];  // tiles per log2(pairs + 1) class (the blend order)
     uint32_t n_heavy;           // tiles of the blend order's heavy classes (BL_HEAVY_CLASS and above)
     uint32_t blend_next[2];     // the blend's next tile in its work list: heavy ones, others
+    uint32_t blend_done;        // CTAs of the blend that have finished
 };
 constexpr size_t COUNTERS_HEAD = 56;  // bytes read back per frame (n_vis .. pix_contribs)
 

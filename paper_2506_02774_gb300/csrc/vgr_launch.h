@@ -14,8 +14,8 @@ void set_last_error(const char* msg);
 // kernel waits (griddepcontrol.wait, its first statement) until the previous
 // one has completed and its writes are visible, so ordering is unchanged and
 // only the launch latency overlaps.  That wait covers a preceding kernel only:
-// a kernel that follows copies, memsets or event records in the stream is
-// launched in plain stream order (PdlScope), so it cannot start before them.
+// a kernel that follows copies, memsets or event records in the stream (the first
+// of a frame) is launched in plain stream order (PdlScope), so it cannot start before them.
 // VGR_PDL=0 in the environment turns it off everywhere.
 bool pdl_enabled();
 struct PdlState {
@@ -58,10 +58,25 @@ struct SceneDev;
 struct FrameParams;
 struct Counters;
 
+// k_frame.cu
+// What a frame starts from: up to three regions of zeros (16-byte units) and the
+// tile ranges, all ones.
+struct FrameClear {
+    uint4* zero[3];
+    size_t zero16[3];
+    uint2* ranges;
+    uint32_t n_ranges;
+};
+// host: the parameters in pinned host memory, as the device sees it
+void launch_frame_begin(const FrameParams* host, FrameParams* dev, const FrameClear& c, int sms, cudaStream_t s);
+
 // k_lod.cu
 void launch_lod_update(const SceneDev& sc, const uint32_t* prev_cut, const uint32_t* n_prev, uint32_t cap_prev,
                        const FrameParams* fp, uint32_t* bitmap, uint32_t* front, uint32_t* counts, Counters* ctr, int grid,
                        bool frustum, bool interp, cudaStream_t s);
+// the whole from-scratch cut in one pass (F_NONMONOTONE: to be redone level by level)
+void launch_lod_dense(const SceneDev& sc, const FrameParams* fp, uint32_t* bitmap, uint32_t* front, uint32_t* counts,
+                      Counters* ctr, int grid, bool frustum, bool interp, cudaStream_t s);
 void launch_lod_level(int level, const SceneDev& sc, const uint32_t* fin, uint32_t* fout, uint32_t cap,
                       const FrameParams* fp, uint32_t* bitmap, uint32_t* front, uint32_t* counts, Counters* ctr, int grid,
                       bool frustum, bool interp, cudaStream_t s);
@@ -141,11 +156,13 @@ constexpr uint32_t BATCH_VIEWS_MAX = 1024;  // views of one batch blend (k_batch
 // k_blend.cu: the persistent blend over a work list of (view << 20 | tile)
 // items in blend order; fps == null: every item is of the view of fp0.  next[0..1]
 // (zero before the launch) hand out the list's tiles; *n_heavy: how many of
-// them, from the start, are of BL_HEAVY_CLASS or above.  depth: hits staged per
+// them, from the start, are of BL_HEAVY_CLASS or above.  The last CTA writes the
+// status of fp0's view, or of the n_views views of fps, to their host buffers;
+// *done (zero before the launch) finds it.  depth: hits staged per
 // chunk (16, 32, 48; 48 needs tiles of 16 or 32); tile: 8, 16 or 32 pixels.
 constexpr uint32_t BL_HEAVY_CLASS = 11;  // class floor(log2(pairs + 1)) + 1: 1023 pairs and more
 void launch_blend(const FrameParams* fp0, const FrameParams* const* fps, const uint32_t* work, uint32_t n_work,
-                  const uint32_t* n_heavy, uint32_t* next, int sms, uint32_t filter, uint32_t exp_mode, uint32_t depth,
+                  const uint32_t* n_heavy, uint32_t* next, uint32_t* done, uint32_t n_views, int sms, uint32_t filter, uint32_t exp_mode, uint32_t depth,
                   uint32_t tile, cudaStream_t s);
 // k_emit.cu: the order of a batch's tiles over all its views (heaviest class
 // first), from each view's tile order and class counts
