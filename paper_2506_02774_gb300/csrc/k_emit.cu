@@ -15,7 +15,8 @@
 // of 512 Gaussians before this left the CTA with the near ones running alone
 // (SM cycles 43 % busy on average) and gathered three half-used sectors each;
 // 1M-leaf box at 1080p (981K slots): 53 -> 21 us, city at 1080p (4.26M slots):
-// 107 -> 61 us.  For each slot the tile-level form of
+// 107 -> 61 us; the records of two slots per lane in flight together: city 56 -> 52
+// (all four, in CTAs of 512 threads: 68).  For each slot the tile-level form of
 // Eq. 4 (paper Sec. 4.2) decides: a kept slot gets key = tile id, a dropped one
 // all ones, which the tile sort's first pass leaves out (the others stay in
 // depth order within a tile, the sort being stable).  The slot's
@@ -36,6 +37,7 @@
 namespace vgr {
 
 constexpr int EM_THREADS = 256;
+constexpr int EM_AHEAD = 2;                   // slots per lane whose records are in flight together
 constexpr int EM_WARPS = EM_THREADS / 32;
 constexpr uint32_t EM_SLOTS = EMIT_SLOTS;   // slots per chunk: 32 runs of a warp
 constexpr uint32_t EM_GAUSS = EM_SLOTS + 1; // Gaussians that may be looked at for a chunk
@@ -126,7 +128,7 @@ __global__ void __launch_bounds__(EM_THREADS, 4) k_emit(const uint32_t* __restri
     pdl_wait();
     __shared__ uint2 s_g[EM_GAUSS];   // per Gaussian: index in the in-front arrays, first slot
     __shared__ uint32_t s_bits[32];   // slots at which a Gaussian starts
-    __shared__ uint32_t s_cnt[EM_THREADS];  // the chunk's kept slots by first digit
+    __shared__ uint32_t s_cnt[256];   // the chunk's kept slots by first digit
     const uint32_t lane = lane_id(), warp = threadIdx.x >> 5, D = 1u << bits;
     const uint32_t n_vis = min(ctr->n_vis, cap_vis);
     const uint64_t cand = ctr->n_cand;
@@ -144,7 +146,7 @@ __global__ void __launch_bounds__(EM_THREADS, 4) k_emit(const uint32_t* __restri
         const uint32_t g1 = ck + 1u < nchunks ? owner[ck + 1u] : n_vis - 1u;  // may start past the chunk
         const uint32_t m = min(g1 - g0 + 1u, EM_GAUSS);
         if (threadIdx.x < 32) s_bits[threadIdx.x] = threadIdx.x == 0 ? 1u : 0u;  // the chunk's first slot has an owner
-        s_cnt[threadIdx.x] = 0u;
+        if (threadIdx.x < 256) s_cnt[threadIdx.x] = 0u;
         __syncthreads();
         for (uint32_t q = threadIdx.x; q < m; q += EM_THREADS) {
             const uint32_t o = slot_off[g0 + q];
@@ -155,49 +157,62 @@ __global__ void __launch_bounds__(EM_THREADS, 4) k_emit(const uint32_t* __restri
         uint32_t total;
         const uint32_t bits_l = s_bits[lane];
         const uint32_t pre_l = warp_excl_scan(__popc(bits_l), &total);  // starts before word 'lane'
+        for (uint32_t r0 = 0; r0 < EM_SLOTS / EM_THREADS; r0 += EM_AHEAD) {
+            uint2 gvs[EM_AHEAD];
+            float4 recA[EM_AHEAD], recB[EM_AHEAD];
 #pragma unroll
-        for (uint32_t r = 0; r < EM_SLOTS / EM_THREADS; ++r) {
-            const uint32_t word = r * EM_WARPS + warp;
-            const uint32_t bits = __shfl_sync(0xFFFFFFFFu, bits_l, word);
-            const uint32_t before = __shfl_sync(0xFFFFFFFFu, pre_l, word);
-            const uint32_t j = j0 + 32u * word + lane;
-            if (32u * word + lane < len) {
-                // the last Gaussian that starts at or before this slot
-                const uint2 gv = s_g[before + __popc(bits & ((2u << lane) - 1u)) - 1u];
-                const float4 A = rec[2 * (size_t)gv.x], B = rec[2 * (size_t)gv.x + 1];
-                const uint32_t local = j - gv.y;
-                const uint32_t rc = __float_as_uint(B.z);
-                const uint32_t w = rc >> 20;
-                // local / w and local % w: local < 2^20 and w <= 2^10, so (local + 1/2) / w is
-                // at least 1 / 2^11 from an integer and its FP32 quotient floors exactly
-                const uint32_t qy = (uint32_t)(((float)local + 0.5f) * __frcp_rn((float)w));
-                const int tx = (int)(rc & 0x3FFu) + (int)(local - qy * w);
-                const int ty = (int)((rc >> 10) & 0x3FFu) + (int)qy;
-                bool keep = true;
-                uint32_t rows = 0xFFu;
-                if (!canonical) {
-                    // the conic is stored pre-scaled (A = -a/2, B = -b, C = -c/2): exact to undo;
-                    // edge optima dy* = (-b / c) dx, dx* = (-b / a) dy: an ulp or two of
-                    // error moves rho_max by far less than the test's 2e-3 slack
-                    const float ca = -2.0f * A.z, cb = -A.w, cc = -2.0f * B.x;
-                    keep = tile_keep(A.x, A.y, ca, cb, cc, __fdividef(-cb, ca), __fdividef(-cb, cc), B.y - TILE_EPS,
-                                     tx, ty, Wf, Hf, T);
-                    // tile rows r with |row0 + r - v| <= half-height, as groups of MR rows
-                    const float row0 = (float)(ty * T) + 0.5f;
-                    const float hh = __half2float(__ushort_as_half((unsigned short)(__float_as_uint(B.w) & 0xFFFFu)));
-                    const float rlo = fmaxf(0.f, ceilf(A.y - hh - row0));
-                    const float rhi = fminf((float)(T - 1), floorf(A.y + hh - row0));
-                    rows = 0u;
-                    if (rlo <= rhi) {
-                        const uint32_t w0 = (uint32_t)rlo / MR, w1 = (uint32_t)rhi / MR;
-                        rows = ((2u << w1) - 1u) & ~((1u << w0) - 1u);
-                    }
+            for (int r = 0; r < EM_AHEAD; ++r) {
+                const uint32_t word = (r0 + r) * EM_WARPS + warp;
+                const uint32_t bits = __shfl_sync(0xFFFFFFFFu, bits_l, word);
+                const uint32_t before = __shfl_sync(0xFFFFFFFFu, pre_l, word);
+                if (32u * word + lane < len) {
+                    // the last Gaussian that starts at or before this slot
+                    gvs[r] = s_g[before + __popc(bits & ((2u << lane) - 1u)) - 1u];
+                    recA[r] = rec[2 * (size_t)gvs[r].x];
+                    recB[r] = rec[2 * (size_t)gvs[r].x + 1];
                 }
-                const uint32_t key = keep ? (uint32_t)ty * TW + (uint32_t)tx : NONE;
-                kept += keep;
-                pair_key[j] = key;
-                pair_val[j] = (gv.x << 8) | rows;
-                if (keep) atomicAdd(&s_cnt[key & (D - 1u)], 1u);
+            }
+#pragma unroll
+            for (int r = 0; r < EM_AHEAD; ++r) {
+                const uint32_t word = (r0 + r) * EM_WARPS + warp;
+                const uint32_t j = j0 + 32u * word + lane;
+                if (32u * word + lane < len) {
+                    const uint2 gv = gvs[r];
+                    const float4 A = recA[r], B = recB[r];
+                    const uint32_t local = j - gv.y;
+                    const uint32_t rc = __float_as_uint(B.z);
+                    const uint32_t w = rc >> 20;
+                    // local / w and local % w: local < 2^20 and w <= 2^10, so (local + 1/2) / w is
+                    // at least 1 / 2^11 from an integer and its FP32 quotient floors exactly
+                    const uint32_t qy = (uint32_t)(((float)local + 0.5f) * __frcp_rn((float)w));
+                    const int tx = (int)(rc & 0x3FFu) + (int)(local - qy * w);
+                    const int ty = (int)((rc >> 10) & 0x3FFu) + (int)qy;
+                    bool keep = true;
+                    uint32_t rows = 0xFFu;
+                    if (!canonical) {
+                        // the conic is stored pre-scaled (A = -a/2, B = -b, C = -c/2): exact to undo;
+                        // edge optima dy* = (-b / c) dx, dx* = (-b / a) dy: an ulp or two of
+                        // error moves rho_max by far less than the test's 2e-3 slack
+                        const float ca = -2.0f * A.z, cb = -A.w, cc = -2.0f * B.x;
+                        keep = tile_keep(A.x, A.y, ca, cb, cc, __fdividef(-cb, ca), __fdividef(-cb, cc), B.y - TILE_EPS,
+                                         tx, ty, Wf, Hf, T);
+                        // tile rows r with |row0 + r - v| <= half-height, as groups of MR rows
+                        const float row0 = (float)(ty * T) + 0.5f;
+                        const float hh = __half2float(__ushort_as_half((unsigned short)(__float_as_uint(B.w) & 0xFFFFu)));
+                        const float rlo = fmaxf(0.f, ceilf(A.y - hh - row0));
+                        const float rhi = fminf((float)(T - 1), floorf(A.y + hh - row0));
+                        rows = 0u;
+                        if (rlo <= rhi) {
+                            const uint32_t w0 = (uint32_t)rlo / MR, w1 = (uint32_t)rhi / MR;
+                            rows = ((2u << w1) - 1u) & ~((1u << w0) - 1u);
+                        }
+                    }
+                    const uint32_t key = keep ? (uint32_t)ty * TW + (uint32_t)tx : NONE;
+                    kept += keep;
+                    pair_key[j] = key;
+                    pair_val[j] = (gv.x << 8) | rows;
+                    if (keep) atomicAdd(&s_cnt[key & (D - 1u)], 1u);
+                }
             }
         }
         __syncthreads();
