@@ -16,7 +16,7 @@
 // long as their number.)  The rows of the tile sort's first pass are written by
 // the emission, so its count kernel is saved there.  Tile sort of 981K slots
 // (1M-leaf box, 1080p): 47 -> 31 us; of 4.26M (city, 1080p): 85 -> 76; of 235K
-// (320 x 180, one pass): 24 -> 12; the standalone sort of 4M 32-bit keys: 191 ->
+// (320 x 180, one pass): 24 -> 12; of 63K (801 x 603): 33 -> 18; the standalone sort of 4M 32-bit keys: 191 ->
 // 171.  Large inputs are bound by the instructions of the ranking (half of the
 // issue slots, the ballots' pipe first); three CTAs an SM at 40 registers were no
 // faster.
@@ -27,14 +27,23 @@ namespace vgr {
 
 constexpr int RS_THREADS = RADIX_THREADS;
 constexpr int RS_WARPS = RS_THREADS / 32;
-constexpr int RS_ITEMS = RADIX_TILE / RADIX_THREADS;
 constexpr uint32_t RS_TILE = RADIX_TILE;
+constexpr int RS_ITEMS = RADIX_TILE / RADIX_THREADS, RS_ITEMS_SMALL = RADIX_TILE_SMALL / RADIX_THREADS;
 static_assert(RS_TILE <= 0xFFFFu, "a row's counts and a tile's places fit 16 bits");
 
-size_t radix_rows(uint64_t n, uint32_t row_len) { return (size_t)((n + row_len - 1) / row_len); }
+size_t radix_rows(uint64_t n, uint32_t row_len) {
+    return (size_t)(row_len ? (n + row_len - 1) / row_len : radix_max_tiles(n));
+}
 size_t radix_groups(uint64_t n, uint32_t row_len) { return (radix_rows(n, row_len) + RADIX_GROUP - 1) / RADIX_GROUP; }
 size_t radix_row_words(uint64_t n, uint32_t row_len, int bits) { return radix_rows(n, row_len) << bits; }
 size_t radix_group_words(uint64_t n, uint32_t row_len, int bits) { return radix_groups(n, row_len) << bits; }
+
+// Keys per thread: few keys go in small tiles over many SMs, since a tile's ranking is
+// a chain over its keys per thread.  The line lies at one small tile per SM: per tile
+// sort, 63K slots (801 x 603, two passes) took 22.9 us in tiles of 4096 and 18.4 in
+// tiles of 1024, and 3.2K slots (one pass) 10.2 and 8.2, but 235K slots (one pass) 12.3
+// and 13.3.
+__device__ __forceinline__ int radix_items(uint32_t n) { return n > RADIX_SMALL_N ? RS_ITEMS : RS_ITEMS_SMALL; }
 
 __device__ __forceinline__ uint32_t radix_n(const uint32_t* n32, const unsigned long long* n64, uint64_t cap) {
     uint64_t n = n32 ? (uint64_t)*n32 : n64 ? (uint64_t)*n64 : cap;
@@ -49,21 +58,26 @@ __global__ void __launch_bounds__(RS_THREADS) k_radix_count(const uint32_t* __re
     pdl_wait();
     __shared__ uint32_t s_cnt[2][256];
     const uint32_t n = radix_n(n32, n64, cap);
-    const uint32_t ntiles = (uint32_t)(((uint64_t)n + RS_TILE - 1) / RS_TILE), D = 1u << bits, t = threadIdx.x;
+    const int items = radix_items(n);
+    const uint32_t tile_keys = items * RS_THREADS;
+    const uint32_t ntiles = (uint32_t)(((uint64_t)n + tile_keys - 1) / tile_keys), D = 1u << bits, t = threadIdx.x;
     if (t < 256) s_cnt[0][t] = s_cnt[1][t] = 0u;
     __syncthreads();
     uint32_t flip = 0;
     for (uint32_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x, flip ^= 1u) {
-        const uint32_t base = tile * RS_TILE + t;  // n < 2^32, and so is a tile's end
+        const uint32_t base = tile * tile_keys + t;  // n < 2^32, and so is a tile's end
         uint32_t key[RS_ITEMS];
 #pragma unroll
         for (int k = 0; k < RS_ITEMS; ++k) {
+            if (k >= items) break;
             const uint32_t i = base + k * RS_THREADS;
             key[k] = i < n ? keys[i] : 0u;
         }
 #pragma unroll
-        for (int k = 0; k < RS_ITEMS; ++k)
+        for (int k = 0; k < RS_ITEMS; ++k) {
+            if (k >= items) break;
             if (base + k * RS_THREADS < n) atomicAdd(&s_cnt[flip][(key[k] >> shift) & (D - 1u)], 1u);
+        }
         __syncthreads();
         if (t < D) {
             const uint32_t c = s_cnt[flip][t];
@@ -92,7 +106,8 @@ __device__ __forceinline__ uint32_t match_digit(uint32_t d, bool valid) {
     return m;
 }
 
-// One digit pass over tiles of RS_TILE pairs (row_tiles rows each):
+// One digit pass over tiles of ITEMS pairs a thread (one row of the tables each, or
+// as many rows of row_len pairs as it holds):
 //  1. the tile's keys and values are requested; meanwhile the tables' entries
 //     before the tile are added up (two digits per thread and load);
 //  2. each warp ranks its contiguous share: peers by one ballot per digit bit,
@@ -105,28 +120,35 @@ __device__ __forceinline__ uint32_t match_digit(uint32_t d, bool valid) {
 // elements are in final key order and each key's run is one contiguous stretch
 // of global positions, so the first and last element of every run it holds give
 // atomicMin updates of (start, ~end), from all ones.
-template <int BITS, bool DROP>
-__global__ void __launch_bounds__(RS_THREADS, 2) k_radix_scatter(
-    const uint32_t* __restrict__ keys_in, const uint32_t* __restrict__ vals_in, uint32_t* __restrict__ keys_out,
-    uint32_t* __restrict__ vals_out, const uint32_t* __restrict__ n32, const unsigned long long* __restrict__ n64,
-    uint64_t cap, int shift, RadixTab tab, uint32_t row_tiles, uint2* __restrict__ ranges, uint32_t n_ranges) {
-    pdl_wait();
+template <uint32_t D>
+struct RadixSmem {
+    __align__(16) uint2 kv[RS_TILE];         // the tile staged digit-sorted: (key, value)
+    __align__(16) uint16_t wc[RS_WARPS][D];  // per-warp digit counts, then per-warp places
+    uint32_t gofs[D];                        // global index minus staged index, per digit
+    uint32_t scan[2][RS_WARPS];
+};
+
+template <int BITS, bool DROP, int ITEMS>
+__device__ __forceinline__ void radix_tiles(
+    RadixSmem<1u << BITS>& sm, uint32_t n, const uint32_t* __restrict__ keys_in, const uint32_t* __restrict__ vals_in,
+    uint32_t* __restrict__ keys_out, uint32_t* __restrict__ vals_out, int shift, RadixTab tab, uint32_t row_len,
+    uint2* __restrict__ ranges, uint32_t n_ranges) {
     constexpr uint32_t D = 1u << BITS, NQ = 2 * RS_THREADS / D;  // rows read at once, two digits a thread
+    constexpr uint32_t tile_keys = ITEMS * RS_THREADS;
     static_assert(D <= RS_THREADS && 2 * RS_THREADS % D == 0 && RS_TILE >= 2 * RS_THREADS, "table layout");
-    __shared__ __align__(16) uint2 s_kv[RS_TILE];   // the tile staged digit-sorted: (key, value)
-    __shared__ __align__(16) uint16_t s_wc[RS_WARPS][D];          // per-warp digit counts, then per-warp places
-    __shared__ uint32_t s_gofs[D];                  // global index minus staged index, per digit
-    __shared__ uint32_t s_scan[2][RS_WARPS];
+    uint2* s_kv = sm.kv;
+    uint16_t (*s_wc)[D] = sm.wc;
+    uint32_t* s_gofs = sm.gofs;
+    uint32_t (*s_scan)[RS_WARPS] = sm.scan;
     // the tables' partial sums lie under the staging buffer: groups, then rows
     uint32_t (*s_grp)[D] = reinterpret_cast<uint32_t (*)[D]>(s_kv);
     uint32_t (*s_row)[D] = reinterpret_cast<uint32_t (*)[D]>(s_kv + RS_THREADS);
-    const uint32_t n = radix_n(n32, n64, cap);
-    const uint32_t ntiles = (uint32_t)(((uint64_t)n + RS_TILE - 1) / RS_TILE);
+    const uint32_t ntiles = (uint32_t)(((uint64_t)n + tile_keys - 1) / tile_keys);
     const uint32_t t = threadIdx.x, lane = lane_id(), warp = t >> 5;
     const uint32_t pair = t % (D / 2), q = t / (D / 2);
     if (blockIdx.x >= ntiles) return;
-    const uint32_t nrows = row_tiles == 1u ? ntiles
-                                           : (uint32_t)(((uint64_t)n + RS_TILE / row_tiles - 1) / (RS_TILE / row_tiles));
+    const uint32_t row_tiles = row_len ? tile_keys / row_len : 1u;
+    const uint32_t nrows = row_len ? (uint32_t)(((uint64_t)n + row_len - 1) / row_len) : ntiles;
     const uint32_t ngroups = (nrows + RADIX_GROUP - 1) / RADIX_GROUP;
     const uint2* groups2 = reinterpret_cast<const uint2*>(tab.groups);
     const uint32_t* rows2 = reinterpret_cast<const uint32_t*>(tab.rows);
@@ -150,17 +172,17 @@ __global__ void __launch_bounds__(RS_THREADS, 2) k_radix_scatter(
         __syncthreads();
     }
     for (uint32_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        const uint32_t base = tile * RS_TILE + warp * (32u * RS_ITEMS) + lane;  // n < 2^32, and so is a tile's end
-        uint32_t key[RS_ITEMS], val[RS_ITEMS], rank[RS_ITEMS];
-        const bool full = n - tile * RS_TILE >= RS_TILE;  // (uniform)
+        const uint32_t base = tile * tile_keys + warp * (32u * ITEMS) + lane;  // n < 2^32, and so is a tile's end
+        uint32_t key[ITEMS], val[ITEMS], rank[ITEMS];
+        const bool full = n - tile * tile_keys >= tile_keys;  // (uniform)
         if (full) {
 #pragma unroll
-            for (int it = 0; it < RS_ITEMS; ++it) key[it] = keys_in[base + it * 32u];
+            for (int it = 0; it < ITEMS; ++it) key[it] = keys_in[base + it * 32u];
 #pragma unroll
-            for (int it = 0; it < RS_ITEMS; ++it) val[it] = vals_in ? vals_in[base + it * 32u] : base + it * 32u;
+            for (int it = 0; it < ITEMS; ++it) val[it] = vals_in ? vals_in[base + it * 32u] : base + it * 32u;
         } else {
 #pragma unroll
-            for (int it = 0; it < RS_ITEMS; ++it) {
+            for (int it = 0; it < ITEMS; ++it) {
                 const uint32_t idx = base + it * 32u;
                 key[it] = idx < n ? keys_in[idx] : 0u;
                 val[it] = idx < n ? (vals_in ? vals_in[idx] : idx) : 0u;
@@ -200,12 +222,13 @@ __global__ void __launch_bounds__(RS_THREADS, 2) k_radix_scatter(
         };
         if (full && !DROP) {
 #pragma unroll
-            for (int it = 0; it < RS_ITEMS; ++it)
+            for (int it = 0; it < ITEMS; ++it) {
                 rank_item(it, true, match_digit<BITS, true>((key[it] >> shift) & (D - 1u), true));
+            }
         } else {
             live = 0u;
 #pragma unroll
-            for (int it = 0; it < RS_ITEMS; ++it) {
+            for (int it = 0; it < ITEMS; ++it) {
                 const bool valid = base + it * 32u < n && !(DROP && key[it] == NONE);
                 live |= (uint32_t)valid << it;
                 rank_item(it, valid, match_digit<BITS, false>((key[it] >> shift) & (D - 1u), valid));
@@ -235,9 +258,10 @@ __global__ void __launch_bounds__(RS_THREADS, 2) k_radix_scatter(
         }
         __syncthreads();
 #pragma unroll
-        for (int it = 0; it < RS_ITEMS; ++it)
+        for (int it = 0; it < ITEMS; ++it) {
             if ((live >> it) & 1u)
                 s_kv[s_wc[warp][(key[it] >> shift) & (D - 1u)] + rank[it]] = make_uint2(key[it], val[it]);
+        }
         __syncthreads();
         for (uint32_t j = t; j < tile_n; j += RS_THREADS) {
             const uint2 kv = s_kv[j];
@@ -257,6 +281,22 @@ __global__ void __launch_bounds__(RS_THREADS, 2) k_radix_scatter(
     }
 }
 
+template <int BITS, bool DROP>
+__global__ void __launch_bounds__(RS_THREADS, 2) k_radix_scatter(
+    const uint32_t* __restrict__ keys_in, const uint32_t* __restrict__ vals_in, uint32_t* __restrict__ keys_out,
+    uint32_t* __restrict__ vals_out, const uint32_t* __restrict__ n32, const unsigned long long* __restrict__ n64,
+    uint64_t cap, int shift, RadixTab tab, uint32_t row_len, uint2* __restrict__ ranges, uint32_t n_ranges) {
+    pdl_wait();
+    __shared__ RadixSmem<1u << BITS> sm;
+    const uint32_t n = radix_n(n32, n64, cap);
+    if (radix_items(n) == RS_ITEMS)
+        radix_tiles<BITS, DROP, RS_ITEMS>(sm, n, keys_in, vals_in, keys_out, vals_out, shift, tab, row_len, ranges,
+                                          n_ranges);
+    else
+        radix_tiles<BITS, DROP, RS_ITEMS_SMALL>(sm, n, keys_in, vals_in, keys_out, vals_out, shift, tab, row_len,
+                                              ranges, n_ranges);
+}
+
 int radix_grid(int sms) { return 2 * sms; }
 
 void launch_radix_count(const uint32_t* keys, const uint32_t* n32, const unsigned long long* n64, uint64_t cap,
@@ -270,7 +310,7 @@ void launch_radix_scatter(const uint32_t* keys_in, const uint32_t* vals_in, uint
                           uint32_t n_ranges) {
 #define VGR_SCATTER_D(B, DR)                                                                                          \
     launch_k(k_radix_scatter<B, DR>, grid, RS_THREADS, s, keys_in, vals_in, keys_out, vals_out, n32, n64, cap, shift, \
-             tab, RS_TILE / row_len, ranges, n_ranges)
+             tab, row_len, ranges, n_ranges)
 #define VGR_SCATTER(B)                   \
     do {                                 \
         if (drop) VGR_SCATTER_D(B, true); \

@@ -655,10 +655,10 @@ constexpr int TILE_PASSES_MAX = 3;  // at most 2^20 tiles
 // chunk, the others one per radix tile.
 size_t tile_group_words(uint64_t cap_pairs, int passes, int bits) {
     return radix_group_words(cap_pairs, EMIT_SLOTS, bits) +
-           (size_t)(passes - 1) * radix_group_words(cap_pairs, RADIX_TILE, bits);
+           (size_t)(passes - 1) * radix_group_words(cap_pairs, 0, bits);
 }
 size_t table_row_words(uint64_t cap_pairs, uint32_t cap_vis) {
-    return std::max(radix_row_words(cap_pairs, EMIT_SLOTS, 8), radix_row_words(cap_vis, RADIX_TILE, 8));
+    return std::max(radix_row_words(cap_pairs, EMIT_SLOTS, 8), radix_row_words(cap_vis, 0, 8));
 }
 
 // the sorts' tables and the slot scan's look-back words; sized from the current capacities
@@ -670,7 +670,7 @@ vgr_status alloc_status(vgr_view* v) {
     if ((s = dalloc(&v->status, ceil_div(v->cap_vis, slot_scan_tile()) + 1, &b)) ||
         (s = dalloc(&v->radix_rows, table_row_words(v->cap_pairs, v->cap_vis), &b)) ||
         (s = dalloc(&v->tile_groups, tile_group_words(v->cap_pairs, TILE_PASSES_MAX, 8), &b)) ||
-        (s = dalloc(&v->depth_groups, 4 * radix_group_words(v->cap_vis, RADIX_TILE, 8), &b)))
+        (s = dalloc(&v->depth_groups, 4 * radix_group_words(v->cap_vis, 0, 8), &b)))
         return s;
     v->status_bytes = b;
     return VGR_OK;
@@ -948,7 +948,7 @@ vgr_status vgr_view_bytes_estimate(const vgr_hierarchy* h, const vgr_view_opts* 
     const uint64_t table_bytes = 8 * (ceil_div(cap_vis, slot_scan_tile()) + 1) +
                                  2 * table_row_words(cap_pairs, (uint32_t)cap_vis) +
                                  4 * (tile_group_words(cap_pairs, TILE_PASSES_MAX, 8) +
-                                      4 * radix_group_words(cap_vis, RADIX_TILE, 8));
+                                      4 * radix_group_words(cap_vis, 0, 8));
     const uint32_t T = o.tile_size ? o.tile_size : TILE_DEFAULT;
     const uint64_t tiles = (uint64_t)((width + T - 1) / T) * ((height + T - 1) / T);
     uint64_t b = 3 * 4 * cap_cut + per_vis * cap_vis + 4 * 4 * cap_pairs + 4 * emit_owner_cap(cap_pairs) + 2 * 4 * n_words + 2 * 4 * N +
@@ -1018,7 +1018,7 @@ uint32_t enqueue_frame(vgr_view* v, int lod, bool radix_depth, int tile_passes, 
     };
     zero(0, v->ctr, cleared_bytes(v->n_words, v->cap_vis));
     zero(1, v->tile_groups, tile_group_words(v->cap_pairs, plan.passes, plan.bits) * sizeof(uint32_t));
-    zero(2, v->depth_groups, radix_depth ? 4 * radix_group_words(v->cap_vis, RADIX_TILE, 8) * sizeof(uint32_t) : 0);
+    zero(2, v->depth_groups, radix_depth ? 4 * radix_group_words(v->cap_vis, 0, 8) * sizeof(uint32_t) : 0);
     clear.ranges = v->ranges;
     clear.n_ranges = n_tiles;
     launch_frame_begin(v->fp_host_dev, v->fp_dev, clear, v->h->num_sms, s);
@@ -1057,11 +1057,11 @@ uint32_t enqueue_frame(vgr_view* v, int lod, bool radix_depth, int tile_passes, 
         for (int p = 0; p < 4; ++p) {
             const uint32_t* kin = p == 0 ? v->vis.depth : sortK[(p + 1) & 1];
             const uint32_t* vin = p == 0 ? nullptr : v->sortV[(p + 1) & 1];
-            const RadixTab tab{v->radix_rows, v->depth_groups + p * radix_group_words(v->cap_vis, RADIX_TILE, 8)};
+            const RadixTab tab{v->radix_rows, v->depth_groups + p * radix_group_words(v->cap_vis, 0, 8)};
             launch_radix_count(kin, &v->ctr->n_front, nullptr, v->cap_vis, 8 * p, 8, tab, grid, s);
             // the last pass writes only the permutation (the sorted keys are not read)
             launch_radix_scatter(kin, vin, p == 3 ? nullptr : sortK[p & 1], v->sortV[p & 1], &v->ctr->n_front,
-                                 nullptr, v->cap_vis, 8 * p, 8, tab, RADIX_TILE, false, grid, s);
+                                 nullptr, v->cap_vis, 8 * p, 8, tab, 0u, false, grid, s);
         }
         launch_slot_scan(order, v->cap_vis, v->vis, v->slot_off, v->slot_owner, v->cap_pairs, v->status,
                          v->ctr, v->fp_dev, v->grid_scan, s);
@@ -1085,7 +1085,7 @@ uint32_t enqueue_frame(vgr_view* v, int lod, bool radix_depth, int tile_passes, 
         }
         launch_radix_scatter(v->pairK[p & 1], v->pairV[p & 1], last ? nullptr : v->pairK[(p + 1) & 1],
                              v->pairV[(p + 1) & 1], nullptr, n, v->cap_pairs, shift, bits, tab,
-                             p == 0 ? EMIT_SLOTS : RADIX_TILE, p == 0, grid, s, last ? v->ranges : nullptr, n_tiles);
+                             p == 0 ? EMIT_SLOTS : 0u, p == 0, grid, s, last ? v->ranges : nullptr, n_tiles);
     }
     v->last_tile_buf = tile_passes & 1;
     mark(VGR_STAGE_RANGES);

@@ -23,8 +23,15 @@ constexpr int MAX_TREE_DEPTH = 64;
 constexpr uint32_t SPIN_LIMIT = 1u << 22;     // bounded waits in look-back scans
 constexpr uint32_t CHILD_SHIFT = 28;          // child word: first_child | n_child << 28
 constexpr uint32_t CHILD_MASK = (1u << CHILD_SHIFT) - 1u;
-constexpr int RADIX_THREADS = 512;            // one radix-sort tile: 512 threads x 8 keys
-constexpr uint32_t RADIX_TILE = RADIX_THREADS * 8;
+constexpr int RADIX_THREADS = 512;
+constexpr uint32_t RADIX_TILE = RADIX_THREADS * 8;        // keys of a radix-sort tile,
+constexpr uint32_t RADIX_TILE_SMALL = RADIX_THREADS * 2;  // and of up to RADIX_SMALL_N keys (k_sort.cu)
+constexpr uint32_t RADIX_SMALL_N = 152 * 1024;
+constexpr uint64_t radix_max_tiles(uint64_t n) {  // of at most n keys
+    const uint64_t large = (n + RADIX_TILE - 1) / RADIX_TILE;
+    const uint64_t small = ((n < RADIX_SMALL_N ? n : RADIX_SMALL_N) + RADIX_TILE_SMALL - 1) / RADIX_TILE_SMALL;
+    return large > small ? large : small;
+}
 constexpr uint32_t RADIX_GROUP = 32;          // rows of digit counts per group
 constexpr int DEPTH_BINS = 6144;              // bins of the depth keys' histogram (k_depth.cu)
 

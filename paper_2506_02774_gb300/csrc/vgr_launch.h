@@ -123,14 +123,15 @@ struct RadixTab {
     uint16_t* rows;
     uint32_t* groups;
 };
+// (row_len: keys per row of the tables, or 0 for one row per tile, of whichever size)
 size_t radix_row_words(uint64_t n, uint32_t row_len, int bits);    // 16-bit words of the rows
 size_t radix_group_words(uint64_t n, uint32_t row_len, int bits);  // 32-bit words of the groups
 int radix_grid(int sms);
-// rows of RADIX_TILE keys
+// one row per tile
 void launch_radix_count(const uint32_t* keys, const uint32_t* n32, const unsigned long long* n64, uint64_t cap,
                         int shift, int bits, RadixTab tab, int grid, cudaStream_t s);
-// bits: 5 to 8; row_len: keys per row of the tables, RADIX_TILE or a divisor of it; the element count is *n32, *n64
-// or (both null) cap, and at most cap
+// bits: 5 to 8; row_len: RADIX_TILE_SMALL or a divisor of it, or 0 for the rows of launch_radix_count; the element
+// count is *n32, *n64 or (both null) cap, and at most cap
 void launch_radix_scatter(const uint32_t* keys_in, const uint32_t* vals_in, uint32_t* keys_out, uint32_t* vals_out,
                           const uint32_t* n32, const unsigned long long* n64, uint64_t cap, int shift, int bits,
                           RadixTab tab, uint32_t row_len, bool drop, int grid, cudaStream_t s, uint2* ranges = nullptr,

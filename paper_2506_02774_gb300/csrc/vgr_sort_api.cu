@@ -17,8 +17,8 @@
 
 namespace vgr {
 
-size_t sort_row_words(uint64_t n) { return radix_row_words(n, RADIX_TILE, 8); }
-size_t sort_group_words(uint64_t n, int passes) { return (size_t)passes * radix_group_words(n, RADIX_TILE, 8); }
+size_t sort_row_words(uint64_t n) { return radix_row_words(n, 0, 8); }
+size_t sort_group_words(uint64_t n, int passes) { return (size_t)passes * radix_group_words(n, 0, 8); }
 
 int sort_passes(uint32_t key_bits) { return (int)((key_bits + 7u) / 8u); }
 
@@ -28,7 +28,7 @@ cudaError_t sort_pairs_enqueue(const uint32_t* keys_in, const uint32_t* vals_in,
                                uint32_t* tmp_keys, uint32_t* tmp_vals, int sms, cudaStream_t s) {
     cudaError_t e = cudaMemsetAsync(groups, 0, sort_group_words(n, passes) * sizeof(uint32_t), s);
     if (e != cudaSuccess) return e;
-    const int grid = (int)std::min<uint64_t>(radix_grid(sms), (n + RADIX_TILE - 1) / RADIX_TILE);
+    const int grid = (int)std::min<uint64_t>(radix_grid(sms), radix_max_tiles(n));
     PdlScope pdl(true);  // the first kernel follows the clear in plain stream order
     // the last pass writes the output; earlier passes alternate backwards
     const uint32_t* kin = keys_in;
@@ -39,7 +39,7 @@ cudaError_t sort_pairs_enqueue(const uint32_t* keys_in, const uint32_t* vals_in,
         uint32_t* vo = to_out ? vals_out : tmp_vals;
         const RadixTab tab{rows, groups + sort_group_words(n, p)};
         launch_radix_count(kin, nullptr, nullptr, n, 8 * p, 8, tab, grid, s);
-        launch_radix_scatter(kin, vin, ko, vo, nullptr, nullptr, n, 8 * p, 8, tab, RADIX_TILE, false, grid, s);
+        launch_radix_scatter(kin, vin, ko, vo, nullptr, nullptr, n, 8 * p, 8, tab, 0u, false, grid, s);
         kin = ko;
         vin = vo;
     }

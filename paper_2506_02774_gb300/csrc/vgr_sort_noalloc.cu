@@ -19,7 +19,7 @@ constexpr uint64_t NA_MAX_N = VGR_SORT_NOALLOC_MAX_N;
 constexpr int NA_MAX_PASSES = 4;
 constexpr size_t na_round(size_t x) { return (x + 255) / 256 * 256; }
 // layout of the static scratch: digit counts of the tiles | of the groups, per pass | ping-pong keys | ping-pong values
-constexpr size_t NA_TILES = (NA_MAX_N + RADIX_TILE - 1) / RADIX_TILE;
+constexpr size_t NA_TILES = radix_max_tiles(NA_MAX_N);
 constexpr size_t NA_GROUPS = (NA_TILES + RADIX_GROUP - 1) / RADIX_GROUP;
 constexpr size_t NA_OFF_GROUPS = na_round(NA_TILES * 256 * sizeof(uint16_t));
 constexpr size_t NA_OFF_TMP = NA_OFF_GROUPS + na_round(NA_MAX_PASSES * NA_GROUPS * 256 * sizeof(uint32_t));
