@@ -52,7 +52,8 @@
 // parts of 32-pixel tiles as items of their own took the blend from 110 to 80 us
 // (1M-leaf box, 1080p), 184 to 161 (city, 1080p), 347 to 162 (1440p, 32-pixel
 // tiles), 81 to 48 and 56 (640 x 360 and 320 x 180 city views), 312 to 208
-// (canonical mode, 960 x 540).
+// (canonical mode, 960 x 540); that mode's pass over the staged records in order
+// took it to 143.
 #include "vgr_internal.cuh"
 #include "vgr_launch.h"
 
@@ -196,7 +197,7 @@ __device__ __forceinline__ bool blend_alpha(const float4& X, float rho, const fl
         alpha = fminf(ALPHA_MAX, ex2_approx(rho));
         return !(rho < LOG2_ALPHA_MIN);
     } else if (MODE == 1) {  // canonical: Eq. 3, then the alpha* test
-        alpha = fminf(ALPHA_MAX, X.w * __expf(rho));
+        alpha = fminf(ALPHA_MAX, X.w * ex2_approx(rho * LOG2E));
         return !(alpha < ALPHA_MIN);
     } else {
         // Eq. 5: nearest of m intervals over [-5.55, 0] (the index is clamped for records that fail Eq. 4 too)
@@ -520,7 +521,15 @@ __device__ __forceinline__ void blend_strips(float4 (*sbuf)[2 + (32 / T > 2 ? 2 
 #pragma unroll
             for (int q = 0; q < (DEPTH + 31) / 32; ++q) {
                 const uint32_t sl = 32u * q + lane;
-                if (sl < (uint32_t)DEPTH)  // each lane its own slots; empty slots reach no pixel
+                if (MODE == 1) {
+                    if (sl < nh) {
+                        blend_prepare<MODE, SR, T>(wA[sl], sbuf[buf][2][warp][sl], sbuf[buf][NP - 1][warp][sl],
+                                                   wC[sl].w, rlo, clo, true);
+                    } else if (sl < (uint32_t)DEPTH) {  // read with the last group
+#pragma unroll
+                        for (int part = 0; part < NP; ++part) sbuf[buf][part][warp][sl] = dummy_part<MODE, SR>(part);
+                    }
+                } else if (sl < (uint32_t)DEPTH)  // each lane its own slots; empty slots reach no pixel
                     pm[sl] = sl < nh ? blend_prepare<MODE, SR, T>(wA[sl], sbuf[buf][2][warp][sl],
                                                                            sbuf[buf][NP - 1][warp][sl],
                                                                            MODE != 0 ? wC[sl].w : 0.f, rlo, clo,
@@ -532,7 +541,7 @@ __device__ __forceinline__ void blend_strips(float4 (*sbuf)[2 + (32 / T > 2 ? 2 
             // depth order from bit 31 down: the transpose of the records' pixel masks
             uint32_t reach[(DEPTH + 31) / 32];
 #pragma unroll
-            for (int q = 0; q < (DEPTH + 31) / 32; ++q) {
+            for (int q = 0; q < (DEPTH + 31) / 32 && MODE != 1; ++q) {
                 const uint32_t sl = 32u * q + 31u - lane;
                 reach[q] = warp_transpose32(sl < (uint32_t)DEPTH ? pm[sl] : 0u);
             }
@@ -560,13 +569,36 @@ __device__ __forceinline__ void blend_strips(float4 (*sbuf)[2 + (32 / T > 2 ? 2 
                         return blend_rho(p, X, R);
                     }
                 };
+                if constexpr (MODE == 1) {
+                    // Every record at every pixel, alpha first: the slots in order, several
+                    // records' reads and exponentials together.  Of those that pass the alpha*
+                    // test (one in twenty) only the bit is kept, and the walk below evaluates
+                    // them again: 960 x 540, 108M evaluations, 143 us; with the rest of the
+                    // blend behind a branch per record 161, as straight code for groups 203.
+                    static_assert(DEPTH == 32, "one word of slots");
+                    constexpr uint32_t G = 8;
+                    evals += nh;
+                    reach[0] = 0u;
+                    for (uint32_t i = 0; i < nh; i += G) {
+                        uint32_t word = 0u;
+#pragma unroll
+                        for (uint32_t g = 0; g < G; ++g) {
+                            float4 X;
+                            float2 R;
+                            float alpha;
+                            load(i + g, X, R);
+                            if (blend_alpha<MODE>(X, rho_of(X, R), s_lut, m, lut_scale, alpha)) word |= 0x80000000u >> g;
+                        }
+                        reach[0] |= word >> i;
+                    }
+                }
 #pragma unroll
                 for (int q = 0; q < (DEPTH + 31) / 32; ++q) {
                     uint32_t mm = reach[q];  // bit 31 - l: slot 32 q + l
                     // BL_GROUP records at a time: their reads, rho and exponentials are
                     // independent of one another and go out together; only the
                     // transmittance runs through them in order
-                    evals += __popc(mm);
+                    if (MODE != 1) evals += __popc(mm);
                     uint32_t at[BL_GROUP], nat[BL_GROUP];
                     auto take = [&](uint32_t* slots) {
 #pragma unroll
@@ -603,10 +635,6 @@ __device__ __forceinline__ void blend_strips(float4 (*sbuf)[2 + (32 / T > 2 ? 2 
                                 use[g] = blend_alpha<MODE>(X, rho_of(X, R), s_lut, m, lut_scale, alpha[g]);
                             }
                         }
-                        if (MODE == 1 && !(use[0] || use[1] || use[2] || use[3])) {  // most fail there
-                            advance();
-                            continue;
-                        }
                         float Tr = p.T;
 #pragma unroll
                         for (int g = 0; g < BL_GROUP; ++g) {
@@ -621,10 +649,11 @@ __device__ __forceinline__ void blend_strips(float4 (*sbuf)[2 + (32 / T > 2 ? 2 
                                 if (use[g] && Tg[g] * (1.f - alpha[g]) < T_MIN) last = g;
                             p.done = true;
                             // not evaluated: what is left of this word, and the group's after the stop
-                            evals -= __popc(left);
+                            if (MODE != 1) evals -= __popc(left);
 #pragma unroll
                             for (int g = 0; g < BL_GROUP; ++g) {
-                                if (g > last && at[g] != (uint32_t)DEPTH) --evals;
+                                if (MODE != 1 && g > last && at[g] != (uint32_t)DEPTH) --evals;
+                                if (MODE == 1 && g == last) evals -= nh - (at[g] + 1u);
                                 if (g >= last) use[g] = false;
                                 if (g == last) Tr = Tg[g];
                             }

@@ -16,10 +16,10 @@
 // long as their number.)  The rows of the tile sort's first pass are written by
 // the emission, so its count kernel is saved there.  Tile sort of 981K slots
 // (1M-leaf box, 1080p): 47 -> 31 us; of 4.26M (city, 1080p): 85 -> 76; of 235K
-// (320 x 180, one pass): 24 -> 12; of 63K (801 x 603): 33 -> 18; the standalone sort of 4M 32-bit keys: 191 ->
-// 171.  Large inputs are bound by the instructions of the ranking (half of the
-// issue slots, the ballots' pipe first); three CTAs an SM at 40 registers were no
-// faster.
+// (320 x 180, one pass): 24 -> 12; of 63K (801 x 603): 23 -> 18 in the smaller tiles;
+// the standalone sort of 4M 32-bit keys: 191 -> 171.  Large inputs are bound by the
+// instructions of the ranking (half of the issue slots, the ballots' pipe first);
+// three CTAs an SM at 40 registers were no faster.
 #include "vgr_internal.cuh"
 #include "vgr_launch.h"
 
