@@ -14,12 +14,18 @@
 // found their bases by look-back took 18-24 us for up to a million keys whatever
 // the traffic: all the tiles were in flight at once, each digit's chain was as
 // long as their number.)  The rows of the tile sort's first pass are written by
-// the emission, so its count kernel is saved there.  Tile sort of 981K slots
-// (1M-leaf box, 1080p): 47 -> 31 us; of 4.26M (city, 1080p): 85 -> 76; of 235K
-// (320 x 180, one pass): 24 -> 12; of 63K (801 x 603): 23 -> 18 in the smaller tiles;
-// the standalone sort of 4M 32-bit keys: 191 -> 171.  Large inputs are bound by the
-// instructions of the ranking (half of the issue slots, the ballots' pipe first);
-// three CTAs an SM at 40 registers were no faster.
+// the emission, so its count kernel is saved there.
+//
+// What bounds it: the instructions of the ranking.  Peers by one ballot per digit
+// bit kept the ballots' pipe and half of the issue slots busy; lane masks OR-ed
+// in shared memory take a third of the instructions, but lanes of one digit queue
+// at its mask, so lane 0's are taken out by a ballot first.  4M random 32-bit
+// keys: 174 us by ballots, 165 by masks alone, 167 with both; 7 different keys:
+// 165, 178, 143; runs of 50 equal keys: 167, 186, 151 (match.any: 233, 138, 137).
+// With the table-based passes the tile sort of 981K slots (1M-leaf box, 1080p) went
+// from 47 to 29 us, of 4.26M (city, 1080p) from 85 to 71, of 235K (320 x 180, one
+// pass) from 24 to 12, of 63K (801 x 603) to 18, the sort of 4M keys from 191 to
+// 167.  Three CTAs an SM at 40 registers were no faster.
 #include "vgr_internal.cuh"
 #include "vgr_launch.h"
 
@@ -88,30 +94,13 @@ __global__ void __launch_bounds__(RS_THREADS) k_radix_count(const uint32_t* __re
     }
 }
 
-// Lanes of the (full) warp with the same digit of BITS bits, among the valid
-// ones; an invalid lane gets the invalid ones.
-template <int BITS, bool ALL>
-__device__ __forceinline__ uint32_t match_digit(uint32_t d, bool valid) {
-    uint32_t m = 0xFFFFFFFFu;
-    if (!ALL) {
-        const uint32_t ok = __ballot_sync(0xFFFFFFFFu, valid);
-        m = valid ? ok : ~ok;
-    }
-#pragma unroll
-    for (int b = 0; b < BITS; ++b) {
-        const bool bit = (d >> b) & 1u;
-        const uint32_t vote = __ballot_sync(0xFFFFFFFFu, bit);
-        m &= bit ? vote : ~vote;
-    }
-    return m;
-}
-
 // One digit pass over tiles of ITEMS pairs a thread (one row of the tables each, or
 // as many rows of row_len pairs as it holds):
 //  1. the tile's keys and values are requested; meanwhile the tables' entries
 //     before the tile are added up (two digits per thread and load);
-//  2. each warp ranks its contiguous share: peers by one ballot per digit bit,
-//     the first of them advances the warp's counter of the digit;
+//  2. each warp ranks its contiguous share, an item per lane at a time: the peers
+//     of lane 0 (same digit) by a ballot, the others' by the digits' lane masks in
+//     shared memory, and the foremost peer advances the warp's counter of its digit;
 //  3. a thread per digit turns the warps' counts into places in the tile;
 //  4. the pairs are staged digit-sorted in shared memory and
 //  5. stored, each digit's run contiguously.
@@ -143,6 +132,9 @@ __device__ __forceinline__ void radix_tiles(
     // the tables' partial sums lie under the staging buffer: groups, then rows
     uint32_t (*s_grp)[D] = reinterpret_cast<uint32_t (*)[D]>(s_kv);
     uint32_t (*s_row)[D] = reinterpret_cast<uint32_t (*)[D]>(s_kv + RS_THREADS);
+    // and so do the warps' peer masks, behind them
+    uint32_t (*s_mask)[D] = reinterpret_cast<uint32_t (*)[D]>(s_kv + 2 * RS_THREADS);
+    static_assert(RS_WARPS * D * sizeof(uint32_t) <= (RS_TILE - 2 * RS_THREADS) * sizeof(uint2), "masks' place");
     const uint32_t ntiles = (uint32_t)(((uint64_t)n + tile_keys - 1) / tile_keys);
     const uint32_t t = threadIdx.x, lane = lane_id(), warp = t >> 5;
     const uint32_t pair = t % (D / 2), q = t / (D / 2);
@@ -206,33 +198,32 @@ __device__ __forceinline__ void radix_tiles(
         }
         seen = g0;
         for (uint32_t i = t; i < RS_WARPS * D / 2; i += RS_THREADS) reinterpret_cast<uint32_t*>(&s_wc[0][0])[i] = 0u;
+        for (uint32_t i = t; i < RS_WARPS * D / 4; i += RS_THREADS)
+            reinterpret_cast<uint4*>(s_mask)[i] = make_uint4(0u, 0u, 0u, 0u);
         __syncthreads();
-        uint32_t live = 0xFFFFFFFFu;  // bit it: the pair takes part
-        auto rank_item = [&](int it, bool valid, uint32_t peers) {
+        uint32_t live = 0u;  // bit it: the pair takes part
+#pragma unroll
+        for (int it = 0; it < ITEMS; ++it) {
             const uint32_t d = (key[it] >> shift) & (D - 1u);
-            const int leader = __ffs(peers) - 1;
+            const bool valid = (full && !DROP) || (base + it * 32u < n && !(DROP && key[it] == NONE));
+            live |= (uint32_t)valid << it;
+            const uint32_t d0 = __shfl_sync(0xFFFFFFFFu, d, 0);
+            const bool as_first = valid && d == d0;
+            const uint32_t first = __ballot_sync(0xFFFFFFFFu, as_first);
+            if (valid && !as_first) atomicOr(&s_mask[warp][d], 1u << lane);
+            __syncwarp();
+            const uint32_t peers = as_first ? first : valid ? s_mask[warp][d] : 1u << lane;
+            __syncwarp();  // read before the foremost clears it
+            const int foremost = __ffs(peers) - 1;
             uint32_t before = 0;
-            if (valid && (int)lane == leader) {
+            if (valid && (int)lane == foremost) {
                 before = s_wc[warp][d];
                 s_wc[warp][d] = (uint16_t)(before + __popc(peers));
+                s_mask[warp][d] = 0u;
             }
-            before = __shfl_sync(0xFFFFFFFFu, before, leader);
+            before = __shfl_sync(0xFFFFFFFFu, before, foremost);
             rank[it] = before + __popc(peers & lanemask_lt());
-            __syncwarp();  // the counters as the next item's leaders read them
-        };
-        if (full && !DROP) {
-#pragma unroll
-            for (int it = 0; it < ITEMS; ++it) {
-                rank_item(it, true, match_digit<BITS, true>((key[it] >> shift) & (D - 1u), true));
-            }
-        } else {
-            live = 0u;
-#pragma unroll
-            for (int it = 0; it < ITEMS; ++it) {
-                const bool valid = base + it * 32u < n && !(DROP && key[it] == NONE);
-                live |= (uint32_t)valid << it;
-                rank_item(it, valid, match_digit<BITS, false>((key[it] >> shift) & (D - 1u), valid));
-            }
+            __syncwarp();  // the counters and masks as the next item's lanes read them
         }
         __syncthreads();
         uint32_t cnt = 0, ofs = 0, tile_n;
@@ -311,10 +302,10 @@ void launch_radix_scatter(const uint32_t* keys_in, const uint32_t* vals_in, uint
 #define VGR_SCATTER_D(B, DR)                                                                                          \
     launch_k(k_radix_scatter<B, DR>, grid, RS_THREADS, s, keys_in, vals_in, keys_out, vals_out, n32, n64, cap, shift, \
              tab, row_len, ranges, n_ranges)
-#define VGR_SCATTER(B)                   \
-    do {                                 \
+#define VGR_SCATTER(B)                    \
+    do {                                  \
         if (drop) VGR_SCATTER_D(B, true); \
-        else VGR_SCATTER_D(B, false);    \
+        else VGR_SCATTER_D(B, false);     \
     } while (0)
     switch (bits) {
         case 5: VGR_SCATTER(5); break;

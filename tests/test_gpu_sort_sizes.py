@@ -1,6 +1,7 @@
 """Key counts at the edges of the pair sort's tiles: a tile holds 1024 keys up to
 152 x 1024 keys and 4096 above, so the edges lie where a tile, a group of 32
-tiles, or the tile size changes.  Stable, against numpy's stable sort: whole
+tiles, or the tile size changes.  Keys at random, in runs of one digit and of few
+digits.  Stable, against numpy's stable sort: whole
 numbers, equal."""
 import numpy as np
 import pytest
@@ -18,10 +19,14 @@ SMALL = 152 * 1024
 
 @pytest.mark.parametrize("n", [1, 1023, 1024, 1025, 32 * 1024, 32 * 1024 + 1, SMALL - 1, SMALL, SMALL + 1,
                                39 * 4096, 64 * 4096 + 1, 304 * 4096, 304 * 4096 + 5])
-@pytest.mark.parametrize("key_bits", [8, 19])
-def test_sort_at_tile_size_edges(n, key_bits):
+@pytest.mark.parametrize("key_bits,kind", [(8, "random"), (19, "random"), (19, "runs"), (19, "few")])
+def test_sort_at_tile_size_edges(n, key_bits, kind):
     rng = np.random.default_rng(n + key_bits)
     keys = rng.integers(0, 1 << key_bits, n, dtype=np.uint32)
+    if kind == "runs":  # of one digit, across warps and tiles
+        keys = (np.arange(n, dtype=np.uint32) // 45) & 0x7FFFF
+    elif kind == "few":  # few digits in every pass
+        keys = keys % 5 * 0x10101
     vals = np.arange(n, dtype=np.uint32)
     order = np.argsort(keys, kind="stable")
     k = torch.from_numpy(keys.view(np.int32)).cuda()
