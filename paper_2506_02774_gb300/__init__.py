@@ -10,6 +10,7 @@ view the library's device buffers as tensors and for streams.
 from __future__ import annotations
 
 import ctypes
+import math
 
 import numpy as np
 
@@ -55,7 +56,7 @@ class _CudaArray:
 def device_tensor(ptr: int, shape, dtype: str):
     """A torch view (no copy) of library-owned device memory."""
     import torch
-    n = int(np.prod(shape)) if len(shape) else 1
+    n = math.prod(shape)
     if n == 0 or not ptr:
         return torch.empty(tuple(shape), dtype=getattr(torch, dtype), device="cuda")
     typestr = {"float32": "<f4", "int32": "<i4", "uint8": "|u1"}[dtype if dtype != "uint32" else "int32"]
@@ -66,8 +67,7 @@ def device_tensor(ptr: int, shape, dtype: str):
 def camera_struct(cam: dict) -> _abi.Camera:
     c = _abi.Camera()
     R = np.asarray(cam["R"], np.float32).reshape(9)
-    for i in range(9):
-        c.R[i] = float(R[i])
+    c.R[:] = R.tolist()
     p = np.asarray(cam["pos"], np.float32)
     for i in range(3):
         c.pos[i] = float(p[i])
@@ -143,15 +143,13 @@ class FrameResult:
         self.width, self.height = int(fr.width), int(fr.height)
         self.cut_count = int(fr.cut_count)
         s = fr.stats
-        self.stats = dict(cut_count=int(s.cut_count), front_count=int(s.front_count),
-                          visible_count=int(s.visible_count),
-                          pair_count=int(s.pair_count), candidate_pairs=int(s.candidate_pairs),
-                          nodes_evaluated=int(s.nodes_evaluated), lod_from_scratch=int(s.lod_from_scratch),
-                          replays=int(s.replays), kernels=int(s.kernels),
-                          pixel_pair_evals=int(s.pixel_pair_evals),
-                          pixel_pair_contribs=int(s.pixel_pair_contribs),
-                          stage_ms={n: float(s.stage_ms[i]) for i, n in enumerate(STAGES)},
-                          frame_ms=float(s.frame_ms))
+        # (the fields' values are Python ints and floats)
+        self.stats = {"cut_count": s.cut_count, "front_count": s.front_count, "visible_count": s.visible_count,
+                      "pair_count": s.pair_count, "candidate_pairs": s.candidate_pairs,
+                      "nodes_evaluated": s.nodes_evaluated, "lod_from_scratch": s.lod_from_scratch,
+                      "replays": s.replays, "kernels": s.kernels, "pixel_pair_evals": s.pixel_pair_evals,
+                      "pixel_pair_contribs": s.pixel_pair_contribs,
+                      "stage_ms": dict(zip(STAGES, s.stage_ms)), "frame_ms": s.frame_ms}
 
     def image(self):
         """H x W x 3 float32 CUDA tensor viewing the view's image buffer."""
