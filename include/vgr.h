@@ -120,12 +120,13 @@ typedef struct {
     uint32_t lod_budget;     /* max nodes one thread explores when expanding a cut node (0 = 4096) */
     uint32_t grid_wide;      /* CTAs of the grid-stride kernels (LoD, preprocess with colour, ranges);
                                 0 = 8 per SM.  Launch geometry only: results do not depend on it. */
-    uint32_t grid_scan;      /* CTAs of the ticketed look-back kernels (compaction, radix passes,
-                                emission); 0 = 4 per SM.  Launch geometry only. */
-    uint32_t test_hooks;     /* 0 in normal use.  VGR_HOOK_WITHHOLD_LOOKBACK: the emission's first
-                                tile never publishes its look-back word, so the later tiles' bounded
-                                waits run out and every frame reports VGR_E_TIMEOUT (the device
-                                stays usable); for testing the timeout path. */
+    uint32_t grid_scan;      /* CTAs of the compaction and the emission (and of the slot scan after a
+                                radix depth sort); 0 = 4 per SM.  Launch geometry only. */
+    uint32_t test_hooks;     /* 0 in normal use.  VGR_HOOK_WITHHOLD_LOOKBACK: depths are ordered by radix
+                                passes, and the first tile of the slot scan behind them never publishes
+                                its look-back word, so the later tiles' bounded waits run out and every
+                                frame reports VGR_E_TIMEOUT (the device stays usable); for testing the
+                                timeout path. */
     uint32_t lod_frustum;    /* 1: frustum-aware granularity test (needs bbox; default 0), see
                                 vgr_render_frame */
     float lod_frustum_guard; /* pixels the frustum test adds beyond each image edge (default 2) */

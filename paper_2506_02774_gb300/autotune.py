@@ -20,7 +20,7 @@ import os
 from . import View
 
 GRID_WIDE_PER_SM = (2, 4, 8, 16)   # grid-stride kernels: LoD, preprocess (with colour), ranges
-GRID_SCAN_PER_SM = (2, 3, 4, 6)    # ticketed look-back kernels: compaction, radix passes, emission
+GRID_SCAN_PER_SM = (2, 3, 4, 6)    # compaction, emission
 BLEND_DEPTHS = (16, 32, 48)        # Gaussians a blend warp stages per chunk
 BATCH_CHAINS = (0, 1, 2, 3, 4, 8)  # views of a batch running at once (0: all)
 TILE_SIZES = (8, 16, 32)           # tile side in pixels

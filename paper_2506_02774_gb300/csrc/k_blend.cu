@@ -812,10 +812,15 @@ __global__ void __launch_bounds__(BL_THREADS, BL_MIN_CTAS) k_blend_wide(const Fr
     // others), the rest of the heavy ones and the rest of the others are claimed
     constexpr uint32_t PARTS = NS / slot_strips(NS);  // slots of a tile (one for a heavy tile of 16 x 16)
     const uint32_t dealt = gridDim.x, mine = blockIdx.x;
-    if (T == 16 && heavy > 0u)
-        blend_strips<0, DEPTH, T>(sbuf, ring, reinterpret_cast<uint32_t*>(s_pm[warp]), it, s_heavy, fp0, fps, work,
-                                  heavy, next, mine < heavy ? mine : NONE, dealt, nullptr, 0u, 0.f, full_walk);
-    const uint32_t light0 = T == 16 && mine < heavy ? NONE : mine, light_base = max(dealt, heavy);
+    uint32_t light0 = mine;
+    if constexpr (T == 16) {
+        if (mine < heavy) light0 = NONE;
+        if (heavy > 0u)
+            blend_strips<0, DEPTH, T>(sbuf, ring, reinterpret_cast<uint32_t*>(s_pm[warp]), it, s_heavy, fp0, fps,
+                                      work, heavy, next, mine < heavy ? mine : NONE, dealt, nullptr, 0u, 0.f,
+                                      full_walk);
+    }
+    const uint32_t light_base = max(dealt, heavy);
     static_assert(T == 32 || PARTS == 1, "slots count tiles where some of them are heavy");
     const uint32_t row = lane / HP, col = 2u * (lane % HP);  // this lane's first pixel in the strip
     for (;;) {

@@ -350,8 +350,6 @@ void launch_preprocess(const SceneDev& sc, const uint32_t* front, const uint32_t
 #undef VGR_PRE_LAUNCH
 }
 
-uint32_t preprocess_tile() { return PRE_THREADS; }
-
 // The visible entries' records as separate arrays (the debug view's layout).
 __global__ void k_debug_records(VisBuffers vis, uint32_t n, uint2* __restrict__ rect, float4* __restrict__ recA,
                                 float4* __restrict__ recB, float4* __restrict__ rgb) {

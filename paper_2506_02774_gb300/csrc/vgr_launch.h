@@ -100,7 +100,6 @@ struct VisBuffers {
 void launch_preprocess(const SceneDev& sc, const uint32_t* front, const uint32_t* n_front, uint32_t cap,
                        const FrameParams* fp, VisBuffers vis, Counters* ctr, uint32_t* depth_bins, bool interp,
                        int grid, cudaStream_t s);
-uint32_t preprocess_tile();
 // The records of n entries as vgr_debug_buffers lays them out
 void launch_debug_records(const VisBuffers& vis, uint32_t n, uint2* rect, float4* recA, float4* recB, float4* rgb,
                           cudaStream_t s);
