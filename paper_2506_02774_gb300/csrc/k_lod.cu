@@ -514,28 +514,35 @@ __global__ void __launch_bounds__(256) k_lod_level(int level, const uint32_t* __
 // warp takes a row of 32 words: a scan of their bit counts gives every word its
 // place, and the warp goes through the words that have bits, lane l storing the
 // id of bit l if it is set (contiguous stores, no barrier, no staging).  Bound by
-// those instructions and, on small scenes, by the kernel's three round trips.
-// Tiles of 1024 words on a look-back chain, their ids unpacked in shared memory
-// bit by bit, took 28 us on the 1M-leaf box (44 tiles for 152 SMs; now 10) and
-// 41 us on the city (26.5M nodes; now 32, while counting adds 10 to the 119 us
-// of its LoD update).
+// those instructions (a bit count per word, at a quarter of the issue rate) and, on
+// small scenes, by the kernel's three round trips.  The words and their places come
+// as broadcasts from shared memory, two words per load: by two shuffles per word the
+// 1M-leaf box took 10 us, now 8.5, the city (26.5M nodes) 32, now 28.  Tiles of 1024
+// words on a look-back chain, their ids unpacked in shared memory bit by bit, took
+// 28 and 41 us (while counting adds 10 to the 119 us of the city's LoD update).
 constexpr int CC_THREADS = 256;
 constexpr int CC_WARPS = CC_THREADS / 32;
 static_assert(CC_TILE_WORDS == CC_THREADS, "one row of 32 words per warp");
 
 // Store the ids of a row's set bits (lane l holds word l, first id id0 + 32 l)
-// from out[at] on.
+// from out[at] on.  s_row: the warp's, for the words and places as broadcasts.
 __device__ __forceinline__ void cc_row(uint32_t word, uint32_t pre, uint32_t id0, uint32_t* __restrict__ out,
-                                       uint32_t cap) {
+                                       uint32_t cap, uint2* s_row) {
     const uint32_t lane = lane_id(), below = lanemask_lt();
     uint32_t some = __ballot_sync(0xFFFFFFFFu, word != 0u);
     if (__popc(some) >= 12) {  // most words have bits: all of them, independent of one another
-#pragma unroll 8
-        for (int w = 0; w < 32; ++w) {
-            const uint32_t bits = __shfl_sync(0xFFFFFFFFu, word, w);
-            const uint32_t p = __shfl_sync(0xFFFFFFFFu, pre, w) + __popc(bits & below);
-            if (((bits >> lane) & 1u) && p < cap) out[p] = id0 + 32u * w + lane;
+        s_row[lane] = make_uint2(word, pre);
+        __syncwarp();
+        const uint4* two = reinterpret_cast<const uint4*>(s_row);
+        const uint32_t id = id0 + lane;
+#pragma unroll
+        for (int w = 0; w < 16; ++w) {
+            const uint4 q = two[w];
+            const uint32_t p0 = q.y + __popc(q.x & below), p1 = q.w + __popc(q.z & below);
+            if (((q.x >> lane) & 1u) && p0 < cap) out[p0] = id + 64u * w;
+            if (((q.z >> lane) & 1u) && p1 < cap) out[p1] = id + 64u * w + 32u;
         }
+        __syncwarp();  // read before the next row's words
         return;
     }
     while (some) {
@@ -556,6 +563,7 @@ __global__ void __launch_bounds__(CC_THREADS) k_cut_compact(uint32_t* __restrict
     pdl_wait();
     __shared__ uint2 s_sum[2][CC_WARPS];
     __shared__ uint32_t s_scan[2][CC_WARPS];
+    __shared__ __align__(16) uint2 s_row[CC_WARPS][32];
     const uint32_t ntiles = n_words / CC_TILE_WORDS;  // the bitmaps are padded to whole tiles
     const uint32_t t = threadIdx.x, warp = t >> 5, lane = lane_id();
     uint32_t oa = 0, ob = 0, seen = 0, flip = 0;  // ids in the tiles before 'seen'
@@ -581,8 +589,8 @@ __global__ void __launch_bounds__(CC_THREADS) k_cut_compact(uint32_t* __restrict
             ob += c.y;
         }
         const uint32_t id0 = (tile * CC_TILE_WORDS + 32u * warp) * 32u;
-        cc_row(a, oa + (pre & 0xFFFFu), id0, cut, cap);
-        cc_row(b, ob + (pre >> 16), id0, front_list, cap);
+        cc_row(a, oa + (pre & 0xFFFFu), id0, cut, cap, s_row[warp]);
+        cc_row(b, ob + (pre >> 16), id0, front_list, cap, s_row[warp]);
         if (a) bitmap[wi] = 0u;
         if (b) front[wi] = 0u;
         if (tile == ntiles - 1 && t == 0) {
