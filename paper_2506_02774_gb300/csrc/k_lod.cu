@@ -59,15 +59,20 @@ __device__ __forceinline__ void load_lodr(const float4* __restrict__ lodr, uint3
         : "l"(lodr + 2 * (size_t)n));
 }
 
-// Set bit n of bm in the lanes where pred holds, one atomic per word: the
-// lanes that hit the same word (the match instruction; a warp's nodes are
-// few words) OR their bits together and the lowest of them stores them.
-// All 32 lanes call it.
-__device__ __forceinline__ void warp_bitmap_set(uint32_t* bm, uint32_t n, bool pred) {
-    const uint32_t w = pred ? n >> 5 : 0xFFFFFFFFu;
+// Set bit n of two bitmaps in the lanes where in_a and in_b hold (in_b implies
+// in_a), one atomic per word: the lanes that hit the same word (the match
+// instruction; a warp's nodes are few words) OR their bits together and the lowest
+// of them stores them.  All 32 lanes call it.
+__device__ __forceinline__ void warp_bitmap_set(uint32_t* a, uint32_t* b, uint32_t n, bool in_a, bool in_b) {
+    const uint32_t w = in_a ? n >> 5 : 0xFFFFFFFFu;
     const uint32_t peers = __match_any_sync(0xFFFFFFFFu, w);
-    const uint32_t bits = __reduce_or_sync(peers, pred ? 1u << (n & 31u) : 0u);
-    if (pred && lane_id() == (uint32_t)(__ffs(peers) - 1)) atomicOr(&bm[w], bits);
+    const uint32_t bit = 1u << (n & 31u);
+    const uint32_t bits_a = __reduce_or_sync(peers, in_a ? bit : 0u);
+    const uint32_t bits_b = __reduce_or_sync(peers, in_b ? bit : 0u);
+    if (in_a && lane_id() == (uint32_t)(__ffs(peers) - 1)) {
+        atomicOr(&a[w], bits_a);
+        if (bits_b) atomicOr(&b[w], bits_b);
+    }
 }
 
 // With weight interpolation the rendered Gaussian of a cut node n is not n's
@@ -348,13 +353,12 @@ __global__ void __launch_bounds__(256) k_lod_update(const uint32_t* __restrict__
 #pragma unroll
         for (int u = 0; u < LOD_UNROLL; ++u) {
             const bool stay = ok[u] && visit(nn[u], cc[u], pp[u], qq[u]);
-            warp_bitmap_set(bitmap, nn[u], stay);
             bool vis = false;
             if (stay) {
                 if (!out.interp || pp[u] == NONE) vis = out.in_front(cc[u], ll[u]);
                 else vis = out.in_front_segment(cc[u], ll[u], qq[u], sc.lmax[pp[u]]);
             }
-            warp_bitmap_set(front, nn[u], vis);
+            warp_bitmap_set(bitmap, front, nn[u], stay, vis);
             in_cut[u] = stay;
             in_front[u] = vis;
         }
@@ -489,8 +493,7 @@ __global__ void __launch_bounds__(256) k_lod_level(int level, const uint32_t* __
             }
         }
         // one atomic per bitmap word and warp (a node's siblings are neighbours)
-        warp_bitmap_set(bitmap, n, is_cut);
-        warp_bitmap_set(front, n, in_front);
+        warp_bitmap_set(bitmap, front, n, is_cut, in_front);
         warp_tile_count<1>(counts, &n, &is_cut, &in_front);
         uint32_t total;
         const uint32_t off = warp_excl_scan(cnt, &total);
