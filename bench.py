@@ -176,10 +176,10 @@ def _frame_bytes(sc: dict, st: dict, W: int, H: int, tile_passes: int) -> dict:
         lod=16 * E + 4 * C + 4 * C + 2 * N / 8,      # node and parent tests, lmax, prev cut read, two bitmaps set
         compact=2 * (N / 8 * 2) + 4 * C + 4 * F,     # two bitmaps read + cleared, cut and in-front ids written
         # ids, centre, covariance + opacity, records out; SH in and rgb out (visible)
-        preprocess=(4 + 16 + 32 + 48) * F + (shb + 16) * V,
-        depth_sort=4 * 2 * 8 * F + 4 * F,            # 4 passes x (key+value) read+write, histogram read
+        preprocess=(4 + 16 + 32 + 40) * F + (shb + 16) * V,
+        depth_sort=4 * F + 24 * V,                   # keys; (key, index) partitioned; order, slot offsets
         color=0,                                     # evaluated in preprocess
-        emit=(4 + 4 + 8 + 32) * V + 8 * P0,          # order, count, rect, record halves; slots
+        emit=(4 + 4 + 32) * V + 8 * P0,              # order, slot offset, record; slots
         tile_sort=tile_passes * 2 * 8 * P0,
         ranges=4 * P + 8 * (W // 16 + 1) * (H // 16 + 1),
         blend=(4 + 48) * P + 12 * W * H,
