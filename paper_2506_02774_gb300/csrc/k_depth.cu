@@ -9,8 +9,8 @@
 //    function of the key (half of the bins logarithmic in z, half linear, over
 //    the depth range the scene's bounds allow: depth_bin);
 //  * k_depth_part scans the bins (every CTA for itself), joins neighbouring
-//    bins into buckets of about 2^q keys (bucket of a bin = its exclusive
-//    prefix >> q, so no bucket holds more than 2^q + its largest bin), and
+//    bins into buckets of about s keys (bucket of a bin = its exclusive prefix
+//    / s, so no bucket holds more than s + its largest bin), and
 //    writes each (key, index << 8 | slot count) to its bucket, at a place
 //    reserved with one atomic per CTA and bucket; the same atomic adds up the
 //    bucket's candidate slots;
@@ -25,10 +25,12 @@
 // Four stable radix passes and a scan of the slot counts did this before; each
 // pass was a chain of look-back round trips (15-21 us for 550K keys whatever
 // the traffic).  Depth order and slots, 1M-leaf box at 1080p (552K visible):
-// 96 -> 26 us; city at 1080p (2.67M visible): 153 -> 67 us.  Bound now by the
+// 96 -> 26 us; city at 1080p (2.67M visible): 153 -> 60 us.  Bound now by the
 // shared-memory atomics and barriers of a CTA's steps (issue slots 35-50 %).
 // A bucket that does not fit a CTA (F_SORT_SKEW: thousands of Gaussians in one
 // bin) makes the host replay the frame with the radix passes of k_sort.cu.
+#include <algorithm>
+
 #include "vgr_internal.cuh"
 #include "vgr_launch.h"
 
@@ -38,8 +40,8 @@ constexpr int DP_THREADS = 512;
 constexpr int DP_ITEMS = 16;
 constexpr int DP_TILE = DP_THREADS * DP_ITEMS;  // entries a CTA partitions at a time
 constexpr int DP_BPT = DEPTH_BINS / DP_THREADS;  // bins per thread
-constexpr uint32_t DP_Q_MIN = 8, DP_Q_MAX = 11;
-constexpr uint32_t DP_BUCKETS = 320;             // buckets aimed at while they stay below 2^DP_Q_MAX keys
+constexpr uint32_t DP_KEYS_MIN = 256, DP_KEYS_MAX = 4096;  // keys aimed at per bucket
+constexpr uint32_t DP_ROUNDS = 3, DP_CTAS = 320;           // rounds of at most so many CTAs shared out evenly
 static_assert(DP_BPT % 4 == 0, "bins are read as uint4");
 
 constexpr int DL_THREADS = 512;
@@ -51,17 +53,29 @@ constexpr uint32_t DL_SUB_BITS = 12, DL_SUB = 1u << DL_SUB_BITS;
 constexpr uint32_t DL_RUN_MAX = 48;     // longest run ranked by comparing its members
 constexpr int DL_SPT = DL_SUB / DL_THREADS;
 
-// log2 of the bucket size for n keys, and the number of bucket ids it makes
-__host__ __device__ inline uint32_t depth_q(uint32_t n) {
-    uint32_t q = DP_Q_MIN;
-    while (q < DP_Q_MAX && (n >> q) > DP_BUCKETS) ++q;
-    return q;
+// The bucket of a key before which there are pre others (below 2^24) is the high word
+// of pre times depth_step(...): pre / s rounded down, for s keys a bucket.  A bucket
+// holds at most s keys and one bin more (s_max: the warps' largest bins), which has to
+// fit its CTA.  Half of a bucket's time does not depend on its keys (sub-bins, scans,
+// barriers), so the fewest whole rounds of k_depth_local's CTAs with buckets of up to
+// DP_KEYS_MAX are shared out evenly, and past DP_ROUNDS rounds the buckets are full.
+// Depth order of the city's frames with buckets of 2048 keys and as here: 5.1M visible
+// 114 and 103 us, 2.9M 70 and 64, 1.4M 42 and 39, 0.94M 35 and 31, 0.67M 31 and 28.
+__device__ __forceinline__ uint32_t depth_step(uint32_t n, const uint32_t* s_max) {
+    const uint32_t ctas = min(gridDim.x, DP_CTAS);
+    if (n < ctas * DP_KEYS_MIN) return 0xFFFFFFFFu / DP_KEYS_MIN + 1u;
+    uint32_t most = 8u;  // for the rounding
+#pragma unroll
+    for (int w = 0; w < DP_THREADS / 32; ++w) most = max(most, s_max[w] + 8u);
+    const uint32_t full = min(max(DL_CAP - min(most, DL_CAP), DP_KEYS_MAX / 2), DP_KEYS_MAX);
+    uint32_t slots = ctas;
+    while (slots < DP_ROUNDS * ctas && n > slots * full) slots += ctas;
+    const uint32_t s = n > slots * full ? full : n / slots + 1u;
+    return 0xFFFFFFFFu / s + 1u;  // 2^32 / s, rounded up
 }
-__host__ __device__ inline uint32_t depth_buckets(uint32_t n) { return (n >> depth_q(n)) + 1u; }
 
 uint32_t depth_bucket_cap(uint32_t cap_vis) {
-    const uint32_t a = DP_BUCKETS + 2u, b = (cap_vis >> DP_Q_MAX) + 2u;
-    return a > b ? a : b;
+    return std::max(DP_ROUNDS * DP_CTAS, cap_vis / (DP_KEYS_MAX / 2)) + 2u;
 }
 
 __global__ void __launch_bounds__(DP_THREADS, 2) k_depth_part(const uint32_t* __restrict__ depth,
@@ -79,7 +93,7 @@ __global__ void __launch_bounds__(DP_THREADS, 2) k_depth_part(const uint32_t* __
     uint32_t* s_base = s_start + cap_buckets + 1;          // [nb] keys of this tile, then their first position
     uint32_t* s_slot = s_base + cap_buckets;               // [nb] candidate slots of this tile
     __shared__ uint32_t s_scan[DP_THREADS / 32];
-    __shared__ uint32_t s_last[DP_THREADS];
+    __shared__ uint32_t s_last[DP_THREADS], s_max[DP_THREADS / 32];
     const uint32_t t = threadIdx.x;
     const uint32_t n = min(ctr->n_front, cap);
     // contiguous chunks, whole rows of DP_THREADS entries
@@ -104,18 +118,24 @@ __global__ void __launch_bounds__(DP_THREADS, 2) k_depth_part(const uint32_t* __
             const uint4 v = reinterpret_cast<const uint4*>(bins)[t * (DP_BPT / 4) + k];
             c[4 * k] = v.x; c[4 * k + 1] = v.y; c[4 * k + 2] = v.z; c[4 * k + 3] = v.w;
         }
-        uint32_t sum = 0;
-#pragma unroll
-        for (int k = 0; k < DP_BPT; ++k) sum += c[k];
-        s_last[t] = c[DP_BPT - 1];
-        uint32_t pre = block_excl_scan<DP_THREADS / 32>(sum, s_scan, &total);
-        const uint32_t q = depth_q(total);
-        nb = min((total >> q) + 1u, cap_buckets);
-        // bucket ids above the previous bin's start at this bin
-        uint32_t id = t == 0 ? NONE : (pre - s_last[t - 1]) >> q;  // NONE + 1 == 0
+        uint32_t sum = 0, most = 0;
 #pragma unroll
         for (int k = 0; k < DP_BPT; ++k) {
-            const uint32_t b = min(pre >> q, nb - 1u);
+            sum += c[k];
+            most = max(most, c[k]);
+        }
+        most = __reduce_max_sync(0xFFFFFFFFu, most);
+        if (lane_id() == 0) s_max[t >> 5] = most;
+        s_last[t] = c[DP_BPT - 1];
+        uint32_t pre = block_excl_scan<DP_THREADS / 32>(sum, s_scan, &total);  // (and a barrier)
+        const uint32_t step = depth_step(total, s_max);
+        nb = min(__umulhi(total, step) + 1u, cap_buckets);
+        if (blockIdx.x == 0 && t == 0) ctr->depth_nb = nb;
+        // bucket ids above the previous bin's start at this bin
+        uint32_t id = t == 0 ? NONE : min(__umulhi(pre - s_last[t - 1], step), nb - 1u);  // NONE + 1 == 0
+#pragma unroll
+        for (int k = 0; k < DP_BPT; ++k) {
+            const uint32_t b = min(__umulhi(pre, step), nb - 1u);
             s_bucket[t * DP_BPT + k] = (uint16_t)b;
             while (id != b) {
                 s_start[++id] = pre;
@@ -210,7 +230,7 @@ __global__ void __launch_bounds__(DL_THREADS, 2) k_depth_local(const uint2* __re
     if (ctr->flags & F_SORT_SKEW) return;
     const DepthMap map = fp->depth;
     const uint32_t n_vis = min(ctr->n_vis, cap_vis);
-    const uint32_t nb = depth_buckets(n_vis);
+    const uint32_t nb = ctr->depth_nb;
     const uint32_t cap_owner = (uint32_t)(cap_pairs / EMIT_SLOTS) + 1u;
     auto slots_of = [&](uint32_t v) -> uint32_t { return (v & 255u) < 255u ? v & 255u : ntile[v >> 8]; };
 #pragma unroll

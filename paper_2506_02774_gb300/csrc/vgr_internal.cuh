@@ -134,6 +134,7 @@ struct Counters {
     uint32_t n_heavy;           // tiles of the blend order's heavy classes (BL_HEAVY_CLASS and above)
     uint32_t blend_next[2];     // the blend's next tile in its work list: heavy ones, others
     uint32_t blend_done;        // CTAs of the blend that have finished
+    uint32_t depth_nb;          // buckets of the depth partition
 };
 constexpr size_t COUNTERS_HEAD = 56;  // bytes read back per frame (n_vis .. pix_contribs)
 

@@ -63,3 +63,21 @@ def test_order(name, half):
         np.testing.assert_array_equal(da["depth_order"], want)
         np.testing.assert_array_equal(db["depth_order"], want)
     v.close(); ref.close(); h.close()
+
+
+@pytest.mark.parametrize("n,equal", [(300_000, 0), (700_000, 3500), (1_400_000, 0), (1_400_000, 4000)])
+def test_order_of_large_frames(n, equal):
+    """More keys than one small bucket per CTA: buckets sized by whole rounds of
+    CTAs, and by the room that a bin of many equal depths leaves."""
+    def depth(r, m):
+        x = r.uniform(20.0, 60.0, m)
+        x[:equal] = 40.0
+        return x
+    h = vgr.Hierarchy(_scene(n, depth))
+    v = vgr.View(h)
+    r = v.render(scenegen.camera((0.0, 15.0, 4.0), 0.0, 333, 211, 160.0), 0.0)
+    d = v.debug()
+    assert r.stats["replays"] <= 1 and r.stats["visible_count"] > 0.9 * n  # (one for the pair buffer, if any)
+    want = np.lexsort((np.arange(d["n_visible"]), d["vis_depth"]))
+    np.testing.assert_array_equal(d["depth_order"], want)
+    v.close(); h.close()
