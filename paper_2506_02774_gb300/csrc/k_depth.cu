@@ -42,6 +42,12 @@ constexpr int DP_TILE = DP_THREADS * DP_ITEMS;  // entries a CTA partitions at a
 constexpr int DP_BPT = DEPTH_BINS / DP_THREADS;  // bins per thread
 constexpr uint32_t DP_KEYS_MIN = 256, DP_KEYS_MAX = 4096;  // keys aimed at per bucket
 constexpr uint32_t DP_ROUNDS = 3, DP_CTAS = 320;           // rounds of at most so many CTAs shared out evenly
+// A bucket's cursor: its keys so far, and above them its candidate slots.  An entry has
+// at most 2^20 slots, so a bucket that fits a CTA has less than 2^33, which one word
+// holds; a tile's share of them is added up in 32 bits, entries of many slots apart.
+constexpr int DP_KEY_BITS = 25;
+constexpr uint32_t DP_FEW_SLOTS = 0xFFFFFFFFu / DP_TILE;
+static_assert(MAX_RANKS < (1u << DP_KEY_BITS), "a cursor counts every key");
 static_assert(DP_BPT % 4 == 0, "bins are read as uint4");
 
 constexpr int DL_THREADS = 512;
@@ -169,7 +175,8 @@ __global__ void __launch_bounds__(DP_THREADS, 2) k_depth_part(const uint32_t* __
                 const uint32_t b = s_bucket[depth_bin(map, key[k])];
                 const uint32_t c = ntile[i];
                 at[k] = (b << 13) | atomicAdd(&s_base[b], 1u);
-                atomicAdd(&s_slot[b], c);
+                if (c <= DP_FEW_SLOTS) atomicAdd(&s_slot[b], c);
+                else atomicAdd(&cursor[b], (unsigned long long)c << DP_KEY_BITS);
                 cnt[k / 4] |= min(c, 255u) << (8 * (k % 4));
             }
         }
@@ -177,8 +184,8 @@ __global__ void __launch_bounds__(DP_THREADS, 2) k_depth_part(const uint32_t* __
         for (uint32_t b = t; b < nb; b += DP_THREADS) {
             const uint32_t c = s_base[b];
             if (c) {
-                const unsigned long long add = (unsigned long long)s_slot[b] << 32 | c;
-                s_base[b] = s_start[b] + (uint32_t)atomicAdd(&cursor[b], add);
+                const unsigned long long add = (unsigned long long)s_slot[b] << DP_KEY_BITS | c;
+                s_base[b] = s_start[b] + ((uint32_t)atomicAdd(&cursor[b], add) & ((1u << DP_KEY_BITS) - 1u));
             }
         }
         __syncthreads();
@@ -256,7 +263,7 @@ __global__ void __launch_bounds__(DL_THREADS, 2) k_depth_local(const uint2* __re
             if (j < n) e[k] = part[start + j];
         }
         unsigned long long sum = 0ull;
-        for (uint32_t p = seen + t; p < b; p += DL_THREADS) sum += cursor[p] >> 32;
+        for (uint32_t p = seen + t; p < b; p += DL_THREADS) sum += cursor[p] >> DP_KEY_BITS;
         seen = b;
 #pragma unroll
         for (int k = 0; k < DL_ITEMS; ++k) {
@@ -342,9 +349,9 @@ __global__ void __launch_bounds__(DL_THREADS, 2) k_depth_local(const uint2* __re
         __syncthreads();
         // first slots: each thread an odd number of neighbours (no bank conflicts)
         const uint32_t per = ((n + DL_THREADS - 1u) / DL_THREADS) | 1u, jb = t * per, je = min(jb + per, n);
-        uint32_t mine = 0, all;
+        uint32_t mine = 0, unused;
         for (uint32_t j = jb; j < je; ++j) mine += slots_of(s_fin[j]);
-        uint32_t run = (uint32_t)slots + block_excl_scan<DL_WARPS>(mine, s_scan2, &all);
+        uint32_t run = (uint32_t)slots + block_excl_scan<DL_WARPS>(mine, s_scan2, &unused);
         for (uint32_t j = jb; j < je; ++j) {
             const uint32_t c = slots_of(s_fin[j]);
             s_off[j] = run;
@@ -359,10 +366,9 @@ __global__ void __launch_bounds__(DL_THREADS, 2) k_depth_local(const uint2* __re
             off[start + j] = s_off[j];
         }
         if (b == nb - 1u && t == 0) {
-            const unsigned long long ns = slots + all;
-            off[n_vis] = (uint32_t)ns;
+            const unsigned long long ns = slots + (cursor[b] >> DP_KEY_BITS);
+            off[n_vis] = (uint32_t)ns;  // (past 2^32 these wrap, and the emission leaves the frame alone)
             ctr->n_cand = ns;
-            if (ns > cap_pairs) atomicOr(&ctr->flags, F_OVF_PAIRS);
         }
         // (the next bucket writes s_kv and s_fin only after barriers that follow these reads)
     }

@@ -107,11 +107,11 @@ __global__ void __launch_bounds__(SS_THREADS) k_slot_scan(const uint32_t* __rest
             }
             run += c[k];
         }
-        if (tile == ntiles - 1 && threadIdx.x == 0) {
-            const uint64_t ns = (uint64_t)s_prefix + total;
-            off[n_vis] = (uint32_t)ns;
-            ctr->n_cand = ns;
-            if (ns > cap_pairs) atomicOr(&ctr->flags, F_OVF_PAIRS);
+        if (threadIdx.x == 0) {
+            // the offsets wrap past 2^32, the frame's count does not.  A tile's own total wraps
+            // only at 2^32 itself (4096 entries of 2^20 slots each)
+            atomicAdd(&ctr->n_cand, total ? (unsigned long long)total : 1ull << 32);
+            if (tile == ntiles - 1) off[n_vis] = s_prefix + total;
         }
         __syncthreads();
     }
@@ -131,8 +131,17 @@ __global__ void __launch_bounds__(EM_THREADS, 4) k_emit(const uint32_t* __restri
     __shared__ uint32_t s_cnt[256];   // the chunk's kept slots by first digit
     const uint32_t lane = lane_id(), warp = threadIdx.x >> 5, D = 1u << bits;
     const uint32_t n_vis = min(ctr->n_vis, cap_vis);
+    // Slots that do not fit their buffers, or 32 bits, may have wrapped offsets, and a
+    // slot scan that timed out leaves wrong ones: the owners then do not ascend, so
+    // nothing is read through them.  Such a frame is replayed or refused.
     const uint64_t cand = ctr->n_cand;
-    const uint32_t ns = (uint32_t)(cand < cap ? cand : cap);
+    const bool timed_out = (ctr->flags & F_SPIN_TIMEOUT) != 0u;
+    if (cand > cap || cand >= 0xFFFFFFFFull || timed_out) {
+        if (blockIdx.x == 0 && threadIdx.x == 0 && !timed_out) atomicOr(&ctr->flags, F_OVF_PAIRS);
+        return;
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) ctr->n_slots = cand;
+    const uint32_t ns = (uint32_t)cand;
     const uint32_t nchunks = n_vis ? (ns + EM_SLOTS - 1u) / EM_SLOTS : 0u;
     const uint32_t TW = fp->tiles_x;
     const int T = (int)fp->tile;

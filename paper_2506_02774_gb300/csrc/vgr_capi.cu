@@ -1077,7 +1077,7 @@ uint32_t enqueue_frame(vgr_view* v, int lod, bool radix_depth, int tile_passes, 
     for (int p = 0; p < plan.passes; ++p) {
         const int bits = p + 1 == plan.passes ? plan.last_bits : plan.bits, shift = plan.bits * p;
         const bool last = p + 1 == plan.passes;
-        const unsigned long long* n = p == 0 ? &v->ctr->n_cand : &v->ctr->n_pairs;
+        const unsigned long long* n = p == 0 ? &v->ctr->n_slots : &v->ctr->n_pairs;
         const int grid = radix_grid(v->h->num_sms);
         if (p > 0) {
             tab.groups = v->tile_groups + tile_group_words(v->cap_pairs, p, plan.bits);

@@ -128,6 +128,7 @@ struct Counters {
     unsigned long long nodes_eval;
     unsigned long long pix_evals;
     unsigned long long pix_contribs;
+    unsigned long long n_slots;  // slots the emission has written: n_cand, or 0 where they do not fit
     uint32_t tickets[TK_COUNT];
     uint32_t frontier_n[MAX_TREE_DEPTH + 2];
     uint32_t tile_buckets[33];  // tiles per log2(pairs + 1) class (the blend order)
