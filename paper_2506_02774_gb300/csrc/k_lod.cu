@@ -101,7 +101,8 @@ struct CutOut {
         if (visible(n, c, lmax[n]) && !(atomicOr(&front_bm[n >> 5], bit) & bit)) fresh |= 1u << 16;
         if (fresh) atomicAdd(&counts[n / CC_TILE_IDS * CC_COUNT_STRIDE], fresh);
     }
-    // a node that only this thread reports; its counts are held back in
+    // a node that only this thread reports (unless the previous cut held one of
+    // its ancestors as well: see k_cut_compact); its counts are held back in
     // (tile, held) while the thread stays in one tile (a subtree's nodes do)
     __device__ __forceinline__ void add(uint32_t n, float4 c, uint32_t& tile, uint32_t& held) const {
         const uint32_t bit = 1u << (n & 31u);
@@ -513,7 +514,13 @@ __global__ void __launch_bounds__(256) k_lod_level(int level, const uint32_t* __
 // Bitmaps -> ascending id lists (the cut, and its in-front part), clearing
 // both bitmaps for the next frame.  The LoD kernels count the bits they set per
 // tile of 256 words, so a tile's place in the lists is the sum of the counts
-// before it: no count is waited for, and the CTAs take tiles in any order.  A
+// before it: no count is waited for, and the CTAs take tiles in any order.  The
+// counts are the bits' as long as every node is reported once.  Where the test is
+// not monotone, an update can leave a node and its descendant in the cut without
+// any of its tests showing it, and the next update then reports nodes twice; so a
+// tile checks its count against its bits, and where they differ F_LOD_FALLBACK has
+// the host replay the frame from the root (one word per tile; until then the lists
+// hold some earlier frame's ids in places, all of them nodes).  A
 // warp takes a row of 32 words: a scan of their bit counts gives every word its
 // place, and the warp goes through the words that have bits, lane l storing the
 // id of bit l if it is set (contiguous stores, no barrier, no staging).  Bound by
@@ -573,6 +580,7 @@ __global__ void __launch_bounds__(CC_THREADS) k_cut_compact(uint32_t* __restrict
     for (uint32_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x, flip ^= 1u) {
         const uint32_t wi = tile * CC_TILE_WORDS + t;
         const uint32_t a = bitmap[wi], b = front[wi];
+        const uint32_t said = t == 0 ? counts[tile * CC_COUNT_STRIDE] : 0u;
         uint32_t sa = 0, sb = 0;
         for (uint32_t j = seen + t; j < tile; j += CC_THREADS) {
             const uint32_t c = counts[j * CC_COUNT_STRIDE];
@@ -596,6 +604,7 @@ __global__ void __launch_bounds__(CC_THREADS) k_cut_compact(uint32_t* __restrict
         cc_row(b, ob + (pre >> 16), id0, front_list, cap, s_row[warp]);
         if (a) bitmap[wi] = 0u;
         if (b) front[wi] = 0u;
+        if (t == 0 && said != total) atomicOr(&ctr->flags, F_LOD_FALLBACK);  // a node was reported twice
         if (tile == ntiles - 1 && t == 0) {
             const uint32_t n = oa + (total & 0xFFFFu);
             *n_cut_out = n;

@@ -37,7 +37,7 @@ constexpr int DEPTH_BINS = 6144;              // bins of the depth keys' histogr
 
 // flags in Counters::flags
 enum : uint32_t {
-    F_LOD_FALLBACK = 1u,   // a thread exceeded its expansion budget: redo the cut top-down
+    F_LOD_FALLBACK = 1u,   // an expansion exceeded its budget, or a node was reported twice: redo the cut top-down
     F_NONMONOTONE = 2u,    // child expands while the parent does not
     F_SPIN_TIMEOUT = 4u,   // a look-back wait ran out
     F_OVF_CUT = 8u,
