@@ -969,7 +969,9 @@ __global__ void __launch_bounds__(BL_THREADS, BL_MIN_CTAS) k_blend_wide(const Fr
                 float aa[G], ab[G];
 #pragma unroll
                 for (int g = 0; g < G; ++g) at[g] = next_slot<DEPTH>(mm, 0);
-                // a pixel outside a record's box fails Eq. 4, so both pixels look at the record
+                // a record that only the neighbour's reach holds is not this pixel's, whatever
+                // its rho: outside the box Eq. 4 fails, but the rounding of rho can pass it for
+                // Gaussians hundreds of pixels long and one wide (a pixel that is done reaches none)
 #pragma unroll
                 for (int g = 0; g < G; ++g) {
                     const float4 X = wY[at[g]];
@@ -977,8 +979,9 @@ __global__ void __launch_bounds__(BL_THREADS, BL_MIN_CTAS) k_blend_wide(const Fr
                     const float rho_a = fmaf(fmaf(X.y, da, X.z), da, X.w), rho_b = fmaf(fmaf(X.y, db, X.z), db, X.w);
                     aa[g] = fminf(ALPHA_MAX, ex2_approx(rho_a));
                     ab[g] = fminf(ALPHA_MAX, ex2_approx(rho_b));
-                    ua[g] = !(rho_a < LOG2_ALPHA_MIN) && !done_a;
-                    ub[g] = !(rho_b < LOG2_ALPHA_MIN) && !done_b;
+                    const uint32_t bit = 0x80000000u >> (at[g] & 31u);  // (slot DEPTH passes at no rho)
+                    ua[g] = !(rho_a < LOG2_ALPHA_MIN) && (reach_a & bit) != 0u;
+                    ub[g] = !(rho_b < LOG2_ALPHA_MIN) && (reach_b & bit) != 0u;
                 }
                 float ta[G], tb[G], Na = Ta, Nb = Tb;
 #pragma unroll
