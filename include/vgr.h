@@ -181,7 +181,11 @@ typedef struct {
  * Device pointers of the intermediate buffers of the last frame (testing).
  * Per-Gaussian arrays are indexed like the in-front list (cut nodes in front
  * of the near plane, ascending node id); entries culled later have
- * vis_ntile = 0 and the depth key 0xFFFFFFFF.
+ * vis_ntile = 0 and the depth key 0xFFFFFFFF.  The records (vis_rect, vis_recA,
+ * vis_recB, vis_rgb) and pair_tile are made by vgr_view_debug, in buffers that it
+ * allocates on first use (VGR_E_NOMEM) and fills again at each call.  A view
+ * whose buffers could not be grown (VGR_E_NOMEM from a frame) has lost some of
+ * them: their arrays are null.
  */
 typedef struct {
     uint32_t n_cut, n_front, n_visible;

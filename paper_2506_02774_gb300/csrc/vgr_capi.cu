@@ -1761,16 +1761,19 @@ vgr_status vgr_view_debug(vgr_view* v, vgr_debug_buffers* o) {
     // the records as separate arrays, made here (the frame keeps them in one 32-byte sector each)
     vgr_status s = VGR_OK;
     VGR_CK(cudaSetDevice(v->h->device));
-    if (!v->dbg_rgb &&
+    // (a view whose buffers could not be grown has lost some: those stay null)
+    const bool records = v->vis.rec && v->vis.rgb && v->vis.ntile, tiles = v->ranges != nullptr;
+    if (records && !v->dbg_rgb &&
         ((s = dalloc(&v->dbg_rect, v->cap_vis, nullptr)) || (s = dalloc(&v->dbg_recA, v->cap_vis, nullptr)) ||
          (s = dalloc(&v->dbg_recB, v->cap_vis, nullptr)) || (s = dalloc(&v->dbg_rgb, v->cap_vis, nullptr)))) {
         dfree(v->dbg_rect); dfree(v->dbg_recA); dfree(v->dbg_recB); dfree(v->dbg_rgb);
         return s;
     }
-    if (!v->dbg_tile && (s = dalloc(&v->dbg_tile, v->cap_pairs, nullptr))) return s;
-    launch_debug_tiles(v->ranges, v->last_tw * v->last_th, v->dbg_tile, v->last_n_pairs, v->stream);
-    launch_debug_records(v->vis, std::min(v->last_n_front, v->cap_vis), v->dbg_rect, v->dbg_recA, v->dbg_recB,
-                         v->dbg_rgb, v->stream);
+    if (tiles && !v->dbg_tile && (s = dalloc(&v->dbg_tile, v->cap_pairs, nullptr))) return s;
+    if (tiles) launch_debug_tiles(v->ranges, v->last_tw * v->last_th, v->dbg_tile, v->last_n_pairs, v->stream);
+    if (records)
+        launch_debug_records(v->vis, std::min(v->last_n_front, v->cap_vis), v->dbg_rect, v->dbg_recA, v->dbg_recB,
+                             v->dbg_rgb, v->stream);
     VGR_CK(cudaGetLastError());
     VGR_CK(cudaStreamSynchronize(v->stream));
     o->vis_rect = reinterpret_cast<const uint32_t*>(v->dbg_rect);
@@ -1778,7 +1781,7 @@ vgr_status vgr_view_debug(vgr_view* v, vgr_debug_buffers* o) {
     o->vis_recB = reinterpret_cast<const float*>(v->dbg_recB);
     o->vis_rgb = reinterpret_cast<const float*>(v->dbg_rgb);
     o->depth_order = v->sortV[1];
-    o->pair_tile = v->dbg_tile;
+    o->pair_tile = tiles ? v->dbg_tile : nullptr;
     o->pair_val = v->pairV[v->last_tile_buf];
     o->tile_range = reinterpret_cast<const uint32_t*>(v->ranges);
     o->tile_size = tile_of(v);
