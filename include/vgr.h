@@ -195,12 +195,14 @@ typedef struct {
     const uint32_t* vis_node;     /* [n_front] node id */
     const uint32_t* vis_depth;    /* [n_front] FP32 depth key bits (0xFFFFFFFF if culled) */
     const uint32_t* vis_ntile;    /* [n_front] candidate tiles (area of vis_rect), 0 if culled */
-    const uint32_t* vis_rect;     /* [2 n_front] candidate tiles: x0 | y0 << 16, x1 | y1 << 16 */
+    const uint32_t* vis_rect;     /* [2 n_front] candidate tiles: x0 | y0 << 16, x1 | y1 << 16 (this and the three
+                                     below: visible entries only, zeros for the others) */
     const float* vis_recA;        /* [4 n_front] u v A B, rho = A dx^2 + B dx dy + C dy^2 */
     const float* vis_recB;        /* [4 n_front] C thr theta h, thr = ln alpha* - ln theta, h = the footprint box's
                                      half-height | half-width << 16 as FP16 bits (rounded up) */
-    const float* vis_rgb;         /* [4 n_front] r g b 0 (visible entries only) */
-    const uint32_t* depth_order;  /* [n_front] in-front index by depth rank; the first n_visible are visible */
+    const float* vis_rgb;         /* [4 n_front] r g b 0 */
+    const uint32_t* depth_order;  /* [n_front] in-front index by depth rank; the first n_visible are visible, the
+                                     others ascend */
     const uint32_t* pair_tile;    /* [n_pairs] tile id, sorted */
     const uint32_t* pair_val;     /* [n_pairs] in-front index << 8 | row mask (bit w: the footprint box reaches
                                      one of the tile's pixel rows w r .. w r + r - 1, r = max(1, tile_size / 8);

@@ -350,12 +350,16 @@ void launch_preprocess(const SceneDev& sc, const uint32_t* front, const uint32_t
 #undef VGR_PRE_LAUNCH
 }
 
-// The visible entries' records as separate arrays (the debug view's layout).
+// The visible entries' records as separate arrays (the debug view's layout), zeros for the others.
 __global__ void k_debug_records(VisBuffers vis, uint32_t n, uint2* __restrict__ rect, float4* __restrict__ recA,
                                 float4* __restrict__ recB, float4* __restrict__ rgb) {
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const uint32_t c = vis.ntile[i];
-        if (c == 0u) continue;
+        if (c == 0u) {
+            rect[i] = make_uint2(0u, 0u);
+            recA[i] = recB[i] = rgb[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+            continue;
+        }
         const float4 a = vis.rec[2 * (size_t)i], b = vis.rec[2 * (size_t)i + 1], col = vis.rgb[i];
         const uint32_t rc = __float_as_uint(b.z);
         const uint32_t x0 = rc & 0x3FFu, y0 = (rc >> 10) & 0x3FFu, w = rc >> 20;
@@ -364,6 +368,27 @@ __global__ void k_debug_records(VisBuffers vis, uint32_t n, uint2* __restrict__ 
         recB[i] = make_float4(b.x, b.y, col.w, b.w);
         rgb[i] = make_float4(col.x, col.y, col.z, 0.f);
     }
+}
+
+// The culled entries behind the n_vis visible ones in the depth order, ascending
+// (their keys are all equal); one CTA.
+__global__ void __launch_bounds__(1024) k_debug_culled(const uint32_t* __restrict__ ntile, uint32_t n, uint32_t n_vis,
+                                                       uint32_t* __restrict__ order) {
+    __shared__ uint32_t s_scan[32];
+    uint32_t at = n_vis;
+    for (uint32_t i0 = 0; i0 < n; i0 += 1024u) {
+        const uint32_t i = i0 + threadIdx.x;
+        const bool culled = i < n && ntile[i] == 0u;
+        uint32_t total;
+        const uint32_t pos = at + block_excl_scan<32>(culled ? 1u : 0u, s_scan, &total);
+        if (culled && pos < n) order[pos] = i;
+        at += total;
+        __syncthreads();  // s_scan is used again
+    }
+}
+
+void launch_debug_culled(const VisBuffers& vis, uint32_t n, uint32_t n_vis, uint32_t* order, cudaStream_t s) {
+    if (n) k_debug_culled<<<1, 1024, 0, s>>>(vis.ntile, n, n_vis, order);
 }
 
 void launch_debug_records(const VisBuffers& vis, uint32_t n, uint2* rect, float4* recA, float4* recB, float4* rgb,

@@ -1771,9 +1771,11 @@ vgr_status vgr_view_debug(vgr_view* v, vgr_debug_buffers* o) {
     }
     if (tiles && !v->dbg_tile && (s = dalloc(&v->dbg_tile, v->cap_pairs, nullptr))) return s;
     if (tiles) launch_debug_tiles(v->ranges, v->last_tw * v->last_th, v->dbg_tile, v->last_n_pairs, v->stream);
-    if (records)
-        launch_debug_records(v->vis, std::min(v->last_n_front, v->cap_vis), v->dbg_rect, v->dbg_recA, v->dbg_recB,
-                             v->dbg_rgb, v->stream);
+    if (records) {
+        const uint32_t n = std::min(v->last_n_front, v->cap_vis);
+        launch_debug_records(v->vis, n, v->dbg_rect, v->dbg_recA, v->dbg_recB, v->dbg_rgb, v->stream);
+        launch_debug_culled(v->vis, n, v->last_n_vis, v->sortV[1], v->stream);
+    }
     VGR_CK(cudaGetLastError());
     VGR_CK(cudaStreamSynchronize(v->stream));
     o->vis_rect = reinterpret_cast<const uint32_t*>(v->dbg_rect);

@@ -103,6 +103,8 @@ void launch_preprocess(const SceneDev& sc, const uint32_t* front, const uint32_t
 // The records of n entries as vgr_debug_buffers lays them out
 void launch_debug_records(const VisBuffers& vis, uint32_t n, uint2* rect, float4* recA, float4* recB, float4* rgb,
                           cudaStream_t s);
+// the culled entries of order[n_vis .. n)
+void launch_debug_culled(const VisBuffers& vis, uint32_t n, uint32_t n_vis, uint32_t* order, cudaStream_t s);
 void prepare_scene(float4* covB, uint32_t n, cudaStream_t s);
 void prepare_scene_half(float4* covB, uint32_t n, cudaStream_t s);
 
