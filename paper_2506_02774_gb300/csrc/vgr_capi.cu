@@ -1537,11 +1537,14 @@ vgr_status finish_impl(vgr_view* v, vgr_frame* out) {
         const int cur = v->parity ^ 1;
         const uint32_t n_cut = v->vstate_host->n_cut[cur];
         if (flags & F_SPIN_TIMEOUT) return fail(VGR_E_TIMEOUT, "a look-back wait timed out");
+        // (such a frame's lists hold nodes that no traversal reaches: what they overflow
+        // counts only after the replay)
         const bool by_level = q.scratch && (flags & F_NONMONOTONE) && frame_lod(v, q) == LOD_DENSE;
         if ((flags & F_NONMONOTONE) && !by_level)
             return fail(VGR_E_NONMONOTONE, "granularity test not monotone: a child expands while its parent does not");
         if (flags & F_OVF_FRONTIER) return fail(VGR_E_OVERFLOW, "frontier overflow");
-        if (flags & F_OVF_VIS) return fail(VGR_E_OVERFLOW, "more than 2^24 cut nodes in front of the camera in one frame");
+        if ((flags & F_OVF_VIS) && !by_level)
+            return fail(VGR_E_OVERFLOW, "more than 2^24 cut nodes in front of the camera in one frame");
         bool again = false;
         if (by_level) {
             v->lod_levels = true;

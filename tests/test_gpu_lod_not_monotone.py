@@ -82,3 +82,27 @@ def test_lists_after_a_missed_frame(kw, graph):
         np.testing.assert_array_equal(v.debug()["vis_node"], ref.debug()["vis_node"])
         assert torch.equal(r.image(), s.image())
     v.close(); ref.close(); h.close()
+
+
+def test_nodes_that_no_traversal_reaches_overflow_nothing():
+    """A tree whose cut is one node, with 2^24 leaves behind a child that expands while
+    its parent does not: the pass over the nodes lists them all, more than a frame may
+    have in front of the camera, and the traversal that follows finds the cut."""
+    kids = [1, 1] + [8] * sum(8 ** k for k in range(8)) + [0] * 8 ** 8  # root, A, then an octree under B
+    n = len(kids)
+    kids = np.array(kids, np.uint8)
+    first = np.where(kids > 0, 1 + np.cumsum(kids, dtype=np.int64) - kids, 0).astype(np.uint32)
+    parent = np.concatenate([[0xFFFFFFFF], np.repeat(np.arange(n, dtype=np.uint32), kids)]).astype(np.uint32)
+    x = np.full(n, 9.99999, np.float32)
+    x[:2] = 19.99999
+    r2 = np.where(kids > 0, np.float32(100.0), np.float32(1e-4)).astype(np.float32)
+    r2[0], r2[1] = 100.0 ** 2, np.float32(19.999985 ** 2)
+    sc = dict(n_nodes=n, sh_degree=0, parent=parent, first_child=first, n_child=kids,
+              mean=np.stack([x, 0 * x, 0 * x], 1), cov6=np.tile(np.array([1e-3, 0, 0, 1e-3, 0, 1e-3], np.float32), (n, 1)),
+              opacity=np.full(n, 0.8, np.float32), sh=np.zeros((n, 1, 3), np.float32), radius2=r2, max_depth=10)
+    h = vgr.Hierarchy(sc)
+    v = vgr.View(h)
+    r = v.render(scenegen.camera((0.0, 0.0, 0.0), 0.0, 64, 48, 64.0), 64.0)
+    assert r.cut().cpu().tolist() == [1] and r.stats["front_count"] == 1
+    assert r.stats["replays"] == 1 and r.stats["lod_from_scratch"] == 1
+    v.close(); h.close()
