@@ -6,8 +6,8 @@
 // pair (key, index) is unique, so no step needs to be stable and none needs a
 // look-back chain:
 //  * preprocess counts the visible keys in DEPTH_BINS bins of a monotone
-//    function of the key (half of the bins logarithmic in z, half linear, over
-//    the depth range the scene's bounds allow: depth_bin);
+//    function of the key (half of the bins logarithmic in z over the depths the
+//    scene's bounds allow, half linear over those of its middle: depth_bin);
 //  * k_depth_part scans the bins (every CTA for itself), joins neighbouring
 //    bins into buckets of about s keys (bucket of a bin = its exclusive prefix
 //    / s, so no bucket holds more than s + its largest bin), and
@@ -28,7 +28,9 @@
 // 96 -> 26 us; city at 1080p (2.67M visible): 153 -> 60 us.  Bound now by the
 // shared-memory atomics and barriers of a CTA's steps (issue slots 35-50 %).
 // A bucket that does not fit a CTA (F_SORT_SKEW: thousands of Gaussians in one
-// bin) makes the host replay the frame with the radix passes of k_sort.cu.
+// bin) makes the host replay the frame with the radix passes of k_sort.cu, and
+// order the view's next 63 frames by them: 82 us for 536K visible (26 here), 130 for
+// 2M (47); the look-back passes of before took 74 and 98.
 #include <algorithm>
 
 #include "vgr_internal.cuh"

@@ -69,12 +69,14 @@ __device__ __forceinline__ uint32_t pack_rect(int x0, int y0, int x1) {
 }
 
 // Monotone map from depth keys to bins: half of the bins logarithmic in z
-// (the key's bits rise like log2 z), half linear, over the depths the scene's
-// bounds allow; keys outside go to the first or last bin.
+// (the key's bits rise like log2 z) over the depths the scene's bounds allow, half
+// linear over the depths of its middle, so that a few nodes far outside take no
+// bins from the others; keys outside go to the first or last bin.
 struct DepthMap {
-    uint32_t key_lo;   // bits of z_lo
-    float z_lo;
+    uint32_t key_lo;     // bits of the logarithmic half's first depth
+    float z_lin;         // first depth of the linear half
     float c_log, c_lin;  // bins per unit of key and of z
+    float lin_max;       // bins of the linear half
 };
 
 // Per-frame parameters, uploaded once per frame (a graph replays them).
@@ -280,8 +282,8 @@ __device__ __forceinline__ float depth_key(float4 m, float R6, float R7, float R
 // same bin.
 __device__ __forceinline__ float depth_coord(const DepthMap& m, uint32_t key) {
     const float a = __fmul_rn(__uint2float_rn(key > m.key_lo ? key - m.key_lo : 0u), m.c_log);
-    const float b = __fmul_rn(fmaxf(__fsub_rn(__uint_as_float(key), m.z_lo), 0.f), m.c_lin);
-    return __fadd_rn(a, b);
+    const float b = __fmul_rn(fmaxf(__fsub_rn(__uint_as_float(key), m.z_lin), 0.f), m.c_lin);
+    return __fadd_rn(a, fminf(b, m.lin_max));
 }
 __device__ __forceinline__ uint32_t depth_bin(const DepthMap& m, uint32_t key) {
     return min(__float2uint_rz(depth_coord(m, key)), (uint32_t)DEPTH_BINS - 1u);
