@@ -54,6 +54,8 @@
 // tiles), 81 to 48 and 56 (640 x 360 and 320 x 180 city views), 312 to 208
 // (canonical mode, 960 x 540); that mode's pass over the staged records in order
 // took it to 143.
+#include <atomic>
+
 #include "vgr_internal.cuh"
 #include "vgr_launch.h"
 
@@ -1112,11 +1114,14 @@ bool blend_wide(uint32_t filter, uint32_t exp_mode, uint32_t depth, uint32_t til
 template <int DEPTH, int T>
 void launch_blend_wide(const FrameParams* fp0, const FrameParams* const* fps, const uint32_t* work, uint32_t n_work,
                        const uint32_t* n_heavy, uint32_t* next, uint32_t* done, uint32_t n_views, int sms, cudaStream_t s) {
-    static int ctas = 0;  // resident CTAs per SM, queried once
+    // resident CTAs per SM, queried once (or by each of the threads that come first: the
+    // answer is the same, on every device that the library runs on)
+    static std::atomic<int> cached{0};
+    int ctas = cached.load(std::memory_order_relaxed);
     if (!ctas) {
-        int n = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_blend_wide<DEPTH, T>, BL_THREADS, 0);
-        ctas = n > 0 ? n : 1;
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas, k_blend_wide<DEPTH, T>, BL_THREADS, 0);
+        ctas = ctas > 0 ? ctas : 1;
+        cached.store(ctas, std::memory_order_relaxed);
     }
     launch_k(k_blend_wide<DEPTH, T>, sms * ctas, BL_THREADS, s, fp0, fps, work, n_work, n_heavy, next, done, n_views);
 }
@@ -1141,12 +1146,12 @@ int occupancy() {
 }
 
 static int blend_ctas_per_sm(uint32_t filter, uint32_t exp_mode, uint32_t depth, uint32_t tile) {
-    // [mode][depth][tile], queried once each
-    static int cache[3][3][3] = {};
+    // [mode][depth][tile], queried once each (as in launch_blend_wide)
+    static std::atomic<int> cache[3][3][3] = {};
     const int md = filter == VGR_FILTER_CANONICAL ? 1 : exp_mode == VGR_EXP_LUT ? 2 : 0;
     const int d = md != 0 ? 1 : depth == 16 ? 0 : (depth == 48 && tile != 8) ? 2 : 1;
     const int t = tile == 8 ? 0 : tile == 32 ? 2 : 1;
-    int& c = cache[md][d][t];
+    int c = cache[md][d][t].load(std::memory_order_relaxed);
     if (!c) {
         switch (md * 9 + d * 3 + t) {
             case 0: c = occupancy<0, 16, 8>(); break;
@@ -1165,6 +1170,7 @@ static int blend_ctas_per_sm(uint32_t filter, uint32_t exp_mode, uint32_t depth,
             case 23: c = occupancy<2, 32, 32>(); break;
             default: c = 1; break;
         }
+        cache[md][d][t].store(c, std::memory_order_relaxed);
     }
     return c;
 }
