@@ -180,8 +180,9 @@ def _frame_bytes(sc: dict, st: dict, W: int, H: int, tile_passes: int) -> dict:
         depth_sort=4 * F + 24 * V,                   # keys; (key, index) partitioned; order, slot offsets
         color=0,                                     # evaluated in preprocess
         emit=(4 + 4 + 32) * V + 8 * P0,              # order, slot offset, record; slots
-        tile_sort=tile_passes * 2 * 8 * P0,
-        ranges=4 * P + 8 * (W // 16 + 1) * (H // 16 + 1),
+        # slots in, the kept pairs out; they pass through every further digit; the last writes no keys
+        tile_sort=8 * P0 + 8 * P + (tile_passes - 1) * 16 * P - 4 * P,
+        ranges=16 * ((W + 15) // 16) * ((H + 15) // 16),  # each tile's range read and written
         blend=(4 + 48) * P + 12 * W * H,
     )
 
@@ -198,7 +199,8 @@ def frame_roofline(fb: dict, stage_ms: dict, frame_ms: float, hbm_gbs: float) ->
                 frac=round(roof_ms / frame_ms, 4), stage_frac=per_stage)
 
 
-def blend_roofline(mean: dict, blend_ms: float, sms: int, peaks: dict, blend_bytes: float, blend_gbs: float) -> dict:
+def blend_roofline(mean: dict, blend_ms: float, sms: int, peaks: dict, blend_bytes: float, blend_gbs: float,
+                   wide: bool) -> dict:
     """The blend (the kernel with the largest share of the frame) against its
     plain-ALU roofline: FP32 lane-instructions the method needs per evaluated
     pixel-pair (dx, dy, rho, Eq. 4 test) and per blended one (exp argument,
@@ -209,7 +211,7 @@ def blend_roofline(mean: dict, blend_ms: float, sms: int, peaks: dict, blend_byt
     t = blend_ms * 1e-3
     peak_t = sms * 128 * peaks["sm_max_mhz"] * 1e6 / 1e12
     units = mean["pair_count"]
-    return dict(bound="alu", stage="blend", kernel="k_blend", achieved=round(ops / t / 1e12, 3),
+    return dict(bound="alu", stage="blend", kernel="k_blend_wide" if wide else "k_blend", achieved=round(ops / t / 1e12, 3),
                 peak=round(peak_t, 2), unit="TFLOP/s", frac=round(ops / t / 1e12 / peak_t, 4),
                 traffic=_traffic("k_blend", "k_blend.cu", units),
                 peak_source="%d SMs x 128 FP32 lanes x %.0f MHz (sm_max_mhz, %s), one op per FP32 "
@@ -555,7 +557,9 @@ def run_ours(args) -> dict:
     shares = {s: float(stage_ms[i]) for i, s in enumerate(vgr.STAGES)}
     hbm_stages = {s: fb[s] / (shares[s] * 1e-3) / 1e9 for s in vgr.STAGES if shares[s] > 0}
     sms = torch.cuda.get_device_properties(dev).multi_processor_count
-    roof_blend = blend_roofline(mean, shares["blend"], sms, peaks, fb["blend"], hbm_stages.get("blend", 0.0))
+    # two pixels per lane where the frame has 32-pixel strips for every resident warp twice over (k_blend.cu)
+    roof_blend = blend_roofline(mean, shares["blend"], sms, peaks, fb["blend"], hbm_stages.get("blend", 0.0),
+                                wide=n_tiles * 8 >= 2 * sms * 4 * 8)
     roof_pre = hbm_roofline("preprocess", "k_preprocess", "k_preprocess.cu", fb["preprocess"], shares["preprocess"],
                             peaks, mean["front_count"])
     out = dict(metric=METRIC, value=round(value, 2), unit="frames/s", n_gpus=ws, steps=args.steps,
