@@ -118,8 +118,9 @@ typedef struct {
     uint64_t cut_capacity;   /* initial capacities; 0 = automatic.  Grown on demand. */
     uint64_t pair_capacity;
     uint32_t lod_budget;     /* max nodes one thread explores when expanding a cut node (0 = 4096) */
-    uint32_t grid_wide;      /* CTAs of the grid-stride kernels (LoD, preprocess with colour, ranges);
-                                0 = 8 per SM.  Launch geometry only: results do not depend on it. */
+    uint32_t grid_wide;      /* CTAs of the LoD update and the level kernels; the pass over the nodes takes
+                                at most 4 per SM of them and preprocess (with colour) at most 2; 0 = 8 per
+                                SM.  Launch geometry only: results do not depend on it. */
     uint32_t grid_scan;      /* CTAs of the compaction and the emission (and of the slot scan after a
                                 radix depth sort); 0 = 4 per SM.  Launch geometry only. */
     uint32_t test_hooks;     /* 0 in normal use.  VGR_HOOK_WITHHOLD_LOOKBACK: depths are ordered by radix
@@ -140,12 +141,14 @@ typedef struct {
 } vgr_view_opts;
 
 enum { VGR_HOOK_WITHHOLD_LOOKBACK = 1,
-       VGR_HOOK_LOD_LEVELS = 8,      /* a cut without a previous one is found level by level, as in trees too
-                                        large for one pass over the nodes (same cut) */
+       VGR_HOOK_FULL_STRIP_WALK = 2, /* the blend walks every record of a strip at every pixel instead of only
+                                        the records whose footprint box covers the pixel (same image, but for
+                                        Gaussians so long and thin that the rounding of their exponent
+                                        passes the alpha* test outside the box) */
        VGR_HOOK_RADIX_DEPTH = 4,     /* order the depths by radix passes, as a frame does whose depths are too
                                         concentrated for the partition (same order) */
-       VGR_HOOK_FULL_STRIP_WALK = 2  /* the blend walks every record of a strip at every pixel instead of only
-                                        the records whose footprint box covers the pixel (same image) */ };
+       VGR_HOOK_LOD_LEVELS = 8       /* a cut without a previous one is found level by level, as a coarse one
+                                        in a very large tree is (same cut) */ };
 
 /* Stages of stage_ms.  The colour (SH -> RGB) is evaluated by the preprocess
  * kernel, so VGR_STAGE_PREPROCESS includes it and VGR_STAGE_COLOR stays

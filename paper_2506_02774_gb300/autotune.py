@@ -19,7 +19,7 @@ import os
 
 from . import View
 
-GRID_WIDE_PER_SM = (2, 4, 8, 16)   # grid-stride kernels: LoD, preprocess (with colour), ranges
+GRID_WIDE_PER_SM = (2, 4, 8, 16)   # LoD update (from scratch at most 4, preprocess at most 2 of them)
 GRID_SCAN_PER_SM = (2, 3, 4, 6)    # compaction, emission
 BLEND_DEPTHS = (16, 32, 48)        # Gaussians a blend warp stages per chunk
 BATCH_CHAINS = (0, 1, 2, 3, 4, 8)  # views of a batch running at once (0: all)

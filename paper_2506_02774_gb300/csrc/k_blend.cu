@@ -406,12 +406,14 @@ __device__ __forceinline__ uint32_t pair_range(int p0, int p1) {
 // B / row terms][warp][slot]; ring: the warp's queue of hit pair values (at a
 // strip's end its pixels); pm: the staged records' pixel masks.
 template <int MODE, int DEPTH, int T>
-__device__ __forceinline__ void blend_strips(float4 (*sbuf)[2 + (32 / T > 2 ? 2 : 1)][BL_WARPS][DEPTH + 1], uint32_t* ring,
+__device__ __forceinline__ void blend_strips(float4 (*sbuf)[2 + (32 / T > 2 ? 2 : 1)][BL_WARPS][DEPTH + 1],
+                                             uint32_t* ring,
                                              uint32_t* pm, volatile WarpItem& it, ClaimRing& claims,
                                              const FrameParams* __restrict__ fp0,
                                              const FrameParams* const* __restrict__ fps,
                                              const uint32_t* __restrict__ work, uint32_t n_work, uint32_t* next,
-                                             uint32_t first, uint32_t base, const float* s_lut, uint32_t m, float lut_scale, bool full_walk) {
+                                             uint32_t first, uint32_t base, const float* s_lut, uint32_t m,
+                                             float lut_scale, bool full_walk) {
     constexpr int SR = 32 / T;                    // rows per strip
     constexpr int NS = T * T / 32;                // strips per tile
     constexpr int MR = T >= 8 ? T / 8 : 1;        // rows per mask bit
@@ -754,7 +756,8 @@ __global__ void __launch_bounds__(BL_THREADS, bl_narrow_ctas(T)) k_blend(const F
     }
     __syncthreads();
     blend_strips<MODE, DEPTH, T>(sbuf, s_ring[warp], s_pm[warp], s_item[warp], s_claims, fp0, fps, work, n_work, next,
-                                 blockIdx.x, gridDim.x, s_lut, m, lut_scale, (fp0->test_hooks & VGR_HOOK_FULL_STRIP_WALK) != 0u);
+                                 blockIdx.x, gridDim.x, s_lut, m, lut_scale,
+                                 (fp0->test_hooks & VGR_HOOK_FULL_STRIP_WALK) != 0u);
     if (lane == 0) flush_item(s_item[warp]);
     finish_blend(done, fp0, fps, n_views);
 }
@@ -918,8 +921,10 @@ __global__ void __launch_bounds__(BL_THREADS, BL_MIN_CTAS) k_blend_wide(const Fr
                         const uint32_t hw = __float_as_uint(b.w);
                         const float by = __half2float(__ushort_as_half((unsigned short)(hw & 0xFFFFu))) + 0.01f;
                         const float bx = __half2float(__ushort_as_half((unsigned short)(hw >> 16))) + 0.01f;
-                        const int c0 = max(__float2int_ru(a.x - bx - clo), 0), c1 = min(__float2int_rd(a.x + bx - clo), T - 1);
-                        int r0 = max(__float2int_ru(a.y - by - rlo), 0), r1 = min(__float2int_rd(a.y + by - rlo), SR - 1);
+                        const int c0 = max(__float2int_ru(a.x - bx - clo), 0);
+                        const int c1 = min(__float2int_rd(a.x + bx - clo), T - 1);
+                        int r0 = max(__float2int_ru(a.y - by - rlo), 0);
+                        int r1 = min(__float2int_rd(a.y + by - rlo), SR - 1);
                         if (SB == 2) {  // rows whose mask bit is clear are out of reach
                             if (!(rows & (1u << (SR * strip / MR)))) r0 = max(r0, MR);
                             if (!(rows & (2u << (SR * strip / MR)))) r1 = min(r1, MR - 1);
@@ -1107,13 +1112,15 @@ void launch_blend_t(const FrameParams* fp0, const FrameParams* const* fps, const
 constexpr uint32_t BL_WIDE_ROUNDS = 2;
 
 bool blend_wide(uint32_t filter, uint32_t exp_mode, uint32_t depth, uint32_t tile, uint32_t n_work, int sms) {
-    return filter == VGR_FILTER_PREEMPTIVE && exp_mode == VGR_EXP_EXACT && depth <= 32 && tile >= 16 &&
-           (tile == 32 || (uint64_t)n_work * (tile * tile / 32) >= (uint64_t)BL_WIDE_ROUNDS * sms * BL_MIN_CTAS * BL_WARPS);
+    if (filter != VGR_FILTER_PREEMPTIVE || exp_mode != VGR_EXP_EXACT || depth > 32 || tile < 16) return false;
+    const uint64_t strips = (uint64_t)n_work * (tile * tile / 32);
+    return tile == 32 || strips >= (uint64_t)BL_WIDE_ROUNDS * sms * BL_MIN_CTAS * BL_WARPS;
 }
 
 template <int DEPTH, int T>
 void launch_blend_wide(const FrameParams* fp0, const FrameParams* const* fps, const uint32_t* work, uint32_t n_work,
-                       const uint32_t* n_heavy, uint32_t* next, uint32_t* done, uint32_t n_views, int sms, cudaStream_t s) {
+                       const uint32_t* n_heavy, uint32_t* next, uint32_t* done, uint32_t n_views, int sms,
+                       cudaStream_t s) {
     // resident CTAs per SM, queried once (or by each of the threads that come first: the
     // answer is the same, on every device that the library runs on)
     static std::atomic<int> cached{0};
@@ -1130,11 +1137,13 @@ void launch_blend_wide(const FrameParams* fp0, const FrameParams* const* fps, co
 // table modes at depth 32.
 template <int T>
 void launch_blend_tile(const FrameParams* fp0, const FrameParams* const* fps, const uint32_t* work, uint32_t n_work,
-                       uint32_t* next, uint32_t* done, uint32_t n_views, int grid, uint32_t filter, uint32_t exp_mode, uint32_t depth, cudaStream_t s) {
+                       uint32_t* next, uint32_t* done, uint32_t n_views, int grid, uint32_t filter, uint32_t exp_mode,
+                       uint32_t depth, cudaStream_t s) {
     if (filter == VGR_FILTER_CANONICAL) launch_blend_t<1, 32, T>(fp0, fps, work, n_work, next, done, n_views, grid, s);
     else if (exp_mode == VGR_EXP_LUT) launch_blend_t<2, 32, T>(fp0, fps, work, n_work, next, done, n_views, grid, s);
     else if (depth == 16) launch_blend_t<0, 16, T>(fp0, fps, work, n_work, next, done, n_views, grid, s);
-    else if (depth == 48 && T != 8) launch_blend_t<0, (T != 8 ? 48 : 32), T>(fp0, fps, work, n_work, next, done, n_views, grid, s);
+    else if (depth == 48 && T != 8)
+        launch_blend_t<0, (T != 8 ? 48 : 32), T>(fp0, fps, work, n_work, next, done, n_views, grid, s);
     else launch_blend_t<0, 32, T>(fp0, fps, work, n_work, next, done, n_views, grid, s);
 }
 
@@ -1176,19 +1185,17 @@ static int blend_ctas_per_sm(uint32_t filter, uint32_t exp_mode, uint32_t depth,
 }
 
 void launch_blend(const FrameParams* fp0, const FrameParams* const* fps, const uint32_t* work, uint32_t n_work,
-                  const uint32_t* n_heavy, uint32_t* next, uint32_t* done, uint32_t n_views, int sms, uint32_t filter, uint32_t exp_mode, uint32_t depth, uint32_t tile,
-                  cudaStream_t s) {
+                  const uint32_t* n_heavy, uint32_t* next, uint32_t* done, uint32_t n_views, int sms, uint32_t filter,
+                  uint32_t exp_mode, uint32_t depth, uint32_t tile, cudaStream_t s) {
     if (blend_wide(filter, exp_mode, depth, tile, n_work, sms)) {
-        if (tile == 32 && depth == 16) launch_blend_wide<16, 32>(fp0, fps, work, n_work, n_heavy, next, done, n_views, sms, s);
-        else if (tile == 32) launch_blend_wide<32, 32>(fp0, fps, work, n_work, n_heavy, next, done, n_views, sms, s);
-        else if (depth == 16) launch_blend_wide<16, 16>(fp0, fps, work, n_work, n_heavy, next, done, n_views, sms, s);
-        else launch_blend_wide<32, 16>(fp0, fps, work, n_work, n_heavy, next, done, n_views, sms, s);
+        auto wide = tile == 32 ? (depth == 16 ? launch_blend_wide<16, 32> : launch_blend_wide<32, 32>)
+                               : (depth == 16 ? launch_blend_wide<16, 16> : launch_blend_wide<32, 16>);
+        wide(fp0, fps, work, n_work, n_heavy, next, done, n_views, sms, s);
         return;
     }
     const int grid = sms * blend_ctas_per_sm(filter, exp_mode, depth, tile);
-    if (tile == 8) launch_blend_tile<8>(fp0, fps, work, n_work, next, done, n_views, grid, filter, exp_mode, depth, s);
-    else if (tile == 32) launch_blend_tile<32>(fp0, fps, work, n_work, next, done, n_views, grid, filter, exp_mode, depth, s);
-    else launch_blend_tile<16>(fp0, fps, work, n_work, next, done, n_views, grid, filter, exp_mode, depth, s);
+    auto narrow = tile == 8 ? launch_blend_tile<8> : tile == 32 ? launch_blend_tile<32> : launch_blend_tile<16>;
+    narrow(fp0, fps, work, n_work, next, done, n_views, grid, filter, exp_mode, depth, s);
 }
 
 }  // namespace vgr

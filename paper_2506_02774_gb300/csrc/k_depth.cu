@@ -393,7 +393,8 @@ cudaError_t depth_sort_init() {
 
 void launch_depth_sort(const VisBuffers& vis, uint32_t cap_vis, const uint32_t* bins, uint2* bstart,
                        unsigned long long* cursor, uint2* part, uint32_t* order, uint32_t* slot_off,
-                       uint32_t* owner, uint64_t cap_pairs, Counters* ctr, const FrameParams* fp, int sms, cudaStream_t s) {
+                       uint32_t* owner, uint64_t cap_pairs, Counters* ctr, const FrameParams* fp, int sms,
+                       cudaStream_t s) {
     const uint32_t cap = cap_vis < MAX_RANKS ? cap_vis : MAX_RANKS;
     const uint32_t cb = depth_bucket_cap(cap);
     launch_ks(k_depth_part, 2 * sms, DP_THREADS, depth_part_smem(cb), s, (const uint32_t*)vis.depth,

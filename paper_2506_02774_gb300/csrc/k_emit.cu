@@ -14,9 +14,9 @@
 // the Gaussian's other slots).  Chunks
 // of 512 Gaussians before this left the CTA with the near ones running alone
 // (SM cycles 43 % busy on average) and gathered three half-used sectors each;
-// 1M-leaf box at 1080p (981K slots): 53 -> 21 us, city at 1080p (4.26M slots):
-// 107 -> 61 us; the records of two slots per lane in flight together: city 56 -> 52
-// (all four, in CTAs of 512 threads: 68).  For each slot the tile-level form of
+// 1M-leaf box at 1080p (981K slots): 53 -> 18 us, city at 1080p (4.26M slots):
+// 107 -> 52 us (with the records of two slots per lane in flight together; one: 56,
+// all four, in CTAs of 512 threads: 68).  For each slot the tile-level form of
 // Eq. 4 (paper Sec. 4.2) decides: a kept slot gets key = tile id, a dropped one
 // all ones, which the tile sort's first pass leaves out (the others stay in
 // depth order within a tile, the sort being stable).  The slot's
@@ -285,7 +285,9 @@ __device__ __forceinline__ void cluster_sync() {
 // word *p of the cluster's CTA 'rank'
 __device__ __forceinline__ uint32_t cluster_load(const uint32_t* p, uint32_t rank) {
     uint32_t a, v;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n"
+                 : "=r"(a)
+                 : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
     asm volatile("ld.shared::cluster.u32 %0, [%1];\n" : "=r"(v) : "r"(a) : "memory");
     return v;
 }

@@ -22,11 +22,11 @@
 //    cut node costs one sector and one round instead of waiting for the
 //    parent's id first; the id itself is read only when the node collapses.
 //  * k_lod_dense: the cut without a previous one (frame 0, tau change, reset,
-//    fallback), in one pass over the nodes of trees that are not too large
-//    for it (DENSE_MAX_NODES in vgr_capi.cu).
-//  * k_lod_level: one level of the from-scratch, top-down traversal, for larger
-//    trees and for views whose test turned out not monotone; frontiers are
-//    appended with one atomic per warp after a warp scan of the child counts.
+//    fallback), in one pass over the nodes.
+//  * k_lod_level: one level of the from-scratch, top-down traversal, for coarse
+//    cuts of large trees (DENSE_ANY_NODES in vgr_capi.cu) and for views whose test
+//    turned out not monotone; frontiers are appended with one atomic per warp after
+//    a warp scan of the child counts.
 #include "vgr_internal.cuh"
 #include "vgr_launch.h"
 
@@ -380,7 +380,8 @@ __global__ void __launch_bounds__(256) k_lod_update(const uint32_t* __restrict__
 // expands and it does not, and no level waits for the one above.  A node that
 // expands under a parent that does not raises F_NONMONOTONE, and the host redoes
 // the frame with k_lod_level.  A warp takes runs of 4 bitmap words and stores each
-// from a ballot, with no atomics but one count per run.  Bound by HBM (the 32-byte node-and-parent records in order, 5.6 TB/s of them):
+// from a ballot, with no atomics but one count per run.  Bound by HBM (the 32-byte
+// node-and-parent records in order, 5.6 TB/s of them):
 // 23 us on the 1M-leaf box against 130 for 12 level kernels, 181 us on the city
 // at tau = 3 against 550 for 16 (tau = 24: 153 and 141, 48: 148 and 106).
 constexpr int LOD_DENSE_UNROLL = 4;

@@ -974,8 +974,10 @@ vgr_status vgr_view_bytes_estimate(const vgr_hierarchy* h, const vgr_view_opts* 
                                       4 * radix_group_words(cap_vis, 0, 8));
     const uint32_t T = o.tile_size ? o.tile_size : TILE_DEFAULT;
     const uint64_t tiles = (uint64_t)((width + T - 1) / T) * ((height + T - 1) / T);
-    uint64_t b = 3 * 4 * cap_cut + per_vis * cap_vis + 4 * 4 * cap_pairs + 4 * emit_owner_cap(cap_pairs) + 2 * 4 * n_words + 2 * 4 * N +
-                 cleared_bytes((uint32_t)n_words, MAX_RANKS) + 8 * (depth_bucket_cap(MAX_RANKS) + 1) + sizeof(ViewState) + sizeof(FrameParams) + 260 * 4 + table_bytes;
+    uint64_t b = 3 * 4 * cap_cut + per_vis * cap_vis + 4 * 4 * cap_pairs + 4 * emit_owner_cap(cap_pairs) +
+                 2 * 4 * n_words + 2 * 4 * N + cleared_bytes((uint32_t)n_words, MAX_RANKS) +
+                 8 * (depth_bucket_cap(MAX_RANKS) + 1) + sizeof(ViewState) + sizeof(FrameParams) + 260 * 4 +
+                 table_bytes;
     b += (uint64_t)width * height * 3 * 4 + tiles * (sizeof(uint2) + 4);
     *bytes = (b + (2u << 20) - 1) / (2u << 20) * (2u << 20);  // device memory is handed out in 2 MiB pieces
     return VGR_OK;
@@ -1017,7 +1019,8 @@ int frame_lod(const vgr_view* v, const PendingFrame& q) {
 uint32_t frame_kernels(const vgr_view* v, int lod, bool radix_depth, int tile_passes) {
     return (lod == LOD_LEVELS ? v->h->max_depth + 1u : 1u) + 1u /*compact*/ + 1u /*preprocess, with colour*/ +
            (radix_depth ? 9u /*4 counts, 4 scatters, slot scan*/ : 2u /*partition, buckets*/) + 1u /*emit*/ +
-           2u * (uint32_t)tile_passes - 1u /*counts but the first, scatters*/ + 1u /*begin*/ + 1u /*tile order (finishes the ranges)*/ + 1u /*blend*/;
+           2u * (uint32_t)tile_passes - 1u /*counts but the first, scatters*/ + 1u /*begin*/ +
+           1u /*tile order (finishes the ranges)*/ + 1u /*blend*/;
 }
 
 // Enqueue one frame.  'lod' selects how its cut is found.  'own_blend' false:

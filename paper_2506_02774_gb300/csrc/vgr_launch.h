@@ -115,7 +115,8 @@ uint32_t depth_bucket_cap(uint32_t cap_vis);  // bucket ids a frame of cap_vis e
 cudaError_t depth_sort_init();                // once per device: the kernels' shared-memory limits
 void launch_depth_sort(const VisBuffers& vis, uint32_t cap_vis, const uint32_t* bins, uint2* bstart,
                        unsigned long long* cursor, uint2* part, uint32_t* order, uint32_t* slot_off,
-                       uint32_t* owner, uint64_t cap_pairs, Counters* ctr, const FrameParams* fp, int sms, cudaStream_t s);
+                       uint32_t* owner, uint64_t cap_pairs, Counters* ctr, const FrameParams* fp, int sms,
+                       cudaStream_t s);
 
 // k_sort.cu
 // Tables of one digit pass: digit counts per row (a tile's keys, or a part of
@@ -141,8 +142,8 @@ void launch_radix_scatter(const uint32_t* keys_in, const uint32_t* vals_in, uint
 // k_emit.cu
 // slot offsets in depth order, into slot_off[cap_vis + 1], after a radix depth sort
 void launch_slot_scan(const uint32_t* order, uint32_t cap_vis, const VisBuffers& vis, uint32_t* slot_off,
-                      uint32_t* owner, uint64_t cap_pairs, unsigned long long* status, Counters* ctr, const FrameParams* fp, int grid,
-                      cudaStream_t s);
+                      uint32_t* owner, uint64_t cap_pairs, unsigned long long* status, Counters* ctr,
+                      const FrameParams* fp, int grid, cudaStream_t s);
 uint32_t emit_owner_cap(uint64_t cap_pairs);  // entries of the owner table (first rank of each emission chunk)
 // 'tab' receives the counts of the keys' low 'bits' bits, one row per EMIT_SLOTS slots; dropped slots (key all ones)
 // are not counted
@@ -164,8 +165,8 @@ constexpr uint32_t BATCH_VIEWS_MAX = 1024;  // views of one batch blend (k_batch
 // chunk (16, 32, 48; 48 needs tiles of 16 or 32); tile: 8, 16 or 32 pixels.
 constexpr uint32_t BL_HEAVY_CLASS = 11;  // class floor(log2(pairs + 1)) + 1: 1023 pairs and more
 void launch_blend(const FrameParams* fp0, const FrameParams* const* fps, const uint32_t* work, uint32_t n_work,
-                  const uint32_t* n_heavy, uint32_t* next, uint32_t* done, uint32_t n_views, int sms, uint32_t filter, uint32_t exp_mode, uint32_t depth,
-                  uint32_t tile, cudaStream_t s);
+                  const uint32_t* n_heavy, uint32_t* next, uint32_t* done, uint32_t n_views, int sms, uint32_t filter,
+                  uint32_t exp_mode, uint32_t depth, uint32_t tile, cudaStream_t s);
 // k_emit.cu: the order of a batch's tiles over all its views (heaviest class
 // first), from each view's tile order and class counts
 void launch_batch_order(const FrameParams* const* fps, uint32_t n_views, const uint32_t* const* orders,
