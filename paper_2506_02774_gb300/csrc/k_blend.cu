@@ -49,8 +49,8 @@
 // What bounds it: large images by their instructions (issue slots 75 % busy),
 // small ones by the chunks of the longest strips (a horizon tile's 2000 to 3500
 // hits).  Groups of four records, first tiles dealt out, two pixels per lane and
-// parts of 32-pixel tiles as items of their own took the blend from 110 to 80 us
-// (1M-leaf box, 1080p), 184 to 161 (city, 1080p), 347 to 162 (1440p, 32-pixel
+// parts of 32-pixel tiles as items of their own took the blend from 110 to 81 us
+// (1M-leaf box, 1080p), 184 to 165 (city, 1080p), 347 to 156 (1440p, 32-pixel
 // tiles), 81 to 48 and 56 (640 x 360 and 320 x 180 city views), 312 to 208
 // (canonical mode, 960 x 540); that mode's pass over the staged records in order
 // took it to 143.
@@ -1108,7 +1108,7 @@ void launch_blend_t(const FrameParams* fp0, const FrameParams* const* fps, const
 // and without: 801 x 603 (15.5K strips, 3.2 rounds) 21.7 and 26.4 us, 640 x 360
 // (7.4K, 1.5 rounds; long horizon tiles) 49.5 and 47.6, 320 x 180 (1.9K) 58.2 and
 // 55.7.  Tiles of 32 pixels always: a strip of one row would stage the hits of
-// the four rows of its mask bit (1440p: 162 us, 347 before).
+// the four rows of its mask bit (1440p: 156 us, 347 before).
 constexpr uint32_t BL_WIDE_ROUNDS = 2;
 
 bool blend_wide(uint32_t filter, uint32_t exp_mode, uint32_t depth, uint32_t tile, uint32_t n_work, int sms) {
